@@ -272,7 +272,7 @@ tn_status tn_contract_slices(tn_plan_t* plan, uint64_t slice_first, uint64_t sli
  * and, when kernel_out is not NULL, the kernel used by each step into
  * kernel_out[n_steps]: 0-2 FP32 SIMT tiles (64x64, 128x16, 256x4), then the
  * tcgen05 kernels 3 TF32 4M, 4 BF16x3 4M, 5 TF32 3M, 6 BF16x3 3M, 7 FP16x3 4M,
- * 8 FP16x3 3M.  Used for plan reports and roofline measurements; synchronises
+ * 8 FP16x3 3M, then 9-10 further FP32 SIMT tiles (128x64, 32x32).  Used for plan reports and roofline measurements; synchronises
  * `stream`. */
 tn_status tn_plan_step_times(tn_plan_t* plan, int32_t reps, double* ms_out, int32_t* kernel_out,
                              void* stream);
@@ -282,7 +282,7 @@ tn_status tn_plan_step_times(tn_plan_t* plan, int32_t reps, double* ms_out, int3
  * complex columns in the TF32 / BF16X3 / FP16X3 modes, each with either
  * write-back order, with the default or a deeper ring of B' slots and, where
  * tn_plan_opts.sm_pairs allows, on one SM or on SM pairs, and the
- * three CUDA-core tilings for steps under 50 us, of low arithmetic intensity
+ * CUDA-core tilings for steps under 50 us, of low arithmetic intensity
  * or in the FP32 mode -- each `reps` times, and keeps the fastest for later
  * calls.  Synchronises `stream`; the arena contents are
  * overwritten (the next call recomputes them). */

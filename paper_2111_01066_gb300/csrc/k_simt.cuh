@@ -1,4 +1,5 @@
-// Complex GEMM on the CUDA cores (complex64, FP32 FMA): the plain FP32 path.
+// Complex GEMM on the CUDA cores (complex64, FP32 FMA): the plain FP32 path and
+// the small steps of the tensor-core modes.
 // Operands are gathered straight from their tensors' storage order, so the
 // index permutation of SI Eq. (2) is folded into the loads (the paper's fused
 // permutation-multiplication, SI figure S7a): each tile covers the lowest
@@ -8,203 +9,455 @@
 
 namespace tnx {
 
-// Shared memory of one tile of a tiling.
-template <int TM, int TN, int TK>
-struct SimtSmem {
-  float2 As[TK][TM];
-  float2 Bs[TK][TN];
-  int64_t offCm[TM];
-  int64_t offCn[TN];
-};
-
-// One (m tile bx, n tile by) of a GEMM for instances bz, bz + gz, ... (the
-// body of both kernels below; every thread of the block calls it).
-template <int TM, int TN, int TK, int RM, int RN>
-__device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int bz, int gz,
-                                          SimtSmem<TM, TN, TK>& sm) {
-  constexpr int NTX = TM / RM, NTY = TN / RN, NT = NTX * NTY;
-  constexpr int AE = (TM * TK + NT - 1) / NT;
-  constexpr int BE = (TK * TN + NT - 1) / NT;
-  auto& As = sm.As;
-  auto& Bs = sm.Bs;
-  auto& offCm = sm.offCm;
-  auto& offCn = sm.offCn;
-  const int tid = threadIdx.x;
-  const int tx = tid % NTX, ty = tid / NTX;
-  const int TMv = 1 << g.tm, TKv = 1 << g.tk, TNv = 1 << g.tn;
-
-  for (int i = tid; i < TK * TM; i += NT) (&As[0][0])[i] = make_float2(0.f, 0.f);
-  for (int i = tid; i < TK * TN; i += NT) (&Bs[0][0])[i] = make_float2(0.f, 0.f);
-  for (int r = tid; r < TM; r += NT) offCm[r] = r < TMv ? deposit_hi((uint64_t)r, g.c_mpos, 0, g.tm) : 0;
-  for (int c = tid; c < TN; c += NT) offCn[c] = c < TNv ? deposit_hi((uint64_t)c, g.c_npos, 0, g.tn) : 0;
-
-  // Each thread's share of a tile, decoded once: element e of the tile has its
-  // bits assigned to tile bits in ascending memory position, so consecutive e
-  // (consecutive threads) read consecutive addresses.
-  int a_sm[AE];
-  int64_t a_off[AE];
-  const int a_elems = 1 << g.a_tbits;
-#pragma unroll
-  for (int j = 0; j < AE; ++j) {
-    const int e = tid + j * NT;
-    a_sm[j] = -1;
-    a_off[j] = 0;
-    if (e < a_elems) {
-      int r = 0, c = 0;
-      int64_t off = 0;
-      for (int t = 0; t < g.a_tbits; ++t)
-        if ((e >> t) & 1) {
-          const int s = g.a_tsel[t];
-          if (s & 64) c |= 1 << (s & 63); else r |= 1 << (s & 63);
-          off += (int64_t)1 << g.a_tpos[t];
-        }
-      a_sm[j] = c * TM + r;
-      a_off[j] = off;
-    }
-  }
-  int b_sm[BE];
-  int64_t b_off[BE];
-  const int b_elems = 1 << g.b_tbits;
-#pragma unroll
-  for (int j = 0; j < BE; ++j) {
-    const int e = tid + j * NT;
-    b_sm[j] = -1;
-    b_off[j] = 0;
-    if (e < b_elems) {
-      int k = 0, n = 0;
-      int64_t off = 0;
-      for (int t = 0; t < g.b_tbits; ++t)
-        if ((e >> t) & 1) {
-          const int s = g.b_tsel[t];
-          if (s & 64) k |= 1 << (s & 63); else n |= 1 << (s & 63);
-          off += (int64_t)1 << g.b_tpos[t];
-        }
-      b_sm[j] = k * TN + n;
-      b_off[j] = off;
-    }
-  }
-  __syncthreads();
-
-  const int nkc = 1 << (g.nk - g.tk);
-  float am = 0.f;   // largest component written (for the FP16 split's scaling)
-  for (int inst = bz; inst < g.n_inst; inst += gz) {
-    const float2* A = g.A + inst_offset(inst, g.a_istride, g.a_bpos, g.nb) +
-                      deposit_hi((uint64_t)bx, g.a_mpos, g.tm, g.nm);
-    const float2* B = g.B + inst_offset(inst, g.b_istride, g.b_bpos, g.nb) +
-                      deposit_hi((uint64_t)by, g.b_npos, g.tn, g.nn);
-    float2* C = g.C + inst_offset(inst, g.c_istride, g.c_bpos, g.nb) +
-                deposit_hi((uint64_t)bx, g.c_mpos, g.tm, g.nm) + deposit_hi((uint64_t)by, g.c_npos, g.tn, g.nn);
-    float2 acc[RM][RN];
-#pragma unroll
-    for (int i = 0; i < RM; ++i)
-#pragma unroll
-      for (int j = 0; j < RN; ++j) acc[i][j] = make_float2(0.f, 0.f);
-    float2 ra[AE], rb[BE];
-    auto load = [&](int kc) {
-      const int64_t ka = deposit_hi((uint64_t)kc, g.a_kpos, g.tk, g.nk);
-      const int64_t kb = deposit_hi((uint64_t)kc, g.b_kpos, g.tk, g.nk);
-#pragma unroll
-      for (int j = 0; j < AE; ++j)
-        if (a_sm[j] >= 0) ra[j] = __ldg(A + ka + a_off[j]);
-#pragma unroll
-      for (int j = 0; j < BE; ++j)
-        if (b_sm[j] >= 0) rb[j] = __ldg(B + kb + b_off[j]);
-    };
-    load(0);
-    for (int kc = 0; kc < nkc; ++kc) {
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < AE; ++j)
-        if (a_sm[j] >= 0) (&As[0][0])[a_sm[j]] = ra[j];
-#pragma unroll
-      for (int j = 0; j < BE; ++j)
-        if (b_sm[j] >= 0) (&Bs[0][0])[b_sm[j]] = rb[j];
-      __syncthreads();
-      if (kc + 1 < nkc) load(kc + 1);
-#pragma unroll 4
-      for (int kk = 0; kk < TKv; ++kk) {
-        float2 a[RM], b[RN];
-#pragma unroll
-        for (int i = 0; i < RM; ++i) a[i] = As[kk][tx + i * NTX];
-#pragma unroll
-        for (int j = 0; j < RN; ++j) b[j] = Bs[kk][ty + j * NTY];
-#pragma unroll
-        for (int i = 0; i < RM; ++i)
-#pragma unroll
-          for (int j = 0; j < RN; ++j) {
-            acc[i][j].x = fmaf(a[i].x, b[j].x, acc[i][j].x);
-            acc[i][j].x = fmaf(-a[i].y, b[j].y, acc[i][j].x);
-            acc[i][j].y = fmaf(a[i].x, b[j].y, acc[i][j].y);
-            acc[i][j].y = fmaf(a[i].y, b[j].x, acc[i][j].y);
-          }
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < RM; ++i)
-#pragma unroll
-      for (int j = 0; j < RN; ++j) {
-        const int r = tx + i * NTX, c = ty + j * NTY;
-        if (r < TMv && c < TNv) {
-          C[offCm[r] + offCn[c]] = acc[i][j];
-          am = fmaxf(am, cabs_max(acc[i][j]));
-        }
-      }
-  }
-  if (g.amax_c) amax_update(g.amax_c, am);   // every thread reaches here (NT is a multiple of 32)
+// ------------------------------------------------------------------ packed FP32 pairs
+// Two independent FP32 FMAs in one instruction (fma.rn.f32x2); each half rounds
+// as fmaf does.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
-// One GEMM: grid (m tiles, n tiles, min(instances, 65535)).
-template <int TM, int TN, int TK, int RM, int RN>
-__global__ void __launch_bounds__((TM / RM) * (TN / RN))
-k_cgemm_simt(const GemmArgs g) {
-  __shared__ SimtSmem<TM, TN, TK> sm;
-  simt_tile<TM, TN, TK, RM, RN>(g, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z, sm);
+// Sum over bits i >= from of bit_{i - from}(x) << pos[i], one bit per lane (the
+// positions are distinct, so the sum is an OR); every lane of the warp calls it.
+__device__ __forceinline__ int64_t warp_deposit(uint32_t x, const int8_t* pos, int from, int to) {
+  const int lane = threadIdx.x & 31;
+  uint64_t v = 0;
+  if (from + lane < to && ((x >> lane) & 1u)) v = (uint64_t)1 << pos[from + lane];
+  const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)v);
+  const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32));
+  return (int64_t)(((uint64_t)hi << 32) | lo);
+}
+__device__ __forceinline__ int64_t warp_inst_offset(uint32_t inst, int64_t istride, const int8_t* bpos, int nb) {
+  return (int64_t)inst * istride + warp_deposit(inst, bpos, 0, nb);
+}
+
+// ---- cluster helpers (split-K over the CTAs of a cluster)
+__device__ __forceinline__ void simt_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t simt_cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ float2 ld_peer_f2(const void* local, uint32_t rank) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(local);
+  uint32_t p;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(a), "r"(rank));
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(p));
+  return v;
+}
+
+constexpr int SIMT_THREADS = 256;
+constexpr int SIMT_MAX_SPLIT = 8;   // CTAs of one split-K cluster (the portable cluster size)
+
+// A tiling: TM x TN outputs per CTA, TK of k per stage, RM x RN outputs per
+// thread, KG groups of threads that each take 1/KG of a stage's k (their sums
+// are added at the end), MINB CTAs per SM that the registers are kept to.  A is
+// staged as two planes (re, im) whose consecutive rows make the packed pairs.
+template <int TM_, int TN_, int TK_, int RM_, int RN_, int KG_, int MINB_>
+struct SimtCfg {
+  static constexpr int TM = TM_, TN = TN_, TK = TK_, RM = RM_, RN = RN_, KG = KG_, MINB = MINB_;
+  static constexpr int NTX = TM / RM, NTY = TN / RN;
+  static_assert(NTX * NTY * KG == SIMT_THREADS, "one thread per RM x RN outputs and k group");
+  static constexpr int RG = RM < 4 ? RM : 4;           // consecutive rows of a thread
+  static constexpr int AS = TM + 4;                    // plane row stride: k-fastest stores stay conflict-free
+  static constexpr bool SPLIT = KG > 1;                // partial tiles: k groups, and CTAs of a split-K cluster
+  struct Stage {
+    float ar[TK][AS];
+    float ai[TK][AS];
+    float2 b[TK][TN + 1];
+  };
+};
+template <class Cfg>
+struct SimtSmem {
+  union alignas(16) {
+    typename Cfg::Stage st[2];
+    // partial tiles of the k groups (column-major); the first one then takes their sum
+    float2 part[Cfg::SPLIT ? Cfg::KG : 1][Cfg::SPLIT ? Cfg::TN : 1][Cfg::SPLIT ? Cfg::TM + 2 : 1];
+  };
+  int64_t offCm[Cfg::TM];
+  int64_t offCn[Cfg::TN];
+  // step of A's and B's k offset from chunk c to c + 1, by the number of
+  // trailing one bits of c
+  int64_t kdA[KMAXR];
+  int64_t kdB[KMAXR];
+};
+
+using SimtBig = SimtCfg<128, 64, 8, 8, 4, 1, 2>;
+using Simt64 = SimtCfg<64, 64, 8, 4, 4, 1, 3>;
+using Simt128x16 = SimtCfg<128, 16, 16, 4, 2, 1, 3>;
+using Simt256x4 = SimtCfg<256, 4, 8, 4, 1, 1, 4>;
+using Simt32 = SimtCfg<32, 32, 32, 4, 4, 4, 2>;
+
+// One thread's pairs of tile elements (2p, 2p + 1) of an operand: the elements
+// of a tile are numbered by the tile bits in ascending memory position, so
+// consecutive threads read consecutive addresses, and a pair is one 16-byte load
+// where the operand's position 0 is a tile bit.
+template <int NP>
+struct PairMap {
+  int64_t off[NP];   // memory offset of the pair's first element
+  int32_t at[NP];    // its (k, row or column) packed as k << 16 | r; -1: no pair
+  int64_t step;      // memory offset of the second from the first
+  int32_t dat;       // the second's packed position less the first's; 0: no second
+};
+template <int NP>
+__device__ __forceinline__ void pair_map(PairMap<NP>& m, int tbits, const int8_t* tpos, const int8_t* tsel) {
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    m.off[j] = 0;
+    m.at[j] = 2 * ((int)threadIdx.x + j * SIMT_THREADS) < (1 << tbits) ? 0 : -1;
+  }
+  m.step = 0;
+  m.dat = 0;
+  if (tbits > 0) {
+    m.step = (int64_t)1 << tpos[0];
+    m.dat = (tsel[0] & 64) ? (1 << (16 + (tsel[0] & 63))) : (1 << tsel[0]);
+  }
+#pragma unroll 4
+  for (int t = 1; t < tbits; ++t) {
+    const int s = tsel[t];
+    const int w = (s & 64) ? (1 << (16 + (s & 63))) : (1 << s);
+    const int64_t o = (int64_t)1 << tpos[t];
+#pragma unroll
+    for (int j = 0; j < NP; ++j)
+      if ((((int)threadIdx.x + j * SIMT_THREADS) >> (t - 1)) & 1) {
+        m.off[j] += o;
+        if (m.at[j] >= 0) m.at[j] += w;
+      }
+  }
+}
+template <int NP>
+__device__ __forceinline__ void pair_load(float4 (&v)[NP], const PairMap<NP>& m, const float2* base, bool vec) {
+#pragma unroll
+  for (int j = 0; j < NP; ++j)
+    if (m.at[j] >= 0) {
+      const float2* p = base + m.off[j];
+      if (vec) {
+        v[j] = __ldg(reinterpret_cast<const float4*>(p));
+      } else {
+        const float2 x = __ldg(p);
+        const float2 y = m.dat ? __ldg(p + m.step) : make_float2(0.f, 0.f);
+        v[j] = make_float4(x.x, x.y, y.x, y.y);
+      }
+    }
+}
+
+// One (m tile bx, n tile by) of a GEMM for instances bz, bz + gz, ... ; with
+// split > 1 CTA `rank` of every `split` consecutive ones takes 1/split of the k
+// chunks and the partial tiles are added over the cluster's shared memory in
+// rank order (deterministic).  Every thread of the block calls it; g is in
+// shared memory.  Rows and columns past the operand's extent hold whatever the
+// stage buffers held: they only reach outputs that are not stored.
+// Large GEMMs are bound by the FP32 pipe's issue slots: a product of two packed
+// FMAs takes half the slots of four scalar ones, and 8 x 4 outputs per thread
+// leave 24 register moves and 8 shared loads per 64 of them; 4096 x 1024 x 4096
+// runs at 56 TFLOP/s (35 with scalar FMAs and 4 x 4 outputs), of about 70.  Small
+// ones are bound by latency: k offsets advance by one table entry per chunk
+// (decoding all k bits per chunk took longer than the chunk's products), and one
+// chunk with its set-up takes about 5 us in a chain of launches (12 before).
+template <class Cfg>
+__device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int bz, int gz, int split, int rank,
+                                          SimtSmem<Cfg>& sm) {
+  constexpr int TM = Cfg::TM, TN = Cfg::TN, TK = Cfg::TK, RM = Cfg::RM, RN = Cfg::RN;
+  constexpr int NTX = Cfg::NTX, RG = Cfg::RG, RP = RM / 2;
+  constexpr int AP = (TM * TK / 2 + SIMT_THREADS - 1) / SIMT_THREADS;
+  constexpr int BP = (TN * TK / 2 + SIMT_THREADS - 1) / SIMT_THREADS;
+  const int tid = threadIdx.x;
+  const int tx = tid % NTX, ty = (tid / NTX) % Cfg::NTY, kg = tid / (NTX * Cfg::NTY);
+  const int TMv = 1 << g.tm, TKv = 1 << g.tk, TNv = 1 << g.tn;
+  const int n_hi = g.nk - g.tk;
+  const int kc_per = (1 << n_hi) / split, kc0 = rank * kc_per;
+
+  // offsets of the tile's rows and columns in C, and the k chunk steps
+  for (int r = tid; r < TM; r += SIMT_THREADS) sm.offCm[r] = r < TMv ? deposit_hi((uint64_t)r, g.c_mpos, 0, g.tm) : 0;
+  if (tid < TN) sm.offCn[tid] = tid < TNv ? deposit_hi((uint64_t)tid, g.c_npos, 0, g.tn) : 0;
+  {
+    const int t = SIMT_THREADS - 1 - tid;   // other threads than the ones above where the tile is small
+    if (t < n_hi) {
+      int64_t a = (int64_t)1 << g.a_kpos[g.tk + t], b = (int64_t)1 << g.b_kpos[g.tk + t];
+      for (int j = 0; j < t; ++j) {
+        a -= (int64_t)1 << g.a_kpos[g.tk + j];
+        b -= (int64_t)1 << g.b_kpos[g.tk + j];
+      }
+      sm.kdA[t] = a;
+      sm.kdB[t] = b;
+    }
+  }
+  PairMap<AP> ma;
+  PairMap<BP> mb;
+  pair_map(ma, g.a_tbits, g.a_tpos, g.a_tsel);
+  pair_map(mb, g.b_tbits, g.b_tpos, g.b_tsel);
+  const bool va = g.a_tbits > 0 && g.a_tpos[0] == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
+  const bool vb = g.b_tbits > 0 && g.b_tpos[0] == 0 && (reinterpret_cast<uintptr_t>(g.B) & 15) == 0;
+  const int64_t abase = warp_deposit((uint32_t)bx, g.a_mpos, g.tm, g.nm) + warp_deposit((uint32_t)kc0, g.a_kpos, g.tk, g.nk);
+  const int64_t bbase = warp_deposit((uint32_t)by, g.b_npos, g.tn, g.nn) + warp_deposit((uint32_t)kc0, g.b_kpos, g.tk, g.nk);
+  const int64_t cbase = warp_deposit((uint32_t)bx, g.c_mpos, g.tm, g.nm) + warp_deposit((uint32_t)by, g.c_npos, g.tn, g.nn);
+  __syncthreads();
+
+  float am = 0.f;   // largest component written (for the FP16 split's scaling)
+  // every CTA of a cluster goes through the same number of rounds (the cluster
+  // barriers), also one without an instance left
+  const int rounds = split > 1 ? (g.n_inst + gz - 1) / gz : 0x7fffffff;
+  for (int it = 0, inst = bz; it < rounds; ++it, inst += gz) {
+    if (bz >= gz || inst >= g.n_inst) {
+      if (split == 1) break;
+      simt_cluster_sync();
+      simt_cluster_sync();
+      continue;
+    }
+    const float2* A = g.A + warp_inst_offset(inst, g.a_istride, g.a_bpos, g.nb) + abase;
+    const float2* B = g.B + warp_inst_offset(inst, g.b_istride, g.b_bpos, g.nb) + bbase;
+    float2* C = g.C + warp_inst_offset(inst, g.c_istride, g.c_bpos, g.nb) + cbase;
+    f32x2 re[RP][RN], im[RP][RN];
+#pragma unroll
+    for (int i = 0; i < RP; ++i)
+#pragma unroll
+      for (int j = 0; j < RN; ++j) re[i][j] = im[i][j] = 0ull;
+    float4 la[AP], lb[BP];
+    auto put = [&](typename Cfg::Stage& st) {
+#pragma unroll
+      for (int j = 0; j < AP; ++j)
+        if (ma.at[j] >= 0) {
+          const int k = ma.at[j] >> 16, r = ma.at[j] & 0xffff;
+          st.ar[k][r] = la[j].x;
+          st.ai[k][r] = la[j].y;
+          if (ma.dat) {
+            const int k2 = (ma.at[j] + ma.dat) >> 16, r2 = (ma.at[j] + ma.dat) & 0xffff;
+            st.ar[k2][r2] = la[j].z;
+            st.ai[k2][r2] = la[j].w;
+          }
+        }
+      auto putb = [&](int at, float x, float y) { st.b[at >> 16][at & 0xffff] = make_float2(x, y); };
+#pragma unroll
+      for (int j = 0; j < BP; ++j)
+        if (mb.at[j] >= 0) {
+          putb(mb.at[j], lb[j].x, lb[j].y);
+          if (mb.dat) putb(mb.at[j] + mb.dat, lb[j].z, lb[j].w);
+        }
+    };
+    auto step = [&](const typename Cfg::Stage& st, int kk) {
+      f32x2 ar[RP], ai[RP];
+#pragma unroll
+      for (int gq = 0; gq < RM / RG; ++gq) {
+        const int r0 = (gq * NTX + tx) * RG;
+        if constexpr (RG == 4) {
+          const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(&st.ar[kk][r0]);
+          const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(&st.ai[kk][r0]);
+          ar[2 * gq] = x.x;
+          ar[2 * gq + 1] = x.y;
+          ai[2 * gq] = y.x;
+          ai[2 * gq + 1] = y.y;
+        } else {
+          ar[gq] = *reinterpret_cast<const f32x2*>(&st.ar[kk][r0]);
+          ai[gq] = *reinterpret_cast<const f32x2*>(&st.ai[kk][r0]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < RN; ++j) {
+        const float2 v = st.b[kk][ty + j * Cfg::NTY];
+        const f32x2 br = pack2(v.x, v.x), bi = pack2(v.y, v.y), nb = pack2(-v.y, -v.y);
+#pragma unroll
+        for (int i = 0; i < RP; ++i) {
+          re[i][j] = fma2(ar[i], br, re[i][j]);
+          im[i][j] = fma2(ar[i], bi, im[i][j]);
+        }
+#pragma unroll
+        for (int i = 0; i < RP; ++i) {
+          re[i][j] = fma2(ai[i], nb, re[i][j]);
+          im[i][j] = fma2(ai[i], br, im[i][j]);
+        }
+      }
+    };
+    pair_load(la, ma, A, va);
+    pair_load(lb, mb, B, vb);
+    put(sm.st[0]);
+    __syncthreads();
+    for (int c = 0; c < kc_per; ++c) {
+      const bool more = c + 1 < kc_per;
+      if (more) {   // the next chunk's loads run under this chunk's products
+        const int t = __ffs(~(kc0 + c)) - 1;   // trailing ones of the chunk index
+        A += sm.kdA[t];
+        B += sm.kdB[t];
+        pair_load(la, ma, A, va);
+        pair_load(lb, mb, B, vb);
+      }
+      const typename Cfg::Stage& st = sm.st[c & 1];
+      if (TKv == TK) {
+#pragma unroll(RM * RN >= 32 ? 4 : 8)
+        for (int kk = 0; kk < TK / Cfg::KG; ++kk) step(st, kk * Cfg::KG + kg);
+      } else {
+        for (int kk = kg; kk < TKv; kk += Cfg::KG) step(st, kk);
+      }
+      if (more) put(sm.st[(c + 1) & 1]);   // last read before the previous barrier
+      __syncthreads();
+    }
+    if constexpr (!Cfg::SPLIT) {
+      const bool vc = g.tm > 0 && g.c_mpos[0] == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+#pragma unroll
+      for (int i = 0; i < RP; ++i) {
+        const int r = ((2 * i / RG) * NTX + tx) * RG + (2 * i) % RG;
+        if (r < TMv) {
+#pragma unroll
+          for (int j = 0; j < RN; ++j) {
+            const int cidx = ty + j * Cfg::NTY;
+            if (cidx < TNv) {
+              const float2 x = unpack2(re[i][j]), y = unpack2(im[i][j]);
+              float2* p = C + sm.offCm[r] + sm.offCn[cidx];
+              am = fmaxf(am, cabs_max(make_float2(x.x, y.x)));
+              if (r + 1 < TMv) {
+                am = fmaxf(am, cabs_max(make_float2(x.y, y.y)));
+                if (vc && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+                  *reinterpret_cast<float4*>(p) = make_float4(x.x, y.x, x.y, y.y);
+                } else {
+                  *p = make_float2(x.x, y.x);
+                  C[sm.offCm[r + 1] + sm.offCn[cidx]] = make_float2(x.y, y.y);
+                }
+              } else {
+                *p = make_float2(x.x, y.x);
+              }
+            }
+          }
+        }
+      }
+    } else {
+      // the k groups' partial tiles to shared memory (the stages are done with:
+      // barrier above), added in group order; with a split, each CTA then adds its
+      // share of the tile's elements over the cluster, in rank order
+#pragma unroll
+      for (int i = 0; i < RP; ++i) {
+        const int r = ((2 * i / RG) * NTX + tx) * RG + (2 * i) % RG;
+#pragma unroll
+        for (int j = 0; j < RN; ++j) {
+          const float2 x = unpack2(re[i][j]), y = unpack2(im[i][j]);
+          *reinterpret_cast<float4*>(&sm.part[kg][ty + j * Cfg::NTY][r]) = make_float4(x.x, y.x, x.y, y.y);
+        }
+      }
+      __syncthreads();
+      const int total = 1 << (g.tm + g.tn);
+      for (int e = tid; e < total; e += SIMT_THREADS) {
+        const int r = e & (TMv - 1), c = e >> g.tm;
+        float2 acc = sm.part[0][c][r];
+#pragma unroll
+        for (int q = 1; q < Cfg::KG; ++q) {
+          acc.x += sm.part[q][c][r].x;
+          acc.y += sm.part[q][c][r].y;
+        }
+        if (split == 1) {
+          C[sm.offCm[r] + sm.offCn[c]] = acc;
+          am = fmaxf(am, cabs_max(acc));
+        } else {
+          sm.part[0][c][r] = acc;   // read by this thread alone so far
+        }
+      }
+      if (split == 1) {
+        __syncthreads();   // the next instance's stages overwrite the partial tiles
+        continue;
+      }
+      simt_cluster_sync();
+      const uint32_t me = simt_cluster_rank(), base = me - (uint32_t)rank;
+      for (int e = rank * SIMT_THREADS + tid; e < total; e += split * SIMT_THREADS) {
+        const int r = e & (TMv - 1), c = e >> g.tm;
+        float2 v[SIMT_MAX_SPLIT];
+#pragma unroll
+        for (int q = 0; q < SIMT_MAX_SPLIT; ++q)
+          if (q < split) v[q] = ld_peer_f2(&sm.part[0][c][r], base + q);
+        float2 acc = v[0];
+#pragma unroll
+        for (int q = 1; q < SIMT_MAX_SPLIT; ++q)
+          if (q < split) {
+            acc.x += v[q].x;
+            acc.y += v[q].y;
+          }
+        C[sm.offCm[r] + sm.offCn[c]] = acc;
+        am = fmaxf(am, cabs_max(acc));
+      }
+      simt_cluster_sync();   // the peers have read this CTA's partial tile
+    }
+  }
+  if (g.amax_c) amax_update(g.amax_c, am);   // every thread reaches here
+}
+
+__device__ __forceinline__ void copy_args(GemmArgs& dst, const GemmArgs* src) {
+  constexpr int words = (int)(sizeof(GemmArgs) / 4);
+  const uint32_t* s = reinterpret_cast<const uint32_t*>(src);
+  uint32_t* d = reinterpret_cast<uint32_t*>(&dst);
+  for (int w = threadIdx.x; w < words; w += blockDim.x) d[w] = s[w];
+}
+
+// One GEMM: grid (m tiles x split, n tiles, min(instances, 65535)); split > 1:
+// clusters of `split` CTAs along x.
+template <class Cfg>
+__global__ void __launch_bounds__(SIMT_THREADS, Cfg::MINB) k_cgemm_simt(const __grid_constant__ GemmArgs g, int split) {
+  __shared__ GemmArgs sg;
+  __shared__ SimtSmem<Cfg> sm;
+  copy_args(sg, &g);
+  __syncthreads();
+  simt_tile<Cfg>(sg, blockIdx.x / split, blockIdx.y, blockIdx.z, gridDim.z, split, blockIdx.x % split, sm);
 }
 
 // Several independent GEMMs in one launch (a group of small steps that
-// neither read nor write what another of the group writes): block b runs
-// block b - start[i] of GEMM i, where start[i] <= b < start[i + 1] (start[n]
-// is the grid size), decoded as (m tile, n tile, instance) with the m tile
-// fastest, exactly as that GEMM's own grid would, with that GEMM's tiling
-// tiling[i] (0: 64x64, 1: 128x16, 2: 256x4; all three use 256 threads).
-__global__ void __launch_bounds__(256)
+// neither read nor write what another of the group writes), on clusters of
+// SIMT_MAX_SPLIT CTAs: block b runs block b - start[i] of GEMM i, where
+// start[i] <= b < start[i + 1] (start[n] is the grid size; every start is a
+// multiple of the cluster size, so a cluster has one GEMM), decoded as (split
+// rank fastest, m tile, n tile, instance), with that GEMM's tiling[i] (0:
+// 64x64, 1: 128x16, 2: 256x4, 3: 32x32; all use 256 threads) and split[i].
+__global__ void __launch_bounds__(SIMT_THREADS, 2)
 k_cgemm_simt_multi(const GemmArgs* __restrict__ gs, const int32_t* __restrict__ start,
-                   const int8_t* __restrict__ tiling, int32_t n) {
+                   const int8_t* __restrict__ tiling, const int8_t* __restrict__ splits, int32_t n) {
   __shared__ GemmArgs sg;
   __shared__ int s_i;
   __shared__ union {   // one tiling per block: their tiles share the space
-    SimtSmem<64, 64, 8> t0;
-    SimtSmem<128, 16, 16> t1;
-    SimtSmem<256, 4, 16> t2;
+    SimtSmem<Simt64> t0;
+    SimtSmem<Simt128x16> t1;
+    SimtSmem<Simt256x4> t2;
+    SimtSmem<Simt32> t3;
   } sm;
   const int b = blockIdx.x;
-  if (threadIdx.x == 0) {
-    int i = 0;
-    while (i + 1 < n && start[i + 1] <= b) ++i;
-    s_i = i;
+  if (threadIdx.x < 32) {   // the last start at or before b
+    int i = -1;
+    for (int t = threadIdx.x; t < n; t += 32)
+      if (start[t] <= b) i = t;
+    i = __reduce_max_sync(0xffffffffu, i);
+    if (threadIdx.x == 0) s_i = i;
   }
   __syncthreads();
   const int i = s_i;
-  {
-    const int words = (int)(sizeof(GemmArgs) / 4);
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(gs + i);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(&sg);
-    for (int w = threadIdx.x; w < words; w += blockDim.x) dst[w] = src[w];
-  }
+  copy_args(sg, gs + i);
   __syncthreads();
+  const int split = splits[i];
   const int gx = 1 << (sg.nm - sg.tm), gy = 1 << (sg.nn - sg.tn);
   const int gz = sg.n_inst < 65535 ? sg.n_inst : 65535;
-  const int lb = b - start[i];
-  const int bx = lb % gx, by = (lb / gx) % gy, bz = lb / (gx * gy);
+  const int lb = b - start[i], rank = lb % split, lt = lb / split;
+  const int bx = lt % gx, by = (lt / gx) % gy, bz = lt / (gx * gy);
+  // blocks past the GEMM's last tile (bz >= gz) fill its last cluster: they run
+  // no instance, only the barriers
   switch (tiling[i]) {   // block-uniform
     case 0:
-      simt_tile<64, 64, 8, 4, 4>(sg, bx, by, bz, gz, sm.t0);
+      simt_tile<Simt64>(sg, bx, by, bz, gz, 1, 0, sm.t0);
       break;
     case 1:
-      simt_tile<128, 16, 16, 4, 2>(sg, bx, by, bz, gz, sm.t1);
+      simt_tile<Simt128x16>(sg, bx, by, bz, gz, 1, 0, sm.t1);
+      break;
+    case 2:
+      simt_tile<Simt256x4>(sg, bx, by, bz, gz, 1, 0, sm.t2);
       break;
     default:
-      simt_tile<256, 4, 16, 4, 1>(sg, bx, by, bz, gz, sm.t2);
+      simt_tile<Simt32>(sg, bx, by, bz, gz, split, rank, sm.t3);
       break;
   }
 }

@@ -33,25 +33,21 @@ namespace tnx {
 enum KernelId {
   K_SIMT_64x64 = 0,   // TM 64, TN 64, TK 8
   K_SIMT_128x16 = 1,  // TM 128, TN 16, TK 16
-  K_SIMT_256x4 = 2,   // TM 256, TN 4, TK 16
+  K_SIMT_256x4 = 2,   // TM 256, TN 4, TK 8
   K_TC_TF32 = 3,      // tcgen05 kind::tf32, tile 128 x (<=128 complex), k chunk 16
   K_TC_BF16X3 = 4,    // tcgen05 kind::f16 bf16 hi/lo split
   K_TC_TF32_3M = 5,   // the same with 3M products (three accumulators per tile)
   K_TC_BF16X3_3M = 6,
   K_TC_FP16X3 = 7,    // tcgen05 kind::f16 fp16 hi/lo split, operands scaled by powers of two
   K_TC_FP16X3_3M = 8,
+  K_SIMT_128x64 = 9,  // TM 128, TN 64, TK 8
+  K_SIMT_32x32 = 10,  // TM 32, TN 32, TK 32; split-K over a cluster's CTAs
   K_COUNT
 };
 struct KernelCfg {
   int tm, tn, tk;  // log2 tile extents
 };
-static const KernelCfg kCfg[K_COUNT] = {{6, 6, 3}, {7, 4, 4}, {8, 2, 4}, {7, 7, 4}, {7, 7, 4}, {7, 7, 4}, {7, 7, 4}, {7, 7, 4}, {7, 7, 4}};
-
-static int pick_simt(const StepDesc& d) {
-  if (d.nn >= 5 && d.nm >= 5) return K_SIMT_64x64;
-  if (d.nn >= 3) return K_SIMT_128x16;
-  return K_SIMT_256x4;
-}
+static const KernelCfg kCfg[K_COUNT] = {{6, 6, 3}, {7, 4, 4}, {8, 2, 3}, {7, 7, 4}, {7, 7, 4}, {7, 7, 4}, {7, 7, 4}, {7, 7, 4}, {7, 7, 4}, {7, 6, 3}, {5, 5, 5}};
 
 static int sm_count() {
   static int n = 0;
@@ -61,6 +57,44 @@ static int sm_count() {
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 1;
   }
   return n;
+}
+
+static bool is_simt(int kid) { return kid >= 0 && kid < K_COUNT && !(kid >= K_TC_TF32 && kid <= K_TC_FP16X3_3M); }
+
+// CUDA-core tiling of a step, from times on a GB300 (us, one launch):
+//  * few outputs (at most two 32x32 tiles per SM): 32x32, whose k groups and
+//    split-K clusters keep the SMs busy -- (log2 m, k, n) = (7, 10, 6): 12 against
+//    148 with 64x64; (10, 6, 8): 9.9 against 14; with more tiles the larger ones
+//    win, (12, 4, 9): 36 against 13 with 128x64;
+//  * n <= 4: 256x4, n <= 16: 128x16 -- (20, 3, 1): 47 with 256x4, 96 with 128x16;
+//    (16, 5, 4): 18 with 128x16, 33 with 64x64;
+//  * n = 32 with k >= 64: 32x32 -- (15, 8, 5): 74 against 110 with 64x64;
+//  * otherwise 128x64 where its tiles fill the SMs -- (12, 10, 12): 2440 against
+//    2710 with 64x64 -- and 64x64 where they do not.
+static int pick_simt(const StepDesc& d, int64_t n_inst) {
+  auto tiles = [&](int tm, int tn) {
+    return ((int64_t)1 << (std::max(d.nm, tm) - tm)) * ((int64_t)1 << (std::max(d.nn, tn) - tn)) * n_inst;
+  };
+  const int64_t sms = sm_count();
+  if (tiles(5, 5) <= 2 * sms || (d.nm < 5 && d.nn >= 5)) return K_SIMT_32x32;
+  if (d.nn <= 2) return K_SIMT_256x4;
+  if (d.nn <= 4) return K_SIMT_128x16;
+  if (d.nn == 5 && d.nk >= 6) return K_SIMT_32x32;
+  if (d.nn >= 6 && d.nm >= 7 && tiles(7, 6) >= 128) return K_SIMT_128x64;
+  return K_SIMT_64x64;
+}
+
+// CTAs of a cluster that share a tile's k loop (1: no split): as many as leave
+// each at least two k chunks and the grid within two CTAs per SM.  A cluster
+// costs 2-4 us, a 32-k chunk of a lone CTA 1-1.5: (8, 8, 6) takes 16 us unsplit,
+// 8.3 over 4 CTAs (2 chunks each), 9.1 over 8; (7, 10, 6) 52, 17 and 12.
+static int simt_split(const GemmArgs& g, int kid) {
+  if (kid != K_SIMT_32x32) return 1;
+  const int64_t tiles = ((int64_t)1 << (g.nm - g.tm)) * ((int64_t)1 << (g.nn - g.tn)) * g.n_inst;
+  const int n_kc = 1 << (g.nk - g.tk);
+  int sp = 1;
+  while (sp < SIMT_MAX_SPLIT && sp * 4 <= n_kc && tiles * sp * 2 <= 2 * (int64_t)sm_count()) sp *= 2;
+  return sp;
 }
 
 // Tile decode tables: the tile's bits in ascending memory position.
@@ -114,21 +148,47 @@ static GemmArgs make_args(const StepDesc& d, int kid, const float2* A, const flo
   return g;
 }
 
+template <class Cfg>
+static void launch_simt_cfg(const GemmArgs& g, dim3 grid, int split, cudaStream_t s) {
+  if (split == 1) {
+    k_cgemm_simt<Cfg><<<grid, SIMT_THREADS, 0, s>>>(g, 1);
+    return;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(SIMT_THREADS);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)split;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  CK(cudaLaunchKernelEx(&cfg, k_cgemm_simt<Cfg>, g, split));
+}
 static void launch_simt(const GemmArgs& g, int kid, cudaStream_t s) {
   if (g.n_inst <= 0) return;
-  const int64_t gx = (int64_t)1 << (g.nm - g.tm);
+  const int split = simt_split(g, kid);
+  const int64_t gx = ((int64_t)1 << (g.nm - g.tm)) * split;
   const int64_t gy = (int64_t)1 << (g.nn - g.tn);
   if (gx > 0x7fffffff || gy > 65535) fail(TN_ERR_UNSUPPORTED, "GEMM grid too large");
   dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)std::min<int32_t>(g.n_inst, 65535));
   switch (kid) {
     case K_SIMT_64x64:
-      k_cgemm_simt<64, 64, 8, 4, 4><<<grid, 256, 0, s>>>(g);
+      launch_simt_cfg<Simt64>(g, grid, 1, s);
       break;
     case K_SIMT_128x16:
-      k_cgemm_simt<128, 16, 16, 4, 2><<<grid, 256, 0, s>>>(g);
+      launch_simt_cfg<Simt128x16>(g, grid, 1, s);
       break;
     case K_SIMT_256x4:
-      k_cgemm_simt<256, 4, 16, 4, 1><<<grid, 256, 0, s>>>(g);
+      launch_simt_cfg<Simt256x4>(g, grid, 1, s);
+      break;
+    case K_SIMT_128x64:
+      launch_simt_cfg<SimtBig>(g, grid, 1, s);
+      break;
+    case K_SIMT_32x32:
+      launch_simt_cfg<Simt32>(g, grid, split, s);
       break;
     default:
       fail(TN_ERR_UNSUPPORTED, "kernel variant not built");
@@ -518,7 +578,8 @@ struct DeviceState {
       int blocks = 0, n = 0;
       GemmArgs* args = nullptr;                // device: n GemmArgs
       int32_t* start = nullptr;                // device: n + 1 block offsets
-      int8_t* tiling = nullptr;                // device: n CUDA-core tilings (kernel ids 0-2)
+      int8_t* tiling = nullptr;                // device: n CUDA-core tilings (simt_multi_tiling)
+      int8_t* split = nullptr;                 // device: n split-K factors
       std::vector<float*> amax;                // FP16X3: result maxima to clear first
     };
     std::vector<Multi> multi;
@@ -550,10 +611,10 @@ static int tc_kernel(int precision, int cmult) {
 // Tensor-core kernels (4M or 3M products) for every step with enough work in
 // the TF32 / BF16X3 / FP16X3 modes; tiny steps (and the FP32 mode) on the CUDA
 // cores, which always form 4M products in FP32.
-static int pick_kernel(int precision, int cmult, const StepDesc& d) {
-  if (precision == TN_PREC_FP32) return pick_simt(d);
+static int pick_kernel(int precision, int cmult, const StepDesc& d, int64_t n_inst) {
+  if (precision == TN_PREC_FP32) return pick_simt(d, n_inst);
   const int work = d.nm + d.nk + d.nn + d.nb;
-  if (work < 20 || d.nm < 4) return pick_simt(d);
+  if (work < 20 || d.nm < 4) return pick_simt(d, n_inst);
   return tc_kernel(precision, cmult);
 }
 
@@ -570,9 +631,26 @@ static GemmArgs step_args(const DeviceState& ds, const StepDesc& d, int kid, int
   return g;
 }
 
+// The tiling index of k_cgemm_simt_multi for a kernel id, -1 for a tiling it does not have.
+static int simt_multi_tiling(int kid) {
+  return kid == K_SIMT_32x32 ? 3 : (kid >= K_SIMT_64x64 && kid <= K_SIMT_256x4 ? kid : -1);
+}
+
 static void launch_simt_multi(const DeviceState::GroupRun::Multi& m, cudaStream_t s) {
   for (float* am : m.amax) CK(cudaMemsetAsync(am, 0, sizeof(float), s));
-  k_cgemm_simt_multi<<<m.blocks, 256, 0, s>>>(m.args, m.start, m.tiling, m.n);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)m.blocks);
+  cfg.blockDim = dim3(SIMT_THREADS);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = SIMT_MAX_SPLIT;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  CK(cudaLaunchKernelEx(&cfg, k_cgemm_simt_multi, (const GemmArgs*)m.args, (const int32_t*)m.start,
+                        (const int8_t*)m.tiling, (const int8_t*)m.split, (int32_t)m.n));
 }
 
 // Dependence flags of a node (bit 0: on the slice id, bit 1: on the closed
@@ -637,7 +715,7 @@ static void build_groups(Plan& p, DeviceState& ds) {
     gr.end = (int)j;
     std::vector<int> simt;
     for (size_t t = i; t < j; ++t) {
-      if (is_tc(ds.launches[t].kid)) gr.singles.push_back((int)t);
+      if (simt_multi_tiling(ds.launches[t].kid) < 0) gr.singles.push_back((int)t);
       else simt.push_back((int)t);
     }
     if (simt.size() == 1) gr.singles.push_back(simt[0]);
@@ -657,7 +735,7 @@ static void build_groups(Plan& p, DeviceState& ds) {
   for (auto& pm : pending) {
     bytes = (bytes + 255) / 256 * 256 + sizeof(GemmArgs) * pm.second.size();
     bytes = (bytes + 15) / 16 * 16 + sizeof(int32_t) * (pm.second.size() + 1);
-    bytes += pm.second.size();   // tilings
+    bytes += 2 * pm.second.size();   // tilings, splits
   }
   std::vector<uint8_t> host(bytes, 0);
   CK(cudaMalloc(&ds.group_buf, bytes));
@@ -672,14 +750,18 @@ static void build_groups(Plan& p, DeviceState& ds) {
     const size_t start_off = off;
     off += sizeof(int32_t) * (pm.second.size() + 1);
     const size_t tiling_off = off;
-    off += pm.second.size();
+    off += 2 * pm.second.size();
     int32_t blocks = 0;
     for (size_t q = 0; q < pm.second.size(); ++q) {
       const GemmArgs& g = ds.launches[pm.second[q]].g;
       std::memcpy(host.data() + args_off + q * sizeof(GemmArgs), &g, sizeof(GemmArgs));
-      host[tiling_off + q] = (uint8_t)ds.launches[pm.second[q]].kid;   // K_SIMT_* are 0..2
-      const int64_t nb = ((int64_t)1 << (g.nm - g.tm)) * ((int64_t)1 << (g.nn - g.tn)) *
-                         std::min<int64_t>(g.n_inst, 65535);
+      const int kid = ds.launches[pm.second[q]].kid, split = simt_split(g, kid);
+      host[tiling_off + q] = (uint8_t)simt_multi_tiling(kid);
+      host[tiling_off + pm.second.size() + q] = (uint8_t)split;
+      // whole clusters: the kernel's blocks past the last tile only keep its barriers
+      int64_t nb = ((int64_t)1 << (g.nm - g.tm)) * ((int64_t)1 << (g.nn - g.tn)) * split *
+                   std::min<int64_t>(g.n_inst, 65535);
+      nb = (nb + SIMT_MAX_SPLIT - 1) / SIMT_MAX_SPLIT * SIMT_MAX_SPLIT;
       if (blocks + nb > 0x7fffffff) fail(TN_ERR_UNSUPPORTED, "step group grid too large");
       std::memcpy(host.data() + start_off + q * sizeof(int32_t), &blocks, sizeof(int32_t));
       blocks += (int32_t)nb;
@@ -690,6 +772,7 @@ static void build_groups(Plan& p, DeviceState& ds) {
     m.args = reinterpret_cast<GemmArgs*>(ds.group_buf + args_off);
     m.start = reinterpret_cast<int32_t*>(ds.group_buf + start_off);
     m.tiling = reinterpret_cast<int8_t*>(ds.group_buf + tiling_off);
+    m.split = m.tiling + pm.second.size();
   }
   CK(cudaMemcpy(ds.group_buf, host.data(), bytes, cudaMemcpyHostToDevice));
 }
@@ -753,7 +836,7 @@ static void ensure_device(Plan& p) {
                     ((int64_t)1 << (d.nk + d.nn + d.nb)) == d.b_elems &&
                     ((int64_t)1 << (d.nm + d.nn + d.nb)) == d.c_elems;
     if (!ok) fail(TN_ERR_PLAN, "internal: step operand outside its extent");
-    const int kid = pick_kernel(p.opts.precision, p.opts.complex_mult, d);
+    const int kid = pick_kernel(p.opts.precision, p.opts.complex_mult, d, (int64_t)1 << d.nb);
     ds->launches.push_back(make_launch(step_args(*ds, d, kid), kid, 64 - __builtin_clzll((uint64_t)d.a_elems) - 1, 1,
                                        d.c_elems, true, -1, (int64_t)256 << 20, 0, p.opts.sm_pairs ? -1 : 0));
   }
@@ -1033,7 +1116,7 @@ static void kernels_changed(Plan& p, DeviceState& ds) {
 // Autotuner: for every step, time the candidate kernels in place (tensor-core
 // tiles of 32, 64 or 128 complex columns in the TF32 / BF16X3 / FP16X3 modes,
 // each with either write-back order, with the default or a deeper B' ring (4,
-// 6 or 8 slots) and on one SM or an SM pair, and the three CUDA-core tilings
+// 6 or 8 slots) and on one SM or an SM pair, and the CUDA-core tilings
 // where the step is small or the mode is FP32) and keep the fastest.  The
 // chunk graph is captured again on the next call.
 extern "C" tn_status tn_plan_autotune(tn_plan_t* h, int32_t reps, void* stream) {
@@ -1095,7 +1178,8 @@ extern "C" tn_status tn_plan_autotune(tn_plan_t* h, int32_t reps, void* stream) 
     const double flops = 8.0 * std::ldexp(1.0, d.nm + d.nk + d.nn + d.nb);
     const double bytes = 8.0 * (double)(d.a_elems + d.b_elems + d.c_elems);
     if (!tc_mode || best < 0.05 || flops / bytes < 48.0)
-      for (int k : {K_SIMT_64x64, K_SIMT_128x16, K_SIMT_256x4}) cands.push_back({k, -1, 0, 0, 0});
+      for (int k : {K_SIMT_64x64, K_SIMT_128x16, K_SIMT_256x4, K_SIMT_128x64, K_SIMT_32x32})
+        cands.push_back({k, -1, 0, 0, 0});
     std::vector<std::array<int, 5>> seen;
     auto key = [](const StepLaunch& L) {
       return std::array<int, 5>{L.kid, L.g.tn, is_tc(L.kid) ? L.tc.epi_ok : 0, is_tc(L.kid) ? L.tc.nbs : 0,
@@ -1159,7 +1243,7 @@ extern "C" tn_status tn_plan_set_tuning(tn_plan_t* h, const int32_t* in, int32_t
   for (size_t i = 0; i < p.steps.size(); ++i) {
     const int32_t* c = in + i * TN_TUNING_INTS;
     const int kid = c[0];
-    const bool simt = kid == K_SIMT_64x64 || kid == K_SIMT_128x16 || kid == K_SIMT_256x4;
+    const bool simt = is_simt(kid);
     if (!simt && !is_tc(kid)) fail(TN_ERR_ARG, "tn_plan_set_tuning: unknown kernel id");
     if (is_tc(kid) && (p.opts.precision == TN_PREC_FP32 || kid != tc_kernel(p.opts.precision, p.opts.complex_mult)))
       fail(TN_ERR_ARG, "tn_plan_set_tuning: tensor-core kernel of another precision or product");
@@ -1569,7 +1653,7 @@ extern "C" tn_status tn_contract_pair(const float* a, const int32_t* aw, int32_t
   d.b_elems = (int64_t)1 << br;
   d.c_elems = (int64_t)1 << cr;
   d.nb = 0;
-  const int kid = pick_kernel(precision, cmult, d);
+  const int kid = pick_kernel(precision, cmult, d, batch);
   GemmArgs g = make_args(d, kid, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
                          reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems);
   Scratch& sc = scratch_for_device();
@@ -1689,7 +1773,7 @@ extern "C" tn_status tn_contract_pair_noalloc(const float* a, const int32_t* aw,
   d.a_elems = (int64_t)1 << ar;
   d.b_elems = (int64_t)1 << br;
   d.c_elems = (int64_t)1 << cr;
-  const int kid = pick_kernel(precision, cmult, d);
+  const int kid = pick_kernel(precision, cmult, d, batch);
   GemmArgs g = make_args(d, kid, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
                          reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems);
   const int64_t cap = (int64_t)(kNoAllocScratchBytes - kNoAllocErrBytes);

@@ -1,0 +1,67 @@
+"""Kernel variants at the sizes where their tiles, splits and dispatch rules change."""
+import numpy as np
+import pytest
+
+from oracle import pairwise
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2111_01066_gb300 import tn
+    torch.cuda.set_device(0)
+    return tn, torch
+
+
+def _pair_case(torch, shape, batch, layout, seed, misaligned=False):
+    nm, nk, nn = shape
+    rng = np.random.default_rng(seed)
+    w = list(range(nm + nk + nn))
+    m, k, n = w[:nm], w[nm:nm + nk], w[nm + nk:]
+    if layout == "kfast":
+        a_w, b_w, c_w = k + m, k + n, m + n
+    else:
+        a_w, b_w, c_w = (list(rng.permutation(v)) for v in (m + k, k + n, m + n))
+    draw = lambda r: ((rng.normal(size=(batch, 2 ** r)) + 1j * rng.normal(size=(batch, 2 ** r))) / 2).astype(np.complex64)
+    a, b = draw(nm + nk), draw(nk + nn)
+
+    def dev(x):   # misaligned: one element past a 16-byte boundary
+        pad = 1 if misaligned else 0
+        t = torch.empty(x.size + pad, dtype=torch.complex64, device="cuda")[pad:].view(x.shape)
+        return t.copy_(torch.from_numpy(x))
+
+    c = dev(np.full((batch, 2 ** (nm + nn)), np.nan, dtype=np.complex64))
+    return (a, a_w, b, b_w, c_w), (dev(a), a_w, dev(b), b_w, c, c_w)
+
+
+@pytest.mark.parametrize("misaligned", [False, True])
+@pytest.mark.parametrize("layout", ["kfast", "random"])
+@pytest.mark.parametrize("shape,batch", [
+    ((5, 5, 5), 1), ((4, 6, 5), 3), ((6, 7, 4), 2), ((0, 1, 0), 1), ((5, 0, 5), 1),        # 32x32: one tile, one chunk
+    ((6, 6, 6), 1), ((5, 8, 5), 1), ((7, 10, 6), 1), ((3, 13, 2), 5), ((6, 8, 1), 7),      # split-K clusters of 2, 4, 8
+    ((3, 2, 17), 1), ((10, 5, 5), 20),                                                      # many 32x32 tiles
+    ((7, 3, 6), 130), ((12, 4, 9), 1), ((8, 2, 13), 3),                                     # 128x64: short and whole k
+    ((14, 3, 2), 2), ((15, 5, 1), 1), ((9, 4, 0), 200), ((12, 6, 4), 5), ((13, 1, 3), 9),  # 256x4 and 128x16
+    ((6, 4, 8), 33), ((5, 6, 9), 70)])                                                      # 64x64
+def test_fp32_tilings_at_their_edges(env, shape, batch, layout, misaligned):
+    """Every CUDA-core tiling the dispatch rule picks, at tile edges, with part
+    tiles, k split over thread groups and clusters, and operands that rule
+    16-byte loads out: within the rounding bound of FP32 sums in any order,
+    |error| <= (2 k + 2) u sum |a| |b|, u = 2^-24 (each component is a sum of 2k
+    products)."""
+    tn, torch = env
+    (a, a_w, b, b_w, c_w), dev = _pair_case(torch, shape, batch, layout, sum(shape) * 100 + batch, misaligned)
+    tn.contract_pair(*dev, batch=batch)
+    tn.device_sync()
+    got = dev[4].cpu().numpy()
+    for i in range(batch):
+        want = pairwise.contract_pair(a[i].astype(np.complex128), a_w, b[i].astype(np.complex128), b_w, c_w)
+        mag = pairwise.contract_pair(np.abs(a[i]).astype(np.complex128), a_w, np.abs(b[i]).astype(np.complex128), b_w,
+                                     c_w).real
+        bound = (2 * 2 ** shape[1] + 2) * 2.0 ** -24 * mag
+        assert np.all(np.abs(got[i].real - want.real) <= bound)
+        assert np.all(np.abs(got[i].imag - want.imag) <= bound)
