@@ -181,7 +181,7 @@ typedef struct tn_plan_stats {
     int64_t  arena_bytes;            /* device arena of one chunk */
     int32_t  k_histogram[40];        /* steps per log2(contracted size k), as figure S4 */
     int32_t  complex_mult;
-    int32_t  n_kernel_launches_per_chunk;  /* before kernels are chosen: slice-dependent steps + 4
+    int32_t  n_kernel_launches_per_chunk;  /* before kernels are chosen: slice-dependent steps + 2
                                               (tn_plan_chunk_launches gives the exact count) */
 } tn_plan_stats;
 
@@ -357,17 +357,16 @@ tn_status tn_plan_rank(const tn_network_t* net, const tn_plan_opts* opts, int32_
 /* Kernels one chunk launches with the kernels chosen so far (after the first
  * tn_contract_slices call; TN_ERR_ARG before): leaf select, every
  * slice-dependent step's kernels (tensor-core steps: B' image + GEMM [+ split-K
- * reduction]; CUDA-core steps: one), the two slice-sum kernels and the chunk
- * advance.  Steps that depend on no slice run once per plan or per batch and
- * are not counted.  Host only. */
+ * reduction]; CUDA-core steps: one) and the slice sum.  Steps that depend on no
+ * slice run once per plan or per batch and are not counted.  Host only. */
 tn_status tn_plan_chunk_launches(const tn_plan_t* plan, int32_t* launches);
 
 /* Kernels the per-batch prologue launches (after the first tn_contract_slices
  * call; TN_ERR_ARG before): the steps that depend on the closed output bits
  * but on no slice run once for every new batch bitstring (main text, section
  * III: the part of the network shared by a batch's slices is contracted once),
- * each with its kernels as in tn_plan_chunk_launches, after one leaf select;
- * 0 when the plan has no such step.  Host only. */
+ * each with its kernels as in tn_plan_chunk_launches, on the leaf select of
+ * the batch's first chunk; 0 when the plan has no such step.  Host only. */
 tn_status tn_plan_batch_launches(const tn_plan_t* plan, int32_t* launches);
 
 /* Wait for the plan's work on `stream` and return its sticky device error, if any. */

@@ -8,50 +8,73 @@
 namespace tnx {
 
 // Materialise every leaf of the chunk: the sliced wires take the bits of the
-// slice id, the closed output wires the bits of the batch's bitstring.
-__global__ void k_leaf_select(const float2* __restrict__ leaf_data, const LeafDesc* __restrict__ leaves,
-                              int n_leaves, float2* __restrict__ arena, const ChunkParam* __restrict__ params,
-                              const unsigned* __restrict__ counter) {
-  const ChunkParam p = params[*counter];
+// slice id, the closed output wires the bits of the batch's bitstring.  Also
+// clears amax[z0, z1) (FP16 split: the maxima the coming steps record).
+__global__ void __launch_bounds__(128) k_leaf_select(const float2* __restrict__ leaf_data,
+                                                     const LeafDesc* __restrict__ leaves, int n_leaves,
+                                                     float2* __restrict__ arena, const ChunkParam* __restrict__ params,
+                                                     const unsigned* __restrict__ counter, float* amax, int z0, int z1) {
+  __shared__ LeafDesc d;
+  static_assert(sizeof(LeafDesc) % 4 == 0, "LeafDesc is copied in 4-byte words");
+  bool waited = false;
+  ChunkParam p{};
   for (int li = blockIdx.x; li < n_leaves; li += gridDim.x) {
-    const LeafDesc& d = leaves[li];
+    __syncthreads();
+    for (int w = threadIdx.x; w < (int)(sizeof(LeafDesc) / 4); w += blockDim.x)
+      reinterpret_cast<uint32_t*>(&d)[w] = reinterpret_cast<const uint32_t*>(leaves + li)[w];
+    __syncthreads();
+    if (!waited) {
+      pdl_wait();
+      p = params[__ldcg(counter)];
+      for (int i = z0 + blockIdx.x * blockDim.x + threadIdx.x; i < z1; i += gridDim.x * blockDim.x) amax[i] = 0.f;
+      waited = true;
+    }
     const int rank = d.rank;
     const int64_t per = (int64_t)1 << rank;
     const int nbat = __popc(d.bmask);
     const int64_t total = per << nbat;
+    // the bits every instance shares, and those that an instance's batch bits set
+    int64_t fix0 = 0;
+    for (int f = 0; f < d.nfixed; ++f) {
+      const int idx = d.fixed_index[f];
+      const uint64_t v = d.fixed_kind[f] == 0 ? ((p.slice_base >> idx) & 1) : ((p.bitstring >> idx) & 1);
+      fix0 |= (int64_t)v << f;
+    }
     for (int64_t e = threadIdx.x; e < total; e += blockDim.x) {
       const uint32_t inst = (uint32_t)(e >> rank);
       const int64_t i = e & (per - 1);
-      uint64_t sid = p.slice_base;
-      for (int t = 0; t < nbat; ++t) sid |= (uint64_t)((inst >> t) & 1u) << d.bslice[t];
-      int64_t fix = 0;
-      for (int f = 0; f < d.nfixed; ++f) {
-        const int idx = d.fixed_index[f];
-        const uint64_t v = d.fixed_kind[f] == 0 ? ((sid >> idx) & 1) : ((p.bitstring >> idx) & 1);
-        fix |= (int64_t)v << f;
-      }
+      int64_t fix = fix0;
+      for (int t = 0; t < nbat; ++t)
+        if ((inst >> t) & 1u)
+          for (int f = 0; f < d.nfixed; ++f)
+            if (d.fixed_kind[f] == 0 && d.fixed_index[f] == d.bslice[t]) fix |= (int64_t)1 << f;
       arena[d.dst_off + e] = leaf_data[d.src_off + fix * per + i];
     }
   }
+  if (!waited) pdl_wait();
 }
 
 // Slice sum of a chunk (main text, section II: the sliced network is the sum of
-// the smaller networks), FP64, in two deterministic passes: k_root_partial sums
-// the slices of group g (slices g*per .. g*per+per-1 of the chunk) for every
-// amplitude j into part[g][j]; k_root_finish adds the groups in order into
-// out[batch][j].  Slices outside the call's range are skipped.
-__global__ void __launch_bounds__(256) k_root_partial(const float2* __restrict__ arena, const RootDesc r, int b,
-                                                     int groups, double2* __restrict__ part,
-                                                     const ChunkParam* __restrict__ params,
-                                                     const unsigned* __restrict__ counter) {
+// the smaller networks) in FP64, deterministic: block (x, g) sums the slices of
+// group g (slices g*per .. g*per+per-1 of the chunk) for its amplitudes j into
+// part[g][j]; the last of the groups' blocks to arrive for the same amplitudes
+// (tickets[x]) adds the groups in order into out[batch][j], and the last block
+// of all advances the chunk counter.  Slices outside the call's range are
+// skipped.  The tickets are zero between launches.
+__global__ void __launch_bounds__(256) k_root_sum(const float2* __restrict__ arena, const RootDesc r, int b,
+                                                 int groups, double2* __restrict__ part,
+                                                 const ChunkParam* __restrict__ params, unsigned* counter,
+                                                 unsigned* tickets) {
   // the group's slices in rounds of 256: their instance offsets in the root
   // (or -1 outside the call's range) are found once per block, then every
   // thread adds its amplitudes over them with four independent FP64
   // accumulators (slice i of a round goes to accumulator i % 4), combined in a
-  // fixed order, so the sum is deterministic.  256 threads, s_off has 256
-  // entries: cnt <= 256 and its padding to a multiple of 4 stays <= 256
+  // fixed order.  256 threads, s_off has 256 entries: cnt <= 256 and its padding
+  // to a multiple of 4 stays <= 256
   __shared__ int64_t s_off[256];
-  const ChunkParam p = params[*counter];
+  __shared__ int s_last;
+  pdl_wait();
+  const ChunkParam p = params[__ldcg(counter)];   // the counter changes under a running kernel: past L1
   const int k = r.rank;
   const int64_t nout = (int64_t)1 << k;
   const uint32_t per = (1u << b) / (uint32_t)groups;
@@ -124,28 +147,42 @@ __global__ void __launch_bounds__(256) k_root_partial(const float2* __restrict__
                                                    (ai[t][0] + ai[t][1]) + (ai[t][2] + ai[t][3]));
       }
   }
-}
-
-__global__ void k_root_finish(const double2* __restrict__ part, int groups, int k,
-                              const ChunkParam* __restrict__ params, const unsigned* __restrict__ counter) {
-  const ChunkParam p = params[*counter];
+  // the last group's block for these amplitudes sums the groups
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&tickets[1 + blockIdx.x], 1u) == (unsigned)groups - 1u;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
   double* __restrict__ out = p.out;
-  const int64_t nout = (int64_t)1 << k;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nout;
-       j += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t j = j0; j < nout; j += jstep) {
     double sr = 0.0, si = 0.0;
-    for (int g = 0; g < groups; ++g) {
-      const double2 v = part[(int64_t)g * nout + j];
-      sr += v.x;
-      si += v.y;
+    // eight loads in flight, added in group order
+    for (int q0 = 0; q0 < groups; q0 += 8) {
+      double2 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        v[u] = q0 + u < groups ? __ldcg(part + (int64_t)(q0 + u) * nout + j) : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (q0 + u < groups) {
+          sr += v[u].x;
+          si += v[u].y;
+        }
     }
     double* o = out + 2 * (p.out_index * nout + j);
     o[0] += sr;
     o[1] += si;
   }
+  if (threadIdx.x == 0) {
+    tickets[1 + blockIdx.x] = 0;
+    // all blocks have read the counter: each did before its arrival above
+    if (atomicAdd(&tickets[0], 1u) == gridDim.x - 1u) {
+      tickets[0] = 0;
+      *counter += 1u;
+    }
+  }
 }
-
-__global__ void k_advance(unsigned* counter) { *counter += 1u; }
 
 // Largest |re|, |im| over n complex values, raised into *out (which the caller
 // zeroes first): the FP16 split's scale of an operand without a producer.

@@ -207,6 +207,7 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
   const int64_t bbase = warp_deposit((uint32_t)by, g.b_npos, g.tn, g.nn) + warp_deposit((uint32_t)kc0, g.b_kpos, g.tk, g.nk);
   const int64_t cbase = warp_deposit((uint32_t)bx, g.c_mpos, g.tm, g.nm) + warp_deposit((uint32_t)by, g.c_npos, g.tn, g.nn);
   __syncthreads();
+  pdl_wait();
 
   float am = 0.f;   // largest component written (for the FP16 split's scaling)
   // every CTA of a cluster goes through the same number of rounds (the cluster

@@ -500,13 +500,14 @@ __global__ void __launch_bounds__(256) k_tc_prep_b(const TcArgs a) {
   const int64_t block_bytes = (int64_t)T::NPL * plane;
   const int per_block = ncp * CPR;              // chunks per plane
   const int tkv = 1 << g.tk, tnv = 1 << a.tnb;
-  const float sc = operand_scale<MODE>(g.amax_b);
   // offsets in B of the k inside a chunk and of the n inside a tile (-1: padding)
   __shared__ int64_t koff[TC_TK];
   __shared__ int64_t noff[128];
   for (int i = threadIdx.x; i < TC_TK; i += blockDim.x) koff[i] = i < tkv ? deposit_hi((uint64_t)i, g.b_kpos, 0, g.tk) : -1;
   for (int i = threadIdx.x; i < 128; i += blockDim.x) noff[i] = i < tnv ? deposit_hi((uint64_t)i, g.b_npos, 0, a.tnb) : -1;
   __syncthreads();
+  pdl_wait();
+  const float sc = operand_scale<MODE>(g.amax_b);
   const int64_t n_blocks = (int64_t)g.n_inst << (a.ls_nt + a.ls_kc);
   // one CTA per (instance, n tile, k chunk) block at a time; threads walk the
   // block's 16-byte chunks in memory order of the image
@@ -566,12 +567,13 @@ __global__ void __launch_bounds__(256) k_tc_prep_b3(const TcArgs a) {
   const int per_block = P::PLANES * rows * CPR;
   const int per_plane = rows * CPR;
   const int tkv = 1 << g.tk, tnv = 1 << a.tnb;
-  const float sc = operand_scale<MODE>(g.amax_b);
   __shared__ int64_t koff[TC_TK];
   __shared__ int64_t noff[128];
   for (int i = threadIdx.x; i < TC_TK; i += blockDim.x) koff[i] = i < tkv ? deposit_hi((uint64_t)i, g.b_kpos, 0, g.tk) : -1;
   for (int i = threadIdx.x; i < 128; i += blockDim.x) noff[i] = i < tnv ? deposit_hi((uint64_t)i, g.b_npos, 0, a.tnb) : -1;
   __syncthreads();
+  pdl_wait();
+  const float sc = operand_scale<MODE>(g.amax_b);
   const int64_t n_blocks = (int64_t)g.n_inst << (a.ls_nt + a.ls_kc);
   for (int64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
     const int kc = (int)(blk & (a.n_kc - 1));
@@ -629,6 +631,7 @@ __global__ void __launch_bounds__(256) k_tc_prep_b3(const TcArgs a) {
 // Split-K: C[i] = sum over splits of the partials, in split order.
 __global__ void k_split_reduce(const float2* __restrict__ part, int n_split, int64_t stride,
                                float2* __restrict__ C, int64_t n, float* amax_c) {
+  pdl_wait();
   float am = 0.f;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     float2 acc = part[i];
@@ -680,9 +683,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
     const int64_t sp = gi & (int64_t)(a.n_split - 1), rest = gi >> a.ls_split;
     return sp | ((j & (int64_t)(a.n_nt - 1)) << a.ls_split) | (rest << (a.ls_split + a.ls_nt));
   };
-  // FP16X3: A and B enter scaled by 2^sa, 2^sb; the epilogue multiplies by 2^-sa 2^-sb (exact)
-  const float sc_a = operand_scale<MODE>(g.amax_a);
-  const float us_a = 1.f / sc_a, us_b = 1.f / operand_scale<MODE>(g.amax_b);
   const int b_slot = P::PLANES * b_plane;
   const int64_t b_slot_g = (int64_t)P::PLANES * b_plane_g;
   const int na = a.na, nbs = a.nbs;
@@ -750,6 +750,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
   if constexpr (PAIR) cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // everything above ran under the kernel before this one
+  pdl_wait();
+  // FP16X3: A and B enter scaled by 2^sa, 2^sb; the epilogue multiplies by 2^-sa 2^-sb (exact)
+  const float sc_a = operand_scale<MODE>(g.amax_a);
+  const float us_a = 1.f / sc_a, us_b = 1.f / operand_scale<MODE>(g.amax_b);
   const int kc_n = a.n_kc;
   const int kc_per = a.n_kc / a.n_split;
 

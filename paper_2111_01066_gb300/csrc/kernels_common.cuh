@@ -5,6 +5,25 @@
 
 namespace tnx {
 
+// Programmatic dependent launch.  Every kernel of a plan or a pairwise
+// contraction is launched with the stream-serialisation attribute: it may start
+// once every CTA of the kernel before it has passed its own pdl_wait, sets itself
+// up under that kernel's run, and waits here until that kernel has completed and
+// its writes are visible.  Before pdl_wait a kernel touches only its arguments,
+// tables written when the plan was built, and its own shared and tensor memory;
+// every thread that touches anything else passes it, so a kernel's completion
+// implies that of all kernels before it.  The next kernel is let go after the
+// wait, not before it: no CTA is then resident while the kernel two before its
+// own still runs, so its first-level cache holds nothing that the kernel before
+// it has overwritten since (read-only loads stay safe).  Without the attribute
+// (a launch outside such a chain) both instructions are no-ops.
+// A chain of small kernels costs 4-6 us a link without it (launch, arguments,
+// decode tables, then the work).
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Per-chunk parameters, read by the kernels from device memory at
 // params[*counter] so that one captured launch sequence serves every chunk.
 struct ChunkParam {

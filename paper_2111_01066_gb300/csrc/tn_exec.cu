@@ -148,24 +148,31 @@ static GemmArgs make_args(const StepDesc& d, int kid, const float2* A, const flo
   return g;
 }
 
-template <class Cfg>
-static void launch_simt_cfg(const GemmArgs& g, dim3 grid, int split, cudaStream_t s) {
-  if (split == 1) {
-    k_cgemm_simt<Cfg><<<grid, SIMT_THREADS, 0, s>>>(g, 1);
-    return;
-  }
+// Launch with programmatic dependent launch where `overlap` (the kernel calls
+// pdl_wait), on clusters of `cluster` CTAs along x where that is above 1.
+template <class... KArgs, class... Args>
+static void klaunch(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t s, int cluster,
+                    bool overlap, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(SIMT_THREADS);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)split;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
-  CK(cudaLaunchKernelEx(&cfg, k_cgemm_simt<Cfg>, g, split));
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  CK(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
+}
+
+template <class Cfg>
+static void launch_simt_cfg(const GemmArgs& g, dim3 grid, int split, cudaStream_t s) {
+  klaunch(k_cgemm_simt<Cfg>, grid, SIMT_THREADS, 0, s, split, true, g, split);
 }
 static void launch_simt(const GemmArgs& g, int kid, cudaStream_t s) {
   if (g.n_inst <= 0) return;
@@ -440,10 +447,15 @@ template <int MODE, int CM>
 static void launch_prep(const TcArgs& t, cudaStream_t s) {
   const int64_t n_blocks = (int64_t)t.g.n_inst * t.n_nt * t.n_kc;
   const int pgrid = (int)std::max<int64_t>(1, std::min<int64_t>(n_blocks, (int64_t)sm_count() * 16));
+  // started under the kernel before it only while it has at most a CTA per SM:
+  // beside a resident GEMM the SM's L1 is a few KB, and a larger grid, which
+  // reads every B entry several times, is slower there than it gains (45 3M
+  // instances of 512 x 256 x 128: 47.8 us a call without the overlap, 55.7 with)
+  const bool overlap = n_blocks <= sm_count();
   if constexpr (CM == 4)
-    k_tc_prep_b<MODE><<<pgrid, 256, 0, s>>>(t);
+    klaunch(k_tc_prep_b<MODE>, dim3(pgrid), 256, 0, s, 1, overlap, t);
   else
-    k_tc_prep_b3<MODE><<<pgrid, 256, 0, s>>>(t);
+    klaunch(k_tc_prep_b3<MODE>, dim3(pgrid), 256, 0, s, 1, overlap, t);
 }
 static void launch_prep_kid(const TcArgs& t, int kid, cudaStream_t s) {
   switch (kid) {
@@ -485,26 +497,16 @@ static void launch_tc(const TcArgs& t, const StepLaunch& L, int grid, cudaStream
   if constexpr (PAIR) {
     // clusters of two CTAs, each pair persistent over the work units
     const int clusters = (int)std::min<int64_t>(t.n_tiles, pair_clusters<MODE, PAIR>());
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * clusters);
-    cfg.blockDim = dim3(TC_THREADS);
-    cfg.dynamicSmemBytes = L.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    CK(cudaLaunchKernelEx(&cfg, k_cgemm_tc<MODE, CM, PAIR>, t, L.tma));
+    klaunch(k_cgemm_tc<MODE, CM, PAIR>, dim3(2 * clusters), TC_THREADS, L.smem, s, 2, true, t, L.tma);
   } else {
-    k_cgemm_tc<MODE, CM, PAIR><<<grid, TC_THREADS, L.smem, s>>>(t, L.tma);
+    klaunch(k_cgemm_tc<MODE, CM, PAIR>, dim3(grid), TC_THREADS, L.smem, s, 1, true, t, L.tma);
   }
 }
 
-static void launch_step(StepLaunch& L, uint8_t* ws, int32_t* err, cudaStream_t s) {
-  if (L.g.amax_c) CK(cudaMemsetAsync(L.g.amax_c, 0, sizeof(float), s));   // the result's maximum, recorded anew
+// clear_amax: the step's recorded maximum starts at zero here (in a chunk or a
+// prologue the leaf select has cleared it)
+static void launch_step(StepLaunch& L, uint8_t* ws, int32_t* err, cudaStream_t s, bool clear_amax) {
+  if (L.g.amax_c && clear_amax) CK(cudaMemsetAsync(L.g.amax_c, 0, sizeof(float), s));   // the result's maximum, recorded anew
   if (!is_tc(L.kid)) {
     launch_simt(L.g, L.kid, s);
     return;
@@ -546,7 +548,8 @@ static void launch_step(StepLaunch& L, uint8_t* ws, int32_t* err, cudaStream_t s
   }
   if (t.n_split > 1) {
     const int rb = (int)std::min<int64_t>((L.c_total + 255) / 256, (int64_t)sm_count() * 8);
-    k_split_reduce<<<rb, 256, 0, s>>>(t.c_part, t.n_split, t.c_part_stride, t.g.C, L.c_total, t.g.amax_c);
+    klaunch(k_split_reduce, dim3(rb), 256, 0, s, 1, true, (const float2*)t.c_part, (int)t.n_split, t.c_part_stride, t.g.C,
+            L.c_total, t.g.amax_c);
   }
 }
 
@@ -563,6 +566,8 @@ struct DeviceState {
   uint8_t* ws = nullptr;
   int64_t ws_bytes = 0;           // capacity of ws
   double2* root_part = nullptr;   // [groups][2^k] partial slice sums
+  unsigned* root_tickets = nullptr;   // arrivals of the slice sum's blocks (zero between launches)
+  int root_blocks = 1;
   float* amax = nullptr;          // FP16X3: largest component of every node (leaves, then steps)
   int root_groups = 1;
   std::vector<StepLaunch> launches;
@@ -580,7 +585,6 @@ struct DeviceState {
       int32_t* start = nullptr;                // device: n + 1 block offsets
       int8_t* tiling = nullptr;                // device: n CUDA-core tilings (simt_multi_tiling)
       int8_t* split = nullptr;                 // device: n split-K factors
-      std::vector<float*> amax;                // FP16X3: result maxima to clear first
     };
     std::vector<Multi> multi;
   };
@@ -590,11 +594,12 @@ struct DeviceState {
   std::vector<uint8_t*> own_imgs;              // B' images built ahead of the chunks (StepLaunch::bimg_own)
   cudaEvent_t done = nullptr;
   bool have_done = false;
-  // the chunk's launch sequence as one CUDA graph, captured after the first
-  // eager chunk; every kernel reads its chunk parameters from device memory
-  cudaGraphExec_t graph = nullptr;
-  bool graph_failed = false;
-  bool eager_done = false;
+  // launch sequences as CUDA graphs, each captured at its second use (the first
+  // runs eagerly): [0] a chunk, [1] a chunk that opens a new batch, with the
+  // batch's prologue; every kernel reads its chunk parameters from device memory
+  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  bool graph_failed[2] = {false, false};
+  bool eager_done[2] = {false, false};
   // prologues: steps whose result depends on no slice run once per plan
   // (dependence flags 0) or once per batch bitstring (flags 2); their results
   // that later steps read sit in the arena's persistent pool
@@ -637,20 +642,8 @@ static int simt_multi_tiling(int kid) {
 }
 
 static void launch_simt_multi(const DeviceState::GroupRun::Multi& m, cudaStream_t s) {
-  for (float* am : m.amax) CK(cudaMemsetAsync(am, 0, sizeof(float), s));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)m.blocks);
-  cfg.blockDim = dim3(SIMT_THREADS);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = SIMT_MAX_SPLIT;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  CK(cudaLaunchKernelEx(&cfg, k_cgemm_simt_multi, (const GemmArgs*)m.args, (const int32_t*)m.start,
-                        (const int8_t*)m.tiling, (const int8_t*)m.split, (int32_t)m.n));
+  klaunch(k_cgemm_simt_multi, dim3((unsigned)m.blocks), SIMT_THREADS, 0, s, SIMT_MAX_SPLIT, true,
+          (const GemmArgs*)m.args, (const int32_t*)m.start, (const int8_t*)m.tiling, (const int8_t*)m.split, (int32_t)m.n);
 }
 
 // Dependence flags of a node (bit 0: on the slice id, bit 1: on the closed
@@ -765,7 +758,6 @@ static void build_groups(Plan& p, DeviceState& ds) {
       if (blocks + nb > 0x7fffffff) fail(TN_ERR_UNSUPPORTED, "step group grid too large");
       std::memcpy(host.data() + start_off + q * sizeof(int32_t), &blocks, sizeof(int32_t));
       blocks += (int32_t)nb;
-      if (g.amax_c) m.amax.push_back(g.amax_c);
     }
     std::memcpy(host.data() + start_off + pm.second.size() * sizeof(int32_t), &blocks, sizeof(int32_t));
     m.blocks = blocks;
@@ -849,10 +841,22 @@ static void ensure_device(Plan& p) {
   ds->ws_bytes = ws;
   ds->root_groups = std::min(1 << p.log2_batch, 64);
   CK(cudaMalloc(&ds->root_part, sizeof(double2) * (size_t)ds->root_groups << p.root.rank));
+  ds->root_blocks = (int)std::min<int64_t>((((int64_t)1 << p.root.rank) + 255) / 256, 4096);
+  CK(cudaMalloc(&ds->root_tickets, sizeof(unsigned) * (size_t)(1 + ds->root_blocks)));
+  CK(cudaMemset(ds->root_tickets, 0, sizeof(unsigned) * (size_t)(1 + ds->root_blocks)));
   if (!in_arena(p.root.off, (int64_t)1 << p.root.rank, 1 << __builtin_popcount(p.root.bmask)))
     fail(TN_ERR_PLAN, "internal: root outside the arena");
   build_groups(p, *ds);
   setup_hoisted(p, *ds);
+}
+
+static void drop_graphs(DeviceState& ds) {
+  for (int w = 0; w < 2; ++w) {
+    if (ds.graph[w]) cudaGraphExecDestroy(ds.graph[w]);
+    ds.graph[w] = nullptr;
+    ds.graph_failed[w] = false;
+    ds.eager_done[w] = false;
+  }
 }
 
 void destroy_device_state(Plan* p) {
@@ -870,10 +874,11 @@ void destroy_device_state(Plan* p) {
   cudaFree(ds->err);
   cudaFree(ds->ws);
   cudaFree(ds->root_part);
+  cudaFree(ds->root_tickets);
   cudaFree(ds->amax);
   cudaFree(ds->group_buf);
   for (uint8_t* b : ds->own_imgs) cudaFree(b);
-  if (ds->graph) cudaGraphExecDestroy(ds->graph);
+  drop_graphs(*ds);
   if (ds->done) cudaEventDestroy(ds->done);
   cudaSetDevice(cur);
   delete ds;
@@ -890,43 +895,55 @@ static void launch_class(Plan& p, cudaStream_t s, Pred in_class) {
     if (!in_class(p.steps[i].dep_flags)) continue;
     const int gi = ds.group_at.empty() ? -1 : ds.group_at[i];
     if (gi < 0) {
-      launch_step(ds.launches[i], ds.ws, ds.err, s);
+      launch_step(ds.launches[i], ds.ws, ds.err, s, false);
       continue;
     }
     const DeviceState::GroupRun& gr = ds.groups[gi];
     for (const auto& m : gr.multi) launch_simt_multi(m, s);
-    for (int t : gr.singles) launch_step(ds.launches[t], ds.ws, ds.err, s);
+    for (int t : gr.singles) launch_step(ds.launches[t], ds.ws, ds.err, s, false);
     i = (size_t)gr.end - 1;
   }
 }
 
-static void run_chunk(Plan& p, cudaStream_t s) {
+// Leaf select with the current chunk's parameters.  FP16X3: it also clears the
+// maxima that the steps of the coming classes record (classes: bit 0
+// slice-dependent steps, bit 1 per-batch ones; 0 the per-plan ones); the
+// execution order keeps each class's steps together.
+static void launch_leaf_select(Plan& p, cudaStream_t s, int classes) {
   DeviceState& ds = *p.dev;
   const int nl = (int)p.leaves.size();
-  k_leaf_select<<<std::max(1, std::min(nl, 4096)), 128, 0, s>>>(ds.leaf_data, ds.leaf_desc, nl, ds.arena,
-                                                                 ds.params, ds.counter);
-  launch_class(p, s, [](int f) { return (f & 1) != 0; });   // slice-dependent steps
-  const int64_t nout = (int64_t)1 << p.root.rank;
-  const int blocks = (int)std::min<int64_t>((nout + 255) / 256, 4096);
-  k_root_partial<<<dim3(blocks, ds.root_groups), 256, 0, s>>>(ds.arena, p.root, p.log2_batch, ds.root_groups,
-                                                               ds.root_part, ds.params, ds.counter);
-  k_root_finish<<<blocks, 256, 0, s>>>(ds.root_part, ds.root_groups, p.root.rank, ds.params, ds.counter);
-  k_advance<<<1, 1, 0, s>>>(ds.counter);
+  int z0 = 0, z1 = 0;
+  if (ds.amax) {
+    for (int i = 0; i < (int)p.steps.size(); ++i) {
+      const int f = p.steps[i].dep_flags;
+      const bool in = classes == 0 ? f == 0 : ((f & 1) && (classes & 1)) || (f == 2 && (classes & 2));
+      if (!in) continue;
+      if (z1 == 0) z0 = nl + i;
+      else if (z1 != nl + i) fail(TN_ERR_PLAN, "internal: steps of a class are not consecutive");
+      z1 = nl + i + 1;
+    }
+  }
+  klaunch(k_leaf_select, dim3((unsigned)std::max(1, std::min(nl, 4096))), 128, 0, s, 1, true,
+          (const float2*)ds.leaf_data,
+          (const LeafDesc*)ds.leaf_desc, nl, ds.arena, (const ChunkParam*)ds.params, (const unsigned*)ds.counter,
+          ds.amax, z0, z1);
 }
 
-// The steps of one dependence class (0: neither slice nor bitstring, 2:
-// bitstring only), after a leaf select with the current chunk's parameters.
+// Whether a class has anything to run: 0, steps that depend on neither the
+// slice nor the bitstring; 2, on the bitstring only; and the B' images of later
+// steps whose B that class completes.
+static bool has_prologue(const Plan& p, int cls) {
+  for (const StepDesc& d : p.steps)
+    if (d.dep_flags == cls) return true;
+  for (const StepLaunch& L : p.dev->launches)
+    if (L.bimg_own && L.bimg_cls == cls) return true;
+  return false;
+}
+
+// The steps and B' images of one prologue class, on the leaves already selected.
 static void run_prologue(Plan& p, cudaStream_t s, int cls) {
   DeviceState& ds = *p.dev;
-  bool any = false;
-  for (const StepDesc& d : p.steps) any = any || d.dep_flags == cls;
-  for (const StepLaunch& L : ds.launches) any = any || (L.bimg_own && L.bimg_cls == cls);
-  if (!any) return;
-  const int nl = (int)p.leaves.size();
-  k_leaf_select<<<std::max(1, std::min(nl, 4096)), 128, 0, s>>>(ds.leaf_data, ds.leaf_desc, nl, ds.arena,
-                                                                 ds.params, ds.counter);
   launch_class(p, s, [cls](int f) { return f == cls; });
-  // the B' images of later steps whose B this class completes
   for (const StepLaunch& L : ds.launches) {
     if (!L.bimg_own || L.bimg_cls != cls) continue;
     TcArgs t = L.tc;
@@ -936,34 +953,48 @@ static void run_prologue(Plan& p, cudaStream_t s, int cls) {
   }
 }
 
+// One chunk; new_batch: with the batch's prologue, which works on the same leaf
+// select (the arena gives no leaf away before its last reader, and the prologue's
+// steps come before the chunk's in the order it was laid out for).
+static void run_chunk(Plan& p, cudaStream_t s, bool new_batch) {
+  DeviceState& ds = *p.dev;
+  launch_leaf_select(p, s, new_batch ? 3 : 1);
+  if (new_batch) run_prologue(p, s, 2);
+  launch_class(p, s, [](int f) { return (f & 1) != 0; });   // slice-dependent steps
+  klaunch(k_root_sum, dim3((unsigned)ds.root_blocks, (unsigned)ds.root_groups), 256, 0, s, 1, true,
+          (const float2*)ds.arena, p.root, p.log2_batch, ds.root_groups, ds.root_part, (const ChunkParam*)ds.params,
+          ds.counter, ds.root_tickets);
+}
+
 // Capture run_chunk once into a graph (on a private stream, thread-local
 // capture mode).  Any failure leaves the plan on eager launches.
-static void capture_chunk_graph(Plan& p) {
+static void capture_chunk_graph(Plan& p, bool new_batch) {
   DeviceState& ds = *p.dev;
-  if (ds.graph || ds.graph_failed) return;
+  const int w = new_batch ? 1 : 0;
+  if (ds.graph[w] || ds.graph_failed[w]) return;
   cudaStream_t cs = nullptr;
   if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
-    ds.graph_failed = true;
+    ds.graph_failed[w] = true;
     return;
   }
   cudaGraph_t graph = nullptr;
   bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
   if (ok) {
     try {
-      run_chunk(p, cs);
+      run_chunk(p, cs, new_batch);
     } catch (const TnError&) {
       ok = false;
     }
     ok = (cudaStreamEndCapture(cs, &graph) == cudaSuccess) && ok;
   }
-  if (ok) ok = cudaGraphInstantiate(&ds.graph, graph, 0) == cudaSuccess;
+  if (ok) ok = cudaGraphInstantiate(&ds.graph[w], graph, 0) == cudaSuccess;
   if (graph) cudaGraphDestroy(graph);
   cudaStreamDestroy(cs);
   if (!ok) {
     cudaGetLastError();
-    ds.graph = nullptr;
-    ds.graph_failed = true;
+    ds.graph[w] = nullptr;
+    ds.graph_failed[w] = true;
   }
 }
 
@@ -1021,6 +1052,7 @@ extern "C" tn_status tn_contract_slices(tn_plan_t* h, uint64_t first, uint64_t c
   if (prm.size() > ds.params_cap) {
     if (ds.params) {
       CK(cudaStreamSynchronize(s));
+      drop_graphs(ds);   // captured with the old buffer's address
       CK(cudaFree(ds.params));
       ds.params = nullptr;
     }
@@ -1029,31 +1061,32 @@ extern "C" tn_status tn_contract_slices(tn_plan_t* h, uint64_t first, uint64_t c
   }
   CK(cudaMemcpyAsync(ds.params, prm.data(), prm.size() * sizeof(ChunkParam), cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(ds.counter, 0, sizeof(unsigned), s));
+  if (!ds.pro0_done) {
+    if (has_prologue(p, 0)) {
+      launch_leaf_select(p, s, 0);
+      run_prologue(p, s, 0);
+    }
+    ds.pro0_done = true;
+  }
+  const bool pro2 = has_prologue(p, 2);
   for (size_t c = 0; c < prm.size(); ++c) {
-    if (c == 0 || prm[c].out_index != prm[c - 1].out_index) {   // first chunk of a batch
-      if (!ds.pro0_done) {
-        run_prologue(p, s, 0);
-        ds.pro0_done = true;
-      }
-      if (!ds.pro2_valid || ds.pro2_bits != prm[c].bitstring) {
-        run_prologue(p, s, 2);
-        ds.pro2_valid = true;
-        ds.pro2_bits = prm[c].bitstring;
-      }
-      CK(cudaGetLastError());
+    const bool new_batch = pro2 && (!ds.pro2_valid || ds.pro2_bits != prm[c].bitstring);
+    const int w = new_batch ? 1 : 0;
+    if (!ds.eager_done[w]) {
+      run_chunk(p, s, new_batch);           // the first one runs eagerly (sets kernel attributes)
+      ds.eager_done[w] = true;
+    } else {
+      capture_chunk_graph(p, new_batch);
+      if (ds.graph[w])
+        CK(cudaGraphLaunch(ds.graph[w], s));
+      else
+        run_chunk(p, s, new_batch);
     }
-    if (!ds.eager_done) {
-      run_chunk(p, s);           // the first chunk runs eagerly (sets kernel attributes)
-      CK(cudaGetLastError());
-      ds.eager_done = true;
-      capture_chunk_graph(p);
-      continue;
-    }
-    if (ds.graph)
-      CK(cudaGraphLaunch(ds.graph, s));
-    else
-      run_chunk(p, s);
     CK(cudaGetLastError());
+    if (new_batch) {
+      ds.pro2_valid = true;
+      ds.pro2_bits = prm[c].bitstring;
+    }
   }
   CK(cudaEventRecord(ds.done, s));
   ds.have_done = true;
@@ -1074,9 +1107,9 @@ extern "C" tn_status tn_plan_step_times(tn_plan_t* h, int32_t reps, double* ms_o
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   for (size_t i = 0; i < p.steps.size(); ++i) {
-    launch_step(ds.launches[i], ds.ws, ds.err, s);  // warm-up
+    launch_step(ds.launches[i], ds.ws, ds.err, s, true);  // warm-up
     CK(cudaEventRecord(e0, s));
-    for (int r = 0; r < reps; ++r) launch_step(ds.launches[i], ds.ws, ds.err, s);
+    for (int r = 0; r < reps; ++r) launch_step(ds.launches[i], ds.ws, ds.err, s, true);
     CK(cudaEventRecord(e1, s));
     CK(cudaEventSynchronize(e1));
     float ms = 0;
@@ -1103,12 +1136,7 @@ static StepLaunch build_choice(const DeviceState& ds, const StepDesc& d, int kid
 static void kernels_changed(Plan& p, DeviceState& ds) {
   build_groups(p, ds);
   setup_hoisted(p, ds);
-  if (ds.graph) {
-    cudaGraphExecDestroy(ds.graph);
-    ds.graph = nullptr;
-  }
-  ds.graph_failed = false;
-  ds.eager_done = false;
+  drop_graphs(ds);
   ds.pro0_done = false;   // the arena may have been overwritten: prologues run again
   ds.pro2_valid = false;
 }
@@ -1144,9 +1172,9 @@ extern "C" tn_status tn_plan_autotune(tn_plan_t* h, int32_t reps, void* stream) 
       }
       ds.ws_bytes = L.ws_bytes;
     }
-    launch_step(L, ds.ws, ds.err, s);  // warm-up
+    launch_step(L, ds.ws, ds.err, s, true);  // warm-up
     CK(cudaEventRecord(e0, s));
-    for (int r = 0; r < reps; ++r) launch_step(L, ds.ws, ds.err, s);
+    for (int r = 0; r < reps; ++r) launch_step(L, ds.ws, ds.err, s, true);
     CK(cudaEventRecord(e1, s));
     CK(cudaEventSynchronize(e1));
     float ms = 0;
@@ -1401,7 +1429,7 @@ extern "C" tn_status tn_plan_chunk_launches(const tn_plan_t* h, int32_t* launche
   if (!h || !launches) fail(TN_ERR_ARG, "tn_plan_chunk_launches: NULL argument");
   const Plan& p = h->plan;
   if (!p.dev) fail(TN_ERR_ARG, "tn_plan_chunk_launches: call after the first tn_contract_slices");
-  *launches = 4 + class_launches(p, [](int f) { return (f & 1) != 0; });
+  *launches = 2 + class_launches(p, [](int f) { return (f & 1) != 0; });
   API_END
 }
 
@@ -1412,7 +1440,7 @@ extern "C" tn_status tn_plan_batch_launches(const tn_plan_t* h, int32_t* launche
   if (!p.dev) fail(TN_ERR_ARG, "tn_plan_batch_launches: call after the first tn_contract_slices");
   int n = class_launches(p, [](int f) { return f == 2; });
   for (const StepLaunch& L : p.dev->launches) n += (L.bimg_own && L.bimg_cls == 2) ? 1 : 0;   // B' images
-  *launches = n > 0 ? n + 1 : 0;   // + the leaf select ahead of them
+  *launches = n;   // on the leaf select of the batch's first chunk
   API_END
 }
 
@@ -1671,7 +1699,7 @@ extern "C" tn_status tn_contract_pair(const float* a, const int32_t* aw, int32_t
     CK(cudaMalloc(&sc.ws, (size_t)L.ws_bytes));
     sc.ws_bytes = L.ws_bytes;
   }
-  launch_step(L, sc.ws, sc.err, (cudaStream_t)stream);
+  launch_step(L, sc.ws, sc.err, (cudaStream_t)stream, true);
   CK(cudaGetLastError());
   API_END
 }
@@ -1797,7 +1825,7 @@ extern "C" tn_status tn_contract_pair_noalloc(const float* a, const int32_t* aw,
   if (g.amax_a)
     operand_maxima(reinterpret_cast<const float2*>(a), batch << ar, reinterpret_cast<const float2*>(b),
                    batch << br, amax, s);
-  launch_step(L, base + kNoAllocErrBytes, err, s);
+  launch_step(L, base + kNoAllocErrBytes, err, s, true);
   CK(cudaGetLastError());
   API_END
 }

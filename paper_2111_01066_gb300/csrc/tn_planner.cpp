@@ -1359,9 +1359,8 @@ extern "C" tn_status tn_plan_info(const tn_plan_t* h, tn_plan_stats* s) {
   for (int i = 0; i < 40; ++i) s->k_histogram[i] = p.stats.khist[i];
   s->complex_mult = p.opts.complex_mult;
   // steps that depend on the slice id run in every chunk (the others run once
-  // per plan or per batch); one kernel each at least, plus leaf select, the
-  // two slice-sum kernels and the chunk advance
-  int per_chunk = 4;
+  // per plan or per batch); one kernel each at least, plus leaf select and slice sum
+  int per_chunk = 2;
   for (const StepDesc& d : p.steps) per_chunk += (d.dep_flags & 1) ? 1 : 0;
   s->n_kernel_launches_per_chunk = per_chunk;
   return TN_OK;

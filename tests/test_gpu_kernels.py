@@ -65,3 +65,32 @@ def test_fp32_tilings_at_their_edges(env, shape, batch, layout, misaligned):
         bound = (2 * 2 ** shape[1] + 2) * 2.0 ** -24 * mag
         assert np.all(np.abs(got[i].real - want.real) <= bound)
         assert np.all(np.abs(got[i].imag - want.imag) <= bound)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16x3"])
+def test_chunk_graphs_across_calls(env, prec):
+    """The chunk's two launch sequences (with and without a batch's prologue) run
+    eagerly, then captured, in calls of few and of many chunks: the parameter
+    buffer (1024 chunks at first) grows after the capture, batches open with a
+    new bitstring or the previous one, and every call gives the state vector's
+    amplitudes."""
+    import rqcgen
+    from oracle import statevector as sv
+    tn, torch = env
+    circ, _, _ = rqcgen.config_circuit("c1")
+    om = 0b111100001111
+    psi = sv.simulate(circ)
+    plan = tn.Plan(tn.Network(circ), open_mask=om, max_log2_intermediate=30, min_log2_slices=5, log2_batch_slices=1,
+                   trials=8, precision=prec)
+    n = 1 << plan.info()["log2_slices"]
+    per = n >> plan.info()["log2_batch_slices"]
+    many = 1024 // per + 3
+    rng = np.random.default_rng(5)
+    draw = lambda count: [int(b) << 4 for b in rng.integers(0, 16, size=count)]
+    for bits in ([0x30], [0x30, 0x30, 0x50], draw(3), draw(many), draw(2)):
+        out = torch.zeros(len(bits) << 8, dtype=torch.complex128, device="cuda")
+        plan.contract_slices(0, n, bits, out)
+        plan.sync()
+        want = np.concatenate([sv.batch_amplitudes(psi, circ.n_qubits, b, om) for b in bits])
+        got = out.cpu().numpy()
+        assert np.linalg.norm(got - want) < (1e-5 if prec == "fp32" else 1e-4) * np.linalg.norm(want)
