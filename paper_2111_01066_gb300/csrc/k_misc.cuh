@@ -216,22 +216,59 @@ __global__ void k_frugal(const double2* __restrict__ a, int64_t count, int n_qub
   }
 }
 
-// sum_i |a_i|^2 in FP64 (one block; count is small)
-__global__ void k_xeb_sum(const double2* __restrict__ a, int64_t n, double* __restrict__ out) {
-  __shared__ double red[1024];
-  double s = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    const double2 v = a[i];
-    s = fma(v.x, v.x, s);
-    s = fma(v.y, v.y, s);
-  }
-  red[threadIdx.x] = s;
+// sum_i |a_i|^2 in FP64, deterministic: every block adds its share (thread t of
+// the grid takes elements t, t + threads, ..., four loads in flight) into
+// part[1 + block]; the last block to arrive (a ticket, zero between launches)
+// adds the blocks' sums in a fixed order into part[0].  Bound by latency up to
+// about 10^5 amplitudes and by HBM above: 10^6 amplitudes (16 MB) took 494 us on
+// one block.  XEB_BLOCKS partial sums at most.
+constexpr int XEB_BLOCKS = 1024, XEB_THREADS = 256;
+__device__ __forceinline__ double block_sum_256(double s, double* red) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  double r = 0.0;
+  for (int w = 0; w < XEB_THREADS / 32; ++w) r += red[w];
+  __syncthreads();
+  return r;
+}
+__global__ void __launch_bounds__(XEB_THREADS) k_xeb_sum(const double2* __restrict__ a, int64_t n, double* part,
+                                                         unsigned* ticket) {
+  __shared__ double red[XEB_THREADS / 32];
+  __shared__ int s_last;
+  double s = 0.0;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < n; i0 += 4 * step) {
+    double2 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = i0 + u * step < n ? a[i0 + u * step] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      s = fma(v[u].x, v[u].x, s);
+      s = fma(v[u].y, v[u].y, s);
+    }
   }
-  if (threadIdx.x == 0) out[0] = red[0];
+  s = block_sum_256(s, red);
+  if (gridDim.x == 1) {
+    if (threadIdx.x == 0) part[0] = s;
+    return;
+  }
+  if (threadIdx.x == 0) {
+    part[1 + blockIdx.x] = s;
+    __threadfence();
+    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double t = 0.0;
+  for (int q = threadIdx.x; q < (int)gridDim.x; q += blockDim.x) t += __ldcg(part + 1 + q);
+  t = block_sum_256(t, red);
+  if (threadIdx.x == 0) {
+    part[0] = t;
+    *ticket = 0u;
+  }
 }
 
 struct PermArgs {

@@ -1479,7 +1479,8 @@ static void operand_maxima(const float2* a, int64_t na, const float2* b, int64_t
 }
 
 struct Scratch {
-  double* xeb = nullptr;
+  double* xeb = nullptr;          // XEB: the sum, then the blocks' partial sums
+  unsigned* xeb_ticket = nullptr; // zero between launches
   int32_t* err = nullptr;
   float* amax = nullptr;   // FP16X3 operand maxima of the last call (A, B)
   unsigned long long* first = nullptr;   // frugal sampling: first accepted draw per sample
@@ -1496,7 +1497,9 @@ static Scratch& scratch_for_device() {
   std::lock_guard<std::mutex> lk(g_scratch_mu);
   Scratch& s = g_scratch[dev];
   if (!s.xeb) {
-    CK(cudaMalloc(&s.xeb, sizeof(double)));
+    CK(cudaMalloc(&s.xeb_ticket, sizeof(unsigned)));
+    CK(cudaMemset(s.xeb_ticket, 0, sizeof(unsigned)));
+    CK(cudaMalloc(&s.xeb, sizeof(double) * (1 + XEB_BLOCKS)));
     CK(cudaMalloc(&s.err, sizeof(int32_t)));
     CK(cudaMemset(s.err, 0, sizeof(int32_t)));
     CK(cudaMalloc(&s.amax, 2 * sizeof(float)));
@@ -1511,9 +1514,13 @@ extern "C" tn_status tn_xeb(const double* amps, int64_t count, int32_t n_qubits,
   if (!amps || !xeb_out) fail(TN_ERR_ARG, "tn_xeb: NULL argument");
   if (count < 1) fail(TN_ERR_ARG, "tn_xeb: count must be >= 1");
   if (n_qubits < 0 || n_qubits > 1023) fail(TN_ERR_ARG, "tn_xeb: n_qubits out of range");
-  double* scratch = scratch_for_device().xeb;
+  Scratch& sc = scratch_for_device();
+  double* scratch = sc.xeb;
   cudaStream_t s = (cudaStream_t)stream;
-  k_xeb_sum<<<1, 1024, 0, s>>>(reinterpret_cast<const double2*>(amps), count, scratch);
+  // a block per 1024 amplitudes (four a thread), at most four blocks per SM
+  const int64_t per = 4 * XEB_THREADS;
+  const int blocks = (int)std::min<int64_t>((count + per - 1) / per, std::min<int64_t>(4 * sm_count(), XEB_BLOCKS));
+  k_xeb_sum<<<blocks, XEB_THREADS, 0, s>>>(reinterpret_cast<const double2*>(amps), count, scratch, sc.xeb_ticket);
   CK(cudaGetLastError());
   double sum = 0;
   CK(cudaMemcpyAsync(&sum, scratch, sizeof(double), cudaMemcpyDeviceToHost, s));

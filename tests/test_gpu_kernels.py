@@ -94,3 +94,18 @@ def test_chunk_graphs_across_calls(env, prec):
         want = np.concatenate([sv.batch_amplitudes(psi, circ.n_qubits, b, om) for b in bits])
         got = out.cpu().numpy()
         assert np.linalg.norm(got - want) < (1e-5 if prec == "fp32" else 1e-4) * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("count", [1, 7, 255, 1024, 1025, 4096, 100003, 4 * 152 * 1024 - 1, 4 * 152 * 1024 + 1, 2000003])
+def test_xeb_block_counts(env, count):
+    """One block, a few, the most, and more rounds than one per block; twice in a
+    row (the ticket is left at zero), the same bits both times.  |error| <= 2^n
+    mean * (terms a thread adds + the trees) * 2^-53, below 1e-12 here."""
+    tn, torch = env
+    rng = np.random.default_rng(count)
+    a = (rng.normal(size=count) + 1j * rng.normal(size=count)) * 2.0 ** -10
+    t = torch.from_numpy(a).cuda()
+    f = tn.xeb(t, 20)
+    want = 2.0 ** 20 * np.mean(a.real ** 2 + a.imag ** 2) - 1.0
+    assert abs(f - want) <= 1e-12 * (1.0 + abs(want))
+    assert tn.xeb(t, 20) == f
