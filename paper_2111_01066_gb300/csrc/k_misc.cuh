@@ -271,15 +271,18 @@ __global__ void __launch_bounds__(XEB_THREADS) k_xeb_sum(const double2* __restri
   }
 }
 
+constexpr int PERM_MAX_T = 12;   // tile bits at most
 struct PermArgs {
   int8_t src_pos[KMAXR];  // output bit p <- input bit src_pos[p]
-  // tiled variant: the tile's bits (input positions), in input order; for each
-  // tile bit its output position; the non-tile bits (input order) and theirs
-  int32_t nt;             // tile bits (<= 10)
-  int8_t t_in[10], t_out[10];
-  int32_t nr;             // remaining bits
+  // tiled variant: tile bit q in input order at input position t_in[q], tile bit
+  // q in output order at output position t_out[q]; an element's shared-memory
+  // slot is the XOR of wcol[q] over its set bits in input order, of rcol[q] over
+  // those in output order
+  int32_t nt;             // tile bits
+  int8_t t_in[PERM_MAX_T], t_out[PERM_MAX_T];
+  int16_t wcol[PERM_MAX_T], rcol[PERM_MAX_T];
+  int32_t nr;             // remaining bits (at most 32), input order
   int8_t r_in[KMAXR], r_out[KMAXR];
-  int32_t t_out_order[10];  // tile bits sorted by output position (indices into t_*)
 };
 
 // Standalone permutation: one thread per output element (coalesced writes,
@@ -298,73 +301,93 @@ __global__ void k_permute_gather(const float2* __restrict__ in, float2* __restri
 }
 
 // Tiled permutation (SI Eq. (2) as a standalone pass): a tile holds every
-// combination of nt <= 10 tile bits: the input's lowest bits and the input bits
-// that feed the output's lowest positions (so reads and writes both run along
-// memory).  Threads read the tile in input order into shared memory and write
-// it back in output order; the remaining nr bits select the tile.  Each
-// thread's in-tile offsets are fixed, so they are computed once; a tile's base
-// is a one-bit-per-lane warp sum.
+// combination of nt = 10 or 12 tile bits: the input's lowest bits and the input
+// bits that feed the output's lowest positions, so reads and writes both run
+// along memory in runs of 2^5 or 2^6 elements, in 16-byte pairs where both
+// arrays are aligned to 16 bytes.  Threads write the tile into shared memory in
+// input order and read it back in output order; the remaining nr bits select the
+// tile.  A persistent block loads its next tile into registers before it writes
+// the current one out.  HBM-bound: what counts is bytes in flight (32 KB a block
+// of 4096 elements, loads of the next tile among them) and the lengths of the
+// runs; a random permutation of 2^27 elements takes 375 us, 5.7 TB/s (557 us,
+// 3.9 TB/s, with 8 KB tiles, 8-byte accesses and no load in flight across the
+// write-back).
+template <int NT>
 __global__ void __launch_bounds__(256) k_permute_tiled(const float2* __restrict__ in, float2* __restrict__ out,
-                                                       int rank, const PermArgs pa, int64_t n_tiles_per_inst,
-                                                       int64_t n_inst) {
-  __shared__ float2 tile[1024];
-  const int tsz = 1 << pa.nt;
+                                                       int rank, const __grid_constant__ PermArgs pa,
+                                                       int64_t n_tiles, int vec) {
+  constexpr int JB = NT - 9, NJ = 1 << JB;   // a thread has NJ pairs: bits 1-8 its index, 0 the pair, 9.. j
+  __shared__ float2 tile[1 << NT];
   const int lane = threadIdx.x & 31;
-  int64_t ioff[4], ooff[4];
-  int sidx[4];
+  int64_t ioff = 0, ooff = 0;
+  int ws = 0, rs = 0;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int e = threadIdx.x + 256 * j;   // element e in input order, element e in output order
-    ioff[j] = -1;
-    ooff[j] = 0;
-    sidx[j] = 0;
-    if (e < tsz) {
-      int64_t io = 0, oo = 0;
-      int si = 0;
-      for (int q = 0; q < pa.nt; ++q)
-        if ((e >> q) & 1) {
-          io += (int64_t)1 << pa.t_in[q];
-          const int i = pa.t_out_order[q];
-          si |= 1 << i;
-          oo += (int64_t)1 << pa.t_out[i];
-        }
-      ioff[j] = io;
-      ooff[j] = oo;
-      sidx[j] = si;
+  for (int q = 1; q <= 8; ++q)
+    if ((threadIdx.x >> (q - 1)) & 1) {
+      ioff += (int64_t)1 << pa.t_in[q];
+      ooff += (int64_t)1 << pa.t_out[q];
+      ws ^= pa.wcol[q];
+      rs ^= pa.rcol[q];
     }
-  }
-  const int64_t total = n_tiles_per_inst * n_inst;
-  for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
-    const int64_t inst = t >> pa.nr;
-    const int64_t r = t & (n_tiles_per_inst - 1);
-    int64_t bi = 0, bo = 0;
-    for (int q0 = 0; q0 < pa.nr; q0 += 32) {
-      const int q = q0 + lane;
-      int64_t vi = 0, vo = 0;
-      if (q < pa.nr && ((r >> q) & 1)) {
-        vi = (int64_t)1 << pa.r_in[q];
-        vo = (int64_t)1 << pa.r_out[q];
-      }
+  auto joff = [&](int j, const int8_t* pos) {
+    int64_t v = 0;
 #pragma unroll
-      for (int o = 16; o; o >>= 1) {
-        vi += __shfl_xor_sync(0xffffffffu, vi, o);
-        vo += __shfl_xor_sync(0xffffffffu, vo, o);
+    for (int q = 0; q < JB; ++q)
+      if ((j >> q) & 1) v += (int64_t)1 << pos[9 + q];
+    return v;
+  };
+  auto jcol = [&](int j, const int16_t* col) {
+    int v = 0;
+#pragma unroll
+    for (int q = 0; q < JB; ++q)
+      if ((j >> q) & 1) v ^= col[9 + q];
+    return v;
+  };
+  // a tile's base in both arrays: one bit per lane, OR over the warp
+  const int64_t rin = lane < pa.nr ? (int64_t)1 << pa.r_in[lane] : 0, rout = lane < pa.nr ? (int64_t)1 << pa.r_out[lane] : 0;
+  auto base = [&](int64_t t, int64_t bit) {
+    const uint64_t v = ((t >> lane) & 1) && lane < pa.nr ? (uint64_t)bit : 0;
+    const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)v), hi = __reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32));
+    return ((t >> pa.nr) << rank) + (int64_t)(((uint64_t)hi << 32) | lo);
+  };
+  float4 v[NJ];
+  auto load = [&](int64_t t) {
+    const float2* p = in + base(t, rin) + ioff;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const float2* q = p + joff(j, pa.t_in);
+      if (vec) {
+        v[j] = __ldcs(reinterpret_cast<const float4*>(q));
+      } else {
+        const float2 x = __ldcs(q), y = __ldcs(q + 1);
+        v[j] = make_float4(x.x, x.y, y.x, y.y);
       }
-      bi += vi;
-      bo += vo;
     }
-    const int64_t ib = (inst << rank) + bi, ob = (inst << rank) + bo;
-    // tile slot of element e: e ^ (bits 5-9 of e), so that runs along either
-    // order spread over the shared-memory banks
+  };
+  int64_t t = blockIdx.x;
+  if (t < n_tiles) load(t);
+  for (; t < n_tiles; t += gridDim.x) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int e = threadIdx.x + 256 * j;
-      if (ioff[j] >= 0) tile[e ^ ((e >> 5) & 31)] = __ldg(in + ib + ioff[j]);
+    for (int j = 0; j < NJ; ++j) {
+      const int s0 = ws ^ jcol(j, pa.wcol);
+      tile[s0] = make_float2(v[j].x, v[j].y);
+      tile[s0 ^ pa.wcol[0]] = make_float2(v[j].z, v[j].w);
     }
     __syncthreads();
+    if (t + gridDim.x < n_tiles) load(t + gridDim.x);
+    float2* p = out + base(t, rout) + ooff;
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (ioff[j] >= 0) out[ob + ooff[j]] = tile[sidx[j] ^ ((sidx[j] >> 5) & 31)];
+    for (int j = 0; j < NJ; ++j) {
+      const int s0 = rs ^ jcol(j, pa.rcol);
+      const float2 x = tile[s0], y = tile[s0 ^ pa.rcol[0]];
+      float2* q = p + joff(j, pa.t_out);
+      if (vec) {
+        __stcs(reinterpret_cast<float4*>(q), make_float4(x.x, x.y, y.x, y.y));
+      } else {
+        __stcs(q, x);
+        __stcs(q + 1, y);
+      }
+    }
     __syncthreads();
   }
 }

@@ -1564,6 +1564,87 @@ extern "C" tn_status tn_frugal_sample(const double* amps, int64_t count, int32_t
   API_END
 }
 
+// Tile bits and shared-memory slots of the tiled permutation with nt tile bits.
+static void permute_tile(PermArgs& pa, int rank, const int32_t* perm, int nt) {
+  std::vector<int> out_of_in(rank);
+  for (int p = 0; p < rank; ++p) out_of_in[perm[p]] = p;
+  // alternately the next input position and the source of the next output
+  // position, so that both runs grow alike
+  std::vector<char> in_tile(rank, 0);
+  for (int n = 0, ni = 0, no = 0; n < nt;) {
+    while (ni < rank && in_tile[ni]) ++ni;
+    if (ni < rank) {
+      in_tile[ni] = 1;
+      ++n;
+    }
+    while (no < rank && in_tile[perm[no]]) ++no;
+    if (n < nt && no < rank) {
+      in_tile[perm[no]] = 1;
+      ++n;
+    }
+  }
+  pa.nt = nt;
+  pa.nr = 0;
+  std::vector<int> in_order, out_order;   // input positions of the tile bits, in either order
+  for (int i = 0; i < rank; ++i) {
+    if (in_tile[i]) {
+      in_order.push_back(i);
+    } else {
+      pa.r_in[pa.nr] = (int8_t)i;
+      pa.r_out[pa.nr] = (int8_t)out_of_in[i];
+      ++pa.nr;
+    }
+  }
+  for (int p = 0; p < rank; ++p)
+    if (in_tile[perm[p]]) out_order.push_back(perm[p]);
+  std::vector<int> q_of_in(rank, -1);
+  for (int q = 0; q < nt; ++q) q_of_in[in_order[q]] = q;
+  // The slot of an element is (4-bit linear map of its bits, bits 4..) in input
+  // order: 8-byte accesses are free of bank conflicts when the 16 elements of a
+  // half warp, which differ in bits 1-4 of either order, differ in that map.  So
+  // the columns of bits 0-3 (the slot stays a permutation), of input-order bits
+  // 1-4 and of output-order bits 1-4 must each be independent.
+  int col[PERM_MAX_T] = {1, 2, 4, 8};
+  int oq[4];
+  for (int i = 0; i < 4; ++i) oq[i] = q_of_in[out_order[i + 1]];
+  auto independent = [](const std::vector<int>& v) {
+    for (int m = 1; m < (1 << v.size()); ++m) {
+      int x = 0;
+      for (size_t i = 0; i < v.size(); ++i)
+        if ((m >> i) & 1) x ^= v[i];
+      if (x == 0) return false;
+    }
+    return true;
+  };
+  for (int c4 = 1; c4 < 16; c4 += 2) {   // odd: independent of the columns of bits 1-3
+    col[4] = c4;
+    std::vector<int> fixed;
+    for (int i = 0; i < 4; ++i)
+      if (oq[i] <= 4) fixed.push_back(col[oq[i]]);
+    if (!independent(fixed)) continue;
+    for (int i = 0; i < 4; ++i) {
+      if (oq[i] <= 4) continue;
+      for (int c = 1; c < 16; ++c) {
+        fixed.push_back(c);
+        if (independent(fixed)) {
+          col[oq[i]] = c;
+          break;
+        }
+        fixed.pop_back();
+      }
+    }
+    break;
+  }
+  for (int q = 0; q < nt; ++q) {
+    pa.t_in[q] = (int8_t)in_order[q];
+    pa.wcol[q] = (int16_t)((q >= 4 ? 1 << q : 0) ^ col[q]);
+  }
+  for (int q = 0; q < nt; ++q) {
+    pa.t_out[q] = (int8_t)out_of_in[out_order[q]];
+    pa.rcol[q] = pa.wcol[q_of_in[out_order[q]]];
+  }
+}
+
 extern "C" tn_status tn_permute(const float* in, float* out, int32_t rank, const int32_t* perm,
                                 int64_t batch, void* stream) {
   API_BEGIN
@@ -1585,53 +1666,21 @@ extern "C" tn_status tn_permute(const float* in, float* out, int32_t rank, const
     k_permute_gather<<<blocks, 256, 0, (cudaStream_t)stream>>>(reinterpret_cast<const float2*>(in),
                                                                reinterpret_cast<float2*>(out), rank, pa, total);
   } else {
-    // tile bits: input positions 0..4 and the inputs of output positions 0..4
-    std::vector<int> out_of_in(rank);
-    for (int p = 0; p < rank; ++p) out_of_in[perm[p]] = p;
-    std::vector<char> in_tile(rank, 0);
-    for (int i = 0; i < 5; ++i) in_tile[i] = 1;
-    for (int p = 0; p < 5; ++p) in_tile[perm[p]] = 1;
-    // widen to 10 tile bits: alternately the next input bit and the source of
-    // the next output bit (longer contiguous runs on both sides)
-    {
-      int nt = 0;
-      for (int i = 0; i < rank; ++i) nt += in_tile[i];
-      int ni = 5, no = 5;
-      while (nt < 10 && (ni < rank || no < rank)) {
-        if (ni < rank && !in_tile[ni] && nt < 10) {
-          in_tile[ni] = 1;
-          ++nt;
-        }
-        ++ni;
-        if (no < rank && !in_tile[perm[no]] && nt < 10) {
-          in_tile[perm[no]] = 1;
-          ++nt;
-        }
-        ++no;
-      }
-    }
-    pa.nt = 0;
-    pa.nr = 0;
-    for (int i = 0; i < rank; ++i) {
-      if (in_tile[i]) {
-        pa.t_in[pa.nt] = (int8_t)i;
-        pa.t_out[pa.nt] = (int8_t)out_of_in[i];
-        ++pa.nt;
-      } else {
-        pa.r_in[pa.nr] = (int8_t)i;
-        pa.r_out[pa.nr] = (int8_t)out_of_in[i];
-        ++pa.nr;
-      }
-    }
-    std::vector<int> ord(pa.nt);
-    for (int q = 0; q < pa.nt; ++q) ord[q] = q;
-    std::sort(ord.begin(), ord.end(), [&](int x, int y) { return pa.t_out[x] < pa.t_out[y]; });
-    for (int q = 0; q < pa.nt; ++q) pa.t_out_order[q] = ord[q];
-    const int64_t tiles = (int64_t)1 << pa.nr;
-    const int blocks = (int)std::min<int64_t>(tiles * batch, (int64_t)sm_count() * 8);
-    k_permute_tiled<<<blocks, 256, 0, (cudaStream_t)stream>>>(reinterpret_cast<const float2*>(in),
-                                                              reinterpret_cast<float2*>(out), rank, pa, tiles,
-                                                              batch);
+    // tiles of 2^12 elements where they give every SM at least four (5.2 TB/s at
+    // rank 24, 5.7 from 28 on; 3.2 and 3.9 with 2^10), else 2^10 (rank 20: 1.5
+    // TB/s, its 8 MB a few microseconds of latency)
+    const int nt = rank >= 12 && (batch << (rank - 12)) >= 4 * (int64_t)sm_count() ? 12 : 10;
+    permute_tile(pa, rank, perm, nt);
+    const int64_t tiles = batch << pa.nr;
+    // 16-byte pairs need both arrays aligned (an instance is 2^rank elements)
+    const int vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+    const int blocks = (int)std::min<int64_t>(tiles, (int64_t)sm_count() * (nt == 12 ? 4 : 8));
+    const float2* x = reinterpret_cast<const float2*>(in);
+    float2* y = reinterpret_cast<float2*>(out);
+    if (nt == 12)
+      k_permute_tiled<12><<<blocks, 256, 0, (cudaStream_t)stream>>>(x, y, rank, pa, tiles, vec);
+    else
+      k_permute_tiled<10><<<blocks, 256, 0, (cudaStream_t)stream>>>(x, y, rank, pa, tiles, vec);
   }
   CK(cudaGetLastError());
   API_END

@@ -109,3 +109,32 @@ def test_xeb_block_counts(env, count):
     want = 2.0 ** 20 * np.mean(a.real ** 2 + a.imag ** 2) - 1.0
     assert abs(f - want) <= 1e-12 * (1.0 + abs(want))
     assert tn.xeb(t, 20) == f
+
+
+@pytest.mark.parametrize("misaligned", [False, True])
+@pytest.mark.parametrize("kind", ["random", "identity", "reverse", "rotate", "swap ends"])
+@pytest.mark.parametrize("rank,batch", [(9, 3), (10, 1), (11, 3), (12, 1), (13, 5), (12, 700), (14, 153), (22, 1)])
+def test_permute_tiles_bit_exact(env, rank, batch, kind, misaligned):
+    """Both tile sizes (4096 elements from four tiles per SM on), one tile to many
+    per block, orders whose tile bits are the same or disjoint on both sides,
+    arrays that rule 16-byte accesses out; nothing outside the output is written."""
+    tn, torch = env
+    perm = {"random": lambda: [int(p) for p in np.random.default_rng(rank).permutation(rank)],
+            "identity": lambda: list(range(rank)), "reverse": lambda: list(range(rank))[::-1],
+            "rotate": lambda: [(p + 4) % rank for p in range(rank)],
+            "swap ends": lambda: [rank - 1] + list(range(1, rank - 1)) + [0]}[kind]()
+    n = batch << rank
+    pad = 1 if misaligned else 0
+    x = torch.arange(n + 2, device="cuda", dtype=torch.float32)[pad:pad + n]
+    x = torch.complex(x, -x)
+    xin = torch.zeros(n + 2, dtype=torch.complex64, device="cuda")
+    xin[pad:pad + n] = x
+    y = torch.full((n + 2,), 7.0, dtype=torch.complex64, device="cuda")
+    tn.permute(xin[pad:pad + n], y[pad:pad + n], rank, perm, batch)
+    at = torch.zeros(1, dtype=torch.int64, device="cuda")
+    for p in perm:
+        at = torch.cat([at, at + (1 << p)])
+    want = x.view(batch, 1 << rank)[:, at].reshape(-1)
+    assert torch.equal(y[pad:pad + n], want)
+    rest = torch.cat([y[:pad], y[pad + n:]])
+    assert torch.all(rest == 7.0)
