@@ -484,146 +484,120 @@ __device__ __forceinline__ void put3m(uint8_t* sa, int row, int h, const float2 
 }
 
 // ------------------------------------------------------------------ B' images
-// One thread per 16-byte chunk of every (instance, n tile, k chunk) block:
-// reads the complex B entries the chunk covers and writes their 2x2 real form
-// (split into hi/lo planes for BF16X3) in the block's shared-memory image.
-// Threads run in memory order of the image, so the writes are contiguous.
-// Padding (k or n beyond the operand) is zero.
-template <int MODE>
-__global__ void __launch_bounds__(256) k_tc_prep_b(const TcArgs a) {
+// A thread takes one row's 16-byte chunk worth of k of one column n of one
+// (instance, n tile, k chunk) block, reads its B entries once (two 16-byte loads
+// where k is B's lowest position) and writes every image chunk they appear in.
+// Blocks are whole warps, so a block's base offset is a warp-wide OR.  Bound by
+// latency for small B (so: no loop, no tables, as many CTAs as chunks allow) and
+// by HBM for large: 45 instances of 256 x 128 in the 3M BF16 form (12 MB in, 35
+// MB out) take about 10 us, 22 when a CTA walked a block with tables and every
+// entry was read once per plane.  Padding (k or n beyond the operand) is zero.
+constexpr int PREP_THREADS = 256;
+template <int MODE, int CM>
+struct TcPrep {
+  using P = TcPl<MODE, CM>;
+  static constexpr int KPT = CM == 4 ? 16 / (2 * P::ESZ) : 16 / P::ESZ;   // complex k per thread
+  static constexpr int LS_KT = KPT == 2 ? 3 : (KPT == 4 ? 2 : 1);         // log2 of threads per column
+  static_assert(KPT << LS_KT == TC_TK, "a column's 16 k are dealt out whole");
+};
+template <int MODE, int CM>
+__global__ void __launch_bounds__(PREP_THREADS) k_tc_prep_b(const __grid_constant__ TcArgs a, int ls_cols) {
   using T = TcT<MODE>;
-  constexpr int KPC = 16 / (2 * T::ESZ);        // complex k per 16-byte chunk (2 or 4)
-  constexpr int CPR = TC_KP * T::ESZ / 16;      // chunks per row (8 or 4)
+  using P = TcPl<MODE, CM>;
+  using Q = TcPrep<MODE, CM>;
+  constexpr int KPT = Q::KPT;
   const GemmArgs& g = a.g;
-  const int ncp = 2 * a.tn_c;
-  const int plane = tc_plane_bytes(ncp, T::ESZ);
-  const int64_t block_bytes = (int64_t)T::NPL * plane;
-  const int per_block = ncp * CPR;              // chunks per plane
-  const int tkv = 1 << g.tk, tnv = 1 << a.tnb;
-  // offsets in B of the k inside a chunk and of the n inside a tile (-1: padding)
-  __shared__ int64_t koff[TC_TK];
-  __shared__ int64_t noff[128];
-  for (int i = threadIdx.x; i < TC_TK; i += blockDim.x) koff[i] = i < tkv ? deposit_hi((uint64_t)i, g.b_kpos, 0, g.tk) : -1;
-  for (int i = threadIdx.x; i < 128; i += blockDim.x) noff[i] = i < tnv ? deposit_hi((uint64_t)i, g.b_npos, 0, a.tnb) : -1;
-  __syncthreads();
+  const int64_t idx = blockIdx.x * (int64_t)PREP_THREADS + threadIdx.x;
+  const int ls_blk = ls_cols + Q::LS_KT;                    // threads of a block (at least a warp)
+  const int64_t blk = idx >> ls_blk;
+  const int c = (int)idx & ((1 << Q::LS_KT) - 1), n = ((int)idx & ((1 << ls_blk) - 1)) >> Q::LS_KT;
+  const int64_t n_blocks = (int64_t)g.n_inst << (a.ls_nt + a.ls_kc);
+  const bool live = blk < n_blocks;                         // warp-uniform
+  const int kc = (int)(blk & (a.n_kc - 1)), nt = (int)((blk >> a.ls_kc) & (a.n_nt - 1));
+  const int inst = live ? (int)(blk >> (a.ls_kc + a.ls_nt)) : 0;
+  const int64_t base = warp_inst_offset((uint32_t)inst, g.b_istride, g.b_bpos, g.nb) +
+                       warp_deposit((uint32_t)kc, g.b_kpos, g.tk, g.nk) + warp_deposit((uint32_t)nt, g.b_npos, a.tnb, g.nn);
+  int64_t off = 0, kw[4];
+#pragma unroll
+  for (int i = 0; i < 7; ++i)
+    if (i < a.tnb && ((n >> i) & 1)) off += (int64_t)1 << g.b_npos[i];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    kw[i] = i < g.tk ? (int64_t)1 << g.b_kpos[i] : 0;
+    if ((c * KPT >> i) & 1) off += kw[i];
+  }
+  const int tkv = 1 << g.tk;
+  const bool n_ok = live && n < (1 << a.tnb);
+  const float2* src = g.B + base + off;
+  const bool v16 = g.tk > 0 && g.b_kpos[0] == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
   pdl_wait();
   const float sc = operand_scale<MODE>(g.amax_b);
-  const int64_t n_blocks = (int64_t)g.n_inst << (a.ls_nt + a.ls_kc);
-  // one CTA per (instance, n tile, k chunk) block at a time; threads walk the
-  // block's 16-byte chunks in memory order of the image
-  for (int64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
-    const int kc = (int)(blk & (a.n_kc - 1));
-    const int nt = (int)((blk >> a.ls_kc) & (a.n_nt - 1));
-    const int inst = (int)(blk >> (a.ls_kc + a.ls_nt));
-    const int64_t base = inst_offset(inst, g.b_istride, g.b_bpos, g.nb) + deposit_hi((uint64_t)kc, g.b_kpos, g.tk, g.nk) +
-                         deposit_hi((uint64_t)nt, g.b_npos, a.tnb, g.nn);
-    uint8_t* dblk = const_cast<uint8_t*>(a.bimg) + blk * block_bytes;
-    for (int q = threadIdx.x; q < per_block; q += blockDim.x) {
-      // q in image order: row within the 8-row group fastest, then chunk, then group
-      const int rlo = q & 7, c = (q >> 3) % CPR, rg = (q >> 3) / CPR;
-      const int row = rg * 8 + rlo;
-      const int t = row & 1, nl = row >> 1;
-      const int64_t no = noff[nl];
-      float vals[2 * KPC];
+  float2 b[KPT];
 #pragma unroll
-      for (int i = 0; i < KPC; ++i) {
-        const int64_t ko = koff[c * KPC + i];
-        float2 b = make_float2(0.f, 0.f);
-        if (no >= 0 && ko >= 0) b = g.B[base + no + ko];
-        // row (n, t), columns (k, u): t = 0 -> (Re, -Im), t = 1 -> (Im, Re)
-        vals[2 * i] = t ? b.y : b.x;
-        vals[2 * i + 1] = t ? b.x : -b.y;
-      }
-      uint8_t* dst = dblk + tc_elem_off(row, c * KPC * 2, T::ESZ);
-      if constexpr (MODE == TC_TF32) {
-        uint32_t w[4];
+  for (int i = 0; i < KPT; i += 2) {
+    const int k = c * KPT + i;
+    int64_t o = 0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) w[i] = to_tf32(vals[i]);
-        *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-      } else {
-        uint32_t hi[4], lo[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) split_pair<MODE>(vals[2 * i] * sc, vals[2 * i + 1] * sc, hi[i], lo[i]);
-        *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4*>(dst + plane) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-      }
+    for (int q = 1; q < 3; ++q)
+      if ((i >> q) & 1) o += kw[q];
+    if (n_ok && k + 1 < tkv && v16) {
+      const float4 t = __ldg(reinterpret_cast<const float4*>(src + o));
+      b[i] = make_float2(t.x, t.y);
+      b[i + 1] = make_float2(t.z, t.w);
+    } else {
+      b[i] = n_ok && k < tkv ? __ldg(src + o) : make_float2(0.f, 0.f);
+      b[i + 1] = n_ok && k + 1 < tkv ? __ldg(src + o + kw[0]) : make_float2(0.f, 0.f);
     }
   }
-}
-
-// 3M B images: per (instance, n tile, k chunk) block the planes of TcPl<MODE, 3>,
-// one plane row per complex column n; one thread per 16-byte chunk in memory
-// order of the image.  Padding (k or n beyond the operand) is zero.
-template <int MODE>
-__global__ void __launch_bounds__(256) k_tc_prep_b3(const TcArgs a) {
-  using P = TcPl<MODE, 3>;
-  constexpr int ESZ = P::ESZ;
-  constexpr int EPC = 16 / ESZ;                 // elements per 16-byte chunk (4 or 8)
-  constexpr int CPR = TC_KP * ESZ / 16;         // chunks per plane row (8 or 4)
-  const GemmArgs& g = a.g;
-  const int rows = a.tn_c;
-  const int plane = tc_plane_bytes(rows, ESZ);
-  const int64_t block_bytes = (int64_t)P::PLANES * plane;
-  const int per_block = P::PLANES * rows * CPR;
-  const int per_plane = rows * CPR;
-  const int tkv = 1 << g.tk, tnv = 1 << a.tnb;
-  __shared__ int64_t koff[TC_TK];
-  __shared__ int64_t noff[128];
-  for (int i = threadIdx.x; i < TC_TK; i += blockDim.x) koff[i] = i < tkv ? deposit_hi((uint64_t)i, g.b_kpos, 0, g.tk) : -1;
-  for (int i = threadIdx.x; i < 128; i += blockDim.x) noff[i] = i < tnv ? deposit_hi((uint64_t)i, g.b_npos, 0, a.tnb) : -1;
-  __syncthreads();
-  pdl_wait();
-  const float sc = operand_scale<MODE>(g.amax_b);
-  const int64_t n_blocks = (int64_t)g.n_inst << (a.ls_nt + a.ls_kc);
-  for (int64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
-    const int kc = (int)(blk & (a.n_kc - 1));
-    const int nt = (int)((blk >> a.ls_kc) & (a.n_nt - 1));
-    const int inst = (int)(blk >> (a.ls_kc + a.ls_nt));
-    const int64_t base = inst_offset(inst, g.b_istride, g.b_bpos, g.nb) + deposit_hi((uint64_t)kc, g.b_kpos, g.tk, g.nk) +
-                         deposit_hi((uint64_t)nt, g.b_npos, a.tnb, g.nn);
-    uint8_t* dblk = const_cast<uint8_t*>(a.bimg) + blk * block_bytes;
-    for (int pq = threadIdx.x; pq < per_block; pq += blockDim.x) {
-      const int pl = pq / per_plane, q = pq % per_plane;
-      const int rlo = q & 7, c = (q >> 3) % CPR, rg = (q >> 3) / CPR;
-      const int n = rg * 8 + rlo;
-      const int half = c / (CPR / 2), k0 = (c % (CPR / 2)) * EPC;   // k0.. within the half's 16 k
-      const int64_t no = noff[n];   // n < tn_c <= 128
-      float2 b[8];
+  if (!live) return;
+  const int plane = tc_plane_bytes(P::ROWS_PER_COL * a.tn_c, T::ESZ);
+  uint8_t* d = const_cast<uint8_t*>(a.bimg) + blk * (int64_t)P::PLANES * plane;
+  if constexpr (CM == 4) {
+    // rows (n, t), columns (k, u): t = 0 -> (Re, -Im), t = 1 -> (Im, Re)
+    uint8_t* d0 = d + tc_elem_off(2 * n, c * KPT * 2, T::ESZ);
+    uint8_t* d1 = d + tc_elem_off(2 * n + 1, c * KPT * 2, T::ESZ);
+    if constexpr (MODE == TC_TF32) {
+      st16(d0, to_tf32(b[0].x), to_tf32(-b[0].y), to_tf32(b[1].x), to_tf32(-b[1].y));
+      st16(d1, to_tf32(b[0].y), to_tf32(b[0].x), to_tf32(b[1].y), to_tf32(b[1].x));
+    } else {
+      uint32_t h0[4], l0[4], h1[4], l1[4];
 #pragma unroll
-      for (int i = 0; i < EPC; ++i) {
-        const int64_t ko = koff[k0 + i];
-        b[i] = (no >= 0 && ko >= 0) ? g.B[base + no + ko] : make_float2(0.f, 0.f);
+      for (int i = 0; i < 4; ++i) {
+        split_pair<MODE>(b[i].x * sc, -b[i].y * sc, h0[i], l0[i]);
+        split_pair<MODE>(b[i].y * sc, b[i].x * sc, h1[i], l1[i]);
       }
-      uint8_t* dst = dblk + (int64_t)pl * plane + tc_elem_off(n, c * EPC, ESZ);
-      if constexpr (MODE == TC_TF32) {
-        // plane 0: [Br | Bi]; plane 1: [Bs | 0]
-        uint32_t w[4];
+      st16(d0, h0[0], h0[1], h0[2], h0[3]);
+      st16(d1, h1[0], h1[1], h1[2], h1[3]);
+      st16(d0 + plane, l0[0], l0[1], l0[2], l0[3]);
+      st16(d1 + plane, l1[0], l1[1], l1[2], l1[3]);
+    }
+  } else {
+    // 3M: one plane row per column, real parts in its first half, imaginary in its second
+    uint8_t* dr = d + tc_elem_off(n, c * KPT, T::ESZ);
+    uint8_t* di = d + tc_elem_off(n, TC_TK + c * KPT, T::ESZ);
+    if constexpr (MODE == TC_TF32) {
+      // plane 0: [Br | Bi]; plane 1: [Bs | 0]
+      st16(dr, to_tf32(b[0].x), to_tf32(b[1].x), to_tf32(b[2].x), to_tf32(b[3].x));
+      st16(di, to_tf32(b[0].y), to_tf32(b[1].y), to_tf32(b[2].y), to_tf32(b[3].y));
+      st16(dr + plane, to_tf32(b[0].x + b[0].y), to_tf32(b[1].x + b[1].y), to_tf32(b[2].x + b[2].y),
+           to_tf32(b[3].x + b[3].y));
+      st16(di + plane, 0u, 0u, 0u, 0u);
+    } else {
+      // plane 0: [Br_hi | Bi_hi]; plane 1: [Br_lo | Bi_lo]; plane 2: [Bs_hi | Bs_lo]
+      uint32_t rh[4], rl[4], ih[4], il[4], sh[4], sl[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float v = pl == 0 ? (half == 0 ? b[i].x : b[i].y) : (half == 0 ? b[i].x + b[i].y : 0.f);
-          w[i] = to_tf32(v);
-        }
-        st16(dst, w[0], w[1], w[2], w[3]);
-      } else {
-        // plane 0: [Br_hi | Bi_hi]; plane 1: [Br_lo | Bi_lo]; plane 2: [Bs_hi | Bs_lo]
-        uint32_t w[4];
-#pragma unroll
-        for (int q2 = 0; q2 < 4; ++q2) {
-          const float2 u = b[2 * q2], v = b[2 * q2 + 1];
-          float x0, x1;
-          if (pl < 2) {
-            x0 = half == 0 ? u.x : u.y;
-            x1 = half == 0 ? v.x : v.y;
-          } else {
-            x0 = u.x + u.y;
-            x1 = v.x + v.y;
-          }
-          uint32_t hi, lo;
-          split_pair<MODE>(x0 * sc, x1 * sc, hi, lo);
-          w[q2] = (pl == 0 || (pl == 2 && half == 0)) ? hi : lo;
-        }
-        st16(dst, w[0], w[1], w[2], w[3]);
+      for (int i = 0; i < 4; ++i) {
+        const float2 u = b[2 * i], w = b[2 * i + 1];
+        split_pair<MODE>(u.x * sc, w.x * sc, rh[i], rl[i]);
+        split_pair<MODE>(u.y * sc, w.y * sc, ih[i], il[i]);
+        split_pair<MODE>((u.x + u.y) * sc, (w.x + w.y) * sc, sh[i], sl[i]);
       }
+      st16(dr, rh[0], rh[1], rh[2], rh[3]);
+      st16(di, ih[0], ih[1], ih[2], ih[3]);
+      st16(dr + plane, rl[0], rl[1], rl[2], rl[3]);
+      st16(di + plane, il[0], il[1], il[2], il[3]);
+      st16(dr + 2 * plane, sh[0], sh[1], sh[2], sh[3]);
+      st16(di + 2 * plane, sl[0], sl[1], sl[2], sl[3]);
     }
   }
 }

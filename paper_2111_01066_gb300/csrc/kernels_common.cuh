@@ -104,4 +104,18 @@ __device__ __forceinline__ int64_t inst_offset(uint32_t inst, int64_t istride, c
   return r;
 }
 
+// Sum over bits i >= from of bit_{i - from}(x) << pos[i], one bit per lane (the
+// positions are distinct, so the sum is an OR); every lane of the warp calls it.
+__device__ __forceinline__ int64_t warp_deposit(uint32_t x, const int8_t* pos, int from, int to) {
+  const int lane = threadIdx.x & 31;
+  uint64_t v = 0;
+  if (from + lane < to && ((x >> lane) & 1u)) v = (uint64_t)1 << pos[from + lane];
+  const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)v);
+  const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32));
+  return (int64_t)(((uint64_t)hi << 32) | lo);
+}
+__device__ __forceinline__ int64_t warp_inst_offset(uint32_t inst, int64_t istride, const int8_t* bpos, int nb) {
+  return (int64_t)inst * istride + warp_deposit(inst, bpos, 0, nb);
+}
+
 }  // namespace tnx

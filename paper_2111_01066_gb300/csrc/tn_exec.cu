@@ -442,20 +442,14 @@ static int pair_clusters() {
   return n;
 }
 
-// The B' images of a tensor-core step into t.bimg: one CTA per image block at a time.
+// The B' images of a tensor-core step into t.bimg.
 template <int MODE, int CM>
 static void launch_prep(const TcArgs& t, cudaStream_t s) {
-  const int64_t n_blocks = (int64_t)t.g.n_inst * t.n_nt * t.n_kc;
-  const int pgrid = (int)std::max<int64_t>(1, std::min<int64_t>(n_blocks, (int64_t)sm_count() * 16));
-  // started under the kernel before it only while it has at most a CTA per SM:
-  // beside a resident GEMM the SM's L1 is a few KB, and a larger grid, which
-  // reads every B entry several times, is slower there than it gains (45 3M
-  // instances of 512 x 256 x 128: 47.8 us a call without the overlap, 55.7 with)
-  const bool overlap = n_blocks <= sm_count();
-  if constexpr (CM == 4)
-    klaunch(k_tc_prep_b<MODE>, dim3(pgrid), 256, 0, s, 1, overlap, t);
-  else
-    klaunch(k_tc_prep_b3<MODE>, dim3(pgrid), 256, 0, s, 1, overlap, t);
+  const int ls_cols = __builtin_ctz((unsigned)t.tn_c);
+  const int64_t threads = ((int64_t)t.g.n_inst * t.n_nt * t.n_kc) << (ls_cols + TcPrep<MODE, CM>::LS_KT);
+  const int64_t grid = (threads + PREP_THREADS - 1) / PREP_THREADS;
+  if (grid > 0x7fffffff) fail(TN_ERR_UNSUPPORTED, "B' image grid too large");
+  klaunch(k_tc_prep_b<MODE, CM>, dim3((unsigned)grid), PREP_THREADS, 0, s, 1, true, t, ls_cols);
 }
 static void launch_prep_kid(const TcArgs& t, int kid, cudaStream_t s) {
   switch (kid) {

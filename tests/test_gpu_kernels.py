@@ -138,3 +138,28 @@ def test_permute_tiles_bit_exact(env, rank, batch, kind, misaligned):
     assert torch.equal(y[pad:pad + n], want)
     rest = torch.cat([y[:pad], y[pad + n:]])
     assert torch.all(rest == 7.0)
+
+
+PAIR_REL = {("tf32", 4): 3e-3, ("tf32", 3): 3e-3, ("bf16x3", 4): 4e-5, ("bf16x3", 3): 4e-5, ("fp16x3", 4): 2e-5,
+            ("fp16x3", 3): 2e-5}
+
+
+@pytest.mark.parametrize("prec,cm", sorted(PAIR_REL))
+@pytest.mark.parametrize("shape,batch,layout,misaligned", [
+    ((14, 2, 9), 1, "random", False), ((13, 3, 9), 1, "kfast", False), ((13, 5, 7), 1, "kfast", True),   # around a k chunk
+    ((14, 6, 3), 5, "kfast", False), ((9, 13, 3), 3, "random", False),                                  # narrow, split k
+    ((4, 10, 6), 40, "random", False), ((6, 6, 9), 17, "kfast", False)])                                # part row tiles
+def test_tensor_core_tiles_at_their_edges(env, shape, batch, layout, misaligned, prec, cm):
+    """Tensor-core contractions around a k chunk (16), with narrow and part
+    tiles, several instances and split k, operands in streaming or any order, or
+    off a 16-byte boundary (no tensor-map or 16-byte loads).  Norm-wise: TF32
+    operands carry 2^-11, the split modes 2^-16 (BF16) or 2^-21 (FP16) plus the
+    tensor cores' 32-bit accumulation over 2^13 products at most."""
+    tn, torch = env
+    (a, a_w, b, b_w, c_w), dev = _pair_case(torch, shape, batch, layout, sum(shape) * 10 + batch, misaligned)
+    tn.contract_pair(*dev, batch=batch, precision=prec, complex_mult=cm)
+    tn.device_sync()
+    got = dev[4].cpu().numpy()
+    for i in {0, batch - 1}:
+        want = pairwise.contract_pair(a[i].astype(np.complex128), a_w, b[i].astype(np.complex128), b_w, c_w)
+        assert np.linalg.norm(got[i] - want) <= PAIR_REL[prec, cm] * np.linalg.norm(want)
