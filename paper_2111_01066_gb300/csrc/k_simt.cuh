@@ -169,8 +169,8 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
   const int kc_per = (1 << n_hi) / split, kc0 = rank * kc_per;
 
   // offsets of the tile's rows and columns in C, and the k chunk steps
-  for (int r = tid; r < TM; r += SIMT_THREADS) sm.offCm[r] = r < TMv ? deposit_hi((uint64_t)r, g.c_mpos, 0, g.tm) : 0;
-  if (tid < TN) sm.offCn[tid] = tid < TNv ? deposit_hi((uint64_t)tid, g.c_npos, 0, g.tn) : 0;
+  for (int r = tid; r < TM; r += SIMT_THREADS) sm.offCm[r] = r < TMv ? deposit_lo<8>((uint32_t)r, g.c_mpos, g.tm) : 0;
+  if (tid < TN) sm.offCn[tid] = tid < TNv ? deposit_lo<6>((uint32_t)tid, g.c_npos, g.tn) : 0;
   {
     const int t = SIMT_THREADS - 1 - tid;   // other threads than the ones above where the tile is small
     if (t < n_hi) {

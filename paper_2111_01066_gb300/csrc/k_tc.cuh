@@ -627,6 +627,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
   using T = TcT<MODE>;
   using P = TcPl<MODE, CM>;
   static_assert(!PAIR || CM == 4, "SM pairs form 4M products");
+  // Set-up is kept short (a launch's fixed cost is what a small step pays): no ring
+  // zeroing where every byte is written, unrolled offset tables, tile bases as
+  // warp-wide ORs, k offsets by one table entry per chunk; with loops over the
+  // argument bank in their place a 2^20 multiply-add step took 9.4 us (8.0 now) and
+  // A gathered in any order 1024 x 64 x 256 28 us (23 now).
   extern __shared__ __align__(1024) uint8_t smem_dyn[];
   // swizzle atoms need 1024-byte aligned slots
   uint8_t* smem_raw = smem_dyn + ((1024 - (smem_u32(smem_dyn) & 1023)) & 1023);
@@ -676,15 +681,31 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
   int64_t* offCm = reinterpret_cast<int64_t*>(tmem_slot + 4);
   float2* epi_stage = reinterpret_cast<float2*>(reinterpret_cast<uint8_t*>(bars) + 4096);
   int64_t* offCn = offCm + TC_M;
+  int64_t* kdA = offCn + 128;
 
-  // zero every slot once: padding rows / columns are never written again
-  for (int i = threadIdx.x; i < (na * P::A_SLOT + nbs * b_slot) / 16; i += blockDim.x)
-    reinterpret_cast<uint4*>(aring)[i] = make_uint4(0, 0, 0, 0);
+  // a contraction of fewer than 16 k leaves the rest of every A row unwritten:
+  // zeroed once.  (Rows past 2^tm hold anything: they reach only accumulator rows
+  // that are not stored.  B' slots are always copied whole.)
+  if (g.tk < 4)
+    for (int i = threadIdx.x; i < na * P::A_SLOT / 16; i += blockDim.x)
+      reinterpret_cast<uint4*>(aring)[i] = make_uint4(0, 0, 0, 0);
   const int tmv = 1 << g.tm, tnv = 1 << a.tnb;
-  for (int r = threadIdx.x; r < TC_M; r += blockDim.x)
-    offCm[r] = r < tmv ? deposit_hi((uint64_t)r, g.c_mpos, 0, g.tm) : 0;
-  for (int c = threadIdx.x; c < 128; c += blockDim.x)
-    offCn[c] = c < tnv ? deposit_hi((uint64_t)c, g.c_npos, 0, a.tnb) : 0;
+  if (threadIdx.x < TC_M) {
+    const int r = threadIdx.x;
+    offCm[r] = r < tmv ? deposit_lo<7>((uint32_t)r, g.c_mpos, g.tm) : 0;
+  } else if (threadIdx.x < 2 * TC_M) {
+    const int c = threadIdx.x - TC_M;
+    offCn[c] = c < tnv ? deposit_lo<7>((uint32_t)c, g.c_npos, a.tnb) : 0;
+  } else if (threadIdx.x < 2 * TC_M + KMAXR && !a.a_tma) {
+    // the gather loaders' step of A's k offset from chunk c to c + 1, by the
+    // number of trailing one bits of c
+    const int t = threadIdx.x - 2 * TC_M;
+    if (g.tk + t < g.nk) {
+      int64_t o = (int64_t)1 << g.a_kpos[g.tk + t];
+      for (int j = 0; j < t; ++j) o -= (int64_t)1 << g.a_kpos[g.tk + j];
+      kdA[t] = o;
+    }
+  }
   if (threadIdx.x == 0) {
     // SM pairs: the even CTA's fullA and tempty also take one arrival from the
     // odd CTA per phase (its chunk in place, its accumulator set drained)
@@ -915,6 +936,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
     }
   } else if (warp >= TC_MMA_WARP + 1) {
     // ---------------------------------------------------------------- loaders
+    // (each wait is voted on by the warp: the tile bases are warp-wide ORs)
     if constexpr (CM == 3) {
       // 3M: one item (tile row, 8 complex k) per thread, gathered from A's
       // storage order into registers; the next slot's item is in flight while
@@ -925,17 +947,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
       const bool rok = row < (1 << g.tm);
       const bool kadj = g.nk > 0 && g.a_kpos[0] == 0;
       int64_t goff[8];
-      const int64_t roff = rok ? deposit_hi((uint64_t)row, g.a_mpos, 0, g.tm) : 0;
+      const int64_t roff = rok ? deposit_lo<7>((uint32_t)row, g.a_mpos, g.tm) : 0;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int k = 8 * h + i;
-        goff[i] = (rok && k < tkv) ? roff + deposit_hi((uint64_t)k, g.a_kpos, 0, g.tk) : -1;
+        goff[i] = (rok && k < tkv) ? roff + deposit_lo<4>((uint32_t)k, g.a_kpos, g.tk) : -1;
       }
       auto tile_base = [&](int64_t tile) -> const float2* {
         const TileIdx ti = tile_decode(tile, a);
         const int mt = own_mt(ti.mt), inst = ti.inst;
-        return g.A + inst_offset(inst, g.a_istride, g.a_bpos, g.nb) +
-               deposit_hi((uint64_t)mt, g.a_mpos, g.tm, g.nm);
+        return g.A + warp_inst_offset((uint32_t)inst, g.a_istride, g.a_bpos, g.nb) +
+               warp_deposit((uint32_t)mt, g.a_mpos, g.tm, g.nm) +
+               warp_deposit((uint32_t)(ti.s * kc_per), g.a_kpos, g.tk, g.nk);
       };
       auto issue = [&](float2(&v)[8], const float2* Ak) {
         const bool v16 = kadj && ((reinterpret_cast<uintptr_t>(Ak) & 15) == 0);
@@ -966,10 +989,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
           ntile = seq_tile(++njt);
           nkc = ntile >= 0 ? (int)(ntile & (int64_t)(a.n_split - 1)) * kc_per : 0;
           if (ntile >= 0) An = tile_base(ntile);
+        } else {
+          An += kdA[__ffs(~kc) - 1];
         }
-        if (ntile >= 0) issue(vn, An + deposit_hi((uint64_t)nkc, g.a_kpos, g.tk, g.nk));
+        if (ntile >= 0) issue(vn, An);
         uint8_t* sa = aring + slot * P::A_SLOT;
-        if (!mbar_wait(smem_u32(&emptyA[slot]), ph ^ 1, abort_flag, a.err)) return false;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&emptyA[slot]), ph ^ 1, abort_flag, a.err))) return false;
         if (rok) put3m<MODE>(sa, row, h, vc, sc_a);
         fence_proxy_async();
         mbar_arrive(smem_u32(&fullA[slot]));
@@ -982,7 +1007,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
         kc = nkc;
         return true;
       };
-      if (tile >= 0) issue(v0, An + deposit_hi((uint64_t)kc, g.a_kpos, g.tk, g.nk));
+      if (tile >= 0) issue(v0, An);
       while (tile >= 0) {
         if (!body(v0, v1) || tile < 0) break;
         if (!body(v1, v0)) break;
@@ -1012,17 +1037,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
         const int c = klanes ? q % CPR : q / TC_M;
         cok[j] = row < (1 << g.tm);
         soff[j] = tc_elem_off(row, c * KPC * 2, T::ESZ);
-        const int64_t roff = deposit_hi((uint64_t)row, g.a_mpos, 0, g.tm);
+        const int64_t roff = deposit_lo<7>((uint32_t)row, g.a_mpos, g.tm);
 #pragma unroll
         for (int i = 0; i < KPC; ++i) {
           const int k = c * KPC + i;
-          goff[j][i] = (cok[j] && k < tkv) ? roff + deposit_hi((uint64_t)k, g.a_kpos, 0, g.tk) : -1;
+          goff[j][i] = (cok[j] && k < tkv) ? roff + deposit_lo<4>((uint32_t)k, g.a_kpos, g.tk) : -1;
         }
       }
       auto tile_base = [&](int64_t tile) -> const float2* {
         const TileIdx ti = tile_decode(tile, a);
         const int mt = own_mt(ti.mt), inst = ti.inst;
-        return g.A + inst_offset(inst, g.a_istride, g.a_bpos, g.nb) + deposit_hi((uint64_t)mt, g.a_mpos, g.tm, g.nm);
+        return g.A + warp_inst_offset((uint32_t)inst, g.a_istride, g.a_bpos, g.nb) +
+               warp_deposit((uint32_t)mt, g.a_mpos, g.tm, g.nm) +
+               warp_deposit((uint32_t)(ti.s * kc_per), g.a_kpos, g.tk, g.nk);
       };
       int slot = 0;
       uint32_t ph = 0;
@@ -1030,12 +1057,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
         bool ok = true;
         int64_t jt = 0;
         for (int64_t tile = seq_tile(0); tile >= 0 && ok; tile = seq_tile(++jt)) {
-          const float2* At = tile_base(tile);
+          const float2* Ak = tile_base(tile);
           const int kc0 = (int)(tile & (int64_t)(a.n_split - 1)) * kc_per;
           for (int kc = kc0; kc < kc0 + kc_per; ++kc) {
-            const float2* Ak = At + deposit_hi((uint64_t)kc, g.a_kpos, g.tk, g.nk);
+            if (kc > kc0) Ak += kdA[__ffs(~(kc - 1)) - 1];
             uint8_t* sa = aring + slot * P::A_SLOT;
-            if (!mbar_wait(smem_u32(&emptyA[slot]), ph ^ 1, abort_flag, a.err)) { ok = false; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&emptyA[slot]), ph ^ 1, abort_flag, a.err))) {
+              ok = false;
+              break;
+            }
             {
               const bool v16 = kadj && ((reinterpret_cast<uintptr_t>(Ak) & 15) == 0);
 #pragma unroll
@@ -1081,8 +1111,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
         int64_t jt = 0;
         int64_t tile = seq_tile(0);
         int kc = tile >= 0 ? (int)(tile & (int64_t)(a.n_split - 1)) * kc_per : 0;
-        const float2* At = tile >= 0 ? tile_base(tile) : g.A;
-        const float2* An = At;     // base of the tile of the prefetched slot
+        const float2* An = tile >= 0 ? tile_base(tile) : g.A;   // the prefetched slot's chunk of A
         auto body = [&](float4(&vc)[NCH][KPC / 2], float4(&vn)[NCH][KPC / 2]) -> bool {
           int64_t ntile = tile, njt = jt;
           int nkc = kc + 1;
@@ -1090,10 +1119,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
             ntile = seq_tile(++njt);
             nkc = ntile >= 0 ? (int)(ntile & (int64_t)(a.n_split - 1)) * kc_per : 0;
             if (ntile >= 0) An = tile_base(ntile);
+          } else {
+            An += kdA[__ffs(~kc) - 1];
           }
-          if (ntile >= 0) issue(vn, An + deposit_hi((uint64_t)nkc, g.a_kpos, g.tk, g.nk));
+          if (ntile >= 0) issue(vn, An);
           uint8_t* sa = aring + slot * P::A_SLOT;
-          if (!mbar_wait(smem_u32(&emptyA[slot]), ph ^ 1, abort_flag, a.err)) return false;
+          if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&emptyA[slot]), ph ^ 1, abort_flag, a.err))) return false;
           {
 #pragma unroll
             for (int j = 0; j < NCH; ++j) {
@@ -1115,13 +1146,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
             slot = 0;
             ph ^= 1;
           }
-          if (ntile != tile) At = An;
           tile = ntile;
           jt = njt;
           kc = nkc;
           return true;
         };
-        if (tile >= 0) issue(v0, At + deposit_hi((uint64_t)kc, g.a_kpos, g.tk, g.nk));
+        if (tile >= 0) issue(v0, An);
         while (tile >= 0) {
           if (!body(v0, v1) || tile < 0) break;
           if (!body(v1, v0)) break;
@@ -1321,26 +1351,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
       const TileIdx ti = tile_decode(tile, a);
       const int nt = ti.nt, mt = own_mt(ti.mt), inst = ti.inst;
       float2* Cb = a.n_split > 1 ? a.c_part + ti.s * a.c_part_stride : g.C;
-      // the tile's base in C: its instance, m-tile and n-tile bits deposited at
-      // their positions in C, one bit per lane, summed over the warp
-      int64_t cb = (int64_t)inst * g.c_istride;
-      {
-        const int n_i = g.nb, n_m = g.nm - g.tm, n_all = g.nb + (g.nm - g.tm) + (g.nn - a.tnb);
-        for (int b0 = 0; b0 < n_all; b0 += 32) {
-          const int bi = b0 + lane;
-          int64_t v = 0;
-          if (bi < n_i) {
-            if ((inst >> bi) & 1) v = (int64_t)1 << g.c_bpos[bi];
-          } else if (bi < n_i + n_m) {
-            if ((mt >> (bi - n_i)) & 1) v = (int64_t)1 << g.c_mpos[g.tm + bi - n_i];
-          } else if (bi < n_all) {
-            if ((nt >> (bi - n_i - n_m)) & 1) v = (int64_t)1 << g.c_npos[a.tnb + bi - n_i - n_m];
-          }
-#pragma unroll
-          for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-          cb += v;
-        }
-      }
+      // the tile's base in C: its instance, m-tile and n-tile bits at their positions
+      const int64_t cb = warp_inst_offset((uint32_t)inst, g.c_istride, g.c_bpos, g.nb) +
+                         warp_deposit((uint32_t)mt, g.c_mpos, g.tm, g.nm) +
+                         warp_deposit((uint32_t)nt, g.c_npos, a.tnb, g.nn);
       float2* C = Cb + cb;
       const bool row_ok = row < tmv;
       const int64_t crow = offCm[row];

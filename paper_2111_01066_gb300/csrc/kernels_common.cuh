@@ -97,10 +97,13 @@ __device__ __forceinline__ int64_t deposit_hi(uint64_t x, const int8_t* pos, int
   return r;
 }
 
-__device__ __forceinline__ int64_t inst_offset(uint32_t inst, int64_t istride, const int8_t* bpos, int nb) {
-  int64_t r = (int64_t)inst * istride;
-  for (int j = 0; j < nb; ++j)
-    if ((inst >> j) & 1) r += (int64_t)1 << bpos[j];
+// the same for from = 0, to = n <= N, unrolled (no loop over the argument bank)
+template <int N>
+__device__ __forceinline__ int64_t deposit_lo(uint32_t x, const int8_t* pos, int n) {
+  int64_t r = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (i < n && ((x >> i) & 1u)) r += (int64_t)1 << pos[i];
   return r;
 }
 
