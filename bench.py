@@ -414,7 +414,7 @@ def pair_bench(args) -> int:
     ms = statistics.mean(times)
     peaks = load_peaks()
     kernel = {"fp32": "simt", "tf32": "tc_tf32", "bf16x3": "tc_bf16x3"}[prec]
-    if prec != "fp32" and (m + k + n + int(math.log2(batch)) < 20 or m < 4):
+    if prec != "fp32" and (m + k + n + math.log2(batch) < 25 or m < 4):
         kernel = "simt"
     r = step_roofline((m, k, n, int(round(math.log2(batch)))), ms, kernel, peaks)
     print(json.dumps({"metric": "pair_contraction", "shape_log2_mkn": [m, k, n], "batch": batch,
@@ -475,7 +475,7 @@ def sweep_bench(args) -> int:
                                               complex_mult=cm, stream=stream)
                 ms = _event_ms(fn, 2, flush, stream)
                 kern = kname[(prec, cm)]
-                if prec != "fp32" and (m + k + n + b < 20 or m < 4):
+                if prec != "fp32" and (m + k + n + b < 25 or m < 4):
                     kern = "simt"
                 r = step_roofline((m, k, n, b), ms, kern, peaks)
                 rows.append({"case": "gemm", "source": source, "mknb_log2": [m, k, n, b], "precision": prec,

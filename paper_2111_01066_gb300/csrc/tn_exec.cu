@@ -306,7 +306,11 @@ static void setup_tma(StepLaunch& L, int a_bits, int64_t n_lin) {
 // TC_MAX_B; the rest of the shared-memory budget goes to A slots)
 // pair_mode: SM pairs (cta_group::2, two m tiles per work unit, half of B' per
 // CTA) where the step allows them -- 4M products and at least two full 128-row
-// m tiles: -1 or 1 uses them there, 0 never
+// m tiles: 1 uses them there, 0 never, -1 unless the step has at most 64 k and 256
+// columns: there B' is a small part of the traffic and a pair's launch and
+// barriers cost more than they save (16384 x 16 x 256: 13.0 us on single SMs, 14.4 on
+// pairs; 2^18 x 64 x 128: 75 and 78; with 1024 columns or 128 k pairs win, 65536 x 64
+// x 1024: 113 and 107, 2^21 x 128 x 128: 704 and 669)
 static bool pair_ok(const GemmArgs& g, int kid) { return !tc_is_3m(kid) && g.tm == 7 && g.nm - g.tm >= 1; }
 static StepLaunch make_launch(const GemmArgs& g, int kid, int a_bits, int64_t n_lin, int64_t c_total = 0,
                               bool allow_split = false, int epi_mode = -1,
@@ -322,7 +326,8 @@ static StepLaunch make_launch(const GemmArgs& g, int kid, int a_bits, int64_t n_
   t.tnb = g.tn;
   const TcGeom geo = tc_geom(kid);
   t.tn_c = std::max(geo.min_tn_c, 1 << g.tn);
-  t.pair = (pair_mode != 0 && pair_ok(g, kid)) ? 1 : 0;
+  const bool pair_pays = g.nk - g.tk > 2 || g.nn - g.tn > 1;
+  t.pair = (pair_mode != 0 && pair_ok(g, kid) && (pair_mode > 0 || pair_pays)) ? 1 : 0;
   t.n_mt = 1 << (g.nm - g.tm - t.pair);
   t.n_nt = 1 << (g.nn - g.tn);
   t.n_kc = 1 << (g.nk - g.tk);
@@ -330,19 +335,30 @@ static StepLaunch make_launch(const GemmArgs& g, int kid, int a_bits, int64_t n_
   const int b_plane = tc_plane_bytes(geo.rows_per_col * t.tn_c, geo.esz);
   const int npl = geo.planes;
   L.ws_bytes = (int64_t)g.n_inst * t.n_nt * t.n_kc * npl * b_plane;
-  // split-K when the output tiles cannot fill the SMs and the k loop is long
-  // (a pair's work unit occupies two SMs)
-  const int64_t unit_sms = 1 + t.pair;
+  // split-K when the output tiles cannot fill the SMs and the k loop is long, by
+  // the modeled time of its work units in waves, each kc / sp chunks and a
+  // write-back, plus the partial tiles' way through memory and the reduction's
+  // launch.  (A chunk of 128 columns takes about 0.6 us, one of few columns the 0.37
+  // in which an SM's share of HBM brings its 16 KB of A; the write-back 3; splitting
+  // whenever a unit fitted made 2048 x 256 x 1024, whose 64 pairs already fill 76,
+  // write four partial results: 36 us, 21 unsplit.)
   t.n_split = 1;
-  if (allow_split && c_total > 0 && t.n_tiles * unit_sms < sm_count() && t.n_kc >= 8) {
-    int sp = 1;
-    // enough tiles for several waves (tail below ~15%), each split >= 4 k chunks
-    while (sp < 32 && t.n_tiles * unit_sms * sp * 2 <= 8 * (int64_t)sm_count() && t.n_kc / (sp * 2) >= 4) sp *= 2;
-    if (sp > 1 && (int64_t)sp * c_total * 8 <= split_cap_bytes) {
-      t.n_split = sp;
+  const int64_t unit_sms = 1 + t.pair, slots = std::max<int64_t>(1, sm_count() / unit_sms);
+  if (allow_split && c_total > 0 && t.n_tiles < slots && t.n_kc >= 8) {
+    const double chunk_us = std::max(0.37, 0.15 + 0.45 * t.tn_c / 128.0), tile_us = 1.0 + 2.0 * t.tn_c / 128.0;
+    auto modeled = [&](int sp) {
+      const double waves = (double)((t.n_tiles * sp + slots - 1) / slots);
+      const double us = waves * (t.n_kc / sp * chunk_us + tile_us);
+      return sp == 1 ? us : us + 3.0 + (2.0 * sp + 1.0) * (double)c_total * 8.0 / 5.5e6;
+    };
+    int best = 1;
+    for (int sp = 2; sp <= 32 && t.n_kc / sp >= 4; sp *= 2)
+      if (modeled(sp) < modeled(best) && (int64_t)sp * c_total * 8 <= split_cap_bytes) best = sp;
+    if (best > 1) {
+      t.n_split = best;
       t.c_part_stride = c_total;
       L.split_off = (L.ws_bytes + 255) / 256 * 256;
-      L.ws_bytes = L.split_off + (int64_t)sp * c_total * 8;
+      L.ws_bytes = L.split_off + (int64_t)best * c_total * 8;
       L.c_total = c_total;
     }
   }
@@ -607,13 +623,17 @@ static int tc_kernel(int precision, int cmult) {
   if (precision == TN_PREC_FP16X3) return cmult == 3 ? K_TC_FP16X3_3M : K_TC_FP16X3;
   return cmult == 3 ? K_TC_BF16X3_3M : K_TC_BF16X3;
 }
-// Tensor-core kernels (4M or 3M products) for every step with enough work in
-// the TF32 / BF16X3 / FP16X3 modes; tiny steps (and the FP32 mode) on the CUDA
-// cores, which always form 4M products in FP32.
+// Tensor-core kernels (4M or 3M products) for the steps with enough work in the
+// TF32 / BF16X3 / FP16X3 modes, from 2^25 multiply-adds over all instances; the
+// rest (and the FP32 mode) on the CUDA cores, which always form 4M products in
+// FP32.  A tensor-core step has a B' image launch, a pipeline to fill and an
+// accumulator to drain, 7-8 us at least in a chain of launches; at 2^20 the CUDA
+// cores take 3.1 us against 8.0, at 2^22 5-6 against 8-10, at 2^24 7.6-9.2 against
+// 9.1-11.8 (16 columns or fewer: 10-16 against 9-17), at 2^25 11.6 against 9.3.
 static int pick_kernel(int precision, int cmult, const StepDesc& d, int64_t n_inst) {
   if (precision == TN_PREC_FP32) return pick_simt(d, n_inst);
-  const int work = d.nm + d.nk + d.nn + d.nb;
-  if (work < 20 || d.nm < 4) return pick_simt(d, n_inst);
+  const double macs = std::ldexp((double)n_inst, d.nm + d.nk + d.nn);
+  if (macs < 33554432.0 || d.nm < 4) return pick_simt(d, n_inst);
   return tc_kernel(precision, cmult);
 }
 
@@ -1867,6 +1887,15 @@ extern "C" tn_status tn_contract_pair_noalloc(const float* a, const int32_t* aw,
   // beside the B' images; otherwise one pass over k
   StepLaunch L = make_launch(g, kid, ar, batch, batch * d.c_elems, true, -1, cap);
   if (L.ws_bytes > cap) L = make_launch(g, kid, ar, batch);
+  // the documented limit is on the operands, not on the kernel that the step's
+  // size selects: what the tensor-core path could not hold is refused from 2^20
+  // multiply-adds an instance on, also where the CUDA cores (no scratch) run it
+  if (!is_tc(kid) && precision != TN_PREC_FP32 && d.nm + d.nk + d.nn >= 20 && d.nm >= 4) {
+    const int tk = tc_kernel(precision, cmult);
+    const GemmArgs gt = make_args(d, tk, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
+                                  reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems);
+    L.ws_bytes = make_launch(gt, tk, ar, batch).ws_bytes;
+  }
   if (L.ws_bytes > cap)
     fail(TN_ERR_ARG, "tn_contract_pair_noalloc: this contraction needs " + std::to_string(L.ws_bytes) +
                          " bytes of scratch; the static array holds " + std::to_string(cap));

@@ -148,7 +148,8 @@ PAIR_REL = {("tf32", 4): 3e-3, ("tf32", 3): 3e-3, ("bf16x3", 4): 4e-5, ("bf16x3"
 @pytest.mark.parametrize("shape,batch,layout,misaligned", [
     ((14, 2, 9), 1, "random", False), ((13, 3, 9), 1, "kfast", False), ((13, 5, 7), 1, "kfast", True),   # around a k chunk
     ((14, 6, 3), 5, "kfast", False), ((9, 13, 3), 3, "random", False),                                  # narrow, split k
-    ((4, 10, 6), 40, "random", False), ((6, 6, 9), 17, "kfast", False)])                                # part row tiles
+    ((4, 10, 6), 40, "random", False), ((6, 6, 9), 17, "kfast", False),                                 # part row tiles
+    ((8, 9, 8), 2, "kfast", False), ((10, 7, 9), 1, "random", False), ((9, 11, 6), 1, "kfast", False)])  # SM pairs
 def test_tensor_core_tiles_at_their_edges(env, shape, batch, layout, misaligned, prec, cm):
     """Tensor-core contractions around a k chunk (16), with narrow and part
     tiles, several instances and split k, operands in streaming or any order, or
