@@ -1700,6 +1700,46 @@ extern "C" tn_status tn_permute(const float* in, float* out, int32_t rank, const
   API_END
 }
 
+// Order of the m and n bits of a pairwise contraction (the tile takes the first
+// ones; any order gives the same sums).  Operands in any order: rows alternate
+// between C's lowest positions and A's, columns between C's and B's, so that a
+// tile's reads and writes both run along memory.  A stored [contracted...,
+// free...] keeps its rows in order, for its tensor-map loads.  In the wires'
+// order of A and B C's stores were mostly single elements: 2^18 x 64 x 128 in random
+// order, TF32, took 208 us (271 with the older gather), 82 with this.
+static void order_pair_bits(StepDesc& d) {
+  // op, cp: positions of the n bits in the operand and in C
+  auto order = [](int n, int8_t* op, int8_t* cp) {
+    int8_t at_op[64], at_c[64], o[MAXR], c[MAXR];   // bit at a position, -1 for none
+    std::memset(at_op, -1, sizeof(at_op));
+    std::memset(at_c, -1, sizeof(at_c));
+    std::memcpy(o, op, sizeof(o));
+    std::memcpy(c, cp, sizeof(c));
+    for (int i = 0; i < n; ++i) {
+      at_op[o[i]] = (int8_t)i;
+      at_c[c[i]] = (int8_t)i;
+    }
+    uint64_t used = 0;
+    for (int k = 0, pc = 0, po = 0; k < n;) {
+      auto take = [&](const int8_t* at, int& pos) {   // the lowest bit of one side not taken yet
+        while (pos < 64 && (at[pos] < 0 || ((used >> at[pos]) & 1))) ++pos;
+        if (pos == 64 || k == n) return;
+        const int i = at[pos];
+        used |= 1ull << i;
+        op[k] = o[i];
+        cp[k] = c[i];
+        ++k;
+      };
+      take(at_c, pc);
+      take(at_op, po);
+    }
+  };
+  bool k_first = true;
+  for (int j = 0; j < d.nk; ++j) k_first = k_first && d.a_kpos[j] == j;
+  if (!(k_first && d.nk >= 4)) order(d.nm, d.a_mpos, d.c_mpos);
+  order(d.nn, d.b_npos, d.c_npos);
+}
+
 extern "C" tn_status tn_contract_pair(const float* a, const int32_t* aw, int32_t ar, const float* b,
                                       const int32_t* bw, int32_t br, float* c, const int32_t* cw,
                                       int32_t cr, int64_t batch, int32_t precision, int32_t cmult,
@@ -1750,6 +1790,7 @@ extern "C" tn_status tn_contract_pair(const float* a, const int32_t* aw, int32_t
   d.a_elems = (int64_t)1 << ar;
   d.b_elems = (int64_t)1 << br;
   d.c_elems = (int64_t)1 << cr;
+  order_pair_bits(d);
   d.nb = 0;
   const int kid = pick_kernel(precision, cmult, d, batch);
   GemmArgs g = make_args(d, kid, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
@@ -1871,6 +1912,7 @@ extern "C" tn_status tn_contract_pair_noalloc(const float* a, const int32_t* aw,
   d.a_elems = (int64_t)1 << ar;
   d.b_elems = (int64_t)1 << br;
   d.c_elems = (int64_t)1 << cr;
+  order_pair_bits(d);
   const int kid = pick_kernel(precision, cmult, d, batch);
   GemmArgs g = make_args(d, kid, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
                          reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems);
