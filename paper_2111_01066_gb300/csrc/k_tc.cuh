@@ -143,8 +143,9 @@ struct TcArgs {
   int32_t na;            // A ring slots (TcPl::A_SLOT bytes each)
   int32_t nbs;           // B' ring slots (one (n tile, k chunk) image each)
   int32_t fa_count;      // arrivals expected on an A slot's "full" barrier
-  int32_t n_acc;         // TMEM accumulator sets (1..8), as many as fit 512 columns: the MMAs
-                         // run up to n_acc tiles ahead of the epilogue (3M 128-column tiles: 1)
+  int32_t n_acc;         // TMEM accumulator sets (1..8, of n_seg accumulators each), as many as
+                         // fit 512 columns: the MMAs run up to n_acc tiles ahead of the epilogue
+                         // (3M 128-column tiles: 1)
   int32_t nmw;           // m bits that are tensor-map rows (contiguous after the k bits)
   int32_t hi_shift;      // storage position where tensor-map dimension 2 starts
   int64_t c2_inst_mul;   // dimension-2 step per linear instance (tn_contract_pair batches)
@@ -159,6 +160,10 @@ struct TcArgs {
   float2* c_part;
   int64_t c_part_stride;
   int32_t ls_split, ls_nt, ls_mt, ls_kc;   // log2 of n_split, n_nt, n_mt, n_kc (powers of two)
+  // a work unit's k chunks are accumulated in n_seg accumulators, one run of
+  // chunks each, which the epilogue adds: as short a chain of 32-bit accumulation
+  // as n_split * n_seg partial results would have, without their way through memory
+  int32_t n_seg, ls_seg_len;   // ls_seg_len: log2 of the chunks of a segment
   // SM pairs: a work unit is a pair of m tiles (n_mt counts pairs); the CTA of
   // cluster rank r takes m tile 2 mt + r and the B' rows [r N'/2, (r + 1) N'/2)
   int32_t pair;
@@ -621,12 +626,16 @@ __global__ void k_split_reduce(const float2* __restrict__ part, int n_split, int
 }
 
 // ------------------------------------------------------------------ the GEMM
-template <int MODE, int CM, bool PAIR>
+// SEG: the k of a work unit may be divided over several accumulators (n_seg > 1);
+// without it n_seg is 1, and the write-back loop keeps its registers for the stores
+// (one kernel for both made write-heavy steps 5-40% slower).
+template <int MODE, int CM, bool PAIR, bool SEG>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constant__ TcArgs a,
                                                               const __grid_constant__ CUtensorMap tma_a) {
   using T = TcT<MODE>;
   using P = TcPl<MODE, CM>;
   static_assert(!PAIR || CM == 4, "SM pairs form 4M products");
+  static_assert(!SEG || CM == 4, "3M accumulators leave no room for segments");
   // Set-up is kept short (a launch's fixed cost is what a small step pays): no ring
   // zeroing where every byte is written, unrolled offset tables, tile bases as
   // warp-wide ORs, k offsets by one table entry per chunk; with loops over the
@@ -638,7 +647,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
   const GemmArgs& g = a.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ncp = 2 * a.tn_c;                                   // real columns of C per tile
-  const int setw = P::ACC_PER_COL * a.tn_c;                     // TMEM columns per accumulator set
+  const int accw = P::ACC_PER_COL * a.tn_c;                     // TMEM columns per accumulator
+  const int setw = SEG ? accw * a.n_seg : accw;                 // and per accumulator set
   const int a_plane = P::A_PLANE;
   // B' planes: the image's (all N' rows) and this CTA's (half of them for a pair)
   const int b_plane_g = tc_plane_bytes(P::ROWS_PER_COL * a.tn_c, T::ESZ);
@@ -1190,8 +1200,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
           break;
         }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * setw);
+        uint32_t d_tmem = tmem_base + (uint32_t)(acc * setw);
+        uint32_t more = 0u;   // 0: a segment's first chunk starts its accumulator
         for (int kc = 0; kc < kc_per; ++kc) {
+          if constexpr (SEG)
+            if (kc > 0 && (kc & ((1 << a.ls_seg_len) - 1)) == 0) {   // the next segment's accumulator
+              d_tmem += (uint32_t)accw;
+              more = 0u;
+            }
           // the chunk's operands are in place (in both CTAs of a pair)
           if (!mbar_wait(smem_u32(&fullA[sa_i]), pha, abort_flag, a.err)) {
             ok = false;
@@ -1208,7 +1224,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
 #pragma unroll
             for (int j = 0; j < TC_KP * T::ESZ / 32; ++j) {
               const uint32_t ko = (uint32_t)(2 * j);
-              const uint32_t first = (kc > 0 || j > 0) ? 1u : 0u;
+              const uint32_t first = j > 0 ? 1u : more;
               mma(d_tmem, da + ko, db + ko, first);
               if constexpr (MODE != TC_TF32) {   // hi*hi + hi*lo + lo*hi
                 mma(d_tmem, da + ko, db + bp + ko, 1u);
@@ -1223,14 +1239,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
 #pragma unroll
               for (int j = 0; j < 2; ++j) {
                 const uint32_t ko = (uint32_t)(2 * j);
-                const uint32_t first = (kc > 0 || j > 0) ? 1u : 0u;
+                const uint32_t first = j > 0 ? 1u : more;
                 mma(d1, da + ko, db + ko, first);
                 mma(d2, da + 4u + ko, db + 4u + ko, first);
                 mma(d3, da + ap + ko, db + bp + ko, first);
               }
             } else {
               // planes H = [Ar_hi | Ai_hi], L = [Ar_lo | Ai_lo], S = [As_hi | As_lo]
-              const uint32_t first = kc > 0 ? 1u : 0u;
+              const uint32_t first = more;
               const uint32_t H = da, L = da + ap, S = da + 2u * ap;
               const uint32_t BH = db, BL = db + bp, BS = db + 2u * bp;
               mma(d1, H, BH, first);
@@ -1244,6 +1260,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
               mma(d3, S + 2u, BS, 1u);
             }
           }
+          more = 1u;
           tc_commit_g<PAIR>(smem_u32(&emptyA[sa_i]));
           da += a_step;
           if (++sa_i == na) {
@@ -1364,6 +1381,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
         float v[32];
         if constexpr (CM == 4) {
           tmem_ld32(tl + (uint32_t)c0, v);
+          if constexpr (SEG)
+            for (int sg = 1; sg < a.n_seg; ++sg) {
+              float w[32];
+              tmem_ld32(tl + (uint32_t)(sg * accw + c0), w);
+#pragma unroll
+              for (int j = 0; j < 32; ++j) v[j] += w[j];
+            }
         } else {
           // Re = T1 - T2, Im = T3 - T1 - T2
           float t[48];

@@ -300,6 +300,48 @@ static void setup_tma(StepLaunch& L, int a_bits, int64_t n_lin) {
   t.c2_inst_mul = n_lin > 1 ? ((int64_t)1 << (a_bits - hi_shift)) : 0;
 }
 
+// How a tile's k chunks are divided: n_split work units (partial tiles through
+// memory) of n_seg accumulators each (in TMEM, acc_cols * tn_c columns apiece).
+// `need`: n_split * n_seg must reach it, so that no chain of 32-bit accumulation
+// gets longer.  Of what fits, the least modeled time: the work units in waves, each
+// its chunks and a write-back, plus the partial tiles' way through memory and the
+// reduction's launch.  A chunk of 128 columns takes about 0.6 us, one of few
+// columns the 0.37 in which an SM's share of HBM brings its 16 KB of A; the
+// write-back 3.  (With partial tiles alone 2048 x 256 x 1024, whose 64 pairs already
+// fill 76, wrote four of them: 36 us.)
+struct TcSplit {
+  int n_split, n_seg;
+  double us;
+};
+static TcSplit tc_split(int64_t n_tiles, int64_t slots, int n_kc, int tn_c, int acc_cols, int64_t c_total,
+                        int64_t cap_bytes, int need) {
+  const double chunk_us = std::max(0.37, 0.15 + 0.45 * tn_c / 128.0), tile_us = 1.0 + 2.0 * tn_c / 128.0;
+  TcSplit best = {0, 1, 0.0};
+  for (int sp = 1; sp <= 32 && (sp == 1 || n_kc / sp >= 4); sp *= 2) {
+    if (sp > 1 && ((n_tiles >= slots && sp > need) || (int64_t)sp * c_total * 8 > cap_bytes)) break;
+    int sg = std::max(1, need / sp);
+    if (sg > 1 && (acc_cols != 2 || sg * acc_cols * tn_c > TC_TMEM_COLS)) continue;   // 4M only, where they fit
+    const double waves = (double)((n_tiles * sp + slots - 1) / slots);
+    double us = waves * (n_kc / sp * chunk_us + tile_us);
+    if (sp > 1) us += 3.0 + (2.0 * sp + 1.0) * (double)c_total * 8.0 / 5.5e6;
+    if (best.n_split == 0 || us < best.us) best = {sp, sg, us};
+  }
+  return best;
+}
+// The parts that a tile's k is divided into at least: when the tiles of the
+// default width (128 columns) cannot fill the SMs, as many as keep eight per SM at
+// most and 4 chunks each.
+static int tc_min_parts(int kid, int nm, int nk, int nn, int64_t n_inst, int64_t c_total, int64_t cap_bytes) {
+  const KernelCfg& k = kCfg[kid];
+  const int tm = std::min(k.tm, nm), tk = std::min(k.tk, nk), tn = std::min(k.tn, nn);
+  const int64_t tiles = n_inst * ((int64_t)1 << (nm - tm)) * ((int64_t)1 << (nn - tn));
+  const int n_kc = 1 << (nk - tk);
+  int sp = 1;
+  if (tiles < sm_count() && n_kc >= 8)
+    while (sp < 32 && tiles * sp * 2 <= 8 * (int64_t)sm_count() && n_kc / (sp * 2) >= 4) sp *= 2;
+  return (int64_t)sp * c_total * 8 <= cap_bytes ? sp : 1;
+}
+
 // epi_mode: -1 chooses the write-back by the coalesced run lengths, 0 forces
 // direct per-column stores, 1 the staged order (where the tile allows it)
 // b_slots: B' ring slots (<= 0: 4 for slots up to 16 KB, else 3; at most
@@ -311,7 +353,33 @@ static void setup_tma(StepLaunch& L, int a_bits, int64_t n_lin) {
 // barriers cost more than they save (16384 x 16 x 256: 13.0 us on single SMs, 14.4 on
 // pairs; 2^18 x 64 x 128: 75 and 78; with 1024 columns or 128 k pairs win, 65536 x 64
 // x 1024: 113 and 107, 2^21 x 128 x 128: 704 and 669)
-static bool pair_ok(const GemmArgs& g, int kid) { return !tc_is_3m(kid) && g.tm == 7 && g.nm - g.tm >= 1; }
+static bool pair_ok(int kid, int nm, int tm) { return !tc_is_3m(kid) && tm == 7 && nm - tm >= 1; }
+static bool pair_pays(int ls_kc, int ls_nt) { return ls_kc > 2 || ls_nt > 1; }
+
+// Default tile width (log2 complex columns): 128, or 64 or 32 where the tiles are
+// few and that takes less modeled time: narrower tiles spread over more SMs and
+// leave room for more accumulators of a divided k (2048 x 256 x 1024: 36 us with 128
+// columns and four partial results, 23 with 64 columns and four accumulators).
+static int tc_tile(int kid, int nm, int nk, int nn, int64_t n_inst, int64_t c_total, int64_t cap_bytes, bool pairs) {
+  const KernelCfg& k = kCfg[kid];
+  const int tm = std::min(k.tm, nm), tk = std::min(k.tk, nk), widest = std::min(k.tn, nn);
+  const int need = tc_min_parts(kid, nm, nk, nn, n_inst, c_total, cap_bytes);
+  if (need == 1) return widest;
+  int best = widest;
+  double best_us = 0.0;
+  for (int tn = widest; tn >= std::min(5, widest); --tn) {
+    const int pair = pairs && pair_ok(kid, nm, tm) && pair_pays(nk - tk, nn - tn) ? 1 : 0;
+    const int64_t units = n_inst * ((int64_t)1 << (nm - tm - pair)) * ((int64_t)1 << (nn - tn));
+    const double us = tc_split(units, sm_count() / (1 + pair), 1 << (nk - tk), std::max(tc_geom(kid).min_tn_c, 1 << tn),
+                               tc_is_3m(kid) ? 3 : 2, c_total, cap_bytes, need).us;
+    if (tn == widest || us < best_us) {
+      best = tn;
+      best_us = us;
+    }
+  }
+  return best;
+}
+
 static StepLaunch make_launch(const GemmArgs& g, int kid, int a_bits, int64_t n_lin, int64_t c_total = 0,
                               bool allow_split = false, int epi_mode = -1,
                               int64_t split_cap_bytes = (int64_t)256 << 20, int b_slots = 0, int pair_mode = -1) {
@@ -326,8 +394,7 @@ static StepLaunch make_launch(const GemmArgs& g, int kid, int a_bits, int64_t n_
   t.tnb = g.tn;
   const TcGeom geo = tc_geom(kid);
   t.tn_c = std::max(geo.min_tn_c, 1 << g.tn);
-  const bool pair_pays = g.nk - g.tk > 2 || g.nn - g.tn > 1;
-  t.pair = (pair_mode != 0 && pair_ok(g, kid) && (pair_mode > 0 || pair_pays)) ? 1 : 0;
+  t.pair = (pair_mode != 0 && pair_ok(kid, g.nm, g.tm) && (pair_mode > 0 || pair_pays(g.nk - g.tk, g.nn - g.tn))) ? 1 : 0;
   t.n_mt = 1 << (g.nm - g.tm - t.pair);
   t.n_nt = 1 << (g.nn - g.tn);
   t.n_kc = 1 << (g.nk - g.tk);
@@ -335,33 +402,25 @@ static StepLaunch make_launch(const GemmArgs& g, int kid, int a_bits, int64_t n_
   const int b_plane = tc_plane_bytes(geo.rows_per_col * t.tn_c, geo.esz);
   const int npl = geo.planes;
   L.ws_bytes = (int64_t)g.n_inst * t.n_nt * t.n_kc * npl * b_plane;
-  // split-K when the output tiles cannot fill the SMs and the k loop is long, by
-  // the modeled time of its work units in waves, each kc / sp chunks and a
-  // write-back, plus the partial tiles' way through memory and the reduction's
-  // launch.  (A chunk of 128 columns takes about 0.6 us, one of few columns the 0.37
-  // in which an SM's share of HBM brings its 16 KB of A; the write-back 3; splitting
-  // whenever a unit fitted made 2048 x 256 x 1024, whose 64 pairs already fill 76,
-  // write four partial results: 36 us, 21 unsplit.)
-  t.n_split = 1;
+  // few output tiles and a long k loop: the k chunks of a tile go to n_split work
+  // units, whose partial tiles are added by k_split_reduce, and to n_seg
+  // accumulators in each (tc_split)
   const int64_t unit_sms = 1 + t.pair, slots = std::max<int64_t>(1, sm_count() / unit_sms);
-  if (allow_split && c_total > 0 && t.n_tiles < slots && t.n_kc >= 8) {
-    const double chunk_us = std::max(0.37, 0.15 + 0.45 * t.tn_c / 128.0), tile_us = 1.0 + 2.0 * t.tn_c / 128.0;
-    auto modeled = [&](int sp) {
-      const double waves = (double)((t.n_tiles * sp + slots - 1) / slots);
-      const double us = waves * (t.n_kc / sp * chunk_us + tile_us);
-      return sp == 1 ? us : us + 3.0 + (2.0 * sp + 1.0) * (double)c_total * 8.0 / 5.5e6;
-    };
-    int best = 1;
-    for (int sp = 2; sp <= 32 && t.n_kc / sp >= 4; sp *= 2)
-      if (modeled(sp) < modeled(best) && (int64_t)sp * c_total * 8 <= split_cap_bytes) best = sp;
-    if (best > 1) {
-      t.n_split = best;
+  t.n_split = 1;
+  t.n_seg = 1;
+  if (allow_split && c_total > 0) {
+    const TcSplit c = tc_split(t.n_tiles, slots, t.n_kc, t.tn_c, tc_is_3m(kid) ? 3 : 2, c_total, split_cap_bytes,
+                               tc_min_parts(kid, g.nm, g.nk, g.nn, g.n_inst, c_total, split_cap_bytes));
+    t.n_split = c.n_split;
+    t.n_seg = c.n_seg;
+    if (t.n_split > 1) {
       t.c_part_stride = c_total;
       L.split_off = (L.ws_bytes + 255) / 256 * 256;
-      L.ws_bytes = L.split_off + (int64_t)best * c_total * 8;
+      L.ws_bytes = L.split_off + (int64_t)t.n_split * c_total * 8;
       L.c_total = c_total;
     }
   }
+  t.ls_seg_len = __builtin_ctz((unsigned)(t.n_kc / (t.n_split * t.n_seg)));
   t.n_tiles *= t.n_split;
   t.ls_split = __builtin_ctz((unsigned)t.n_split);
   t.ls_nt = g.nn - g.tn;
@@ -422,7 +481,7 @@ static StepLaunch make_launch(const GemmArgs& g, int kid, int a_bits, int64_t n_
   t.fa_count = (t.a_tma && kid == K_TC_TF32) ? 1 : (t.a_tma ? TC_LOAD_THREADS / 2 : TC_LOAD_THREADS);
   // as many accumulator sets as fit the 512 TMEM columns (at most 8): narrow
   // tiles let the MMAs run several tiles ahead of the epilogue
-  t.n_acc = std::max(1, std::min(TC_MAX_ACC, TC_TMEM_COLS / ((tc_is_3m(kid) ? 3 : 2) * t.tn_c)));
+  t.n_acc = std::max(1, std::min(TC_MAX_ACC, TC_TMEM_COLS / ((tc_is_3m(kid) ? 3 : 2) * t.tn_c * t.n_seg)));
   L.smem = std::max(t.na * geo.a_slot + t.nbs * b_slot + 4096 + epi_bytes + 1024, TC_MIN_SMEM);
   return L;
 }
@@ -449,7 +508,8 @@ static int pair_clusters() {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int q = 0;
-  if (cudaOccupancyMaxActiveClusters(&q, k_cgemm_tc<MODE, 4, PAIR>, &cfg) != cudaSuccess || q <= 0) {
+  CK(cudaFuncSetAttribute(k_cgemm_tc<MODE, 4, PAIR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_MAX_SMEM));
+  if (cudaOccupancyMaxActiveClusters(&q, k_cgemm_tc<MODE, 4, PAIR, false>, &cfg) != cudaSuccess || q <= 0) {
     cudaGetLastError();
     q = sm_count() / 2;
   }
@@ -490,9 +550,8 @@ static void launch_prep_kid(const TcArgs& t, int kid, cudaStream_t s) {
   }
 }
 
-template <int MODE, int CM, bool PAIR>
-static void launch_tc(const TcArgs& t, const StepLaunch& L, int grid, cudaStream_t s) {
-  if (!L.bimg_own) launch_prep<MODE, CM>(t, s);   // else built ahead by a prologue
+template <int MODE, int CM, bool PAIR, bool SEG>
+static void launch_tc_kernel(const TcArgs& t, const StepLaunch& L, int grid, cudaStream_t s) {
   // the shared-memory opt-in is a per-device function attribute: one bit per
   // device (ids < 64) records that it was set there; two threads racing on the
   // same bit both set the same value, which is harmless
@@ -501,16 +560,26 @@ static void launch_tc(const TcArgs& t, const StepLaunch& L, int grid, cudaStream
   CK(cudaGetDevice(&dev));
   const uint64_t bit = dev < 64 ? (1ULL << dev) : 0;
   if (!bit || !(attr_set.load(std::memory_order_acquire) & bit)) {
-    CK(cudaFuncSetAttribute(k_cgemm_tc<MODE, CM, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_MAX_SMEM));
+    CK(cudaFuncSetAttribute(k_cgemm_tc<MODE, CM, PAIR, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_MAX_SMEM));
     attr_set.fetch_or(bit, std::memory_order_acq_rel);
   }
   if constexpr (PAIR) {
     // clusters of two CTAs, each pair persistent over the work units
     const int clusters = (int)std::min<int64_t>(t.n_tiles, pair_clusters<MODE, PAIR>());
-    klaunch(k_cgemm_tc<MODE, CM, PAIR>, dim3(2 * clusters), TC_THREADS, L.smem, s, 2, true, t, L.tma);
+    klaunch(k_cgemm_tc<MODE, CM, PAIR, SEG>, dim3(2 * clusters), TC_THREADS, L.smem, s, 2, true, t, L.tma);
   } else {
-    klaunch(k_cgemm_tc<MODE, CM, PAIR>, dim3(grid), TC_THREADS, L.smem, s, 1, true, t, L.tma);
+    klaunch(k_cgemm_tc<MODE, CM, PAIR, SEG>, dim3(grid), TC_THREADS, L.smem, s, 1, true, t, L.tma);
   }
+}
+template <int MODE, int CM, bool PAIR>
+static void launch_tc(const TcArgs& t, const StepLaunch& L, int grid, cudaStream_t s) {
+  if (!L.bimg_own) launch_prep<MODE, CM>(t, s);   // else built ahead by a prologue
+  if constexpr (CM == 4)
+    if (t.n_seg > 1) {
+      launch_tc_kernel<MODE, CM, PAIR, true>(t, L, grid, s);
+      return;
+    }
+  launch_tc_kernel<MODE, CM, PAIR, false>(t, L, grid, s);
 }
 
 // clear_amax: the step's recorded maximum starts at zero here (in a chunk or a
@@ -843,7 +912,10 @@ static void ensure_device(Plan& p) {
                     ((int64_t)1 << (d.nm + d.nn + d.nb)) == d.c_elems;
     if (!ok) fail(TN_ERR_PLAN, "internal: step operand outside its extent");
     const int kid = pick_kernel(p.opts.precision, p.opts.complex_mult, d, (int64_t)1 << d.nb);
-    ds->launches.push_back(make_launch(step_args(*ds, d, kid), kid, 64 - __builtin_clzll((uint64_t)d.a_elems) - 1, 1,
+    const int tn = is_tc(kid) ? tc_tile(kid, d.nm, d.nk, d.nn, (int64_t)1 << d.nb, d.c_elems, (int64_t)256 << 20,
+                                        p.opts.sm_pairs != 0)
+                              : -1;
+    ds->launches.push_back(make_launch(step_args(*ds, d, kid, tn), kid, 64 - __builtin_clzll((uint64_t)d.a_elems) - 1, 1,
                                        d.c_elems, true, -1, (int64_t)256 << 20, 0, p.opts.sm_pairs ? -1 : 0));
   }
   int64_t ws = 16;
@@ -1794,7 +1866,9 @@ extern "C" tn_status tn_contract_pair(const float* a, const int32_t* aw, int32_t
   d.nb = 0;
   const int kid = pick_kernel(precision, cmult, d, batch);
   GemmArgs g = make_args(d, kid, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
-                         reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems);
+                         reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems,
+                         is_tc(kid) ? tc_tile(kid, d.nm, d.nk, d.nn, batch, batch * d.c_elems, (int64_t)256 << 20, true)
+                                    : -1);
   Scratch& sc = scratch_for_device();
   if (precision == TN_PREC_FP16X3 && is_tc(kid)) {   // operand maxima for the FP16 scaling (one extra read)
     operand_maxima(reinterpret_cast<const float2*>(a), batch << ar, reinterpret_cast<const float2*>(b),
@@ -1915,7 +1989,10 @@ extern "C" tn_status tn_contract_pair_noalloc(const float* a, const int32_t* aw,
   order_pair_bits(d);
   const int kid = pick_kernel(precision, cmult, d, batch);
   GemmArgs g = make_args(d, kid, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
-                         reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems);
+                         reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems,
+                         is_tc(kid) ? tc_tile(kid, d.nm, d.nk, d.nn, batch, batch * d.c_elems,
+                                              (int64_t)(kNoAllocScratchBytes - kNoAllocErrBytes), true)
+                                    : -1);
   const int64_t cap = (int64_t)(kNoAllocScratchBytes - kNoAllocErrBytes);
   uint8_t* base = static_cast<uint8_t*>(noalloc_scratch_address());
   int32_t* err = reinterpret_cast<int32_t*>(base);
