@@ -52,11 +52,17 @@ constexpr int SIMT_MAX_SPLIT = 8;   // CTAs of one split-K cluster (the portable
 
 // A tiling: TM x TN outputs per CTA, TK of k per stage, RM x RN outputs per
 // thread, KG groups of threads that each take 1/KG of a stage's k (their sums
-// are added at the end), MINB CTAs per SM that the registers are kept to.  A is
-// staged as two planes (re, im) whose consecutive rows make the packed pairs.
-template <int TM_, int TN_, int TK_, int RM_, int RN_, int KG_, int MINB_>
+// are added at the end), MINB CTAs per SM that the registers are kept to, NST
+// stages, filled by asynchronous copies NST - 1 chunks ahead or (REGS) through
+// registers one chunk ahead.  Copies need no registers and hide the latency of
+// operands that come from HBM, but move 4 bytes at a time (the two planes), twice
+// the L1 requests of the register path's 16-byte loads.  A is staged as two planes (re, im) whose consecutive rows make the
+// packed pairs.
+template <int TM_, int TN_, int TK_, int RM_, int RN_, int KG_, int MINB_, int NST_, bool REGS_>
 struct SimtCfg {
   static constexpr int TM = TM_, TN = TN_, TK = TK_, RM = RM_, RN = RN_, KG = KG_, MINB = MINB_;
+  static constexpr int NST = NST_;
+  static constexpr bool REGS = REGS_;
   static constexpr int NTX = TM / RM, NTY = TN / RN;
   static_assert(NTX * NTY * KG == SIMT_THREADS, "one thread per RM x RN outputs and k group");
   static constexpr int RG = RM < 4 ? RM : 4;           // consecutive rows of a thread
@@ -71,7 +77,7 @@ struct SimtCfg {
 template <class Cfg>
 struct SimtSmem {
   union alignas(16) {
-    typename Cfg::Stage st[2];
+    typename Cfg::Stage st[Cfg::NST];
     // partial tiles of the k groups (column-major); the first one then takes their sum
     float2 part[Cfg::SPLIT ? Cfg::KG : 1][Cfg::SPLIT ? Cfg::TN : 1][Cfg::SPLIT ? Cfg::TM + 2 : 1];
   };
@@ -83,16 +89,16 @@ struct SimtSmem {
   int64_t kdB[KMAXR];
 };
 
-using SimtBig = SimtCfg<128, 64, 8, 8, 4, 1, 2>;
-using Simt64 = SimtCfg<64, 64, 8, 4, 4, 1, 3>;
-using Simt128x16 = SimtCfg<128, 16, 16, 4, 2, 1, 3>;
-using Simt256x4 = SimtCfg<256, 4, 8, 4, 1, 1, 4>;
-using Simt32 = SimtCfg<32, 32, 32, 4, 4, 4, 2>;
+using SimtBig = SimtCfg<128, 64, 8, 8, 4, 1, 2, 3, false>;
+using SimtBigR = SimtCfg<128, 64, 8, 8, 4, 1, 2, 2, true>;
+using Simt64 = SimtCfg<64, 64, 8, 4, 4, 1, 3, 2, true>;
+using Simt128x16 = SimtCfg<128, 16, 16, 4, 2, 1, 3, 2, false>;
+using Simt256x4 = SimtCfg<256, 4, 8, 4, 1, 1, 4, 2, false>;
+using Simt32 = SimtCfg<32, 32, 32, 4, 4, 4, 2, 2, false>;
 
 // One thread's pairs of tile elements (2p, 2p + 1) of an operand: the elements
 // of a tile are numbered by the tile bits in ascending memory position, so
-// consecutive threads read consecutive addresses, and a pair is one 16-byte load
-// where the operand's position 0 is a tile bit.
+// consecutive threads read consecutive addresses.
 template <int NP>
 struct PairMap {
   int64_t off[NP];   // memory offset of the pair's first element
@@ -126,6 +132,33 @@ __device__ __forceinline__ void pair_map(PairMap<NP>& m, int tbits, const int8_t
       }
   }
 }
+// Asynchronous copies global -> shared of 4 and 8 bytes (no registers between)
+__device__ __forceinline__ void cp_async_f1(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_f2(float2* dst, const float2* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait_groups() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Loads that stay where they are written: left to the compiler, the next chunk's
+// loads moved down to their use, behind the products they should run under.
+__device__ __forceinline__ float4 ldv4(const float2* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float2 ldv2(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
 template <int NP>
 __device__ __forceinline__ void pair_load(float4 (&v)[NP], const PairMap<NP>& m, const float2* base, bool vec) {
 #pragma unroll
@@ -133,10 +166,10 @@ __device__ __forceinline__ void pair_load(float4 (&v)[NP], const PairMap<NP>& m,
     if (m.at[j] >= 0) {
       const float2* p = base + m.off[j];
       if (vec) {
-        v[j] = __ldg(reinterpret_cast<const float4*>(p));
+        v[j] = ldv4(p);
       } else {
-        const float2 x = __ldg(p);
-        const float2 y = m.dat ? __ldg(p + m.step) : make_float2(0.f, 0.f);
+        const float2 x = ldv2(p);
+        const float2 y = m.dat ? ldv2(p + m.step) : make_float2(0.f, 0.f);
         v[j] = make_float4(x.x, x.y, y.x, y.y);
       }
     }
@@ -151,10 +184,11 @@ __device__ __forceinline__ void pair_load(float4 (&v)[NP], const PairMap<NP>& m,
 // Large GEMMs are bound by the FP32 pipe's issue slots: a product of two packed
 // FMAs takes half the slots of four scalar ones, and 8 x 4 outputs per thread
 // leave 24 register moves and 8 shared loads per 64 of them; 4096 x 1024 x 4096
-// runs at 56 TFLOP/s (35 with scalar FMAs and 4 x 4 outputs), of about 70.  Small
-// ones are bound by latency: k offsets advance by one table entry per chunk
-// (decoding all k bits per chunk took longer than the chunk's products), and one
-// chunk with its set-up takes about 5 us in a chain of launches (12 before).
+// runs at 55 TFLOP/s (35 with scalar FMAs and 4 x 4 outputs), 2^17 x 256 x 256 at 52
+// (34), of about 70.  Small ones are bound by latency: k offsets advance by one
+// table entry per chunk (decoding all k bits per chunk took longer than the
+// chunk's products), and one chunk with its set-up takes about 3 us in a chain of
+// launches (12 before).
 template <class Cfg>
 __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int bz, int gz, int split, int rank,
                                           SimtSmem<Cfg>& sm) {
@@ -187,11 +221,17 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
   PairMap<BP> mb;
   pair_map(ma, g.a_tbits, g.a_tpos, g.a_tsel);
   pair_map(mb, g.b_tbits, g.b_tpos, g.b_tsel);
-  const bool va = g.a_tbits > 0 && g.a_tpos[0] == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
-  const bool vb = g.b_tbits > 0 && g.b_tpos[0] == 0 && (reinterpret_cast<uintptr_t>(g.B) & 15) == 0;
   const int64_t abase = warp_deposit((uint32_t)bx, g.a_mpos, g.tm, g.nm) + warp_deposit((uint32_t)kc0, g.a_kpos, g.tk, g.nk);
   const int64_t bbase = warp_deposit((uint32_t)by, g.b_npos, g.tn, g.nn) + warp_deposit((uint32_t)kc0, g.b_kpos, g.tk, g.nk);
   const int64_t cbase = warp_deposit((uint32_t)bx, g.c_mpos, g.tm, g.nm) + warp_deposit((uint32_t)by, g.c_npos, g.tn, g.nn);
+  const float2 *A0, *B0;
+  float2* C0;
+  auto inst_bases = [&](int inst) {
+    A0 = g.A + warp_inst_offset(inst, g.a_istride, g.a_bpos, g.nb) + abase;
+    B0 = g.B + warp_inst_offset(inst, g.b_istride, g.b_bpos, g.nb) + bbase;
+    C0 = g.C + warp_inst_offset(inst, g.c_istride, g.c_bpos, g.nb) + cbase;
+  };
+  inst_bases(bz);
   __syncthreads();
   pdl_wait();
 
@@ -206,34 +246,32 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
       simt_cluster_sync();
       continue;
     }
-    const float2* A = g.A + warp_inst_offset(inst, g.a_istride, g.a_bpos, g.nb) + abase;
-    const float2* B = g.B + warp_inst_offset(inst, g.b_istride, g.b_bpos, g.nb) + bbase;
-    float2* C = g.C + warp_inst_offset(inst, g.c_istride, g.c_bpos, g.nb) + cbase;
+    if (it > 0) inst_bases(inst);
+    const float2* A = A0;
+    const float2* B = B0;
+    float2* C = C0;
     f32x2 re[RP][RN], im[RP][RN];
 #pragma unroll
     for (int i = 0; i < RP; ++i)
 #pragma unroll
       for (int j = 0; j < RN; ++j) re[i][j] = im[i][j] = 0ull;
-    float4 la[AP], lb[BP];
-    auto put = [&](typename Cfg::Stage& st) {
+    auto issue = [&](typename Cfg::Stage& st) {
+      auto put_a = [&](int at, const float2* p) {
+        cp_async_f1(&st.ar[at >> 16][at & 0xffff], &p->x);
+        cp_async_f1(&st.ai[at >> 16][at & 0xffff], &p->y);
+      };
 #pragma unroll
       for (int j = 0; j < AP; ++j)
         if (ma.at[j] >= 0) {
-          const int k = ma.at[j] >> 16, r = ma.at[j] & 0xffff;
-          st.ar[k][r] = la[j].x;
-          st.ai[k][r] = la[j].y;
-          if (ma.dat) {
-            const int k2 = (ma.at[j] + ma.dat) >> 16, r2 = (ma.at[j] + ma.dat) & 0xffff;
-            st.ar[k2][r2] = la[j].z;
-            st.ai[k2][r2] = la[j].w;
-          }
+          put_a(ma.at[j], A + ma.off[j]);
+          if (ma.dat) put_a(ma.at[j] + ma.dat, A + ma.off[j] + ma.step);
         }
-      auto putb = [&](int at, float x, float y) { st.b[at >> 16][at & 0xffff] = make_float2(x, y); };
 #pragma unroll
       for (int j = 0; j < BP; ++j)
         if (mb.at[j] >= 0) {
-          putb(mb.at[j], lb[j].x, lb[j].y);
-          if (mb.dat) putb(mb.at[j] + mb.dat, lb[j].z, lb[j].w);
+          const int at = mb.at[j], a2 = at + mb.dat;
+          cp_async_f2(&st.b[at >> 16][at & 0xffff], B + mb.off[j]);
+          if (mb.dat) cp_async_f2(&st.b[a2 >> 16][a2 & 0xffff], B + mb.off[j] + mb.step);
         }
     };
     auto step = [&](const typename Cfg::Stage& st, int kk) {
@@ -269,29 +307,86 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
         }
       }
     };
-    pair_load(la, ma, A, va);
-    pair_load(lb, mb, B, vb);
-    put(sm.st[0]);
-    __syncthreads();
-    for (int c = 0; c < kc_per; ++c) {
-      const bool more = c + 1 < kc_per;
-      if (more) {   // the next chunk's loads run under this chunk's products
-        const int t = __ffs(~(kc0 + c)) - 1;   // trailing ones of the chunk index
-        A += sm.kdA[t];
-        B += sm.kdB[t];
+    constexpr int NST = Cfg::NST;
+    if constexpr (Cfg::REGS) {
+      static_assert(!Cfg::REGS || (Cfg::KG == 1 && NST == 2), "one k group, two stages");
+      float4 la[AP], lb[BP];
+      const bool va = g.a_tbits > 0 && g.a_tpos[0] == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
+      const bool vb = g.b_tbits > 0 && g.b_tpos[0] == 0 && (reinterpret_cast<uintptr_t>(g.B) & 15) == 0;
+      auto load = [&]() {
         pair_load(la, ma, A, va);
         pair_load(lb, mb, B, vb);
-      }
-      const typename Cfg::Stage& st = sm.st[c & 1];
-      if (TKv == TK) {
-#pragma unroll(RM * RN >= 32 ? 4 : 8)
-        for (int kk = 0; kk < TK / Cfg::KG; ++kk) step(st, kk * Cfg::KG + kg);
-      } else {
-        for (int kk = kg; kk < TKv; kk += Cfg::KG) step(st, kk);
-      }
-      if (more) put(sm.st[(c + 1) & 1]);   // last read before the previous barrier
+      };
+      auto put = [&](typename Cfg::Stage& st) {
+        auto put_a = [&](int at, float x, float y) {
+          st.ar[at >> 16][at & 0xffff] = x;
+          st.ai[at >> 16][at & 0xffff] = y;
+        };
+#pragma unroll
+        for (int j = 0; j < AP; ++j)
+          if (ma.at[j] >= 0) {
+            put_a(ma.at[j], la[j].x, la[j].y);
+            if (ma.dat) put_a(ma.at[j] + ma.dat, la[j].z, la[j].w);
+          }
+#pragma unroll
+        for (int j = 0; j < BP; ++j)
+          if (mb.at[j] >= 0) {
+            const int at = mb.at[j], a2 = at + mb.dat;
+            st.b[at >> 16][at & 0xffff] = make_float2(lb[j].x, lb[j].y);
+            if (mb.dat) st.b[a2 >> 16][a2 & 0xffff] = make_float2(lb[j].z, lb[j].w);
+          }
+      };
+      load();
+      put(sm.st[0]);
       __syncthreads();
+      for (int c = 0; c < kc_per; ++c) {
+        const bool more = c + 1 < kc_per;
+        if (more) {
+          const int t = __ffs(~(kc0 + c)) - 1;
+          A += sm.kdA[t];
+          B += sm.kdB[t];
+          load();
+        }
+        const typename Cfg::Stage& st = sm.st[c & 1];
+        if (TKv == TK) {
+#pragma unroll(RM * RN >= 32 ? 4 : 8)
+          for (int kk = 0; kk < TK; ++kk) step(st, kk);
+        } else {
+          for (int kk = 0; kk < TKv; ++kk) step(st, kk);
+        }
+        if (more) put(sm.st[(c + 1) & 1]);
+        __syncthreads();
+      }
+    } else {
+      // NST - 1 chunks in flight ahead of the one being multiplied; a chunk's stage
+      // was last read before the barrier that lets its copies be issued
+      auto next = [&](int c) {   // chunk c's copies, as one group (empty past the end)
+        if (c < kc_per) {
+          if (c > 0) {
+            const int t = __ffs(~(kc0 + c - 1)) - 1;   // trailing ones of the chunk before
+            A += sm.kdA[t];
+            B += sm.kdB[t];
+          }
+          issue(sm.st[c % NST]);
+        }
+        cp_async_commit_group();
+      };
+#pragma unroll
+      for (int c = 0; c < NST - 1; ++c) next(c);
+      for (int c = 0; c < kc_per; ++c) {
+        cp_async_wait_groups<NST - 2>();
+        __syncthreads();
+        next(c + NST - 1);
+        const typename Cfg::Stage& st = sm.st[c % NST];
+        if (TKv == TK) {
+#pragma unroll(RM * RN >= 32 ? 4 : 8)
+          for (int kk = 0; kk < TK / Cfg::KG; ++kk) step(st, kk * Cfg::KG + kg);
+        } else {
+          for (int kk = kg; kk < TKv; kk += Cfg::KG) step(st, kk);
+        }
+      }
     }
+    __syncthreads();   // the stages are free for the partial tiles or the next instance
     if constexpr (!Cfg::SPLIT) {
       const bool vc = g.tm > 0 && g.c_mpos[0] == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
 #pragma unroll
@@ -321,8 +416,7 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
         }
       }
     } else {
-      // the k groups' partial tiles to shared memory (the stages are done with:
-      // barrier above), added in group order; with a split, each CTA then adds its
+      // the k groups' partial tiles to shared memory, added in group order; with a split, each CTA then adds its
       // share of the tile's elements over the cluster, in rank order
 #pragma unroll
       for (int i = 0; i < RP; ++i) {
