@@ -256,6 +256,9 @@ tn_status tn_plan_model_time(const tn_plan_t* plan, double peak_flops, double pe
  * The first call on a plan allocates the plan's device arena, workspace and
  * the B' image buffers of steps whose B operand depends on no slice (all freed
  * by tn_plan_destroy) and uploads the leaf tensors; that call synchronises.
+ * Plans of small chunks hold several arenas, 64 MB (and max_arena_bytes) at most,
+ * and run that many chunks of a call side by side, of one batch or of several;
+ * the amplitudes are the same bits as chunk by chunk.
  * Steps that depend on no slice, and those B' images, are computed once per
  * plan, or once per batch when they depend on the closed bits (main text,
  * section III: the major part of the network is shared by a correlated batch).

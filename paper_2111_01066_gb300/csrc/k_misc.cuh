@@ -8,12 +8,21 @@
 namespace tnx {
 
 // Materialise every leaf of the chunk: the sliced wires take the bits of the
-// slice id, the closed output wires the bits of the batch's bitstring.  Also
-// clears amax[z0, z1) (FP16 split: the maxima the coming steps record).
+// slice id, the closed output wires the bits of the batch's bitstring.  Lane
+// blockIdx.y does so for the chunk params[counter + lane] in its own arena: the
+// chunks of several lanes then run through the same launches, as further instances
+// of every step, which is what chains of steps too small for the GPU wait for (a
+// chunk of 11 steps of 2^11 multiply-adds or less takes 36 us of launches, nine of
+// them side by side hardly more).  Also clears amax[z0, z1) of the lane (FP16 split:
+// the maxima the coming steps record).
 __global__ void __launch_bounds__(128) k_leaf_select(const float2* __restrict__ leaf_data,
                                                      const LeafDesc* __restrict__ leaves, int n_leaves,
                                                      float2* __restrict__ arena, const ChunkParam* __restrict__ params,
-                                                     const unsigned* __restrict__ counter, float* amax, int z0, int z1) {
+                                                     const unsigned* __restrict__ counter, int64_t lane_stride,
+                                                     float* amax, int amax_lane, int z0, int z1) {
+  const int lane = blockIdx.y;
+  arena += lane * lane_stride;
+  amax += (int64_t)lane * amax_lane;
   __shared__ LeafDesc d;
   static_assert(sizeof(LeafDesc) % 4 == 0, "LeafDesc is copied in 4-byte words");
   bool waited = false;
@@ -25,7 +34,7 @@ __global__ void __launch_bounds__(128) k_leaf_select(const float2* __restrict__ 
     __syncthreads();
     if (!waited) {
       pdl_wait();
-      p = params[__ldcg(counter)];
+      p = params[__ldcg(counter) + lane];
       for (int i = z0 + blockIdx.x * blockDim.x + threadIdx.x; i < z1; i += gridDim.x * blockDim.x) amax[i] = 0.f;
       waited = true;
     }
@@ -55,16 +64,16 @@ __global__ void __launch_bounds__(128) k_leaf_select(const float2* __restrict__ 
 }
 
 // Slice sum of a chunk (main text, section II: the sliced network is the sum of
-// the smaller networks) in FP64, deterministic: block (x, g) sums the slices of
-// group g (slices g*per .. g*per+per-1 of the chunk) for its amplitudes j into
-// part[g][j]; the last of the groups' blocks to arrive for the same amplitudes
-// (tickets[x]) adds the groups in order into out[batch][j], and the last block
-// of all advances the chunk counter.  Slices outside the call's range are
+// the smaller networks) in FP64, deterministic: block (x, g, lane) sums the slices of
+// group g (slices g*per .. g*per+per-1 of the lane's chunk) for its amplitudes j into
+// part[lane][g][j]; the last of the blocks to arrive for the same amplitudes
+// (tickets[x]) adds lanes and groups in order into out[batch][j], and the last block
+// of all advances the chunk counter by the lanes.  Slices outside the call's range are
 // skipped.  The tickets are zero between launches.
 __global__ void __launch_bounds__(256) k_root_sum(const float2* __restrict__ arena, const RootDesc r, int b,
                                                  int groups, double2* __restrict__ part,
                                                  const ChunkParam* __restrict__ params, unsigned* counter,
-                                                 unsigned* tickets) {
+                                                 unsigned* tickets, int64_t lane_stride) {
   // the group's slices in rounds of 256: their instance offsets in the root
   // (or -1 outside the call's range) are found once per block, then every
   // thread adds its amplitudes over them with four independent FP64
@@ -74,7 +83,10 @@ __global__ void __launch_bounds__(256) k_root_sum(const float2* __restrict__ are
   __shared__ int64_t s_off[256];
   __shared__ int s_last;
   pdl_wait();
-  const ChunkParam p = params[__ldcg(counter)];   // the counter changes under a running kernel: past L1
+  const int lane = blockIdx.z, lanes = gridDim.z;
+  const unsigned first = __ldcg(counter);   // changes under a running kernel: past L1
+  const ChunkParam p = params[first + lane];
+  arena += lane * lane_stride;
   const int k = r.rank;
   const int64_t nout = (int64_t)1 << k;
   const uint32_t per = (1u << b) / (uint32_t)groups;
@@ -143,43 +155,65 @@ __global__ void __launch_bounds__(256) k_root_sum(const float2* __restrict__ are
     for (int t = 0; t < MAXJ; ++t)
       if (t < nj) {
         const int64_t j = j0 + (int64_t)(jj0 + t) * jstep;
-        part[(int64_t)g * nout + j] = make_double2((ar[t][0] + ar[t][1]) + (ar[t][2] + ar[t][3]),
+        part[((int64_t)lane * groups + g) * nout + j] = make_double2((ar[t][0] + ar[t][1]) + (ar[t][2] + ar[t][3]),
                                                    (ai[t][0] + ai[t][1]) + (ai[t][2] + ai[t][3]));
       }
   }
-  // the last group's block for these amplitudes sums the groups
+  // the last block for these amplitudes sums lanes and groups
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&tickets[1 + blockIdx.x], 1u) == (unsigned)groups - 1u;
+  const int parts = lanes * groups;
+  if (threadIdx.x == 0) s_last = atomicAdd(&tickets[1 + blockIdx.x], 1u) == (unsigned)parts - 1u;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  double* __restrict__ out = p.out;
   for (int64_t j = j0; j < nout; j += jstep) {
-    double sr = 0.0, si = 0.0;
-    // eight loads in flight, added in group order
-    for (int q0 = 0; q0 < groups; q0 += 8) {
+    double* o = nullptr;         // the batch's amplitude: lanes of one batch follow each other
+    double ar0 = 0.0, ai0 = 0.0;
+    double sr = 0.0, si = 0.0;   // the lane's sum
+    // eight loads in flight, added in order
+    for (int q0 = 0; q0 < parts; q0 += 8) {
       double2 v[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        v[u] = q0 + u < groups ? __ldcg(part + (int64_t)(q0 + u) * nout + j) : make_double2(0.0, 0.0);
+        v[u] = q0 + u < parts ? __ldcg(part + (int64_t)(q0 + u) * nout + j) : make_double2(0.0, 0.0);
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (q0 + u < groups) {
+        if (q0 + u < parts) {
           sr += v[u].x;
           si += v[u].y;
+          const int l = (q0 + u) / groups;
+          if (q0 + u == (l + 1) * groups - 1) {   // the lane is complete
+            const ChunkParam& pl = params[first + l];
+            if (pl.valid_lo < pl.valid_hi) {      // (a lane without slices only fills the launch)
+              double* ol = pl.out + 2 * (pl.out_index * nout + j);
+              if (ol != o) {
+                if (o) {
+                  o[0] = ar0;
+                  o[1] = ai0;
+                }
+                o = ol;
+                ar0 = o[0];
+                ai0 = o[1];
+              }
+              ar0 += sr;
+              ai0 += si;
+            }
+            sr = si = 0.0;
+          }
         }
     }
-    double* o = out + 2 * (p.out_index * nout + j);
-    o[0] += sr;
-    o[1] += si;
+    if (o) {
+      o[0] = ar0;
+      o[1] = ai0;
+    }
   }
   if (threadIdx.x == 0) {
     tickets[1 + blockIdx.x] = 0;
     // all blocks have read the counter: each did before its arrival above
     if (atomicAdd(&tickets[0], 1u) == gridDim.x - 1u) {
       tickets[0] = 0;
-      *counter += 1u;
+      *counter = first + (unsigned)lanes;
     }
   }
 }

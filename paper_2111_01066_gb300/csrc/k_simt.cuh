@@ -469,7 +469,8 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
       simt_cluster_sync();   // the peers have read this CTA's partial tile
     }
   }
-  if (g.amax_c) amax_update(g.amax_c, am);   // every thread reaches here
+  // every thread reaches here; with several lanes a block has one instance (bz)
+  if (g.amax_c) amax_update(g.amax_c + (int64_t)(bz >> (g.nb - g.ls_lanes)) * g.amax_lane, am);
 }
 
 __device__ __forceinline__ void copy_args(GemmArgs& dst, const GemmArgs* src) {

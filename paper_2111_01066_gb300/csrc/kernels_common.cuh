@@ -64,6 +64,11 @@ struct GemmArgs {
   const float* amax_a;
   const float* amax_b;
   float* amax_c;
+  // lanes (chunks run side by side, one arena each, see k_leaf_select): their bits
+  // are the highest of the instance index; lane l records its maximum at
+  // amax_c + l * amax_lane
+  int32_t ls_lanes;                // log2 of the lanes (0: one)
+  int32_t amax_lane;
 };
 
 static_assert(sizeof(GemmArgs) % 4 == 0, "GemmArgs is copied to shared memory in 4-byte words");

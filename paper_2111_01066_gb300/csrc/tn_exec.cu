@@ -90,7 +90,8 @@ static int pick_simt(const StepDesc& d, int64_t n_inst) {
 // 8.3 over 4 CTAs (2 chunks each), 9.1 over 8; (7, 10, 6) 52, 17 and 12.
 static int simt_split(const GemmArgs& g, int kid) {
   if (kid != K_SIMT_32x32) return 1;
-  const int64_t tiles = ((int64_t)1 << (g.nm - g.tm)) * ((int64_t)1 << (g.nn - g.tn)) * g.n_inst;
+  // of one lane: the same sums however many chunks run side by side
+  const int64_t tiles = ((int64_t)1 << (g.nm - g.tm)) * ((int64_t)1 << (g.nn - g.tn)) * (g.n_inst >> g.ls_lanes);
   const int n_kc = 1 << (g.nk - g.tk);
   int sp = 1;
   while (sp < SIMT_MAX_SPLIT && sp * 4 <= n_kc && tiles * sp * 2 <= 2 * (int64_t)sm_count()) sp *= 2;
@@ -639,6 +640,44 @@ static void launch_step(StepLaunch& L, uint8_t* ws, int32_t* err, cudaStream_t s
 }
 
 // ------------------------------------------------------------------ plan device state
+// groups of small independent steps (StepDesc::group): per group, the steps
+// [first, end) and the launches that run them -- one multi-step launch for
+// all its CUDA-core steps (each block with its step's tiling), single
+// launches for its tensor-core steps; rebuilt whenever the kernels are
+// chosen again
+struct GroupRun {
+  int first = 0, end = 0;
+  std::vector<int> singles;                  // steps launched alone
+  struct Multi {
+    int blocks = 0, n = 0;
+    GemmArgs* args = nullptr;                // device: n GemmArgs
+    int32_t* start = nullptr;                // device: n + 1 block offsets
+    int8_t* tiling = nullptr;                // device: n CUDA-core tilings (simt_multi_tiling)
+    int8_t* split = nullptr;                 // device: n split-K factors
+  };
+  std::vector<Multi> multi;
+};
+
+// The launches of a plan for 2^ls lanes: CUDA-core steps with the lanes as further
+// instances, tensor-core steps once per lane (lane l > 0 in more[l - 1]), so that
+// a chunk's result does not depend on what runs beside it.
+struct LaunchSet {
+  int ls = 0;
+  bool built = false;
+  std::vector<StepLaunch> launches;
+  std::vector<std::vector<StepLaunch>> more;   // [lane - 1][step], tensor-core steps only
+  std::vector<GroupRun> groups;
+  std::vector<int> group_at;                   // per step: its group run's index, or -1
+  uint8_t* group_buf = nullptr;                // device memory of every Multi's arrays
+  // the launch sequences as CUDA graphs, each captured at its second use (the
+  // first runs eagerly): [0] a chunk per lane, [1] with the prologue of new
+  // batches; every kernel reads its chunk parameters from device memory
+  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  bool graph_failed[2] = {false, false};
+  bool eager_done[2] = {false, false};
+};
+constexpr int MAX_LS_LANES = 4;
+
 struct DeviceState {
   int device = -1;
   float2* arena = nullptr;
@@ -653,44 +692,26 @@ struct DeviceState {
   double2* root_part = nullptr;   // [groups][2^k] partial slice sums
   unsigned* root_tickets = nullptr;   // arrivals of the slice sum's blocks (zero between launches)
   int root_blocks = 1;
-  float* amax = nullptr;          // FP16X3: largest component of every node (leaves, then steps)
+  float* amax = nullptr;          // FP16X3: largest component of every node (leaves, then steps), per lane
+  int amax_nodes = 0;
   int root_groups = 1;
-  std::vector<StepLaunch> launches;
-  // groups of small independent steps (StepDesc::group): per group, the steps
-  // [first, end) and the launches that run them -- one multi-step launch for
-  // all its CUDA-core steps (each block with its step's tiling), single
-  // launches for its tensor-core steps; rebuilt whenever the kernels are
-  // chosen again
-  struct GroupRun {
-    int first = 0, end = 0;
-    std::vector<int> singles;                  // steps launched alone
-    struct Multi {
-      int blocks = 0, n = 0;
-      GemmArgs* args = nullptr;                // device: n GemmArgs
-      int32_t* start = nullptr;                // device: n + 1 block offsets
-      int8_t* tiling = nullptr;                // device: n CUDA-core tilings (simt_multi_tiling)
-      int8_t* split = nullptr;                 // device: n split-K factors
-    };
-    std::vector<Multi> multi;
-  };
-  std::vector<GroupRun> groups;
-  std::vector<int> group_at;                   // per step: its group run's index, or -1
-  uint8_t* group_buf = nullptr;                // device memory of every Multi's arrays
+  LaunchSet set[MAX_LS_LANES + 1];
+  std::vector<StepLaunch>& launches = set[0].launches;
+  int ls_lanes = 0;               // lanes that the arena has room for (log2)
+  int64_t lane_stride = 0;        // elements between the lanes' arenas (a power of two where there are several)
   std::vector<uint8_t*> own_imgs;              // B' images built ahead of the chunks (StepLaunch::bimg_own)
   cudaEvent_t done = nullptr;
   bool have_done = false;
-  // launch sequences as CUDA graphs, each captured at its second use (the first
-  // runs eagerly): [0] a chunk, [1] a chunk that opens a new batch, with the
-  // batch's prologue; every kernel reads its chunk parameters from device memory
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};
-  bool graph_failed[2] = {false, false};
-  bool eager_done[2] = {false, false};
   // prologues: steps whose result depends on no slice run once per plan
   // (dependence flags 0) or once per batch bitstring (flags 2); their results
-  // that later steps read sit in the arena's persistent pool
-  bool pro0_done = false;
-  bool pro2_valid = false;
-  uint64_t pro2_bits = 0;
+  // that later steps read sit in the arena's persistent pool, each lane's in its own
+  int pro0_lanes = 0;             // lanes whose per-plan steps have run
+  bool pro2_valid[1 << MAX_LS_LANES] = {false};
+  uint64_t pro2_bits[1 << MAX_LS_LANES] = {0};
+  void forget_prologues() {
+    pro0_lanes = 0;
+    for (bool& v : pro2_valid) v = false;
+  }
 };
 
 static int tc_kernel(int precision, int cmult) {
@@ -714,13 +735,21 @@ static int pick_kernel(int precision, int cmult, const StepDesc& d, int64_t n_in
 
 // Launch arguments of plan step d for kernel kid; FP16X3 plans also get the
 // maxima of the step's operands (to scale them) and of its result (to record).
-static GemmArgs step_args(const DeviceState& ds, const StepDesc& d, int kid, int tn_log = -1) {
-  GemmArgs g = make_args(d, kid, ds.arena + d.a_off, ds.arena + d.b_off, ds.arena + d.c_off, 1 << d.nb, 0, 0, 0,
-                         tn_log);
+// lane: the arena of that lane alone; ls > 0: all of 2^ls lanes as instances.
+static GemmArgs step_args(const DeviceState& ds, const StepDesc& d, int kid, int tn_log = -1, int lane = 0, int ls = 0) {
+  float2* arena = ds.arena + lane * ds.lane_stride;
+  GemmArgs g = make_args(d, kid, arena + d.a_off, arena + d.b_off, arena + d.c_off, 1 << (d.nb + ls), 0, 0, 0, tn_log);
+  for (int t = 0; t < ls; ++t)
+    g.a_bpos[d.nb + t] = g.b_bpos[d.nb + t] = g.c_bpos[d.nb + t] =
+        (int8_t)(__builtin_ctzll((uint64_t)ds.lane_stride) + t);
+  g.nb = d.nb + ls;
+  g.ls_lanes = ls;
   if (ds.amax) {
-    g.amax_a = ds.amax + d.a_node;
-    g.amax_b = ds.amax + d.b_node;
-    g.amax_c = ds.amax + d.c_node;
+    float* amax = ds.amax + (int64_t)lane * ds.amax_nodes;
+    g.amax_a = amax + d.a_node;
+    g.amax_b = amax + d.b_node;
+    g.amax_c = amax + d.c_node;
+    g.amax_lane = ls ? ds.amax_nodes : 0;
   }
   return g;
 }
@@ -730,7 +759,7 @@ static int simt_multi_tiling(int kid) {
   return kid == K_SIMT_32x32 ? 3 : (kid >= K_SIMT_64x64 && kid <= K_SIMT_256x4 ? kid : -1);
 }
 
-static void launch_simt_multi(const DeviceState::GroupRun::Multi& m, cudaStream_t s) {
+static void launch_simt_multi(const GroupRun::Multi& m, cudaStream_t s) {
   klaunch(k_cgemm_simt_multi, dim3((unsigned)m.blocks), SIMT_THREADS, 0, s, SIMT_MAX_SPLIT, true,
           (const GemmArgs*)m.args, (const int32_t*)m.start, (const int8_t*)m.tiling, (const int8_t*)m.split, (int32_t)m.n);
 }
@@ -759,7 +788,9 @@ static void setup_hoisted(Plan& p, DeviceState& ds) {
     L.bimg_own = nullptr;
     L.bimg_cls = -1;
     const StepDesc& d = p.steps[i];
-    if (!is_tc(L.kid) || !(d.dep_flags & 1)) continue;
+    // (several lanes: a batch's prologue may run for one lane in one set of launches
+    // and its chunks in another; the images are then built with every launch)
+    if (ds.ls_lanes > 0 || !is_tc(L.kid) || !(d.dep_flags & 1)) continue;
     const int bf = node_flags(p, d.b_node);
     if (bf & 1) continue;
     const int64_t img = L.tc.n_split > 1 ? L.split_off : L.ws_bytes;
@@ -775,7 +806,7 @@ static void setup_hoisted(Plan& p, DeviceState& ds) {
 }
 
 // Group runs from the plan's step groups and the kernels chosen so far.
-static void build_groups(Plan& p, DeviceState& ds) {
+static void build_groups(const Plan& p, LaunchSet& ds) {
   if (ds.group_buf) {
     CK(cudaFree(ds.group_buf));
     ds.group_buf = nullptr;
@@ -792,7 +823,7 @@ static void build_groups(Plan& p, DeviceState& ds) {
       i = j;
       continue;
     }
-    DeviceState::GroupRun gr;
+    GroupRun gr;
     gr.first = (int)i;
     gr.end = (int)j;
     std::vector<int> simt;
@@ -802,7 +833,7 @@ static void build_groups(Plan& p, DeviceState& ds) {
     }
     if (simt.size() == 1) gr.singles.push_back(simt[0]);
     if (simt.size() >= 2) {
-      DeviceState::GroupRun::Multi m;
+      GroupRun::Multi m;
       m.n = (int)simt.size();
       gr.multi.push_back(m);
       pending.push_back({ds.groups.size(), simt});
@@ -858,6 +889,55 @@ static void build_groups(Plan& p, DeviceState& ds) {
   CK(cudaMemcpy(ds.group_buf, host.data(), bytes, cudaMemcpyHostToDevice));
 }
 
+// Step d's launch with one kernel choice (as the autotuner builds its candidates).
+static StepLaunch build_choice(const DeviceState& ds, const StepDesc& d, int kid, int tn_log, int epi, int bslots,
+                               int pair, int lane = 0) {
+  return make_launch(step_args(ds, d, kid, tn_log, lane), kid, 64 - __builtin_clzll((uint64_t)d.a_elems) - 1, 1,
+                     d.c_elems, true, epi, (int64_t)256 << 20, bslots, pair);
+}
+
+// The launch set of 2^ls lanes, built from the kernels chosen for one lane.
+static void ensure_set(Plan& p, DeviceState& ds, int ls) {
+  LaunchSet& st = ds.set[ls];
+  if (st.built) return;
+  if (ls > 0) {
+    st.ls = ls;
+    st.launches.clear();
+    st.more.assign(((size_t)1 << ls) - 1, {});
+    for (size_t i = 0; i < p.steps.size(); ++i) {
+      const StepDesc& d = p.steps[i];
+      const StepLaunch& one = ds.launches[i];
+      if (is_tc(one.kid)) {
+        st.launches.push_back(one);
+        for (int l = 1; l < (1 << ls); ++l)
+          st.more[l - 1].push_back(build_choice(ds, d, one.kid, one.g.tn, one.tc.epi_ok, one.tc.nbs, one.tc.pair, l));
+      } else {
+        const GemmArgs g = step_args(ds, d, one.kid, -1, 0, ls);
+        st.launches.push_back(make_launch(g, one.kid, 0, 1));
+        for (auto& m : st.more) m.push_back(StepLaunch());
+      }
+    }
+  }
+  build_groups(p, st);
+  st.built = true;
+}
+
+static int ceil_log2(int64_t v) { return v <= 1 ? 0 : 64 - __builtin_clzll((uint64_t)(v - 1)); }
+
+// Lanes of a plan (log2): as many as keep their arenas in 64 MB -- in L2, and of
+// plans whose chunks are so small that they are launches and latency rather than
+// work -- and under the caller's bound, at most 16.
+static int lanes_of(const Plan& p) {
+  const int64_t cap = std::min<int64_t>((int64_t)64 << 20, p.opts.max_arena_bytes > 0 ? p.opts.max_arena_bytes : INT64_MAX);
+  const int64_t arena = (int64_t)sizeof(float2) << ceil_log2(std::max<int64_t>(p.arena_elems, 32));
+  const int64_t part = (int64_t)sizeof(double2) * std::min(1 << p.log2_batch, 64) << p.root.rank;
+  int nb = 0;
+  for (const StepDesc& d : p.steps) nb = std::max(nb, d.nb);
+  int ls = 0;
+  while (ls < MAX_LS_LANES && (arena << (ls + 1)) <= cap && (part << (ls + 1)) <= cap && nb + ls + 1 < KMAXB) ++ls;
+  return ls;
+}
+
 static void ensure_device(Plan& p) {
   int dev = 0;
   CK(cudaGetDevice(&dev));
@@ -869,7 +949,17 @@ static void ensure_device(Plan& p) {
   p.dev = ds;
   ds->device = dev;
   const size_t ab = std::max<size_t>(256, (size_t)p.arena_elems * sizeof(float2));
-  if (cudaMalloc(&ds->arena, ab) != cudaSuccess) {
+  ds->ls_lanes = lanes_of(p);
+  if (ds->ls_lanes > 0) {   // several arenas; where they cannot be had, one
+    ds->lane_stride = (int64_t)1 << ceil_log2(std::max<int64_t>(p.arena_elems, 32));
+    if (cudaMalloc(&ds->arena, ((size_t)ds->lane_stride * sizeof(float2)) << ds->ls_lanes) != cudaSuccess) {
+      cudaGetLastError();
+      ds->arena = nullptr;
+      ds->ls_lanes = 0;
+      ds->lane_stride = 0;
+    }
+  }
+  if (!ds->arena && cudaMalloc(&ds->arena, ab) != cudaSuccess) {
     cudaGetLastError();
     fail(TN_ERR_OOM, "arena allocation of " + std::to_string(ab) + " bytes failed");
   }
@@ -886,11 +976,14 @@ static void ensure_device(Plan& p) {
   CK(cudaEventCreateWithFlags(&ds->done, cudaEventDisableTiming));
   if (p.opts.precision == TN_PREC_FP16X3) {
     // leaves' maxima are constants of the plan; the steps' are recorded per chunk
-    const size_t nn = p.leaves.size() + p.steps.size();
-    CK(cudaMalloc(&ds->amax, sizeof(float) * std::max<size_t>(nn, 1)));
-    CK(cudaMemset(ds->amax, 0, sizeof(float) * std::max<size_t>(nn, 1)));
+    const size_t nn = std::max<size_t>(p.leaves.size() + p.steps.size(), 1);
+    ds->amax_nodes = (int)nn;
+    CK(cudaMalloc(&ds->amax, (sizeof(float) * nn) << ds->ls_lanes));
+    CK(cudaMemset(ds->amax, 0, (sizeof(float) * nn) << ds->ls_lanes));
     if (!p.leaf_amax.empty())
-      CK(cudaMemcpy(ds->amax, p.leaf_amax.data(), sizeof(float) * p.leaf_amax.size(), cudaMemcpyHostToDevice));
+      for (int l = 0; l < (1 << ds->ls_lanes); ++l)
+        CK(cudaMemcpy(ds->amax + l * nn, p.leaf_amax.data(), sizeof(float) * p.leaf_amax.size(),
+                      cudaMemcpyHostToDevice));
   }
   // bounds of every operand inside the arena, checked once on the host
   const int64_t ae = p.arena_elems;
@@ -932,23 +1025,24 @@ static void ensure_device(Plan& p) {
   }
   ds->ws_bytes = ws;
   ds->root_groups = std::min(1 << p.log2_batch, 64);
-  CK(cudaMalloc(&ds->root_part, sizeof(double2) * (size_t)ds->root_groups << p.root.rank));
+  CK(cudaMalloc(&ds->root_part, (sizeof(double2) * (size_t)ds->root_groups << p.root.rank) << ds->ls_lanes));
   ds->root_blocks = (int)std::min<int64_t>((((int64_t)1 << p.root.rank) + 255) / 256, 4096);
   CK(cudaMalloc(&ds->root_tickets, sizeof(unsigned) * (size_t)(1 + ds->root_blocks)));
   CK(cudaMemset(ds->root_tickets, 0, sizeof(unsigned) * (size_t)(1 + ds->root_blocks)));
   if (!in_arena(p.root.off, (int64_t)1 << p.root.rank, 1 << __builtin_popcount(p.root.bmask)))
     fail(TN_ERR_PLAN, "internal: root outside the arena");
-  build_groups(p, *ds);
+  ensure_set(p, *ds, 0);
   setup_hoisted(p, *ds);
 }
 
 static void drop_graphs(DeviceState& ds) {
-  for (int w = 0; w < 2; ++w) {
-    if (ds.graph[w]) cudaGraphExecDestroy(ds.graph[w]);
-    ds.graph[w] = nullptr;
-    ds.graph_failed[w] = false;
-    ds.eager_done[w] = false;
-  }
+  for (LaunchSet& st : ds.set)
+    for (int w = 0; w < 2; ++w) {
+      if (st.graph[w]) cudaGraphExecDestroy(st.graph[w]);
+      st.graph[w] = nullptr;
+      st.graph_failed[w] = false;
+      st.eager_done[w] = false;
+    }
 }
 
 void destroy_device_state(Plan* p) {
@@ -968,7 +1062,7 @@ void destroy_device_state(Plan* p) {
   cudaFree(ds->root_part);
   cudaFree(ds->root_tickets);
   cudaFree(ds->amax);
-  cudaFree(ds->group_buf);
+  for (LaunchSet& st : ds->set) cudaFree(st.group_buf);
   for (uint8_t* b : ds->own_imgs) cudaFree(b);
   drop_graphs(*ds);
   if (ds->done) cudaEventDestroy(ds->done);
@@ -981,18 +1075,23 @@ void destroy_device_state(Plan* p) {
 // of independent small steps runs as its multi-step launches, then the rest of
 // the group alone.
 template <class Pred>
-static void launch_class(Plan& p, cudaStream_t s, Pred in_class) {
+static void launch_class(Plan& p, cudaStream_t s, LaunchSet& st, Pred in_class) {
   DeviceState& ds = *p.dev;
+  auto one = [&](int i) {
+    launch_step(st.launches[i], ds.ws, ds.err, s, false);
+    if (is_tc(st.launches[i].kid))
+      for (auto& lane : st.more) launch_step(lane[i], ds.ws, ds.err, s, false);
+  };
   for (size_t i = 0; i < p.steps.size(); ++i) {
     if (!in_class(p.steps[i].dep_flags)) continue;
-    const int gi = ds.group_at.empty() ? -1 : ds.group_at[i];
+    const int gi = st.group_at.empty() ? -1 : st.group_at[i];
     if (gi < 0) {
-      launch_step(ds.launches[i], ds.ws, ds.err, s, false);
+      one((int)i);
       continue;
     }
-    const DeviceState::GroupRun& gr = ds.groups[gi];
+    const GroupRun& gr = st.groups[gi];
     for (const auto& m : gr.multi) launch_simt_multi(m, s);
-    for (int t : gr.singles) launch_step(ds.launches[t], ds.ws, ds.err, s, false);
+    for (int t : gr.singles) one(t);
     i = (size_t)gr.end - 1;
   }
 }
@@ -1001,7 +1100,7 @@ static void launch_class(Plan& p, cudaStream_t s, Pred in_class) {
 // maxima that the steps of the coming classes record (classes: bit 0
 // slice-dependent steps, bit 1 per-batch ones; 0 the per-plan ones); the
 // execution order keeps each class's steps together.
-static void launch_leaf_select(Plan& p, cudaStream_t s, int classes) {
+static void launch_leaf_select(Plan& p, cudaStream_t s, int classes, int ls) {
   DeviceState& ds = *p.dev;
   const int nl = (int)p.leaves.size();
   int z0 = 0, z1 = 0;
@@ -1015,10 +1114,10 @@ static void launch_leaf_select(Plan& p, cudaStream_t s, int classes) {
       z1 = nl + i + 1;
     }
   }
-  klaunch(k_leaf_select, dim3((unsigned)std::max(1, std::min(nl, 4096))), 128, 0, s, 1, true,
+  klaunch(k_leaf_select, dim3((unsigned)std::max(1, std::min(nl, 4096)), 1u << ls), 128, 0, s, 1, true,
           (const float2*)ds.leaf_data,
           (const LeafDesc*)ds.leaf_desc, nl, ds.arena, (const ChunkParam*)ds.params, (const unsigned*)ds.counter,
-          ds.amax, z0, z1);
+          ds.lane_stride, ds.amax, ds.amax_nodes, z0, z1);
 }
 
 // Whether a class has anything to run: 0, steps that depend on neither the
@@ -1033,10 +1132,10 @@ static bool has_prologue(const Plan& p, int cls) {
 }
 
 // The steps and B' images of one prologue class, on the leaves already selected.
-static void run_prologue(Plan& p, cudaStream_t s, int cls) {
+static void run_prologue(Plan& p, cudaStream_t s, LaunchSet& st, int cls) {
   DeviceState& ds = *p.dev;
-  launch_class(p, s, [cls](int f) { return f == cls; });
-  for (const StepLaunch& L : ds.launches) {
+  launch_class(p, s, st, [cls](int f) { return f == cls; });
+  for (const StepLaunch& L : st.launches) {
     if (!L.bimg_own || L.bimg_cls != cls) continue;
     TcArgs t = L.tc;
     t.bimg = L.bimg_own;
@@ -1045,48 +1144,47 @@ static void run_prologue(Plan& p, cudaStream_t s, int cls) {
   }
 }
 
-// One chunk; new_batch: with the batch's prologue, which works on the same leaf
-// select (the arena gives no leaf away before its last reader, and the prologue's
-// steps come before the chunk's in the order it was laid out for).
-static void run_chunk(Plan& p, cudaStream_t s, bool new_batch) {
+// One chunk per lane; new_batch: with their batches' prologues, which work on the
+// same leaf select (the arena gives no leaf away before its last reader, and the
+// prologue's steps come before the chunk's in the order it was laid out for).
+static void run_chunk(Plan& p, cudaStream_t s, LaunchSet& st, bool new_batch) {
   DeviceState& ds = *p.dev;
-  launch_leaf_select(p, s, new_batch ? 3 : 1);
-  if (new_batch) run_prologue(p, s, 2);
-  launch_class(p, s, [](int f) { return (f & 1) != 0; });   // slice-dependent steps
-  klaunch(k_root_sum, dim3((unsigned)ds.root_blocks, (unsigned)ds.root_groups), 256, 0, s, 1, true,
+  launch_leaf_select(p, s, new_batch ? 3 : 1, st.ls);
+  if (new_batch) run_prologue(p, s, st, 2);
+  launch_class(p, s, st, [](int f) { return (f & 1) != 0; });   // slice-dependent steps
+  klaunch(k_root_sum, dim3((unsigned)ds.root_blocks, (unsigned)ds.root_groups, 1u << st.ls), 256, 0, s, 1, true,
           (const float2*)ds.arena, p.root, p.log2_batch, ds.root_groups, ds.root_part, (const ChunkParam*)ds.params,
-          ds.counter, ds.root_tickets);
+          ds.counter, ds.root_tickets, ds.lane_stride);
 }
 
 // Capture run_chunk once into a graph (on a private stream, thread-local
 // capture mode).  Any failure leaves the plan on eager launches.
-static void capture_chunk_graph(Plan& p, bool new_batch) {
-  DeviceState& ds = *p.dev;
+static void capture_chunk_graph(Plan& p, LaunchSet& st, bool new_batch) {
   const int w = new_batch ? 1 : 0;
-  if (ds.graph[w] || ds.graph_failed[w]) return;
+  if (st.graph[w] || st.graph_failed[w]) return;
   cudaStream_t cs = nullptr;
   if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
-    ds.graph_failed[w] = true;
+    st.graph_failed[w] = true;
     return;
   }
   cudaGraph_t graph = nullptr;
   bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
   if (ok) {
     try {
-      run_chunk(p, cs, new_batch);
+      run_chunk(p, cs, st, new_batch);
     } catch (const TnError&) {
       ok = false;
     }
     ok = (cudaStreamEndCapture(cs, &graph) == cudaSuccess) && ok;
   }
-  if (ok) ok = cudaGraphInstantiate(&ds.graph[w], graph, 0) == cudaSuccess;
+  if (ok) ok = cudaGraphInstantiate(&st.graph[w], graph, 0) == cudaSuccess;
   if (graph) cudaGraphDestroy(graph);
   cudaStreamDestroy(cs);
   if (!ok) {
     cudaGetLastError();
-    ds.graph[w] = nullptr;
-    ds.graph_failed[w] = true;
+    st.graph[w] = nullptr;
+    st.graph_failed[w] = true;
   }
 }
 
@@ -1141,44 +1239,74 @@ extern "C" tn_status tn_contract_slices(tn_plan_t* h, uint64_t first, uint64_t c
       prm.push_back(c);
     }
   if (ds.have_done) CK(cudaStreamWaitEvent(s, ds.done, 0));
-  if (prm.size() > ds.params_cap) {
+  // Runs of chunks side by side: as many as there are lanes.  A rest that is no
+  // power of two is filled up with copies of its last chunk that count no slices
+  // where a chunk is little work, else it is divided into powers of two.
+  struct Run {
+    size_t at;
+    int ls;
+  };
+  std::vector<Run> runs;
+  std::vector<ChunkParam> lanes;
+  const bool fill = p.stats.flops_chunk <= 5e8;
+  for (size_t i = 0; i < prm.size();) {
+    const size_t q = std::min(prm.size() - i, (size_t)1 << ds.ls_lanes);
+    int ls = 0;
+    while (fill ? ((size_t)1 << ls) < q : ((size_t)2 << ls) <= q) ++ls;
+    runs.push_back({lanes.size(), ls});
+    for (size_t l = 0; l < ((size_t)1 << ls); ++l) {
+      lanes.push_back(prm[std::min(i + l, prm.size() - 1)]);
+      if (l >= q) lanes.back().valid_lo = lanes.back().valid_hi = 0;
+    }
+    i += std::min(q, (size_t)1 << ls);
+  }
+  if (lanes.size() > ds.params_cap) {
     if (ds.params) {
       CK(cudaStreamSynchronize(s));
       drop_graphs(ds);   // captured with the old buffer's address
       CK(cudaFree(ds.params));
       ds.params = nullptr;
     }
-    ds.params_cap = std::max<size_t>(prm.size(), 1024);
+    ds.params_cap = std::max<size_t>(lanes.size(), 1024);
     CK(cudaMalloc(&ds.params, ds.params_cap * sizeof(ChunkParam)));
   }
-  CK(cudaMemcpyAsync(ds.params, prm.data(), prm.size() * sizeof(ChunkParam), cudaMemcpyHostToDevice, s));
+  CK(cudaMemcpyAsync(ds.params, lanes.data(), lanes.size() * sizeof(ChunkParam), cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(ds.counter, 0, sizeof(unsigned), s));
-  if (!ds.pro0_done) {
-    if (has_prologue(p, 0)) {
-      launch_leaf_select(p, s, 0);
-      run_prologue(p, s, 0);
+  const bool pro0 = has_prologue(p, 0), pro2 = has_prologue(p, 2);
+  for (const Run& r : runs) {
+    const int n = 1 << r.ls;
+    ensure_set(p, ds, r.ls);
+    LaunchSet& st = ds.set[r.ls];
+    if (ds.pro0_lanes < n) {
+      if (pro0) {
+        launch_leaf_select(p, s, 0, r.ls);
+        run_prologue(p, s, st, 0);
+      }
+      ds.pro0_lanes = n;
     }
-    ds.pro0_done = true;
-  }
-  const bool pro2 = has_prologue(p, 2);
-  for (size_t c = 0; c < prm.size(); ++c) {
-    const bool new_batch = pro2 && (!ds.pro2_valid || ds.pro2_bits != prm[c].bitstring);
+    bool new_batch = false;
+    for (int l = 0; l < n && pro2; ++l)
+      new_batch = new_batch || !ds.pro2_valid[l] || ds.pro2_bits[l] != lanes[r.at + l].bitstring;
     const int w = new_batch ? 1 : 0;
-    if (!ds.eager_done[w]) {
-      run_chunk(p, s, new_batch);           // the first one runs eagerly (sets kernel attributes)
-      ds.eager_done[w] = true;
+    if (!st.eager_done[w]) {
+      run_chunk(p, s, st, new_batch);           // the first one runs eagerly (sets kernel attributes)
+      st.eager_done[w] = true;
     } else {
-      capture_chunk_graph(p, new_batch);
-      if (ds.graph[w])
-        CK(cudaGraphLaunch(ds.graph[w], s));
+      capture_chunk_graph(p, st, new_batch);
+      if (st.graph[w])
+        CK(cudaGraphLaunch(st.graph[w], s));
       else
-        run_chunk(p, s, new_batch);
+        run_chunk(p, s, st, new_batch);
     }
     CK(cudaGetLastError());
-    if (new_batch) {
-      ds.pro2_valid = true;
-      ds.pro2_bits = prm[c].bitstring;
+    for (int l = 0; l < n && new_batch; ++l) {
+      ds.pro2_valid[l] = true;
+      ds.pro2_bits[l] = lanes[r.at + l].bitstring;
     }
+    // one batch's prologue is kept, the last one's (for its further slices), however
+    // many lanes there are: a batch that comes back is contracted again
+    const uint64_t last = lanes[r.at + n - 1].bitstring;
+    for (int l = 0; l < (1 << MAX_LS_LANES); ++l) ds.pro2_valid[l] = ds.pro2_valid[l] && ds.pro2_bits[l] == last;
   }
   CK(cudaEventRecord(ds.done, s));
   ds.have_done = true;
@@ -1212,25 +1340,17 @@ extern "C" tn_status tn_plan_step_times(tn_plan_t* h, int32_t reps, double* ms_o
   CK(cudaGetLastError());
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  ds.pro0_done = false;   // the arena was overwritten: prologues run again
-  ds.pro2_valid = false;
+  ds.forget_prologues();   // the arena was overwritten: they run again
   API_END
-}
-
-// Step d's launch with one kernel choice (as the autotuner builds its candidates).
-static StepLaunch build_choice(const DeviceState& ds, const StepDesc& d, int kid, int tn_log, int epi, int bslots,
-                               int pair) {
-  return make_launch(step_args(ds, d, kid, tn_log), kid, 64 - __builtin_clzll((uint64_t)d.a_elems) - 1, 1,
-                     d.c_elems, true, epi, (int64_t)256 << 20, bslots, pair);
 }
 
 // After the kernels of a plan changed: group runs, chunk graph and prologues anew.
 static void kernels_changed(Plan& p, DeviceState& ds) {
-  build_groups(p, ds);
-  setup_hoisted(p, ds);
   drop_graphs(ds);
-  ds.pro0_done = false;   // the arena may have been overwritten: prologues run again
-  ds.pro2_valid = false;
+  for (LaunchSet& st : ds.set) st.built = false;
+  ensure_set(p, ds, 0);
+  setup_hoisted(p, ds);
+  ds.forget_prologues();   // the arena may have been overwritten: they run again
 }
 
 // Autotuner: for every step, time the candidate kernels in place (tensor-core
@@ -1503,12 +1623,13 @@ static int class_launches(const Plan& p, Pred in_class) {
   };
   for (size_t i = 0; i < p.steps.size(); ++i) {
     if (!in_class(p.steps[i].dep_flags)) continue;
-    const int gi = p.dev->group_at.empty() ? -1 : p.dev->group_at[i];
+    const LaunchSet& st = p.dev->set[0];
+    const int gi = st.group_at.empty() ? -1 : st.group_at[i];
     if (gi < 0) {
       n += kernels_of((int)i);
       continue;
     }
-    const auto& gr = p.dev->groups[gi];
+    const GroupRun& gr = st.groups[gi];
     n += (int)gr.multi.size();
     for (int t : gr.singles) n += kernels_of(t);
     i = (size_t)gr.end - 1;

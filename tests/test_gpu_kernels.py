@@ -164,3 +164,40 @@ def test_tensor_core_tiles_at_their_edges(env, shape, batch, layout, misaligned,
     for i in {0, batch - 1}:
         want = pairwise.contract_pair(a[i].astype(np.complex128), a_w, b[i].astype(np.complex128), b_w, c_w)
         assert np.linalg.norm(got[i] - want) <= PAIR_REL[prec, cm] * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("prec,slices,chunk", [("fp32", 0, 0), ("fp32", 5, 2), ("bf16x3", 4, 0), ("fp16x3", 4, 1)])
+def test_chunks_side_by_side(env, prec, slices, chunk):
+    """Chunks of one call run side by side, 16 at most, filled up to a power of
+    two: any number of batches, in one call or one by one, whole or in ragged slice
+    ranges, gives the same bits, and the state vector's amplitudes."""
+    import rqcgen
+    from oracle import statevector as sv
+    tn, torch = env
+    circ = rqcgen.sycamore_style(4, 4, 9, 7, 0)
+    om = 0b1111110000000000
+    psi = sv.simulate(circ)
+    net = tn.Network(circ)
+    make = lambda: tn.Plan(net, open_mask=om, max_log2_intermediate=30, min_log2_slices=slices, trials=8,
+                           log2_batch_slices=chunk, precision=prec)
+    n = 1 << make().info()["log2_slices"]
+    rng = np.random.default_rng(3)
+    plan = make()
+    for count in (1, 3, 2, 17, 16, 5):
+        bits = [int(b) for b in rng.integers(0, 1 << 10, size=count)]
+        out = torch.zeros(count << 6, dtype=torch.complex128, device="cuda")
+        cuts = sorted({0, n // 3, n})
+        for a, b in zip(cuts, cuts[1:]):
+            plan.contract_slices(a, b - a, bits, out)
+        plan.sync()
+        alone = torch.zeros_like(out)
+        single = make()
+        for i, b in enumerate(bits):
+            for lo, hi in zip(cuts, cuts[1:]):
+                single.contract_slices(lo, hi - lo, [b], alone[i << 6:(i + 1) << 6])
+        single.sync()
+        want = np.concatenate([sv.batch_amplitudes(psi, circ.n_qubits, b, om) for b in bits])
+        got = out.cpu().numpy()
+        assert np.linalg.norm(got - want) < (1e-5 if prec == "fp32" else 1e-4) * np.linalg.norm(want)
+        if n // 3 == 0 or chunk == 0:   # one chunk per range: also the same bits
+            assert torch.equal(torch.view_as_real(out), torch.view_as_real(alone))
