@@ -232,21 +232,22 @@ __global__ void k_amax(const float2* __restrict__ x, int64_t n, float* out) {
 // first draw with u * M < 2^n |a|^2 is the sample.  Every draw is tested in
 // parallel and the smallest accepted t per sample kept.  The products are
 // rounded separately (no fused multiply-add), as the decision's definition
-// states them.  A candidate outside [0, count) is skipped and flagged.
+// states them.  first[0] becomes 0 when a candidate is outside [0, count) (it is
+// skipped), first[1 + s] is sample s's draw; all are ~0 before.
 __global__ void k_frugal(const double2* __restrict__ a, int64_t count, int n_qubits, double m_bound,
                          const int64_t* __restrict__ cand, const double* __restrict__ u, int64_t n_draws,
-                         int64_t n_samples, unsigned long long* first, int32_t* bad) {
+                         int64_t n_samples, unsigned long long* first) {
   const int64_t total = n_draws * n_samples;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t c = cand[i];
     if (c < 0 || c >= count) {
-      atomicExch(bad, 1);
+      atomicExch(first, 0ull);
       continue;
     }
     const double2 v = a[c];
     const double p = __dadd_rn(__dmul_rn(v.x, v.x), __dmul_rn(v.y, v.y));
     if (__dmul_rn(u[i], m_bound) < ldexp(p, n_qubits))
-      atomicMin(first + i / n_draws, (unsigned long long)(i % n_draws));
+      atomicMin(first + 1 + i / n_draws, (unsigned long long)(i % n_draws));
   }
 }
 

@@ -1691,14 +1691,16 @@ static void operand_maxima(const float2* a, int64_t na, const float2* b, int64_t
   k_amax<<<std::max(gb, 1), 256, 0, s>>>(b, nb, amax + 1);
 }
 
+constexpr int64_t kHostWords = 8192;
 struct Scratch {
   double* xeb = nullptr;          // XEB: the sum, then the blocks' partial sums
   unsigned* xeb_ticket = nullptr; // zero between launches
   int32_t* err = nullptr;
   float* amax = nullptr;   // FP16X3 operand maxima of the last call (A, B)
-  unsigned long long* first = nullptr;   // frugal sampling: first accepted draw per sample
+  unsigned long long* first = nullptr;   // frugal sampling: ~0 unless a candidate was out of range, then the
+                                         // first accepted draw per sample (~0: none)
   int64_t first_cap = 0;
-  int32_t* bad = nullptr;
+  unsigned long long* host = nullptr;    // page-locked: results on their way to the caller
   uint8_t* ws = nullptr;
   int64_t ws_bytes = 0;
 };
@@ -1716,7 +1718,7 @@ static Scratch& scratch_for_device() {
     CK(cudaMalloc(&s.err, sizeof(int32_t)));
     CK(cudaMemset(s.err, 0, sizeof(int32_t)));
     CK(cudaMalloc(&s.amax, 2 * sizeof(float)));
-    CK(cudaMalloc(&s.bad, sizeof(int32_t)));
+    CK(cudaMallocHost(&s.host, kHostWords * sizeof(unsigned long long)));
   }
   return s;
 }
@@ -1735,9 +1737,10 @@ extern "C" tn_status tn_xeb(const double* amps, int64_t count, int32_t n_qubits,
   const int blocks = (int)std::min<int64_t>((count + per - 1) / per, std::min<int64_t>(4 * sm_count(), XEB_BLOCKS));
   k_xeb_sum<<<blocks, XEB_THREADS, 0, s>>>(reinterpret_cast<const double2*>(amps), count, scratch, sc.xeb_ticket);
   CK(cudaGetLastError());
-  double sum = 0;
-  CK(cudaMemcpyAsync(&sum, scratch, sizeof(double), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(sc.host, scratch, sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  double sum = 0;
+  std::memcpy(&sum, sc.host, sizeof(double));
   *xeb_out = std::ldexp(sum / (double)count, n_qubits) - 1.0;
   API_END
 }
@@ -1753,27 +1756,31 @@ extern "C" tn_status tn_frugal_sample(const double* amps, int64_t count, int32_t
   if (n_draws > ((int64_t)1 << 40) / n_samples) fail(TN_ERR_ARG, "tn_frugal_sample: too many draws");
   Scratch& sc = scratch_for_device();
   cudaStream_t s = (cudaStream_t)stream;
-  if (n_samples > sc.first_cap) {
+  const int64_t words = n_samples + 1;
+  if (words > sc.first_cap) {
     CK(cudaStreamSynchronize(s));
     if (sc.first) CK(cudaFree(sc.first));
     sc.first = nullptr;
-    CK(cudaMalloc(&sc.first, sizeof(unsigned long long) * (size_t)n_samples));
-    sc.first_cap = n_samples;
+    sc.first_cap = 0;
+    CK(cudaMalloc(&sc.first, sizeof(unsigned long long) * (size_t)words));
+    sc.first_cap = words;
   }
-  CK(cudaMemsetAsync(sc.first, 0xff, sizeof(unsigned long long) * (size_t)n_samples, s));
-  CK(cudaMemsetAsync(sc.bad, 0, sizeof(int32_t), s));
+  CK(cudaMemsetAsync(sc.first, 0xff, sizeof(unsigned long long) * (size_t)words, s));
   const int64_t total = n_draws * n_samples;
   const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sm_count() * 16);
   k_frugal<<<blocks, 256, 0, s>>>(reinterpret_cast<const double2*>(amps), count, n_qubits, m_bound, candidates,
-                                  uniforms, n_draws, n_samples, sc.first, sc.bad);
+                                  uniforms, n_draws, n_samples, sc.first);
   CK(cudaGetLastError());
-  std::vector<unsigned long long> f((size_t)n_samples);
-  int32_t bad = 0;
-  CK(cudaMemcpyAsync(f.data(), sc.first, sizeof(unsigned long long) * f.size(), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(&bad, sc.bad, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  std::vector<unsigned long long> many;   // more samples than the page-locked area holds
+  unsigned long long* f = sc.host;
+  if (words > kHostWords) {
+    many.resize((size_t)words);
+    f = many.data();
+  }
+  CK(cudaMemcpyAsync(f, sc.first, sizeof(unsigned long long) * (size_t)words, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  if (bad) fail(TN_ERR_ARG, "tn_frugal_sample: a candidate index is outside [0, count)");
-  for (int64_t i = 0; i < n_samples; ++i) first_out[i] = f[i] == ~0ULL ? -1 : (int64_t)f[i];
+  if (f[0] != ~0ULL) fail(TN_ERR_ARG, "tn_frugal_sample: a candidate index is outside [0, count)");
+  std::memcpy(first_out, f + 1, sizeof(int64_t) * (size_t)n_samples);   // ~0 is -1: no accepted draw
   API_END
 }
 

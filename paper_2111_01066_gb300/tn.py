@@ -7,6 +7,7 @@ CPU fallback: if the shared library is missing the import of this module fails.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 from typing import List, Optional, Sequence, Tuple
@@ -82,7 +83,7 @@ _SIGS = {
     "tn_plan_step_shape": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32] + [ctypes.POINTER(ctypes.c_int32)] * 4),
     "tn_frugal_sample": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_double,
                                         ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_int64,
-                                        ctypes.POINTER(ctypes.c_int64), ctypes.c_void_p]),
+                                        ctypes.c_void_p, ctypes.c_void_p]),
     "tn_plan_select": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(tn_plan_opts), ctypes.c_int32,
                                       ctypes.c_uint64, ctypes.c_void_p, ctypes.POINTER(ctypes.c_void_p),
                                       ctypes.POINTER(ctypes.c_double)]),
@@ -116,16 +117,16 @@ _SIGS = {
     "tn_xeb": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32,
                               ctypes.POINTER(ctypes.c_double), ctypes.c_void_p]),
     "tn_permute": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
-                                  ctypes.POINTER(ctypes.c_int32), ctypes.c_int64, ctypes.c_void_p]),
-    "tn_contract_pair": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32), ctypes.c_int32,
-                                        ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32), ctypes.c_int32,
-                                        ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32), ctypes.c_int32,
+                                  ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]),
+    "tn_contract_pair": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
+                                        ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
+                                        ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
                                         ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p]),
     "tn_selftest_bounded_wait": (ctypes.c_int, [ctypes.c_int32, ctypes.POINTER(ctypes.c_int32), ctypes.c_void_p]),
     "tn_device_sync": (ctypes.c_int, [ctypes.c_void_p]),
-    "tn_contract_pair_noalloc": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32), ctypes.c_int32,
-                                                ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32), ctypes.c_int32,
-                                                ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32), ctypes.c_int32,
+    "tn_contract_pair_noalloc": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
+                                                ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
+                                                ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
                                                 ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p]),
 }
 
@@ -154,6 +155,15 @@ def _check(status: int) -> None:
     if status != TN_OK:
         msg = load().tn_last_error()
         raise TnError(status, msg.decode() if msg else "")
+
+
+def _ints(seq):
+    """int32 buffer of a sequence of integers and its address (the buffer must outlive the call)."""
+    try:
+        buf = array.array("i", seq)
+    except (TypeError, OverflowError):   # other numbers: converted one by one, wrapped to 32 bits
+        buf = array.array("i", _i32(seq)[:len(seq)])
+    return buf, buf.buffer_info()[0]
 
 
 def _i32(seq) -> ctypes.Array:
@@ -394,26 +404,24 @@ def contract_pair_noalloc(a, a_wires, b, b_wires, c, c_wires, batch: int = 1, pr
     """tn_contract_pair_noalloc on complex64 CUDA tensors (scratch from the
     library's static device array; nothing is allocated)."""
     p = PREC[precision] if isinstance(precision, str) else int(precision)
-    _check(load().tn_contract_pair_noalloc(ctypes.c_void_p(a.data_ptr()), _i32(a_wires), len(a_wires),
-                                           ctypes.c_void_p(b.data_ptr()), _i32(b_wires), len(b_wires),
-                                           ctypes.c_void_p(c.data_ptr()), _i32(c_wires), len(c_wires),
-                                           batch, p, complex_mult, _stream_handle(stream)))
+    (ab, aw), (bb, bw), (cb, cw) = _ints(a_wires), _ints(b_wires), _ints(c_wires)
+    _check(load().tn_contract_pair_noalloc(a.data_ptr(), aw, len(ab), b.data_ptr(), bw, len(bb), c.data_ptr(), cw,
+                                           len(cb), batch, p, complex_mult, _stream_handle(stream)))
 
 
 def permute(inp, out, rank: int, perm: Sequence[int], batch: int = 1, stream=None) -> None:
     """tn_permute on complex64 CUDA tensors."""
-    _check(load().tn_permute(ctypes.c_void_p(inp.data_ptr()), ctypes.c_void_p(out.data_ptr()), rank,
-                             _i32(perm), batch, _stream_handle(stream)))
+    buf, at = _ints(perm)
+    _check(load().tn_permute(inp.data_ptr(), out.data_ptr(), rank, at, batch, _stream_handle(stream)))
 
 
 def contract_pair(a, a_wires, b, b_wires, c, c_wires, batch: int = 1, precision: str = "fp32",
                   complex_mult: int = 4, stream=None) -> None:
     """tn_contract_pair on complex64 CUDA tensors."""
     p = PREC[precision] if isinstance(precision, str) else int(precision)
-    _check(load().tn_contract_pair(ctypes.c_void_p(a.data_ptr()), _i32(a_wires), len(a_wires),
-                                   ctypes.c_void_p(b.data_ptr()), _i32(b_wires), len(b_wires),
-                                   ctypes.c_void_p(c.data_ptr()), _i32(c_wires), len(c_wires),
-                                   batch, p, complex_mult, _stream_handle(stream)))
+    (ab, aw), (bb, bw), (cb, cw) = _ints(a_wires), _ints(b_wires), _ints(c_wires)
+    _check(load().tn_contract_pair(a.data_ptr(), aw, len(ab), b.data_ptr(), bw, len(bb), c.data_ptr(), cw,
+                                   len(cb), batch, p, complex_mult, _stream_handle(stream)))
 
 
 def frugal_sample(amplitudes, n_qubits: int, m_bound: float, candidates, uniforms, stream=None) -> List[int]:
@@ -422,12 +430,12 @@ def frugal_sample(amplitudes, n_qubits: int, m_bound: float, candidates, uniform
     accepted draw of each sample (-1 if none)."""
     n_samples, n_draws = (int(candidates.shape[0]), int(candidates.shape[1])) if candidates.dim() == 2 \
         else (1, int(candidates.numel()))
-    out = (ctypes.c_int64 * n_samples)()
+    out = np.empty(n_samples, dtype=np.int64)
     _check(load().tn_frugal_sample(ctypes.c_void_p(amplitudes.data_ptr()), amplitudes.numel(), n_qubits,
                                    float(m_bound), ctypes.c_void_p(candidates.data_ptr()),
-                                   ctypes.c_void_p(uniforms.data_ptr()), n_draws, n_samples, out,
+                                   ctypes.c_void_p(uniforms.data_ptr()), n_draws, n_samples, out.ctypes.data,
                                    _stream_handle(stream)))
-    return list(out)
+    return out.tolist()
 
 
 def select_plan(network: Network, n_candidates: int, bitstring: int, stream=None, open_mask: int = 0,
