@@ -66,9 +66,9 @@ __global__ void __launch_bounds__(128) k_leaf_select(const float2* __restrict__ 
 // Slice sum of a chunk (main text, section II: the sliced network is the sum of
 // the smaller networks) in FP64, deterministic: block (x, g, lane) sums the slices of
 // group g (slices g*per .. g*per+per-1 of the lane's chunk) for its amplitudes j into
-// part[lane][g][j]; the last of the blocks to arrive for the same amplitudes
-// (tickets[x]) adds lanes and groups in order into out[batch][j], and the last block
-// of all advances the chunk counter by the lanes.  Slices outside the call's range are
+// part[lane][g][j]; the last of the lane's blocks to arrive for the same amplitudes
+// adds its groups, the last lane's block adds the lanes into out[batch][j], both in
+// order, and the last block of all advances the chunk counter by the lanes.  Slices outside the call's range are
 // skipped.  The tickets are zero between launches.
 __global__ void __launch_bounds__(256) k_root_sum(const float2* __restrict__ arena, const RootDesc r, int b,
                                                  int groups, double2* __restrict__ part,
@@ -159,62 +159,82 @@ __global__ void __launch_bounds__(256) k_root_sum(const float2* __restrict__ are
                                                    (ai[t][0] + ai[t][1]) + (ai[t][2] + ai[t][3]));
       }
   }
-  // the last block for these amplitudes sums lanes and groups
-  __threadfence();
-  __syncthreads();
-  const int parts = lanes * groups;
-  if (threadIdx.x == 0) s_last = atomicAdd(&tickets[1 + blockIdx.x], 1u) == (unsigned)parts - 1u;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
+  // the last block of the lane for these amplitudes sums its groups in order ...
+  auto arrive_last = [&](unsigned* ticket, int of) {   // whether this block is the last of `of` at the ticket
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s_last = atomicAdd(ticket, 1u) == (unsigned)of - 1u;
+      if (s_last) *ticket = 0u;
+    }
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last != 0;
+  };
+  if (!arrive_last(&tickets[1 + gridDim.x + blockIdx.x * lanes + lane], groups)) return;
   for (int64_t j = j0; j < nout; j += jstep) {
-    double* o = nullptr;         // the batch's amplitude: lanes of one batch follow each other
-    double ar0 = 0.0, ai0 = 0.0;
-    double sr = 0.0, si = 0.0;   // the lane's sum
-    // eight loads in flight, added in order
-    for (int q0 = 0; q0 < parts; q0 += 8) {
+    double2* pj = part + (int64_t)lane * groups * nout + j;
+    double sr = 0.0, si = 0.0;
+    // eight loads in flight, added in group order
+    for (int q0 = 0; q0 < groups; q0 += 8) {
       double2 v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        v[u] = q0 + u < parts ? __ldcg(part + (int64_t)(q0 + u) * nout + j) : make_double2(0.0, 0.0);
+      for (int u = 0; u < 8; ++u) v[u] = q0 + u < groups ? __ldcg(pj + (q0 + u) * nout) : make_double2(0.0, 0.0);
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (q0 + u < parts) {
+        if (q0 + u < groups) {
           sr += v[u].x;
           si += v[u].y;
-          const int l = (q0 + u) / groups;
-          if (q0 + u == (l + 1) * groups - 1) {   // the lane is complete
-            const ChunkParam& pl = params[first + l];
-            if (pl.valid_lo < pl.valid_hi) {      // (a lane without slices only fills the launch)
-              double* ol = pl.out + 2 * (pl.out_index * nout + j);
-              if (ol != o) {
-                if (o) {
-                  o[0] = ar0;
-                  o[1] = ai0;
-                }
-                o = ol;
-                ar0 = o[0];
-                ai0 = o[1];
-              }
-              ar0 += sr;
-              ai0 += si;
-            }
-            sr = si = 0.0;
-          }
         }
     }
-    if (o) {
-      o[0] = ar0;
-      o[1] = ai0;
+    if (lanes > 1) {
+      *pj = make_double2(sr, si);
+    } else {
+      double* o = p.out + 2 * (p.out_index * nout + j);
+      o[0] += sr;
+      o[1] += si;
     }
   }
-  if (threadIdx.x == 0) {
-    tickets[1 + blockIdx.x] = 0;
-    // all blocks have read the counter: each did before its arrival above
-    if (atomicAdd(&tickets[0], 1u) == gridDim.x - 1u) {
-      tickets[0] = 0;
-      *counter = first + (unsigned)lanes;
+  // ... and the last lane's adds the lanes in order, those of one batch onto one value
+  if (lanes > 1) {
+    if (!arrive_last(&tickets[1 + blockIdx.x], lanes)) return;
+    for (int64_t j = j0; j < nout; j += jstep) {
+      double* o = nullptr;
+      double ar0 = 0.0, ai0 = 0.0;
+      for (int l0 = 0; l0 < lanes; l0 += 8) {
+        double2 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          v[u] = l0 + u < lanes ? __ldcg(part + (int64_t)(l0 + u) * groups * nout + j) : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (l0 + u >= lanes) break;
+          const ChunkParam& pl = params[first + l0 + u];
+          if (pl.valid_lo >= pl.valid_hi) continue;   // a lane without slices only fills the launch
+          double* ol = pl.out + 2 * (pl.out_index * nout + j);
+          if (ol != o) {
+            if (o) {
+              o[0] = ar0;
+              o[1] = ai0;
+            }
+            o = ol;
+            ar0 = o[0];
+            ai0 = o[1];
+          }
+          ar0 += v[u].x;
+          ai0 += v[u].y;
+        }
+      }
+      if (o) {
+        o[0] = ar0;
+        o[1] = ai0;
+      }
     }
+  }
+  // all blocks have read the counter: each did before its arrival above
+  if (threadIdx.x == 0 && atomicAdd(&tickets[0], 1u) == gridDim.x - 1u) {
+    tickets[0] = 0u;
+    *counter = first + (unsigned)lanes;
   }
 }
 

@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(SIMT_THREADS, Cfg::MINB) k_cgemm_simt(const __
 
 // Several independent GEMMs in one launch (a group of small steps that
 // neither read nor write what another of the group writes), on clusters of
-// SIMT_MAX_SPLIT CTAs: block b runs block b - start[i] of GEMM i, where
+// SIMT_MAX_SPLIT CTAs where one of them splits its k: block b runs block b - start[i] of GEMM i, where
 // start[i] <= b < start[i + 1] (start[n] is the grid size; every start is a
 // multiple of the cluster size, so a cluster has one GEMM), decoded as (split
 // rank fastest, m tile, n tile, instance), with that GEMM's tiling[i] (0:

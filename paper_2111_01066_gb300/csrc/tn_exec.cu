@@ -650,6 +650,7 @@ struct GroupRun {
   std::vector<int> singles;                  // steps launched alone
   struct Multi {
     int blocks = 0, n = 0;
+    int cluster = 1;                         // SIMT_MAX_SPLIT where a step's k is split
     GemmArgs* args = nullptr;                // device: n GemmArgs
     int32_t* start = nullptr;                // device: n + 1 block offsets
     int8_t* tiling = nullptr;                // device: n CUDA-core tilings (simt_multi_tiling)
@@ -677,15 +678,16 @@ struct LaunchSet {
   bool eager_done[2] = {false, false};
 };
 constexpr int MAX_LS_LANES = 4;
+constexpr size_t PARAMS_AT = 64;
 
 struct DeviceState {
   int device = -1;
   float2* arena = nullptr;
   float2* leaf_data = nullptr;
   LeafDesc* leaf_desc = nullptr;
+  unsigned* counter = nullptr;    // one buffer: the chunk counter, then (at PARAMS_AT) the chunks' parameters
   ChunkParam* params = nullptr;
   size_t params_cap = 0;
-  unsigned* counter = nullptr;
   int32_t* err = nullptr;
   uint8_t* ws = nullptr;
   int64_t ws_bytes = 0;           // capacity of ws
@@ -760,7 +762,7 @@ static int simt_multi_tiling(int kid) {
 }
 
 static void launch_simt_multi(const GroupRun::Multi& m, cudaStream_t s) {
-  klaunch(k_cgemm_simt_multi, dim3((unsigned)m.blocks), SIMT_THREADS, 0, s, SIMT_MAX_SPLIT, true,
+  klaunch(k_cgemm_simt_multi, dim3((unsigned)m.blocks), SIMT_THREADS, 0, s, m.cluster, true,
           (const GemmArgs*)m.args, (const int32_t*)m.start, (const int8_t*)m.tiling, (const int8_t*)m.split, (int32_t)m.n);
 }
 
@@ -865,6 +867,8 @@ static void build_groups(const Plan& p, LaunchSet& ds) {
     const size_t tiling_off = off;
     off += 2 * pm.second.size();
     int32_t blocks = 0;
+    for (int t : pm.second)
+      if (simt_split(ds.launches[t].g, ds.launches[t].kid) > 1) m.cluster = SIMT_MAX_SPLIT;
     for (size_t q = 0; q < pm.second.size(); ++q) {
       const GemmArgs& g = ds.launches[pm.second[q]].g;
       std::memcpy(host.data() + args_off + q * sizeof(GemmArgs), &g, sizeof(GemmArgs));
@@ -874,7 +878,7 @@ static void build_groups(const Plan& p, LaunchSet& ds) {
       // whole clusters: the kernel's blocks past the last tile only keep its barriers
       int64_t nb = ((int64_t)1 << (g.nm - g.tm)) * ((int64_t)1 << (g.nn - g.tn)) * split *
                    std::min<int64_t>(g.n_inst, 65535);
-      nb = (nb + SIMT_MAX_SPLIT - 1) / SIMT_MAX_SPLIT * SIMT_MAX_SPLIT;
+      nb = (nb + m.cluster - 1) / m.cluster * m.cluster;
       if (blocks + nb > 0x7fffffff) fail(TN_ERR_UNSUPPORTED, "step group grid too large");
       std::memcpy(host.data() + start_off + q * sizeof(int32_t), &blocks, sizeof(int32_t));
       blocks += (int32_t)nb;
@@ -970,7 +974,6 @@ static void ensure_device(Plan& p) {
   CK(cudaMalloc(&ds->leaf_desc, std::max<size_t>(1, p.leaves.size()) * sizeof(LeafDesc)));
   CK(cudaMemcpy(ds->leaf_desc, p.leaves.data(), p.leaves.size() * sizeof(LeafDesc),
                 cudaMemcpyHostToDevice));
-  CK(cudaMalloc(&ds->counter, sizeof(unsigned)));
   CK(cudaMalloc(&ds->err, sizeof(int32_t)));
   CK(cudaMemset(ds->err, 0, sizeof(int32_t)));
   CK(cudaEventCreateWithFlags(&ds->done, cudaEventDisableTiming));
@@ -1027,8 +1030,9 @@ static void ensure_device(Plan& p) {
   ds->root_groups = std::min(1 << p.log2_batch, 64);
   CK(cudaMalloc(&ds->root_part, (sizeof(double2) * (size_t)ds->root_groups << p.root.rank) << ds->ls_lanes));
   ds->root_blocks = (int)std::min<int64_t>((((int64_t)1 << p.root.rank) + 255) / 256, 4096);
-  CK(cudaMalloc(&ds->root_tickets, sizeof(unsigned) * (size_t)(1 + ds->root_blocks)));
-  CK(cudaMemset(ds->root_tickets, 0, sizeof(unsigned) * (size_t)(1 + ds->root_blocks)));
+  const size_t tickets = 1 + (size_t)ds->root_blocks * (1 + ((size_t)1 << ds->ls_lanes));
+  CK(cudaMalloc(&ds->root_tickets, sizeof(unsigned) * tickets));
+  CK(cudaMemset(ds->root_tickets, 0, sizeof(unsigned) * tickets));
   if (!in_arena(p.root.off, (int64_t)1 << p.root.rank, 1 << __builtin_popcount(p.root.bmask)))
     fail(TN_ERR_PLAN, "internal: root outside the arena");
   ensure_set(p, *ds, 0);
@@ -1055,7 +1059,6 @@ void destroy_device_state(Plan* p) {
   cudaFree(ds->arena);
   cudaFree(ds->leaf_data);
   cudaFree(ds->leaf_desc);
-  cudaFree(ds->params);
   cudaFree(ds->counter);
   cudaFree(ds->err);
   cudaFree(ds->ws);
@@ -1264,14 +1267,20 @@ extern "C" tn_status tn_contract_slices(tn_plan_t* h, uint64_t first, uint64_t c
     if (ds.params) {
       CK(cudaStreamSynchronize(s));
       drop_graphs(ds);   // captured with the old buffer's address
-      CK(cudaFree(ds.params));
+      CK(cudaFree(ds.counter));
+      ds.counter = nullptr;
       ds.params = nullptr;
     }
-    ds.params_cap = std::max<size_t>(lanes.size(), 1024);
-    CK(cudaMalloc(&ds.params, ds.params_cap * sizeof(ChunkParam)));
+    ds.params_cap = 0;
+    const size_t cap = std::max<size_t>(lanes.size(), 1024);
+    CK(cudaMalloc(&ds.counter, PARAMS_AT + cap * sizeof(ChunkParam)));
+    ds.params = reinterpret_cast<ChunkParam*>(reinterpret_cast<uint8_t*>(ds.counter) + PARAMS_AT);
+    ds.params_cap = cap;
   }
-  CK(cudaMemcpyAsync(ds.params, lanes.data(), lanes.size() * sizeof(ChunkParam), cudaMemcpyHostToDevice, s));
-  CK(cudaMemsetAsync(ds.counter, 0, sizeof(unsigned), s));
+  // the counter (zero) and the parameters in one copy
+  std::vector<uint8_t> up(PARAMS_AT + lanes.size() * sizeof(ChunkParam), 0);
+  std::memcpy(up.data() + PARAMS_AT, lanes.data(), lanes.size() * sizeof(ChunkParam));
+  CK(cudaMemcpyAsync(ds.counter, up.data(), up.size(), cudaMemcpyHostToDevice, s));
   const bool pro0 = has_prologue(p, 0), pro2 = has_prologue(p, 2);
   for (const Run& r : runs) {
     const int n = 1 << r.ls;
