@@ -17,8 +17,8 @@ namespace tnx {
 // the maxima the coming steps record).
 __global__ void __launch_bounds__(128) k_leaf_select(const float2* __restrict__ leaf_data,
                                                      const LeafDesc* __restrict__ leaves, int n_leaves,
-                                                     float2* __restrict__ arena, const ChunkParam* __restrict__ params,
-                                                     const unsigned* __restrict__ counter, int64_t lane_stride,
+                                                     float2* arena, const ChunkParam* params,
+                                                     const unsigned* counter, int64_t lane_stride,
                                                      float* amax, int amax_lane, int z0, int z1) {
   const int lane = blockIdx.y;
   arena += lane * lane_stride;
@@ -70,9 +70,9 @@ __global__ void __launch_bounds__(128) k_leaf_select(const float2* __restrict__ 
 // adds its groups, the last lane's block adds the lanes into out[batch][j], both in
 // order, and the last block of all advances the chunk counter by the lanes.  Slices outside the call's range are
 // skipped.  The tickets are zero between launches.
-__global__ void __launch_bounds__(256) k_root_sum(const float2* __restrict__ arena, const RootDesc r, int b,
-                                                 int groups, double2* __restrict__ part,
-                                                 const ChunkParam* __restrict__ params, unsigned* counter,
+__global__ void __launch_bounds__(256) k_root_sum(const float2* arena, const RootDesc r, int b,
+                                                 int groups, double2* part,
+                                                 const ChunkParam* params, unsigned* counter,
                                                  unsigned* tickets, int64_t lane_stride) {
   // the group's slices in rounds of 256: their instance offsets in the root
   // (or -1 outside the call's range) are found once per block, then every

@@ -546,12 +546,12 @@ __global__ void __launch_bounds__(PREP_THREADS) k_tc_prep_b(const __grid_constan
     for (int q = 1; q < 3; ++q)
       if ((i >> q) & 1) o += kw[q];
     if (n_ok && k + 1 < tkv && v16) {
-      const float4 t = __ldg(reinterpret_cast<const float4*>(src + o));
+      const float4 t = *reinterpret_cast<const float4*>(src + o);
       b[i] = make_float2(t.x, t.y);
       b[i + 1] = make_float2(t.z, t.w);
     } else {
-      b[i] = n_ok && k < tkv ? __ldg(src + o) : make_float2(0.f, 0.f);
-      b[i + 1] = n_ok && k + 1 < tkv ? __ldg(src + o + kw[0]) : make_float2(0.f, 0.f);
+      b[i] = n_ok && k < tkv ? src[o] : make_float2(0.f, 0.f);
+      b[i + 1] = n_ok && k + 1 < tkv ? src[o + kw[0]] : make_float2(0.f, 0.f);
     }
   }
   if (!live) return;
@@ -608,8 +608,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_tc_prep_b(const __grid_constan
 }
 
 // Split-K: C[i] = sum over splits of the partials, in split order.
-__global__ void k_split_reduce(const float2* __restrict__ part, int n_split, int64_t stride,
-                               float2* __restrict__ C, int64_t n, float* amax_c) {
+__global__ void k_split_reduce(const float2* part, int n_split, int64_t stride, float2* C, int64_t n, float* amax_c) {
   pdl_wait();
   float am = 0.f;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -976,12 +975,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
         for (int q = 0; q < 4; ++q) {
           const int64_t o0 = goff[2 * q], o1 = goff[2 * q + 1];
           if (v16 && o1 >= 0) {
-            const float4 t = __ldg(reinterpret_cast<const float4*>(Ak + o0));
+            const float4 t = *reinterpret_cast<const float4*>(Ak + o0);
             v[2 * q] = make_float2(t.x, t.y);
             v[2 * q + 1] = make_float2(t.z, t.w);
           } else {
-            v[2 * q] = o0 >= 0 ? __ldg(Ak + o0) : make_float2(0.f, 0.f);
-            v[2 * q + 1] = o1 >= 0 ? __ldg(Ak + o1) : make_float2(0.f, 0.f);
+            v[2 * q] = o0 >= 0 ? Ak[o0] : make_float2(0.f, 0.f);
+            v[2 * q + 1] = o1 >= 0 ? Ak[o1] : make_float2(0.f, 0.f);
           }
         }
       };
@@ -1110,10 +1109,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_cgemm_tc(const __grid_constan
             for (int h = 0; h < KPC / 2; ++h) {
               const int64_t o0 = goff[j][2 * h], o1 = goff[j][2 * h + 1];
               if (v16 && o1 >= 0) {
-                v[j][h] = __ldg(reinterpret_cast<const float4*>(Ak + o0));
+                v[j][h] = *reinterpret_cast<const float4*>(Ak + o0);
               } else {
-                const float2 x = o0 >= 0 ? __ldg(Ak + o0) : make_float2(0.f, 0.f);
-                const float2 y = o1 >= 0 ? __ldg(Ak + o1) : make_float2(0.f, 0.f);
+                const float2 x = o0 >= 0 ? Ak[o0] : make_float2(0.f, 0.f);
+                const float2 y = o1 >= 0 ? Ak[o1] : make_float2(0.f, 0.f);
                 v[j][h] = make_float4(x.x, x.y, y.x, y.y);
               }
             }

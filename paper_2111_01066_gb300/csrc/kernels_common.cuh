@@ -9,14 +9,14 @@ namespace tnx {
 // contraction is launched with the stream-serialisation attribute: it may start
 // once every CTA of the kernel before it has passed its own pdl_wait, sets itself
 // up under that kernel's run, and waits here until that kernel has completed and
-// its writes are visible.  Before pdl_wait a kernel touches only its arguments,
+// its writes are visible (to ordinary loads: what another kernel of the chain
+// writes is never read as read-only data).  Before pdl_wait a kernel touches only its arguments,
 // tables written when the plan was built, and its own shared and tensor memory;
 // every thread that touches anything else passes it, so a kernel's completion
 // implies that of all kernels before it.  The next kernel is let go after the
 // wait, not before it: no CTA is then resident while the kernel two before its
-// own still runs, so its first-level cache holds nothing that the kernel before
-// it has overwritten since (read-only loads stay safe).  Without the attribute
-// (a launch outside such a chain) both instructions are no-ops.
+// own still runs.  Without the attribute (a launch outside such a chain) both
+// instructions are no-ops.
 // A chain of small kernels costs 4-6 us a link without it (launch, arguments,
 // decode tables, then the work).
 __device__ __forceinline__ void pdl_wait() {
@@ -78,7 +78,8 @@ static_assert(sizeof(GemmArgs) % 4 == 0, "GemmArgs is copied to shared memory in
 // maximum is zero, subnormal or not recorded).
 __device__ __forceinline__ int fp16_scale_exp(const float* amax) {
   if (!amax) return 0;
-  const int be = (int)((__float_as_uint(*amax) >> 23) & 255u);
+  // past L1: the maxima share sectors with ones that running kernels raise
+  const int be = (int)((__float_as_uint(__ldcg(amax)) >> 23) & 255u);
   if (be == 0 || be == 255) return 0;
   const int s = 14 - (be - 127);
   return s < -126 ? -126 : (s > 126 ? 126 : s);

@@ -61,16 +61,16 @@ static int sm_count() {
 
 static bool is_simt(int kid) { return kid >= 0 && kid < K_COUNT && !(kid >= K_TC_TF32 && kid <= K_TC_FP16X3_3M); }
 
-// CUDA-core tiling of a step, from times on a GB300 (us, one launch):
+// CUDA-core tiling of a step, from times on a GB300 (us a launch, log2 m, k, n):
 //  * few outputs (at most two 32x32 tiles per SM): 32x32, whose k groups and
-//    split-K clusters keep the SMs busy -- (log2 m, k, n) = (7, 10, 6): 12 against
-//    148 with 64x64; (10, 6, 8): 9.9 against 14; with more tiles the larger ones
-//    win, (12, 4, 9): 36 against 13 with 128x64;
-//  * n <= 4: 256x4, n <= 16: 128x16 -- (20, 3, 1): 47 with 256x4, 96 with 128x16;
-//    (16, 5, 4): 18 with 128x16, 33 with 64x64;
-//  * n = 32 with k >= 64: 32x32 -- (15, 8, 5): 74 against 110 with 64x64;
-//  * otherwise 128x64 where its tiles fill the SMs -- (12, 10, 12): 2440 against
-//    2710 with 64x64 -- and 64x64 where they do not.
+//    split-K clusters keep the SMs busy -- (7, 10, 6): 8.6 against 148 with 64x64;
+//    (10, 6, 8): 8.1 against 14; with more tiles the larger ones win, (12, 4, 9): 36
+//    against 12 with 128x64;
+//  * n <= 4: 256x4, n <= 16: 128x16 -- (20, 3, 1): 44 with 256x4, 96 with 128x16;
+//    (16, 5, 4): 15 with 128x16, 30 with 64x64;
+//  * n = 32 with k >= 64: 32x32 -- (15, 8, 5): 70 against 105 with 64x64;
+//  * otherwise 128x64 where its tiles fill the SMs -- (12, 10, 12): 2513 against
+//    2639 with 64x64 -- and 64x64 where they do not.
 static int pick_simt(const StepDesc& d, int64_t n_inst) {
   auto tiles = [&](int tm, int tn) {
     return ((int64_t)1 << (std::max(d.nm, tm) - tm)) * ((int64_t)1 << (std::max(d.nn, tn) - tn)) * n_inst;
@@ -86,8 +86,9 @@ static int pick_simt(const StepDesc& d, int64_t n_inst) {
 
 // CTAs of a cluster that share a tile's k loop (1: no split): as many as leave
 // each at least two k chunks and the grid within two CTAs per SM.  A cluster
-// costs 2-4 us, a 32-k chunk of a lone CTA 1-1.5: (8, 8, 6) takes 16 us unsplit,
-// 8.3 over 4 CTAs (2 chunks each), 9.1 over 8; (7, 10, 6) 52, 17 and 12.
+// costs 2-4 us, a 32-k chunk of a lone CTA 1-1.5 (in a chain of launches without
+// overlap (8, 8, 6) took 16 us unsplit, 8.3 over 4 CTAs with 2 chunks each, 9.1 over
+// 8; (7, 10, 6) 52, 17 and 12).
 static int simt_split(const GemmArgs& g, int kid) {
   if (kid != K_SIMT_32x32) return 1;
   // of one lane: the same sums however many chunks run side by side
