@@ -54,10 +54,11 @@ constexpr int SIMT_MAX_SPLIT = 8;   // CTAs of one split-K cluster (the portable
 // thread, KG groups of threads that each take 1/KG of a stage's k (their sums
 // are added at the end), MINB CTAs per SM that the registers are kept to, NST
 // stages, filled by asynchronous copies NST - 1 chunks ahead or (REGS) through
-// registers one chunk ahead.  Copies need no registers and hide the latency of
-// operands that come from HBM, but move 4 bytes at a time (the two planes), twice
-// the L1 requests of the register path's 16-byte loads.  A is staged as two planes (re, im) whose consecutive rows make the
-// packed pairs.
+// registers one chunk ahead.  Copies need no registers, which the small tilings'
+// short loops want; they move 4 bytes at a time (the two planes of A), twice the L1
+// requests of the register path's 16-byte loads, which is faster where a loop is
+// long (2^17 x 256 x 256: 1198 us against 1310 with 128x64).  A is staged as two planes
+// (re, im) whose consecutive rows make the packed pairs.
 template <int TM_, int TN_, int TK_, int RM_, int RN_, int KG_, int MINB_, int NST_, bool REGS_>
 struct SimtCfg {
   static constexpr int TM = TM_, TN = TN_, TK = TK_, RM = RM_, RN = RN_, KG = KG_, MINB = MINB_;
@@ -89,8 +90,7 @@ struct SimtSmem {
   int64_t kdB[KMAXR];
 };
 
-using SimtBig = SimtCfg<128, 64, 8, 8, 4, 1, 2, 3, false>;
-using SimtBigR = SimtCfg<128, 64, 8, 8, 4, 1, 2, 2, true>;
+using SimtBig = SimtCfg<128, 64, 8, 8, 4, 1, 2, 2, true>;
 using Simt64 = SimtCfg<64, 64, 8, 4, 4, 1, 3, 2, true>;
 using Simt128x16 = SimtCfg<128, 16, 16, 4, 2, 1, 3, 2, false>;
 using Simt256x4 = SimtCfg<256, 4, 8, 4, 1, 1, 4, 2, false>;
@@ -184,7 +184,7 @@ __device__ __forceinline__ void pair_load(float4 (&v)[NP], const PairMap<NP>& m,
 // Large GEMMs are bound by the FP32 pipe's issue slots: a product of two packed
 // FMAs takes half the slots of four scalar ones, and 8 x 4 outputs per thread
 // leave 24 register moves and 8 shared loads per 64 of them; 4096 x 1024 x 4096
-// runs at 55 TFLOP/s (35 with scalar FMAs and 4 x 4 outputs), 2^17 x 256 x 256 at 52
+// runs at 57 TFLOP/s (35 with scalar FMAs and 4 x 4 outputs), 2^17 x 256 x 256 at 57
 // (34), of about 70.  Small ones are bound by latency: k offsets advance by one
 // table entry per chunk (decoding all k bits per chunk took longer than the
 // chunk's products), and one chunk with its set-up takes about 3 us in a chain of
@@ -197,7 +197,11 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
   constexpr int AP = (TM * TK / 2 + SIMT_THREADS - 1) / SIMT_THREADS;
   constexpr int BP = (TN * TK / 2 + SIMT_THREADS - 1) / SIMT_THREADS;
   const int tid = threadIdx.x;
-  const int tx = tid % NTX, ty = (tid / NTX) % Cfg::NTY, kg = tid / (NTX * Cfg::NTY);
+  // a warp covers 8 x 4 threads of the tile: it then reads 8 distinct 16-byte pieces
+  // of A's planes and 4 of B per k, against 16 and 2 in rows of 16 (3-6% on large
+  // GEMMs)
+  const int kg = tid / (NTX * Cfg::NTY), w = (tid / 32) % (NTX * Cfg::NTY / 32);
+  const int tx = (w % (NTX / 8)) * 8 + tid % 8, ty = (w / (NTX / 8)) * 4 + (tid % 32) / 8;
   const int TMv = 1 << g.tm, TKv = 1 << g.tk, TNv = 1 << g.tn;
   const int n_hi = g.nk - g.tk;
   const int kc_per = (1 << n_hi) / split, kc0 = rank * kc_per;
@@ -349,7 +353,7 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
         }
         const typename Cfg::Stage& st = sm.st[c & 1];
         if (TKv == TK) {
-#pragma unroll(RM * RN >= 32 ? 4 : 8)
+#pragma unroll 8
           for (int kk = 0; kk < TK; ++kk) step(st, kk);
         } else {
           for (int kk = 0; kk < TKv; ++kk) step(st, kk);
@@ -379,7 +383,7 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
         next(c + NST - 1);
         const typename Cfg::Stage& st = sm.st[c % NST];
         if (TKv == TK) {
-#pragma unroll(RM * RN >= 32 ? 4 : 8)
+#pragma unroll 8
           for (int kk = 0; kk < TK / Cfg::KG; ++kk) step(st, kk * Cfg::KG + kg);
         } else {
           for (int kk = kg; kk < TKv; kk += Cfg::KG) step(st, kk);

@@ -194,13 +194,7 @@ static void launch_simt(const GemmArgs& g, int kid, cudaStream_t s) {
       launch_simt_cfg<Simt256x4>(g, grid, 1, s);
       break;
     case K_SIMT_128x64:
-      // from 2048 columns on A's tiles are read again from L2, whose latency the
-      // register path hides, with fewer requests: 4096 x 1024 x 4096 2515 us against 2705
-      // with asynchronous copies, 2^17 x 256 x 256 1436 against 1318
-      if (g.nn >= 11)
-        launch_simt_cfg<SimtBigR>(g, grid, 1, s);
-      else
-        launch_simt_cfg<SimtBig>(g, grid, 1, s);
+      launch_simt_cfg<SimtBig>(g, grid, 1, s);
       break;
     case K_SIMT_32x32:
       launch_simt_cfg<Simt32>(g, grid, split, s);
