@@ -70,6 +70,10 @@ __global__ void __launch_bounds__(128) k_leaf_select(const float2* __restrict__ 
 // adds its groups, the last lane's block adds the lanes into out[batch][j], both in
 // order, and the last block of all advances the chunk counter by the lanes.  Slices outside the call's range are
 // skipped.  The tickets are zero between launches.
+// MAXJ: amplitudes that a thread holds in registers, 1 where the grid has a thread
+// for each: the registers of four, mostly unused, let two blocks on an SM (4096
+// slices of 4096 amplitudes: 206-215 us, 157 with one).
+template <int MAXJ>
 __global__ void __launch_bounds__(256) k_root_sum(const float2* arena, const RootDesc r, int b,
                                                  int groups, double2* part,
                                                  const ChunkParam* params, unsigned* counter,
@@ -98,7 +102,6 @@ __global__ void __launch_bounds__(256) k_root_sum(const float2* arena, const Roo
   // number of times, even where it has no amplitude: the pass count depends
   // on the grid only
   const int my_n = j0 < nout ? (int)((nout - 1 - j0) / jstep) + 1 : 0;
-  constexpr int MAXJ = 4;   // amplitudes per thread held in registers
   const int64_t max_n = (nout + jstep - 1) / jstep;
   const int passes = (int)((max_n + MAXJ - 1) / MAXJ);
   double ar[MAXJ][4], ai[MAXJ][4];

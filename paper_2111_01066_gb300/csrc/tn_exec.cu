@@ -1150,9 +1150,10 @@ static void run_chunk(Plan& p, cudaStream_t s, LaunchSet& st, bool new_batch) {
   launch_leaf_select(p, s, new_batch ? 3 : 1, st.ls);
   if (new_batch) run_prologue(p, s, st, 2);
   launch_class(p, s, st, [](int f) { return (f & 1) != 0; });   // slice-dependent steps
-  klaunch(k_root_sum, dim3((unsigned)ds.root_blocks, (unsigned)ds.root_groups, 1u << st.ls), 256, 0, s, 1, true,
-          (const float2*)ds.arena, p.root, p.log2_batch, ds.root_groups, ds.root_part, (const ChunkParam*)ds.params,
-          ds.counter, ds.root_tickets, ds.lane_stride);
+  const bool one = ((int64_t)1 << p.root.rank) <= (int64_t)ds.root_blocks * 256;   // amplitude per thread
+  klaunch(one ? k_root_sum<1> : k_root_sum<4>, dim3((unsigned)ds.root_blocks, (unsigned)ds.root_groups, 1u << st.ls),
+          256, 0, s, 1, true, (const float2*)ds.arena, p.root, p.log2_batch, ds.root_groups, ds.root_part,
+          (const ChunkParam*)ds.params, ds.counter, ds.root_tickets, ds.lane_stride);
 }
 
 // Capture run_chunk once into a graph (on a private stream, thread-local
