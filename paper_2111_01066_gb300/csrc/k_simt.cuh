@@ -473,8 +473,9 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
       simt_cluster_sync();   // the peers have read this CTA's partial tile
     }
   }
-  // every thread reaches here; with several lanes a block has one instance (bz)
-  if (g.amax_c) amax_update(g.amax_c + (int64_t)(bz >> (g.nb - g.ls_lanes)) * g.amax_lane, am);
+  // every thread reaches here; with several lanes a block has one instance (bz; past
+  // the last one in a block that only fills a cluster)
+  if (g.amax_c && bz < gz) amax_update(g.amax_c + (int64_t)(bz >> (g.nb - g.ls_lanes)) * g.amax_lane, am);
 }
 
 __device__ __forceinline__ void copy_args(GemmArgs& dst, const GemmArgs* src) {
