@@ -469,7 +469,9 @@ tn_status tn_device_sync(void* stream);
  *     the library holds it until the process exits.  A contraction whose
  *     scratch exceeds it even without split-K (tensor-core paths: about 16
  *     bytes per complex entry of B per batch instance, after padding k to 16
- *     and n to 8) fails with TN_ERR_ARG before anything is launched.
+ *     and n to 8) fails with TN_ERR_ARG before anything is launched; one of
+ *     instances under 2^20 multiply-adds runs on the CUDA cores instead, which
+ *     form FP32 products and need no scratch.
  *   - No cudaMalloc, cudaFree or allocating library routine is called.  The
  *     first call on each device looks the array's device address up (with
  *     that device current); make that first call before any stream capture.

@@ -2053,6 +2053,8 @@ extern "C" tn_status tn_selftest_bounded_wait(int32_t wait_ms, int32_t* device_s
 // library holds the array until the process exits.
 constexpr size_t kNoAllocScratchBytes = (size_t)32 << 20;   // 32 MiB
 constexpr size_t kNoAllocErrBytes = 256;                     // error word, then the B' images
+// log2 of the multiply-adds an instance has at least where scratch beyond the array is an error
+constexpr int kNoAllocLog2Refused = 20;
 static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocScratchBytes];
 
 static std::mutex g_noalloc_mu;
@@ -2126,7 +2128,7 @@ extern "C" tn_status tn_contract_pair_noalloc(const float* a, const int32_t* aw,
   d.b_elems = (int64_t)1 << br;
   d.c_elems = (int64_t)1 << cr;
   order_pair_bits(d);
-  const int kid = pick_kernel(precision, cmult, d, batch);
+  int kid = pick_kernel(precision, cmult, d, batch);
   GemmArgs g = make_args(d, kid, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
                          reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems,
                          is_tc(kid) ? tc_tile(kid, d.nm, d.nk, d.nn, batch, batch * d.c_elems,
@@ -2145,10 +2147,17 @@ extern "C" tn_status tn_contract_pair_noalloc(const float* a, const int32_t* aw,
   // beside the B' images; otherwise one pass over k
   StepLaunch L = make_launch(g, kid, ar, batch, batch * d.c_elems, true, -1, cap);
   if (L.ws_bytes > cap) L = make_launch(g, kid, ar, batch);
+  // many small instances whose B' images do not fit together: the CUDA cores, which
+  // need no scratch (4096 x (128 x 32 x 32): 64 MiB of images)
+  if (is_tc(kid) && L.ws_bytes > cap && d.nm + d.nk + d.nn < kNoAllocLog2Refused) {
+    kid = pick_simt(d, batch);
+    g = make_args(d, kid, g.A, g.B, g.C, (int32_t)batch, d.a_elems, d.b_elems, d.c_elems);
+    L = make_launch(g, kid, ar, batch);
+  }
   // the documented limit is on the operands, not on the kernel that the step's
   // size selects: what the tensor-core path could not hold is refused from 2^20
-  // multiply-adds an instance on, also where the CUDA cores (no scratch) run it
-  if (!is_tc(kid) && precision != TN_PREC_FP32 && d.nm + d.nk + d.nn >= 20 && d.nm >= 4) {
+  // multiply-adds an instance on (kNoAllocLog2Refused), also where the CUDA cores (no scratch) run it
+  if (!is_tc(kid) && precision != TN_PREC_FP32 && d.nm + d.nk + d.nn >= kNoAllocLog2Refused && d.nm >= 4) {
     const int tk = tc_kernel(precision, cmult);
     const GemmArgs gt = make_args(d, tk, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
                                   reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems);

@@ -95,3 +95,33 @@ def test_noalloc_rejects_scratch_beyond_the_static_array(env):
     st = _noalloc(tn, ta, a_w, tb, b_w, tc, c_w, 1, "bf16x3", 4, torch)
     assert st == tn.TN_ERR_ARG
     assert b"static array" in tn.load().tn_last_error()
+
+
+@pytest.mark.parametrize("prec,cm", [("tf32", 4), ("bf16x3", 4), ("fp16x3", 4), ("tf32", 3), ("bf16x3", 3)])
+@pytest.mark.parametrize("shape,batch", [((7, 5, 5), 4096), ((4, 4, 4), 16384), ((6, 7, 6), 512), ((5, 9, 5), 200)])
+def test_noalloc_takes_many_small_instances(env, prec, cm, shape, batch):
+    """Instances under 2^20 multiply-adds are accepted whatever their number:
+    where the B' images of all of them exceed the static array they run on the
+    CUDA cores, within the rounding bound of FP32 sums in any order,
+    |error| <= (2 k + 2) u sum |a| |b|, u = 2^-24 (each component is a sum of 2k
+    products)."""
+    tn, torch = env
+    nm, nk, nn = shape
+    rng = np.random.default_rng(sum(shape) + batch)
+    wires = list(range(nm + nk + nn))
+    m_w, k_w, n_w = wires[:nm], wires[nm:nm + nk], wires[nm + nk:]
+    a_w, b_w, c_w = k_w + m_w, list(rng.permutation(k_w + n_w)), list(rng.permutation(m_w + n_w))
+    a, b, ta, tb = _operands(torch, rng, batch, a_w, b_w)
+    tc = torch.full((batch, 2 ** len(c_w)), float("nan"), dtype=torch.complex64, device="cuda")
+    st = _noalloc(tn, ta, a_w, tb, b_w, tc, c_w, batch, prec, cm, torch)
+    assert st == tn.TN_OK, tn.load().tn_last_error()
+    tn.device_sync()
+    got = tc.cpu().numpy()
+    assert np.all(np.isfinite(got.view(np.float32)))
+    for i in {0, 1, batch // 2, batch - 1}:
+        want = pairwise.contract_pair(a[i].astype(np.complex128), a_w, b[i].astype(np.complex128), b_w, c_w)
+        mag = pairwise.contract_pair(np.abs(a[i]).astype(np.complex128), a_w, np.abs(b[i]).astype(np.complex128), b_w,
+                                     c_w).real
+        bound = (2 * 2 ** nk + 2) * 2.0 ** -24 * mag
+        assert np.all(np.abs(got[i].real - want.real) <= bound)
+        assert np.all(np.abs(got[i].imag - want.imag) <= bound)
