@@ -2129,12 +2129,17 @@ extern "C" tn_status tn_contract_pair_noalloc(const float* a, const int32_t* aw,
   d.c_elems = (int64_t)1 << cr;
   order_pair_bits(d);
   int kid = pick_kernel(precision, cmult, d, batch);
+  const int64_t cap = (int64_t)(kNoAllocScratchBytes - kNoAllocErrBytes);
+  // bytes left for partial sums beside the B' images, whose size no tile width changes
+  int64_t part_cap = cap;
+  if (is_tc(kid)) {
+    const GemmArgs gw = make_args(d, kid, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
+                                  reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems);
+    part_cap = std::max<int64_t>(0, cap - (make_launch(gw, kid, ar, batch).ws_bytes + 255) / 256 * 256);
+  }
   GemmArgs g = make_args(d, kid, reinterpret_cast<const float2*>(a), reinterpret_cast<const float2*>(b),
                          reinterpret_cast<float2*>(c), (int32_t)batch, d.a_elems, d.b_elems, d.c_elems,
-                         is_tc(kid) ? tc_tile(kid, d.nm, d.nk, d.nn, batch, batch * d.c_elems,
-                                              (int64_t)(kNoAllocScratchBytes - kNoAllocErrBytes), true)
-                                    : -1);
-  const int64_t cap = (int64_t)(kNoAllocScratchBytes - kNoAllocErrBytes);
+                         is_tc(kid) ? tc_tile(kid, d.nm, d.nk, d.nn, batch, batch * d.c_elems, part_cap, true) : -1);
   uint8_t* base = static_cast<uint8_t*>(noalloc_scratch_address());
   int32_t* err = reinterpret_cast<int32_t*>(base);
   float* amax = reinterpret_cast<float*>(base + 16);   // FP16X3 operand maxima, inside the header
@@ -2143,9 +2148,11 @@ extern "C" tn_status tn_contract_pair_noalloc(const float* a, const int32_t* aw,
     g.amax_a = amax;
     g.amax_b = amax + 1;
   }
-  // split-K as tn_contract_pair chooses it, as long as the partial sums fit
-  // beside the B' images; otherwise one pass over k
-  StepLaunch L = make_launch(g, kid, ar, batch, batch * d.c_elems, true, -1, cap);
+  // split-K as tn_contract_pair chooses it, among the choices whose partial sums
+  // fit beside the B' images.  (Chosen against the whole array, 16 partial tiles of 12 x
+  // 1024 x 2^14 x 8 did not fit where 8 do, and one pass over k instead took 383 us
+  // with an error of 1.1e-4; 8 take 353 us with 1.5e-5.)
+  StepLaunch L = make_launch(g, kid, ar, batch, batch * d.c_elems, true, -1, part_cap);
   if (L.ws_bytes > cap) L = make_launch(g, kid, ar, batch);
   // many small instances whose B' images do not fit together: the CUDA cores, which
   // need no scratch (4096 x (128 x 32 x 32): 64 MiB of images)

@@ -125,3 +125,26 @@ def test_noalloc_takes_many_small_instances(env, prec, cm, shape, batch):
         bound = (2 * 2 ** nk + 2) * 2.0 ** -24 * mag
         assert np.all(np.abs(got[i].real - want.real) <= bound)
         assert np.all(np.abs(got[i].imag - want.imag) <= bound)
+
+
+@pytest.mark.parametrize("shape,batch", [((10, 14, 3), 12), ((12, 14, 4), 3), ((12, 15, 3), 3), ((11, 14, 4), 5),
+                                         ((11, 16, 3), 3)])
+def test_noalloc_divides_k_beside_the_images(env, shape, batch):
+    """Partial sums and B' images that fill the static array between them: k is
+    still divided as far as both fit, so the tensor cores' 32-bit accumulation
+    runs over at most 2^13 of the k (norm-wise 4e-5 at BF16x3; it grows with the
+    length of the chain, and one pass over these k is 1.1e-4 to 4.6e-4 off)."""
+    tn, torch = env
+    nm, nk, nn = shape
+    wires = list(range(nm + nk + nn))
+    m_w, k_w, n_w = wires[:nm], wires[nm:nm + nk], wires[nm + nk:]
+    g = torch.Generator(device="cuda").manual_seed(sum(shape))
+    draw = lambda r: torch.randn((batch, 1 << r), generator=g, dtype=torch.complex64, device="cuda")
+    ta, tb = draw(nm + nk), draw(nk + nn)
+    tc = torch.full((batch, 1 << (nm + nn)), float("nan"), dtype=torch.complex64, device="cuda")
+    st = _noalloc(tn, ta, k_w + m_w, tb, k_w + n_w, tc, m_w + n_w, batch, "bf16x3", 4, torch)
+    assert st == tn.TN_OK, tn.load().tn_last_error()
+    tn.device_sync()
+    want = torch.bmm(tb.view(batch, 1 << nn, 1 << nk).to(torch.complex128),
+                     ta.view(batch, 1 << nm, 1 << nk).to(torch.complex128).transpose(1, 2)).reshape(batch, -1)
+    assert float((tc.to(torch.complex128) - want).norm() / want.norm()) <= 4e-5
