@@ -39,11 +39,12 @@
  * stream) so that this header needs no CUDA include.
  *
  * Concurrency: a plan is used by one host thread at a time; different plans may
- * run on different streams.  tn_contract_pair, tn_xeb and tn_frugal_sample
- * share one small per-device scratch area (result word, error word, B' images
- * of tn_contract_pair, grown on demand), so calls of these that may overlap on
- * the same device -- from several host threads, or queued on streams that run
- * concurrently -- must be serialised by the caller.
+ * run on different streams.  tn_xeb and tn_frugal_sample, which return with
+ * their result, run one at a time per device, whatever threads and streams call
+ * them.  tn_contract_pair keeps its scratch (error word, FP16X3 maxima, B'
+ * images) in one per-device area, grown on demand, so calls of it that may
+ * overlap on the same device -- from several host threads, or queued on streams
+ * that run concurrently -- must be serialised by the caller.
  */
 #ifndef TN_GB300_H
 #define TN_GB300_H

@@ -1685,8 +1685,6 @@ extern "C" void tn_plan_destroy(tn_plan_t* h) {
   delete h;
 }
 
-// Per-device scratch of the calls that have no plan: the XEB sum, the error
-// word and the B' workspace of tn_contract_pair.
 // FP16X3 calls without a plan: the maxima of A and B by one reduction pass each
 static void operand_maxima(const float2* a, int64_t na, const float2* b, int64_t nb, float* amax, cudaStream_t s) {
   CK(cudaMemsetAsync(amax, 0, 2 * sizeof(float), s));
@@ -1696,10 +1694,16 @@ static void operand_maxima(const float2* a, int64_t na, const float2* b, int64_t
   k_amax<<<std::max(gb, 1), 256, 0, s>>>(b, nb, amax + 1);
 }
 
+// Per-device scratch of the calls that have no plan: the XEB sum, the sampling
+// results, the error word and the B' workspace of tn_contract_pair.
 constexpr int64_t kHostWords = 8192;
 struct Scratch {
+  // held by tn_xeb and tn_frugal_sample from their launch to their result: the
+  // buffers they share, and the ticket, then serve one call at a time
+  std::mutex sync_calls;
   double* xeb = nullptr;          // XEB: the sum, then the blocks' partial sums
   unsigned* xeb_ticket = nullptr; // zero between launches
+  bool xeb_ticket_zero = false;   // false while a launch's end has not been seen
   int32_t* err = nullptr;
   float* amax = nullptr;   // FP16X3 operand maxima of the last call (A, B)
   unsigned long long* first = nullptr;   // frugal sampling: ~0 unless a candidate was out of range, then the
@@ -1716,13 +1720,16 @@ static Scratch& scratch_for_device() {
   CK(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_scratch_mu);
   Scratch& s = g_scratch[dev];
-  if (!s.xeb) {
-    CK(cudaMalloc(&s.xeb_ticket, sizeof(unsigned)));
-    CK(cudaMemset(s.xeb_ticket, 0, sizeof(unsigned)));
-    CK(cudaMalloc(&s.xeb, sizeof(double) * (1 + XEB_BLOCKS)));
-    CK(cudaMalloc(&s.err, sizeof(int32_t)));
-    CK(cudaMemset(s.err, 0, sizeof(int32_t)));
-    CK(cudaMalloc(&s.amax, 2 * sizeof(float)));
+  if (!s.host) {   // the last of them: what an earlier, failed call allocated is kept
+    if (!s.xeb_ticket) CK(cudaMalloc(&s.xeb_ticket, sizeof(unsigned)));
+    if (!s.xeb) CK(cudaMalloc(&s.xeb, sizeof(double) * (1 + XEB_BLOCKS)));
+    if (!s.err) {
+      int32_t* err = nullptr;
+      CK(cudaMalloc(&err, sizeof(int32_t)));
+      CK(cudaMemset(err, 0, sizeof(int32_t)));
+      s.err = err;
+    }
+    if (!s.amax) CK(cudaMalloc(&s.amax, 2 * sizeof(float)));
     CK(cudaMallocHost(&s.host, kHostWords * sizeof(unsigned long long)));
   }
   return s;
@@ -1735,8 +1742,11 @@ extern "C" tn_status tn_xeb(const double* amps, int64_t count, int32_t n_qubits,
   if (count < 1) fail(TN_ERR_ARG, "tn_xeb: count must be >= 1");
   if (n_qubits < 0 || n_qubits > 1023) fail(TN_ERR_ARG, "tn_xeb: n_qubits out of range");
   Scratch& sc = scratch_for_device();
+  std::lock_guard<std::mutex> one(sc.sync_calls);
   double* scratch = sc.xeb;
   cudaStream_t s = (cudaStream_t)stream;
+  if (!sc.xeb_ticket_zero) CK(cudaMemsetAsync(sc.xeb_ticket, 0, sizeof(unsigned), s));
+  sc.xeb_ticket_zero = false;
   // a block per 1024 amplitudes (four a thread), at most four blocks per SM
   const int64_t per = 4 * XEB_THREADS;
   const int blocks = (int)std::min<int64_t>((count + per - 1) / per, std::min<int64_t>(4 * sm_count(), XEB_BLOCKS));
@@ -1744,6 +1754,7 @@ extern "C" tn_status tn_xeb(const double* amps, int64_t count, int32_t n_qubits,
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(sc.host, scratch, sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  sc.xeb_ticket_zero = true;
   double sum = 0;
   std::memcpy(&sum, sc.host, sizeof(double));
   *xeb_out = std::ldexp(sum / (double)count, n_qubits) - 1.0;
@@ -1760,6 +1771,7 @@ extern "C" tn_status tn_frugal_sample(const double* amps, int64_t count, int32_t
   if (!(m_bound > 0.0) || !std::isfinite(m_bound)) fail(TN_ERR_ARG, "tn_frugal_sample: m_bound must be positive");
   if (n_draws > ((int64_t)1 << 40) / n_samples) fail(TN_ERR_ARG, "tn_frugal_sample: too many draws");
   Scratch& sc = scratch_for_device();
+  std::lock_guard<std::mutex> one(sc.sync_calls);
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t words = n_samples + 1;
   if (words > sc.first_cap) {

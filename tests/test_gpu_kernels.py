@@ -111,6 +111,38 @@ def test_xeb_block_counts(env, count):
     assert tn.xeb(t, 20) == f
 
 
+def test_scoring_calls_from_several_threads(env):
+    """tn_xeb and tn_frugal_sample share one scratch area per device: calls from
+    several threads, each on a stream of its own, give what they give alone,
+    and leave the area fit for the next call."""
+    import threading
+    tn, torch = env
+    rng = np.random.default_rng(11)
+    jobs = []
+    for t, count in enumerate((3001, 100003, 500000, 1 << 20)):
+        a = torch.from_numpy((rng.normal(size=count) + 1j * rng.normal(size=count)) * 2.0 ** -10).cuda()
+        cand = torch.from_numpy(rng.integers(0, count, size=(50 + t, 16))).cuda()
+        u = torch.from_numpy(rng.random((50 + t, 16))).cuda()
+        jobs.append((a, cand, u, tn.xeb(a, 20), tn.frugal_sample(a, 20, 10.0, cand, u)))
+    wrong = []
+
+    def work(job, stream):
+        a, cand, u, f, first = job
+        for _ in range(100):
+            if tn.xeb(a, 20, stream=stream) != f or tn.frugal_sample(a, 20, 10.0, cand, u, stream=stream) != first:
+                wrong.append(a.numel())
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(j, torch.cuda.Stream())) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
+    for a, cand, u, f, first in jobs:
+        assert tn.xeb(a, 20) == f and tn.frugal_sample(a, 20, 10.0, cand, u) == first
+
+
 @pytest.mark.parametrize("misaligned", [False, True])
 @pytest.mark.parametrize("kind", ["random", "identity", "reverse", "rotate", "swap ends"])
 @pytest.mark.parametrize("rank,batch", [(9, 3), (10, 1), (11, 3), (12, 1), (13, 5), (12, 700), (14, 153), (22, 1)])
