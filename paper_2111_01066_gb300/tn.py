@@ -159,10 +159,15 @@ def _check(status: int) -> None:
 
 def _ints(seq):
     """int32 buffer of a sequence of integers and its address (the buffer must outlive the call)."""
-    try:
-        buf = array.array("i", seq)
-    except (TypeError, OverflowError):   # other numbers: converted one by one, wrapped to 32 bits
-        buf = array.array("i", _i32(seq)[:len(seq)])
+    n = len(seq)
+    if type(seq) is list or type(seq) is tuple:
+        try:
+            buf = array.array("i", seq)
+            return buf, buf.buffer_info()[0]
+        except (TypeError, OverflowError):   # other numbers
+            pass
+    # one by one, wrapped to 32 bits (array.array would take bytes for the items' memory)
+    buf = array.array("i", _i32(seq)[:n])
     return buf, buf.buffer_info()[0]
 
 

@@ -429,3 +429,17 @@ def test_step_groups_are_consecutive_independent_and_small(tn, name):
             assert sum(shapes[i]) < 20
             for x in nodes[i]:
                 assert x - n_leaves not in members or x < n_leaves
+
+
+@pytest.mark.parametrize("seq", [[2, 0, 1], (2, 0, 1), b"\x02\x00\x01", bytearray(b"\x02\x00\x01"), np.array([2, 0, 1]),
+                                 np.array([2.0, 0.0, 1.0]), [2.0, 0, 1], range(3), [2 ** 32 + 2, 0, 1], [], "201"])
+def test_integer_lists_of_any_kind(tn, seq):
+    """Wires and permutations reach C item by item, whatever sequence holds them."""
+    buf, at = tn._ints(seq)
+    assert list(buf) == [int(v) - (2 ** 32 if int(v) > 2 ** 31 else 0) for v in seq]
+    assert at == buf.buffer_info()[0] and buf.itemsize == 4
+
+
+def test_integer_lists_need_a_length(tn):
+    with pytest.raises(TypeError):
+        tn._ints(iter([1, 2]))
