@@ -256,7 +256,9 @@ tn_status tn_plan_model_time(const tn_plan_t* plan, double peak_flops, double pe
  *   stream           cudaStream_t; the call is asynchronous on it.
  * The first call on a plan allocates the plan's device arena, workspace and
  * the B' image buffers of steps whose B operand depends on no slice (all freed
- * by tn_plan_destroy) and uploads the leaf tensors; that call synchronises.
+ * by tn_plan_destroy) and uploads the leaf tensors; that call synchronises.  A
+ * later call allocates and waits only where it has more chunks than any before
+ * and than 1024 (their parameters).
  * Plans of small chunks hold several arenas, 64 MB (and max_arena_bytes) at most,
  * and run that many chunks of a call side by side, of one batch or of several;
  * the amplitudes are the same bits as chunk by chunk.

@@ -646,25 +646,22 @@ struct GroupRun {
   struct Multi {
     int blocks = 0, n = 0;
     int cluster = 1;                         // SIMT_MAX_SPLIT where a step's k is split
-    GemmArgs* args = nullptr;                // device: n GemmArgs
-    int32_t* start = nullptr;                // device: n + 1 block offsets
-    int8_t* tiling = nullptr;                // device: n CUDA-core tilings (simt_multi_tiling)
-    int8_t* split = nullptr;                 // device: n split-K factors
+    // offsets in DeviceState::group_buf: n GemmArgs, n + 1 block offsets (int32), n
+    // CUDA-core tilings (simt_multi_tiling), n split-K factors
+    size_t args_at = 0, start_at = 0, tiling_at = 0, split_at = 0;
   };
   std::vector<Multi> multi;
 };
 
 // The launches of a plan for 2^ls lanes: CUDA-core steps with the lanes as further
-// instances, tensor-core steps once per lane (lane l > 0 in more[l - 1]), so that
+// instances, tensor-core steps once per lane (lane l > 0 in more[step][l - 1]), so that
 // a chunk's result does not depend on what runs beside it.
 struct LaunchSet {
   int ls = 0;
-  bool built = false;
   std::vector<StepLaunch> launches;
-  std::vector<std::vector<StepLaunch>> more;   // [lane - 1][step], tensor-core steps only
+  std::vector<std::vector<StepLaunch>> more;   // [step][lane - 1], tensor-core steps only (empty: one lane)
   std::vector<GroupRun> groups;
   std::vector<int> group_at;                   // per step: its group run's index, or -1
-  uint8_t* group_buf = nullptr;                // device memory of every Multi's arrays
   // the launch sequences as CUDA graphs, each captured at its second use (the
   // first runs eagerly): [0] a chunk per lane, [1] with the prologue of new
   // batches; every kernel reads its chunk parameters from device memory
@@ -694,6 +691,7 @@ struct DeviceState {
   int root_groups = 1;
   LaunchSet set[MAX_LS_LANES + 1];
   std::vector<StepLaunch>& launches = set[0].launches;
+  uint8_t* group_buf = nullptr;   // the arrays of every set's multi-step launches
   int ls_lanes = 0;               // lanes that the arena has room for (log2)
   int64_t lane_stride = 0;        // elements between the lanes' arenas (a power of two where there are several)
   std::vector<uint8_t*> own_imgs;              // B' images built ahead of the chunks (StepLaunch::bimg_own)
@@ -730,24 +728,28 @@ static int pick_kernel(int precision, int cmult, const StepDesc& d, int64_t n_in
   return tc_kernel(precision, cmult);
 }
 
-// Launch arguments of plan step d for kernel kid; FP16X3 plans also get the
-// maxima of the step's operands (to scale them) and of its result (to record).
-// lane: the arena of that lane alone; ls > 0: all of 2^ls lanes as instances.
-static GemmArgs step_args(const DeviceState& ds, const StepDesc& d, int kid, int tn_log = -1, int lane = 0, int ls = 0) {
+// Launch arguments of plan step d for kernel kid in one lane's arena; FP16X3 plans also
+// get the maxima of the step's operands (to scale them) and of its result (to record).
+static GemmArgs step_args(const DeviceState& ds, const StepDesc& d, int kid, int tn_log = -1, int lane = 0) {
   float2* arena = ds.arena + lane * ds.lane_stride;
-  GemmArgs g = make_args(d, kid, arena + d.a_off, arena + d.b_off, arena + d.c_off, 1 << (d.nb + ls), 0, 0, 0, tn_log);
-  for (int t = 0; t < ls; ++t)
-    g.a_bpos[d.nb + t] = g.b_bpos[d.nb + t] = g.c_bpos[d.nb + t] =
-        (int8_t)(__builtin_ctzll((uint64_t)ds.lane_stride) + t);
-  g.nb = d.nb + ls;
-  g.ls_lanes = ls;
+  GemmArgs g = make_args(d, kid, arena + d.a_off, arena + d.b_off, arena + d.c_off, 1 << d.nb, 0, 0, 0, tn_log);
   if (ds.amax) {
     float* amax = ds.amax + (int64_t)lane * ds.amax_nodes;
     g.amax_a = amax + d.a_node;
     g.amax_b = amax + d.b_node;
     g.amax_c = amax + d.c_node;
-    g.amax_lane = ls ? ds.amax_nodes : 0;
   }
+  return g;
+}
+// The same with the lanes 0 .. 2^ls - 1 as further instances, from the arguments of lane 0.
+static GemmArgs lanes_args(const DeviceState& ds, GemmArgs g, int ls) {
+  for (int t = 0; t < ls; ++t)
+    g.a_bpos[g.nb + t] = g.b_bpos[g.nb + t] = g.c_bpos[g.nb + t] =
+        (int8_t)(__builtin_ctzll((uint64_t)ds.lane_stride) + t);
+  g.nb += ls;
+  g.n_inst <<= ls;
+  g.ls_lanes = ls;
+  g.amax_lane = ds.amax ? ds.amax_nodes : 0;
   return g;
 }
 
@@ -756,9 +758,11 @@ static int simt_multi_tiling(int kid) {
   return kid == K_SIMT_32x32 ? 3 : (kid >= K_SIMT_64x64 && kid <= K_SIMT_256x4 ? kid : -1);
 }
 
-static void launch_simt_multi(const GroupRun::Multi& m, cudaStream_t s) {
+static void launch_simt_multi(const DeviceState& ds, const GroupRun::Multi& m, cudaStream_t s) {
+  const uint8_t* buf = ds.group_buf;
   klaunch(k_cgemm_simt_multi, dim3((unsigned)m.blocks), SIMT_THREADS, 0, s, m.cluster, true,
-          (const GemmArgs*)m.args, (const int32_t*)m.start, (const int8_t*)m.tiling, (const int8_t*)m.split, (int32_t)m.n);
+          reinterpret_cast<const GemmArgs*>(buf + m.args_at), reinterpret_cast<const int32_t*>(buf + m.start_at),
+          reinterpret_cast<const int8_t*>(buf + m.tiling_at), reinterpret_cast<const int8_t*>(buf + m.split_at), (int32_t)m.n);
 }
 
 // Dependence flags of a node (bit 0: on the slice id, bit 1: on the closed
@@ -802,15 +806,12 @@ static void setup_hoisted(Plan& p, DeviceState& ds) {
   }
 }
 
-// Group runs from the plan's step groups and the kernels chosen so far.
-static void build_groups(const Plan& p, LaunchSet& ds) {
-  if (ds.group_buf) {
-    CK(cudaFree(ds.group_buf));
-    ds.group_buf = nullptr;
-  }
+// Group runs from the plan's step groups and the kernels chosen so far.  The arrays of
+// their multi-step launches are appended to `host`, the image of group_buf, and addressed
+// by their offsets in it.
+static void build_groups(const Plan& p, LaunchSet& ds, std::vector<uint8_t>& host) {
   ds.groups.clear();
   ds.group_at.assign(p.steps.size(), -1);
-  std::vector<std::pair<size_t, std::vector<int>>> pending;   // (group run, steps) of each Multi
   for (size_t i = 0; i < p.steps.size();) {
     const int gid = p.steps[i].group;
     size_t j = i + 1;
@@ -832,60 +833,36 @@ static void build_groups(const Plan& p, LaunchSet& ds) {
     if (simt.size() >= 2) {
       GroupRun::Multi m;
       m.n = (int)simt.size();
+      m.args_at = (host.size() + 255) / 256 * 256;
+      m.start_at = (m.args_at + sizeof(GemmArgs) * simt.size() + 15) / 16 * 16;
+      m.tiling_at = m.start_at + sizeof(int32_t) * (simt.size() + 1);
+      m.split_at = m.tiling_at + simt.size();
+      host.resize(m.split_at + simt.size(), 0);
+      for (int t : simt)
+        if (simt_split(ds.launches[t].g, ds.launches[t].kid) > 1) m.cluster = SIMT_MAX_SPLIT;
+      int32_t blocks = 0;
+      for (size_t q = 0; q < simt.size(); ++q) {
+        const GemmArgs& g = ds.launches[simt[q]].g;
+        const int kid = ds.launches[simt[q]].kid, split = simt_split(g, kid);
+        std::memcpy(host.data() + m.args_at + q * sizeof(GemmArgs), &g, sizeof(GemmArgs));
+        host[m.tiling_at + q] = (uint8_t)simt_multi_tiling(kid);
+        host[m.split_at + q] = (uint8_t)split;
+        // whole clusters: the kernel's blocks past the last tile only keep its barriers
+        int64_t nb = ((int64_t)1 << (g.nm - g.tm)) * ((int64_t)1 << (g.nn - g.tn)) * split *
+                     std::min<int64_t>(g.n_inst, 65535);
+        nb = (nb + m.cluster - 1) / m.cluster * m.cluster;
+        if (blocks + nb > 0x7fffffff) fail(TN_ERR_UNSUPPORTED, "step group grid too large");
+        std::memcpy(host.data() + m.start_at + q * sizeof(int32_t), &blocks, sizeof(int32_t));
+        blocks += (int32_t)nb;
+      }
+      std::memcpy(host.data() + m.start_at + simt.size() * sizeof(int32_t), &blocks, sizeof(int32_t));
+      m.blocks = blocks;
       gr.multi.push_back(m);
-      pending.push_back({ds.groups.size(), simt});
     }
     for (size_t t = i; t < j; ++t) ds.group_at[t] = (int)ds.groups.size();
     ds.groups.push_back(gr);
     i = j;
   }
-  if (pending.empty()) return;
-  // one device buffer: every Multi's GemmArgs, then its block offsets
-  size_t bytes = 0;
-  for (auto& pm : pending) {
-    bytes = (bytes + 255) / 256 * 256 + sizeof(GemmArgs) * pm.second.size();
-    bytes = (bytes + 15) / 16 * 16 + sizeof(int32_t) * (pm.second.size() + 1);
-    bytes += 2 * pm.second.size();   // tilings, splits
-  }
-  std::vector<uint8_t> host(bytes, 0);
-  CK(cudaMalloc(&ds.group_buf, bytes));
-  size_t off = 0;
-  std::vector<size_t> next_multi(ds.groups.size(), 0);
-  for (auto& pm : pending) {
-    auto& m = ds.groups[pm.first].multi[next_multi[pm.first]++];
-    off = (off + 255) / 256 * 256;
-    const size_t args_off = off;
-    off += sizeof(GemmArgs) * pm.second.size();
-    off = (off + 15) / 16 * 16;
-    const size_t start_off = off;
-    off += sizeof(int32_t) * (pm.second.size() + 1);
-    const size_t tiling_off = off;
-    off += 2 * pm.second.size();
-    int32_t blocks = 0;
-    for (int t : pm.second)
-      if (simt_split(ds.launches[t].g, ds.launches[t].kid) > 1) m.cluster = SIMT_MAX_SPLIT;
-    for (size_t q = 0; q < pm.second.size(); ++q) {
-      const GemmArgs& g = ds.launches[pm.second[q]].g;
-      std::memcpy(host.data() + args_off + q * sizeof(GemmArgs), &g, sizeof(GemmArgs));
-      const int kid = ds.launches[pm.second[q]].kid, split = simt_split(g, kid);
-      host[tiling_off + q] = (uint8_t)simt_multi_tiling(kid);
-      host[tiling_off + pm.second.size() + q] = (uint8_t)split;
-      // whole clusters: the kernel's blocks past the last tile only keep its barriers
-      int64_t nb = ((int64_t)1 << (g.nm - g.tm)) * ((int64_t)1 << (g.nn - g.tn)) * split *
-                   std::min<int64_t>(g.n_inst, 65535);
-      nb = (nb + m.cluster - 1) / m.cluster * m.cluster;
-      if (blocks + nb > 0x7fffffff) fail(TN_ERR_UNSUPPORTED, "step group grid too large");
-      std::memcpy(host.data() + start_off + q * sizeof(int32_t), &blocks, sizeof(int32_t));
-      blocks += (int32_t)nb;
-    }
-    std::memcpy(host.data() + start_off + pm.second.size() * sizeof(int32_t), &blocks, sizeof(int32_t));
-    m.blocks = blocks;
-    m.args = reinterpret_cast<GemmArgs*>(ds.group_buf + args_off);
-    m.start = reinterpret_cast<int32_t*>(ds.group_buf + start_off);
-    m.tiling = reinterpret_cast<int8_t*>(ds.group_buf + tiling_off);
-    m.split = m.tiling + pm.second.size();
-  }
-  CK(cudaMemcpy(ds.group_buf, host.data(), bytes, cudaMemcpyHostToDevice));
 }
 
 // Step d's launch with one kernel choice (as the autotuner builds its candidates).
@@ -895,30 +872,37 @@ static StepLaunch build_choice(const DeviceState& ds, const StepDesc& d, int kid
                      d.c_elems, true, epi, (int64_t)256 << 20, bslots, pair);
 }
 
-// The launch set of 2^ls lanes, built from the kernels chosen for one lane.
-static void ensure_set(Plan& p, DeviceState& ds, int ls) {
-  LaunchSet& st = ds.set[ls];
-  if (st.built) return;
-  if (ls > 0) {
-    st.ls = ls;
-    st.launches.clear();
-    st.more.assign(((size_t)1 << ls) - 1, {});
-    for (size_t i = 0; i < p.steps.size(); ++i) {
-      const StepDesc& d = p.steps[i];
-      const StepLaunch& one = ds.launches[i];
-      if (is_tc(one.kid)) {
-        st.launches.push_back(one);
-        for (int l = 1; l < (1 << ls); ++l)
-          st.more[l - 1].push_back(build_choice(ds, d, one.kid, one.g.tn, one.tc.epi_ok, one.tc.nbs, one.tc.pair, l));
-      } else {
-        const GemmArgs g = step_args(ds, d, one.kid, -1, 0, ls);
-        st.launches.push_back(make_launch(g, one.kid, 0, 1));
-        for (auto& m : st.more) m.push_back(StepLaunch());
+// The launch sets of every number of lanes, built from the kernels chosen for one lane:
+// all of them at once, so that no later call allocates or waits, whatever its number
+// of chunks.
+static void build_sets(Plan& p, DeviceState& ds) {
+  std::vector<uint8_t> host;
+  for (int ls = 0; ls <= ds.ls_lanes; ++ls) {
+    LaunchSet& st = ds.set[ls];
+    if (ls > 0) {
+      st.ls = ls;
+      st.launches.clear();
+      st.launches.reserve(p.steps.size());
+      st.more.assign(p.steps.size(), {});
+      for (size_t i = 0; i < p.steps.size(); ++i) {
+        const StepDesc& d = p.steps[i];
+        const StepLaunch& one = ds.launches[i];
+        if (is_tc(one.kid)) {
+          st.launches.push_back(one);
+          for (int l = 1; l < (1 << ls); ++l)
+            st.more[i].push_back(build_choice(ds, d, one.kid, one.g.tn, one.tc.epi_ok, one.tc.nbs, one.tc.pair, l));
+        } else {
+          st.launches.push_back(make_launch(lanes_args(ds, one.g, ls), one.kid, 0, 1));
+        }
       }
     }
+    build_groups(p, st, host);
   }
-  build_groups(p, st);
-  st.built = true;
+  if (ds.group_buf) CK(cudaFree(ds.group_buf));
+  ds.group_buf = nullptr;
+  if (host.empty()) return;
+  CK(cudaMalloc(&ds.group_buf, host.size()));
+  CK(cudaMemcpy(ds.group_buf, host.data(), host.size(), cudaMemcpyHostToDevice));
 }
 
 static int ceil_log2(int64_t v) { return v <= 1 ? 0 : 64 - __builtin_clzll((uint64_t)(v - 1)); }
@@ -1030,8 +1014,8 @@ static void ensure_device(Plan& p) {
   CK(cudaMemset(ds->root_tickets, 0, sizeof(unsigned) * tickets));
   if (!in_arena(p.root.off, (int64_t)1 << p.root.rank, 1 << __builtin_popcount(p.root.bmask)))
     fail(TN_ERR_PLAN, "internal: root outside the arena");
-  ensure_set(p, *ds, 0);
   setup_hoisted(p, *ds);
+  build_sets(p, *ds);
 }
 
 static void drop_graphs(DeviceState& ds) {
@@ -1060,7 +1044,7 @@ void destroy_device_state(Plan* p) {
   cudaFree(ds->root_part);
   cudaFree(ds->root_tickets);
   cudaFree(ds->amax);
-  for (LaunchSet& st : ds->set) cudaFree(st.group_buf);
+  cudaFree(ds->group_buf);
   for (uint8_t* b : ds->own_imgs) cudaFree(b);
   drop_graphs(*ds);
   if (ds->done) cudaEventDestroy(ds->done);
@@ -1077,8 +1061,8 @@ static void launch_class(Plan& p, cudaStream_t s, LaunchSet& st, Pred in_class) 
   DeviceState& ds = *p.dev;
   auto one = [&](int i) {
     launch_step(st.launches[i], ds.ws, ds.err, s, false);
-    if (is_tc(st.launches[i].kid))
-      for (auto& lane : st.more) launch_step(lane[i], ds.ws, ds.err, s, false);
+    if (!st.more.empty())
+      for (StepLaunch& lane : st.more[i]) launch_step(lane, ds.ws, ds.err, s, false);
   };
   for (size_t i = 0; i < p.steps.size(); ++i) {
     if (!in_class(p.steps[i].dep_flags)) continue;
@@ -1088,7 +1072,7 @@ static void launch_class(Plan& p, cudaStream_t s, LaunchSet& st, Pred in_class) 
       continue;
     }
     const GroupRun& gr = st.groups[gi];
-    for (const auto& m : gr.multi) launch_simt_multi(m, s);
+    for (const auto& m : gr.multi) launch_simt_multi(ds, m, s);
     for (int t : gr.singles) one(t);
     i = (size_t)gr.end - 1;
   }
@@ -1280,7 +1264,6 @@ extern "C" tn_status tn_contract_slices(tn_plan_t* h, uint64_t first, uint64_t c
   const bool pro0 = has_prologue(p, 0), pro2 = has_prologue(p, 2);
   for (const Run& r : runs) {
     const int n = 1 << r.ls;
-    ensure_set(p, ds, r.ls);
     LaunchSet& st = ds.set[r.ls];
     if (ds.pro0_lanes < n) {
       if (pro0) {
@@ -1352,9 +1335,8 @@ extern "C" tn_status tn_plan_step_times(tn_plan_t* h, int32_t reps, double* ms_o
 // After the kernels of a plan changed: group runs, chunk graph and prologues anew.
 static void kernels_changed(Plan& p, DeviceState& ds) {
   drop_graphs(ds);
-  for (LaunchSet& st : ds.set) st.built = false;
-  ensure_set(p, ds, 0);
   setup_hoisted(p, ds);
+  build_sets(p, ds);
   ds.forget_prologues();   // the arena may have been overwritten: they run again
 }
 

@@ -233,3 +233,32 @@ def test_chunks_side_by_side(env, prec, slices, chunk):
         assert np.linalg.norm(got - want) < (1e-5 if prec == "fp32" else 1e-4) * np.linalg.norm(want)
         if n // 3 == 0 or chunk == 0:   # one chunk per range: also the same bits
             assert torch.equal(torch.view_as_real(out), torch.view_as_real(alone))
+
+
+def test_later_calls_do_not_wait(env):
+    """Only the first call of a plan synchronises: calls with other numbers of
+    chunks return while earlier work of another stream still runs (half a second of
+    sleep on the legacy stream, which a blocking copy would wait for)."""
+    import time
+    import rqcgen
+    tn, torch = env
+    circ = rqcgen.sycamore_style(4, 4, 9, 7, 0)
+    plan = tn.Plan(tn.Network(circ), open_mask=0b1111110000000000, max_log2_intermediate=30, trials=8)
+    out = torch.zeros(16 << 6, dtype=torch.complex128, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    plan.contract_slices(0, 1, [1], out, stream=side)
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda._sleep(1000)   # its kernel is loaded
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.default_stream()):
+        e0.record()
+        torch.cuda._sleep(1_000_000_000)
+        e1.record()
+    t0 = time.perf_counter()
+    for count in (2, 5, 3, 16, 9, 16, 1):
+        plan.contract_slices(0, 1, [4 * i + count for i in range(count)], out, stream=side)
+    host = time.perf_counter() - t0
+    side.synchronize()
+    torch.cuda.synchronize()
+    assert e0.elapsed_time(e1) > 400.0 and host < 0.2
