@@ -220,6 +220,7 @@ struct StepLaunch {
   // batch) into bimg_own; null: built with every launch in the workspace
   uint8_t* bimg_own = nullptr;
   int bimg_cls = -1;
+  int64_t bimg_lane = 0;   // bytes from one lane's images to the next one's
 };
 
 static bool is_tc(int kid) { return kid >= K_TC_TF32 && kid <= K_TC_FP16X3_3M; }
@@ -778,9 +779,11 @@ static int node_flags(const Plan& p, int node) {
 }
 
 // B' images of per-chunk tensor-core steps whose B depends on no slice: one
-// buffer each, built by the prologue of B's class (once per plan, or once per
-// batch bitstring) instead of with every chunk.  Where a buffer cannot be had
-// the step keeps building its images per launch.
+// buffer each per lane, built by the prologue of B's class (once per plan, or once
+// per batch bitstring) instead of with every chunk, for the lane's own arena: they
+// are as valid as the results of that prologue in that lane, whichever launch set
+// runs it and reads them.  Where the buffers cannot be had the step keeps building its
+// images per launch.
 static void setup_hoisted(Plan& p, DeviceState& ds) {
   for (uint8_t* b : ds.own_imgs) cudaFree(b);
   ds.own_imgs.clear();
@@ -788,21 +791,21 @@ static void setup_hoisted(Plan& p, DeviceState& ds) {
     StepLaunch& L = ds.launches[i];
     L.bimg_own = nullptr;
     L.bimg_cls = -1;
+    L.bimg_lane = 0;
     const StepDesc& d = p.steps[i];
-    // (several lanes: a batch's prologue may run for one lane in one set of launches
-    // and its chunks in another; the images are then built with every launch)
-    if (ds.ls_lanes > 0 || !is_tc(L.kid) || !(d.dep_flags & 1)) continue;
+    if (!is_tc(L.kid) || !(d.dep_flags & 1)) continue;
     const int bf = node_flags(p, d.b_node);
     if (bf & 1) continue;
-    const int64_t img = L.tc.n_split > 1 ? L.split_off : L.ws_bytes;
+    const int64_t img = ((L.tc.n_split > 1 ? L.split_off : L.ws_bytes) + 255) / 256 * 256;
     uint8_t* buf = nullptr;
-    if (img <= 0 || cudaMalloc(&buf, (size_t)img) != cudaSuccess) {
+    if (img <= 0 || cudaMalloc(&buf, (size_t)img << ds.ls_lanes) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
     ds.own_imgs.push_back(buf);
     L.bimg_own = buf;
     L.bimg_cls = bf;
+    L.bimg_lane = img;
   }
 }
 
@@ -889,8 +892,12 @@ static void build_sets(Plan& p, DeviceState& ds) {
         const StepLaunch& one = ds.launches[i];
         if (is_tc(one.kid)) {
           st.launches.push_back(one);
-          for (int l = 1; l < (1 << ls); ++l)
-            st.more[i].push_back(build_choice(ds, d, one.kid, one.g.tn, one.tc.epi_ok, one.tc.nbs, one.tc.pair, l));
+          for (int l = 1; l < (1 << ls); ++l) {
+            StepLaunch L = build_choice(ds, d, one.kid, one.g.tn, one.tc.epi_ok, one.tc.nbs, one.tc.pair, l);
+            if (one.bimg_own) L.bimg_own = one.bimg_own + l * one.bimg_lane;
+            L.bimg_cls = one.bimg_cls;
+            st.more[i].push_back(L);
+          }
         } else {
           st.launches.push_back(make_launch(lanes_args(ds, one.g, ls), one.kid, 0, 1));
         }
@@ -1117,12 +1124,17 @@ static bool has_prologue(const Plan& p, int cls) {
 static void run_prologue(Plan& p, cudaStream_t s, LaunchSet& st, int cls) {
   DeviceState& ds = *p.dev;
   launch_class(p, s, st, [cls](int f) { return f == cls; });
-  for (const StepLaunch& L : st.launches) {
-    if (!L.bimg_own || L.bimg_cls != cls) continue;
+  auto images = [&](const StepLaunch& L) {
+    if (!L.bimg_own || L.bimg_cls != cls) return;
     TcArgs t = L.tc;
     t.bimg = L.bimg_own;
     t.err = ds.err;
     launch_prep_kid(t, L.kid, s);
+  };
+  for (size_t i = 0; i < st.launches.size(); ++i) {
+    images(st.launches[i]);
+    if (!st.more.empty())
+      for (const StepLaunch& L : st.more[i]) images(L);
   }
 }
 

@@ -235,6 +235,61 @@ def test_chunks_side_by_side(env, prec, slices, chunk):
             assert torch.equal(torch.view_as_real(out), torch.view_as_real(alone))
 
 
+@pytest.fixture(scope="module")
+def wide_plans(env):
+    """35 qubits, 14 cycles, 8 chunks of one slice: a plan of several lanes whose
+    chunks hold tensor-core steps (from 2^25 multiply-adds), some of them with a
+    B that depends on no slice; and the same circuit's FP32 amplitudes."""
+    import rqcgen
+    tn, torch = env
+    circ = rqcgen.sycamore_style(5, 7, 14, 44, 0)
+    net = tn.Network(circ)
+    make = lambda prec, cm=4, arena=0: tn.Plan(net, open_mask=255 << 27, max_log2_intermediate=26, trials=8,
+                                               precision=prec, complex_mult=cm, max_arena_bytes=arena,
+                                               forced_slices=[(34, 22), (34, 21), (34, 20)])
+    bits = [int(b) for b in np.random.default_rng(9).integers(0, 1 << 27, size=3)]
+    ref = torch.zeros(3 << 8, dtype=torch.complex128, device="cuda")
+    make("fp32").contract_slices(0, 8, bits, ref)
+    torch.cuda.synchronize()
+    return make, bits, ref
+
+
+@pytest.mark.parametrize("prec,cm", [("tf32", 4), ("bf16x3", 4), ("fp16x3", 4), ("bf16x3", 3), ("fp16x3", 3)])
+def test_lanes_with_tensor_core_steps(env, wide_plans, prec, cm):
+    """Tensor-core steps run once per lane, each lane with its own operands, FP16
+    maxima and B' images: calls of several chunks, of one batch or of several, give
+    the bits of a plan that gets them one chunk a call, and the FP32
+    amplitudes; images of a B that no slice changes are built with its prologue,
+    not with every chunk, in either."""
+    tn, torch = env
+    make, bits, ref = wide_plans
+    many = make(prec, cm)
+    one = make(prec, cm, arena=many.info()["arena_bytes"])   # room for one lane
+    assert one.step_shapes() == many.step_shapes()
+    want = torch.zeros_like(ref)
+    for i, b in enumerate(bits):
+        for c in range(8):
+            one.contract_slices(c, 1, [b], want[i << 8:(i + 1) << 8])
+    kernels = [k for _, k in one.step_times(1)]
+    flags = [one.step_layout(i)["dep_flags"] for i in range(len(kernels))]
+    tc = sum(k.startswith("tc") and bool(f & 1) for k, f in zip(kernels, flags))
+    assert tc >= 2
+    rel = {"tf32": 2e-2, "bf16x3": 1e-4, "fp16x3": 1e-4}[prec]
+    assert float((want - ref).norm() / ref.norm()) < rel
+    for cuts, batches in (([0, 8], [[0, 1, 2]]), ([0, 1, 8], [[0], [1, 2]]), ([0, 3, 4, 8], [[2], [1], [0]]),
+                          ([0, 2, 4, 6, 8], [[0, 1], [2]])):
+        out = torch.zeros_like(ref)
+        for group in batches:
+            part = torch.zeros(len(group) << 8, dtype=torch.complex128, device="cuda")
+            for lo, hi in zip(cuts, cuts[1:]):
+                many.contract_slices(lo, hi - lo, [bits[i] for i in group], part)
+            for j, i in enumerate(group):
+                out[i << 8:(i + 1) << 8] = part[j << 8:(j + 1) << 8]
+        many.sync()
+        assert torch.equal(torch.view_as_real(out), torch.view_as_real(want)), (cuts, batches)
+    assert many.chunk_launches() == one.chunk_launches()
+
+
 def test_later_calls_do_not_wait(env):
     """Only the first call of a plan synchronises: calls with other numbers of
     chunks return while earlier work of another stream still runs (half a second of
