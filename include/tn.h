@@ -260,11 +260,13 @@ tn_status tn_plan_model_time(const tn_plan_t* plan, double peak_flops, double pe
  * later call allocates and waits only where it has more chunks than any before
  * and than 1024 (their parameters).
  * Plans of small chunks hold several arenas, 64 MB (and max_arena_bytes) at most,
- * and run that many chunks of a call side by side, of one batch or of several;
- * the amplitudes are the same bits as chunk by chunk.
+ * and run up to that many chunks of a call side by side, of one batch or of
+ * several, fewer where the shared part below is the larger work; the amplitudes
+ * are the same bits as chunk by chunk.
  * Steps that depend on no slice, and those B' images, are computed once per
  * plan, or once per batch when they depend on the closed bits (main text,
- * section III: the major part of the network is shared by a correlated batch).
+ * section III: the major part of the network is shared by a correlated batch),
+ * in every arena that the call's chunks run in.
  * A range beyond 2^S, n_batches < 1 or a NULL pointer gives TN_ERR_ARG.  Not
  * thread-safe per plan. */
 tn_status tn_contract_slices(tn_plan_t* plan, uint64_t slice_first, uint64_t slice_count,

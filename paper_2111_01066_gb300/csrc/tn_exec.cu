@@ -694,6 +694,11 @@ struct DeviceState {
   std::vector<StepLaunch>& launches = set[0].launches;
   uint8_t* group_buf = nullptr;   // the arrays of every set's multi-step launches
   int ls_lanes = 0;               // lanes that the arena has room for (log2)
+  // rough times that a call's lanes are chosen by (set_lane_times)
+  double chain_us = 0.0;          // a chunk's launches that its lanes share
+  double pro_chain_us = 0.0;      // the same of a batch's prologue
+  double pro_us[2] = {0.0, 0.0};  // one lane's part of the prologue: per plan, per batch
+  bool tc_chunk = false;          // a chunk or its batch's prologue has tensor-core steps
   int64_t lane_stride = 0;        // elements between the lanes' arenas (a power of two where there are several)
   std::vector<uint8_t*> own_imgs;              // B' images built ahead of the chunks (StepLaunch::bimg_own)
   cudaEvent_t done = nullptr;
@@ -912,6 +917,75 @@ static void build_sets(Plan& p, DeviceState& ds) {
   CK(cudaMemcpy(ds.group_buf, host.data(), host.size(), cudaMemcpyHostToDevice));
 }
 
+// Launches for the steps of a class in plan order: CUDA-core ones, which all lanes
+// share, into *shared, kernels of tensor-core steps, which run once per lane, into *alone.
+template <class Pred>
+static void class_launches(const Plan& p, Pred in_class, int* shared, int* alone) {
+  const LaunchSet& st = p.dev->set[0];
+  *shared = *alone = 0;
+  auto one = [&](int i) {
+    const StepLaunch& L = st.launches[i];
+    if (is_tc(L.kid)) *alone += (L.tc.n_split > 1 ? 3 : 2) - (L.bimg_own ? 1 : 0);
+    else ++*shared;
+  };
+  for (size_t i = 0; i < p.steps.size(); ++i) {
+    if (!in_class(p.steps[i].dep_flags)) continue;
+    const int gi = st.group_at.empty() ? -1 : st.group_at[i];
+    if (gi < 0) {
+      one((int)i);
+      continue;
+    }
+    const GroupRun& gr = st.groups[gi];
+    *shared += (int)gr.multi.size();
+    for (int t : gr.singles) one(t);
+    i = (size_t)gr.end - 1;
+  }
+}
+
+// Rough times of the parts that the choice of lanes trades: a launch of a chain of
+// small steps takes about 3 us, a prologue's multiply-adds about 8 flops at 30
+// TFLOP/s on the CUDA cores, and a tensor-core step 8 us at least.
+static void set_lane_times(const Plan& p, DeviceState& ds) {
+  int shared, alone;
+  class_launches(p, [](int f) { return (f & 1) != 0; }, &shared, &alone);
+  ds.chain_us = 3.0 * (2 + shared);
+  class_launches(p, [](int f) { return f == 2; }, &shared, &alone);
+  ds.pro_chain_us = 3.0 * shared;
+  ds.tc_chunk = false;
+  ds.pro_us[0] = ds.pro_us[1] = 0.0;
+  for (size_t i = 0; i < p.steps.size(); ++i) {
+    const StepDesc& d = p.steps[i];
+    const bool tc = is_tc(ds.launches[i].kid);
+    if (d.dep_flags != 0) ds.tc_chunk = ds.tc_chunk || tc;
+    if (d.dep_flags & 1) continue;
+    const double us = std::ldexp(8.0, d.nm + d.nk + d.nn + d.nb) / 1e6 / (tc ? 500.0 : 30.0) + (tc ? 8.0 : 0.0);
+    ds.pro_us[d.dep_flags == 0 ? 0 : 1] += us;
+  }
+}
+
+// Lanes of a call (log2) for `chunks` chunks of each of `batches` batches: the more,
+// the fewer chains of launches, but a batch's prologue runs in min(lanes, chunks)
+// arenas.  Measured (us; all lanes, and what this takes): 30 + 6 qubits of which only the
+// 6 are sliced, prologue of 2^24.8 multiply-adds, 16 chunks of 2^11: 16 lanes 329, 8
+// lanes 231; 36 + 6 qubits, 2^26.7, 4 chunks: 4 lanes 254, 2 lanes 227, and four such
+// batches 821 with 8 lanes, 899 with 2.
+static int lanes_of_call(const DeviceState& ds, size_t batches, size_t chunks) {
+  const size_t total = batches * chunks;
+  int best = 0;
+  double best_us = 0.0;
+  for (int ls = 0; ls <= ds.ls_lanes && (ls == 0 || ((size_t)1 << (ls - 1)) < total); ++ls) {
+    const size_t n = (size_t)1 << ls, runs = (total + n - 1) / n;
+    const double us = (double)runs * ds.chain_us + (double)std::min(runs, batches) * ds.pro_chain_us +
+                      (double)(batches * std::min(n, chunks)) * ds.pro_us[1] +
+                      (double)std::max(0, (int)n - ds.pro0_lanes) * ds.pro_us[0];
+    if (ls == 0 || us <= best_us) {
+      best = ls;
+      best_us = us;
+    }
+  }
+  return best;
+}
+
 static int ceil_log2(int64_t v) { return v <= 1 ? 0 : 64 - __builtin_clzll((uint64_t)(v - 1)); }
 
 // Lanes of a plan (log2): as many as keep their arenas in 64 MB -- in L2, and of
@@ -1023,6 +1097,7 @@ static void ensure_device(Plan& p) {
     fail(TN_ERR_PLAN, "internal: root outside the arena");
   setup_hoisted(p, *ds);
   build_sets(p, *ds);
+  set_lane_times(p, *ds);
 }
 
 static void drop_graphs(DeviceState& ds) {
@@ -1234,18 +1309,20 @@ extern "C" tn_status tn_contract_slices(tn_plan_t* h, uint64_t first, uint64_t c
       prm.push_back(c);
     }
   if (ds.have_done) CK(cudaStreamWaitEvent(s, ds.done, 0));
-  // Runs of chunks side by side: as many as there are lanes.  A rest that is no
+  // Runs of chunks side by side: as many as the call has lanes.  A rest that is no
   // power of two is filled up with copies of its last chunk that count no slices
-  // where a chunk is little work, else it is divided into powers of two.
+  // where a chunk is little work and all its launches are shared by the lanes, else
+  // it is divided into powers of two.
   struct Run {
     size_t at;
     int ls;
   };
   std::vector<Run> runs;
   std::vector<ChunkParam> lanes;
-  const bool fill = p.stats.flops_chunk <= 5e8;
+  const bool fill = p.stats.flops_chunk <= 5e8 && !ds.tc_chunk;
+  const int ls_call = lanes_of_call(ds, (size_t)n_batches, prm.size() / (size_t)n_batches);
   for (size_t i = 0; i < prm.size();) {
-    const size_t q = std::min(prm.size() - i, (size_t)1 << ds.ls_lanes);
+    const size_t q = std::min(prm.size() - i, (size_t)1 << ls_call);
     int ls = 0;
     while (fill ? ((size_t)1 << ls) < q : ((size_t)2 << ls) <= q) ++ls;
     runs.push_back({lanes.size(), ls});
@@ -1349,6 +1426,7 @@ static void kernels_changed(Plan& p, DeviceState& ds) {
   drop_graphs(ds);
   setup_hoisted(p, ds);
   build_sets(p, ds);
+  set_lane_times(p, ds);
   ds.forget_prologues();   // the arena may have been overwritten: they run again
 }
 
@@ -1612,36 +1690,14 @@ extern "C" tn_status tn_plan_select_list(const tn_network_t* net, const tn_plan_
   API_END
 }
 
-// Kernels launch_class launches for the steps of a class (memsets not counted).
-template <class Pred>
-static int class_launches(const Plan& p, Pred in_class) {
-  int n = 0;
-  auto kernels_of = [&](int i) {
-    const StepLaunch& L = p.dev->launches[i];
-    return is_tc(L.kid) ? (L.tc.n_split > 1 ? 3 : 2) - (L.bimg_own ? 1 : 0) : 1;
-  };
-  for (size_t i = 0; i < p.steps.size(); ++i) {
-    if (!in_class(p.steps[i].dep_flags)) continue;
-    const LaunchSet& st = p.dev->set[0];
-    const int gi = st.group_at.empty() ? -1 : st.group_at[i];
-    if (gi < 0) {
-      n += kernels_of((int)i);
-      continue;
-    }
-    const GroupRun& gr = st.groups[gi];
-    n += (int)gr.multi.size();
-    for (int t : gr.singles) n += kernels_of(t);
-    i = (size_t)gr.end - 1;
-  }
-  return n;
-}
-
 extern "C" tn_status tn_plan_chunk_launches(const tn_plan_t* h, int32_t* launches) {
   API_BEGIN
   if (!h || !launches) fail(TN_ERR_ARG, "tn_plan_chunk_launches: NULL argument");
   const Plan& p = h->plan;
   if (!p.dev) fail(TN_ERR_ARG, "tn_plan_chunk_launches: call after the first tn_contract_slices");
-  *launches = 2 + class_launches(p, [](int f) { return (f & 1) != 0; });
+  int shared, alone;
+  class_launches(p, [](int f) { return (f & 1) != 0; }, &shared, &alone);
+  *launches = 2 + shared + alone;
   API_END
 }
 
@@ -1650,7 +1706,9 @@ extern "C" tn_status tn_plan_batch_launches(const tn_plan_t* h, int32_t* launche
   if (!h || !launches) fail(TN_ERR_ARG, "tn_plan_batch_launches: NULL argument");
   const Plan& p = h->plan;
   if (!p.dev) fail(TN_ERR_ARG, "tn_plan_batch_launches: call after the first tn_contract_slices");
-  int n = class_launches(p, [](int f) { return f == 2; });
+  int shared, alone;
+  class_launches(p, [](int f) { return f == 2; }, &shared, &alone);
+  int n = shared + alone;
   for (const StepLaunch& L : p.dev->launches) n += (L.bimg_own && L.bimg_cls == 2) ? 1 : 0;   // B' images
   *launches = n;   // on the leaf select of the batch's first chunk
   API_END

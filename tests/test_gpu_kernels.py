@@ -290,6 +290,64 @@ def test_lanes_with_tensor_core_steps(env, wide_plans, prec, cm):
     assert many.chunk_launches() == one.chunk_launches()
 
 
+def test_lanes_weigh_a_heavy_prologue(env):
+    """30 closed qubits beside 6 open ones of which alone wires are sliced: the
+    prologue of a batch (2^24.8 multiply-adds) outweighs its 16 chunks (2^11).
+    More lanes save launches but repeat the prologue, so a call of all chunks takes
+    no longer than the same chunks in two calls of half the lanes (329 us
+    against 231 with as many lanes as there is room for), and gives the same bits."""
+    import rqcgen
+    tn, torch = env
+    big, small = rqcgen.sycamore_style(5, 6, 14, 17, 0), rqcgen.sycamore_style(2, 3, 8, 18, 0)
+    n = big.n_qubits
+    circ = rqcgen.Circuit(n + 6, np.concatenate([big.gate_qubits, np.where(small.gate_qubits >= 0,
+                                                                           small.gate_qubits + n, -1)]),
+                          list(big.gate_matrices) + list(small.gate_matrices),
+                          np.concatenate([big.gate_layer, small.gate_layer]))
+    net = tn.Network(circ)
+    per = net.gates_per_qubit()
+    make = lambda **kw: tn.Plan(net, open_mask=63 << n, max_log2_intermediate=26, trials=8,
+                                forced_slices=[(n + j, per[n + j] - 2) for j in range(4)], **kw)
+    plan = make()
+    work = {0: 0.0, 1: 0.0, 2: 0.0}
+    for i, shape in enumerate(plan.step_shapes()):
+        f = plan.step_layout(i)["dep_flags"]
+        work[1 if f & 1 else f] += 2.0 ** sum(shape)
+    assert work[2] > 100 * work[1]
+    single = make(max_arena_bytes=plan.info()["arena_bytes"])   # room for one lane
+    rng = np.random.default_rng(4)
+    draw = lambda: [int(b) for b in rng.integers(0, 1 << n, size=1)]
+
+    def amplitudes(p, bits, parts):
+        out = torch.zeros(64, dtype=torch.complex128, device="cuda")
+        for lo in range(0, 16, 16 // parts):
+            p.contract_slices(lo, 16 // parts, bits, out)
+        return torch.view_as_real(out)
+
+    for _ in range(3):
+        bits = draw()
+        want = amplitudes(single, bits, 16)
+        assert float(want.abs().max()) > 0.0
+        for parts in (1, 2, 4):
+            assert torch.equal(amplitudes(plan, bits, parts), want)
+
+    def us(parts):
+        best = float("inf")
+        for _ in range(5):
+            torch.cuda.synchronize()
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(20):
+                amplitudes(plan, draw(), parts)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1) * 50)
+        return best
+
+    whole, halves = us(1), us(2)
+    assert whole < 1.15 * halves, (whole, halves)
+
+
 def test_later_calls_do_not_wait(env):
     """Only the first call of a plan synchronises: calls with other numbers of
     chunks return while earlier work of another stream still runs (half a second of
