@@ -325,9 +325,10 @@ tn_status tn_plan_set_tuning(tn_plan_t* plan, const int32_t* in, int32_t n);
  * slice time is smallest is kept, not the one with the fewest flops).  Builds
  * n_candidates plans from *opts with seeds seed, seed+1, ... and memory weights
  * cycling through w, w/4, 4w (w = opts->mem_weight or 32), times chunks of
- * each on `stream` (after an untimed warm-up call with the same bitstring, the
- * fastest of three timed calls of one chunk), estimates the time for all 2^S
- * slices as chunk time x 2^(S-b), and returns the fastest plan in *out (its
+ * each on `stream` (after untimed warm-up calls with the same bitstring, the
+ * fastest of three timed calls of one chunk, or of as many as the plan has
+ * arenas for, see tn_contract_slices), estimates the time for all 2^S slices
+ * from it in proportion, and returns the fastest plan in *out (its
  * device state is released; the first contract call re-creates it).
  * cand_seconds (HOST, [n_candidates], may be NULL) receives each estimate, -1
  * for a candidate that could not be built or run (e.g. its arena does not

@@ -1589,9 +1589,9 @@ extern "C" tn_status tn_plan_set_tuning(tn_plan_t* h, const int32_t* in, int32_t
   API_END
 }
 
-// Time one chunk of every candidate (seed and memory weight per candidate, the
-// rest from *opts) after an untimed warm-up chunk, and keep the plan whose
-// estimate for all 2^S slices is smallest.
+// Time a few chunks of every candidate (seed and memory weight per candidate, the
+// rest from *opts) after an untimed warm-up, and keep the plan whose estimate for
+// all 2^S slices is smallest.
 static void select_among(const tn_network_t* net, const tn_plan_opts* opts, int32_t n_candidates,
                          const uint64_t* seeds, const double* weights, uint64_t bitstring, void* stream,
                          tn_plan_t** out, double* cand_seconds) {
@@ -1621,14 +1621,16 @@ static void select_among(const tn_network_t* net, const tn_plan_opts* opts, int3
       amps_bytes = need;
     }
     double est = -1.0;
-    // warm-up (device state, prologues, graph capture), then the fastest of
-    // three timed chunks
+    // warm-up (device state, prologues, graph capture), then the fastest of three
+    // timed calls of as many chunks as the plan runs side by side
     if (tn_contract_slices(h, 0, chunk, &bitstring, 1, amps, s) == TN_OK) {
+      const int log2_timed = std::min((int)p.sliced.size(), p.log2_batch + p.dev->ls_lanes);
+      const uint64_t timed = 1ULL << log2_timed;
       float best_ms = -1.f;
-      tn_status st = TN_OK;
+      tn_status st = timed > chunk ? tn_contract_slices(h, 0, timed, &bitstring, 1, amps, s) : TN_OK;
       for (int r = 0; r < 3 && st == TN_OK; ++r) {
         CK(cudaEventRecord(e0, s));
-        st = tn_contract_slices(h, 0, chunk, &bitstring, 1, amps, s);
+        st = tn_contract_slices(h, 0, timed, &bitstring, 1, amps, s);
         CK(cudaEventRecord(e1, s));
         CK(cudaEventSynchronize(e1));
         float ms = 0.f;
@@ -1636,7 +1638,7 @@ static void select_among(const tn_network_t* net, const tn_plan_opts* opts, int3
         if (best_ms < 0.f || ms < best_ms) best_ms = ms;
       }
       if (st == TN_OK && tn_plan_sync(h, s) == TN_OK)
-        est = (double)best_ms / 1e3 * std::ldexp(1.0, (int)p.sliced.size() - p.log2_batch);
+        est = (double)best_ms / 1e3 * std::ldexp(1.0, (int)p.sliced.size() - log2_timed);
     }
     CK(cudaStreamSynchronize(s));
     destroy_device_state(&p);

@@ -375,3 +375,27 @@ def test_later_calls_do_not_wait(env):
     side.synchronize()
     torch.cuda.synchronize()
     assert e0.elapsed_time(e1) > 400.0 and host < 0.2
+
+
+def test_selection_estimates_calls_of_many_chunks(env):
+    """A candidate's estimate for all slices is what the chosen plan then takes: a
+    plan of small chunks runs several side by side, and is timed so."""
+    import rqcgen
+    tn, torch = env
+    circ = rqcgen.sycamore_style(4, 4, 9, 7, 0)
+    om = 0b1111110000000000
+    plan, est = tn.select_plan(tn.Network(circ), 3, 5, open_mask=om, max_log2_intermediate=30, min_log2_slices=5,
+                               trials=8, log2_batch_slices=1)
+    info = plan.info()
+    assert info["log2_slices"] - info["log2_batch_slices"] >= 4
+    out = torch.zeros(1 << 6, dtype=torch.complex128, device="cuda")
+    best = float("inf")
+    for _ in range(20):
+        torch.cuda.synchronize()
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        plan.contract_slices(0, 1 << info["log2_slices"], [5], out)
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, e0.elapsed_time(e1) * 1e-3)
+    assert best / 2.5 < min(est) < 2.5 * best, (est, best)
