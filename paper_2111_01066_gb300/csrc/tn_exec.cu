@@ -1002,16 +1002,7 @@ static int lanes_of(const Plan& p) {
   return ls;
 }
 
-static void ensure_device(Plan& p) {
-  int dev = 0;
-  CK(cudaGetDevice(&dev));
-  if (p.dev) {
-    if (p.dev->device != dev) fail(TN_ERR_ARG, "plan was first used on another device");
-    return;
-  }
-  auto* ds = new DeviceState;
-  p.dev = ds;
-  ds->device = dev;
+static void build_device_state(Plan& p, DeviceState* ds) {
   const size_t ab = std::max<size_t>(256, (size_t)p.arena_elems * sizeof(float2));
   ds->ls_lanes = lanes_of(p);
   if (ds->ls_lanes > 0) {   // several arenas; where they cannot be had, one
@@ -1100,6 +1091,25 @@ static void ensure_device(Plan& p) {
   set_lane_times(p, *ds);
 }
 
+// The plan's device state, built by its first call; one that could not be built whole
+// is taken down again, so that a later call starts anew.
+static void ensure_device(Plan& p) {
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  if (p.dev) {
+    if (p.dev->device != dev) fail(TN_ERR_ARG, "plan was first used on another device");
+    return;
+  }
+  p.dev = new DeviceState;
+  p.dev->device = dev;
+  try {
+    build_device_state(p, p.dev);
+  } catch (...) {
+    destroy_device_state(&p);
+    throw;
+  }
+}
+
 static void drop_graphs(DeviceState& ds) {
   for (LaunchSet& st : ds.set)
     for (int w = 0; w < 2; ++w) {
@@ -1133,6 +1143,27 @@ void destroy_device_state(Plan* p) {
   cudaSetDevice(cur);
   delete ds;
   p->dev = nullptr;
+}
+
+// A workspace of at least `bytes` (synchronises the device).  Where it cannot be had
+// the old one is, or else the plan starts anew with its next call; fails either way.
+static void grow_workspace(Plan& p, int64_t bytes, const char* who) {
+  DeviceState& ds = *p.dev;
+  if (bytes <= ds.ws_bytes) return;
+  drop_graphs(ds);   // captured with the old workspace's address
+  CK(cudaFree(ds.ws));
+  ds.ws = nullptr;
+  if (cudaMalloc(&ds.ws, (size_t)bytes) == cudaSuccess) {
+    ds.ws_bytes = bytes;
+    return;
+  }
+  cudaGetLastError();
+  ds.ws = nullptr;
+  if (cudaMalloc(&ds.ws, (size_t)ds.ws_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    destroy_device_state(&p);
+  }
+  fail(TN_ERR_OOM, std::string(who) + ": workspace allocation of " + std::to_string(bytes) + " bytes failed");
 }
 
 // The steps whose dependence flags satisfy `in_class`, in plan order; a group
@@ -1421,11 +1452,17 @@ extern "C" tn_status tn_plan_step_times(tn_plan_t* h, int32_t reps, double* ms_o
   API_END
 }
 
-// After the kernels of a plan changed: group runs, chunk graph and prologues anew.
+// After the kernels of a plan changed: launch sets, graphs and prologues anew (a plan
+// whose sets cannot be built starts anew with its next call).
 static void kernels_changed(Plan& p, DeviceState& ds) {
   drop_graphs(ds);
-  setup_hoisted(p, ds);
-  build_sets(p, ds);
+  try {
+    setup_hoisted(p, ds);
+    build_sets(p, ds);
+  } catch (...) {
+    destroy_device_state(&p);
+    throw;
+  }
   set_lane_times(p, ds);
   ds.forget_prologues();   // the arena may have been overwritten: they run again
 }
@@ -1452,14 +1489,7 @@ extern "C" tn_status tn_plan_autotune(tn_plan_t* h, int32_t reps, void* stream) 
   auto time_launch = [&](StepLaunch& L) -> double {
     if (L.ws_bytes > ds.ws_bytes) {
       CK(cudaStreamSynchronize(s));
-      CK(cudaFree(ds.ws));
-      ds.ws = nullptr;
-      ds.ws_bytes = 0;
-      if (cudaMalloc(&ds.ws, (size_t)L.ws_bytes) != cudaSuccess) {
-        cudaGetLastError();
-        fail(TN_ERR_OOM, "autotune workspace allocation failed");
-      }
-      ds.ws_bytes = L.ws_bytes;
+      grow_workspace(p, L.ws_bytes, "tn_plan_autotune");
     }
     launch_step(L, ds.ws, ds.err, s, true);  // warm-up
     CK(cudaEventRecord(e0, s));
@@ -1574,16 +1604,7 @@ extern "C" tn_status tn_plan_set_tuning(tn_plan_t* h, const int32_t* in, int32_t
     }
     ws = std::max(ws, next[i].ws_bytes);
   }
-  if (ws > ds.ws_bytes) {   // a larger workspace (synchronises the device through cudaFree)
-    CK(cudaFree(ds.ws));
-    ds.ws = nullptr;
-    ds.ws_bytes = 0;
-    if (cudaMalloc(&ds.ws, (size_t)ws) != cudaSuccess) {
-      cudaGetLastError();
-      fail(TN_ERR_OOM, "tn_plan_set_tuning: workspace allocation failed");
-    }
-    ds.ws_bytes = ws;
-  }
+  grow_workspace(p, ws, "tn_plan_set_tuning");
   ds.launches.swap(next);
   kernels_changed(p, ds);
   API_END

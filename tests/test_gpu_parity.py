@@ -196,6 +196,25 @@ def test_c1_range_errors(env):
     assert float(out.abs().max()) == 0.0
 
 
+def test_arena_beyond_the_memory_is_refused_every_time(env):
+    """A plan whose arena no allocation can hold (53 qubits in four slices, 689 GiB)
+    is refused by its first call and by the next ones alike: no call runs on a
+    device state that could not be built whole."""
+    tn, torch = env
+    circ = rqcgen.sycamore_style(6, 9, 20, 5, 1)
+    n = circ.n_qubits
+    plan = tn.Plan(tn.Network(circ), open_mask=63 << (n - 6), max_log2_intermediate=34, trials=8,
+                   max_arena_bytes=1 << 45)
+    assert plan.info()["arena_bytes"] > torch.cuda.get_device_properties(0).total_memory
+    out = torch.zeros(1 << 6, dtype=torch.complex128, device="cuda")
+    for _ in range(3):
+        with pytest.raises(tn.TnError) as e:
+            plan.contract_slices(0, 1, [0], out)
+        assert e.value.status == tn.TN_ERR_OOM
+    torch.cuda.synchronize()
+    assert float(torch.view_as_real(out).abs().max()) == 0.0
+
+
 @pytest.mark.parametrize("prec,cm", [("fp32", 4), ("tf32", 4), ("bf16x3", 4), ("tf32", 3), ("bf16x3", 3),
                                      ("fp16x3", 4), ("fp16x3", 3)])
 def test_c2_against_golden(env, prec, cm):
