@@ -192,17 +192,67 @@ def test_tensor_core_tiles_at_their_edges(env, shape, batch, layout, misaligned,
     (a, a_w, b, b_w, c_w), dev = _pair_case(torch, shape, batch, layout, sum(shape) * 10 + batch, misaligned)
     tn.contract_pair(*dev, batch=batch, precision=prec, complex_mult=cm)
     tn.device_sync()
+    fp32 = torch.empty_like(dev[4])
+    tn.contract_pair(*dev[:4], fp32, dev[5], batch=batch)   # on the tensor cores: not the bits of the FP32 call
+    assert not torch.equal(torch.view_as_real(dev[4]), torch.view_as_real(fp32))
     got = dev[4].cpu().numpy()
     for i in {0, batch - 1}:
         want = pairwise.contract_pair(a[i].astype(np.complex128), a_w, b[i].astype(np.complex128), b_w, c_w)
         assert np.linalg.norm(got[i] - want) <= PAIR_REL[prec, cm] * np.linalg.norm(want)
 
 
-@pytest.mark.parametrize("prec,slices,chunk", [("fp32", 0, 0), ("fp32", 5, 2), ("bf16x3", 4, 0), ("fp16x3", 4, 1)])
+@pytest.mark.parametrize("misaligned", [False, True])
+@pytest.mark.parametrize("layout", ["kfast", "random"])
+@pytest.mark.parametrize("shape,batch", [((18, 7, 0), 1), ((17, 7, 1), 1), ((16, 7, 2), 1), ((14, 3, 2), 70), ((15, 10, 1), 3),
+                                         ((4, 9, 0), 4100)])
+@pytest.mark.parametrize("prec,cm", sorted(PAIR_REL))
+def test_tensor_core_padded_columns(env, prec, cm, shape, batch, layout, misaligned):
+    """Fewer columns than the narrowest tile has (8, or 16 with 3M): the images'
+    other columns are zero and no result of theirs is stored.  Against 64 bits,
+    and on the tensor cores: not the bits of the FP32 call."""
+    tn, torch = env
+    nm, nk, nn = shape
+    g = torch.Generator(device="cuda").manual_seed(sum(shape))
+    rng = np.random.default_rng(sum(shape))
+    w = list(range(nm + nk + nn))
+    m, k, n = w[:nm], w[nm:nm + nk], w[nm + nk:]
+    a_w, b_w, c_w = (k + m, k + n, m + n) if layout == "kfast" else \
+        tuple([int(x) for x in rng.permutation(v)] for v in (m + k, k + n, m + n))
+    pad = 1 if misaligned else 0
+
+    def draw(r):
+        t = torch.randn((batch << r) + pad, generator=g, dtype=torch.complex64, device="cuda")
+        return t[pad:].view(batch, 1 << r)
+
+    def ordered(x, have, want):
+        at = torch.zeros(1, dtype=torch.int64, device="cuda")
+        for q in want:
+            at = torch.cat([at, at + (1 << have.index(q))])
+        return x[:, at]
+
+    a, b = draw(nm + nk), draw(nk + nn)
+    buf = torch.full(((batch << (nm + nn)) + 2,), 7.0, dtype=torch.complex64, device="cuda")
+    c = buf[pad:pad + (batch << (nm + nn))].view(batch, -1)
+    tn.contract_pair(a, a_w, b, b_w, c, c_w, batch=batch, precision=prec, complex_mult=cm)
+    tn.device_sync()
+    x = ordered(a, a_w, k + m).view(batch, 1 << nm, 1 << nk).to(torch.complex128)
+    y = ordered(b, b_w, k + n).view(batch, 1 << nn, 1 << nk).to(torch.complex128)
+    want = ordered(torch.bmm(y, x.transpose(1, 2)).reshape(batch, -1), m + n, c_w)
+    assert float((c.to(torch.complex128) - want).norm() / want.norm()) <= PAIR_REL[prec, cm]
+    assert torch.all(buf[:pad] == 7.0) and torch.all(buf[pad + (batch << (nm + nn)):] == 7.0)
+    fp32 = torch.empty_like(c)
+    tn.contract_pair(a, a_w, b, b_w, fp32, c_w, batch=batch)
+    assert not torch.equal(torch.view_as_real(c), torch.view_as_real(fp32))
+
+
+@pytest.mark.parametrize("prec,slices,chunk", [("fp32", 0, 0), ("fp32", 5, 2), ("tf32", 4, 2), ("bf16x3", 4, 0),
+                                               ("fp16x3", 4, 1)])
 def test_chunks_side_by_side(env, prec, slices, chunk):
     """Chunks of one call run side by side, 16 at most, filled up to a power of
-    two: any number of batches, in one call or one by one, whole or in ragged slice
-    ranges, gives the same bits, and the state vector's amplitudes."""
+    two: any number of batches, whole or in ragged slice ranges, gives the bits of
+    a plan with room for one lane that gets one chunk a call, and the state
+    vector's amplitudes; with the CUDA-core steps that these sizes have, then
+    with tensor-core kernels wherever they can run."""
     import rqcgen
     from oracle import statevector as sv
     tn, torch = env
@@ -210,29 +260,41 @@ def test_chunks_side_by_side(env, prec, slices, chunk):
     om = 0b1111110000000000
     psi = sv.simulate(circ)
     net = tn.Network(circ)
-    make = lambda: tn.Plan(net, open_mask=om, max_log2_intermediate=30, min_log2_slices=slices, trials=8,
-                           log2_batch_slices=chunk, precision=prec)
-    n = 1 << make().info()["log2_slices"]
-    rng = np.random.default_rng(3)
+    make = lambda arena=0: tn.Plan(net, open_mask=om, max_log2_intermediate=30, min_log2_slices=slices, trials=8,
+                                   log2_batch_slices=chunk, precision=prec, max_arena_bytes=arena)
     plan = make()
-    for count in (1, 3, 2, 17, 16, 5):
-        bits = [int(b) for b in rng.integers(0, 1 << 10, size=count)]
-        out = torch.zeros(count << 6, dtype=torch.complex128, device="cuda")
-        cuts = sorted({0, n // 3, n})
-        for a, b in zip(cuts, cuts[1:]):
-            plan.contract_slices(a, b - a, bits, out)
-        plan.sync()
-        alone = torch.zeros_like(out)
-        single = make()
-        for i, b in enumerate(bits):
+    single = make(plan.info()["arena_bytes"])
+    assert single.step_shapes() == plan.step_shapes()
+    n, per = 1 << plan.info()["log2_slices"], 1 << plan.info()["log2_batch_slices"]
+    rng = np.random.default_rng(3)
+    for tensor_cores in ([False, True] if prec != "fp32" else [False]):
+        if tensor_cores:
+            kid = {v: k for k, v in tn.Plan.KERNELS.items()}["tc_" + prec]
+            forced = [(kid, -1, 0, 0, 1) if shape[0] >= 4 else t
+                      for t, shape in zip(plan.get_tuning(), plan.step_shapes())]
+            for p in (plan, single):
+                p.set_tuning(forced)
+            assert sum(t[0] == kid for t in plan.get_tuning()) >= 3
+        for count in (1, 3, 2, 17, 16, 5):
+            bits = [int(b) for b in rng.integers(0, 1 << 10, size=count)]
+            out = torch.zeros(count << 6, dtype=torch.complex128, device="cuda")
+            alone = torch.zeros_like(out)
+            cuts = sorted({0, n // 3, n})
             for lo, hi in zip(cuts, cuts[1:]):
-                single.contract_slices(lo, hi - lo, [b], alone[i << 6:(i + 1) << 6])
-        single.sync()
-        want = np.concatenate([sv.batch_amplitudes(psi, circ.n_qubits, b, om) for b in bits])
-        got = out.cpu().numpy()
-        assert np.linalg.norm(got - want) < (1e-5 if prec == "fp32" else 1e-4) * np.linalg.norm(want)
-        if n // 3 == 0 or chunk == 0:   # one chunk per range: also the same bits
-            assert torch.equal(torch.view_as_real(out), torch.view_as_real(alone))
+                plan.contract_slices(lo, hi - lo, bits, out)
+                for i, b in enumerate(bits):
+                    at = lo
+                    while at < hi:
+                        end = min(hi, (at // per + 1) * per)
+                        single.contract_slices(at, end - at, [b], alone[i << 6:(i + 1) << 6])
+                        at = end
+            plan.sync()
+            single.sync()
+            want = np.concatenate([sv.batch_amplitudes(psi, circ.n_qubits, b, om) for b in bits])
+            got = out.cpu().numpy()
+            tol = {"fp32": 1e-5, "tf32": 2e-2 if tensor_cores else 1e-5}.get(prec, 1e-4)
+            assert np.linalg.norm(got - want) < tol * np.linalg.norm(want)
+            assert torch.equal(torch.view_as_real(out), torch.view_as_real(alone)), (count, tensor_cores)
 
 
 @pytest.fixture(scope="module")

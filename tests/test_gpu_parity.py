@@ -226,6 +226,18 @@ def test_c2_against_golden(env, prec, cm):
     n_sl = 1 << plan.info()["log2_slices"]
     got = _run_plan(tn, torch, plan, 0, n_sl, [cb], 10)
     _check_plan(got, want, circ.n_qubits, prec, f"c2 {prec} {cm}M")
+    if prec == "fp32":
+        return
+    # its steps are small enough for the CUDA cores: the tensor-core kernel put on
+    # the larger ones, from 2^20 multiply-adds on
+    kid = {v: k for k, v in tn.Plan.KERNELS.items()}["tc_" + prec + ("_3m" if cm == 3 else "")]
+    forced = [(kid, -1, 0, 0, int(cm == 4)) if shape[0] >= 4 and sum(shape) >= 20 else t
+              for t, shape in zip(plan.get_tuning(), plan.step_shapes())]
+    plan.set_tuning(forced)
+    assert sum(t[0] == kid for t in plan.get_tuning()) >= 6
+    for _ in range(2):
+        got = _run_plan(tn, torch, plan, 0, n_sl, [cb], 10)
+        _check_plan(got, want, circ.n_qubits, prec, f"c2 {prec} {cm}M, tensor cores")
 
 
 def _pool_candidates(name):
@@ -448,10 +460,18 @@ SHAPES = [  # (m bits, k bits, n bits): several tiles, ragged (smaller than a ti
 ]
 
 
-TC_SHAPES = [  # big enough for the tensor-core kernel (m >= 4 bits, >= 2^20 multiply-adds)
-    (10, 4, 6), (12, 5, 3), (8, 8, 8), (7, 13, 2), (14, 2, 4), (9, 6, 7), (16, 3, 1),
+TC_SHAPES = [  # big enough for the tensor-core kernels (m >= 4 bits, >= 2^25 multiply-adds)
+    (12, 5, 8), (13, 9, 3), (8, 9, 8), (8, 15, 2), (15, 6, 4), (10, 8, 7), (13, 6, 6),
     (8, 14, 5), (9, 13, 3), (7, 12, 8),   # few output tiles, long k: split-K
 ]
+
+
+def _on_tensor_cores(tn, torch, got, ta, a_w, tb, b_w, c_w, batch):
+    """Whether a result came from the tensor cores: the CUDA cores form the same
+    FP32 products in every precision, so theirs is the FP32 call's bit for bit."""
+    fp32 = torch.empty_like(got)
+    tn.contract_pair(ta, a_w, tb, b_w, fp32, c_w, batch=batch, precision="fp32")
+    return not torch.equal(torch.view_as_real(got), torch.view_as_real(fp32))
 
 
 @pytest.mark.parametrize("prec", ["fp32", "tf32", "bf16x3", "fp16x3"])
@@ -473,6 +493,7 @@ def test_contract_pair(env, shape, batch, prec):
     tc = torch.empty((batch, 2 ** len(c_w)), dtype=torch.complex64, device="cuda")
     tn.contract_pair(ta, a_w, tb, b_w, tc, c_w, batch=batch, precision=prec)
     tn.device_sync()     # synchronises; raises if a bounded device wait ran out
+    assert prec == "fp32" or shape in SHAPES or _on_tensor_cores(tn, torch, tc, ta, a_w, tb, b_w, c_w, batch)
     got = tc.cpu().numpy()
     for i in range(batch):
         want = pairwise.contract_pair(a[i], a_w, b[i], b_w, c_w)
@@ -490,7 +511,8 @@ PAIR_TOL_3M = {"tf32": 6e-3, "bf16x3": 1e-4, "fp16x3": 4e-5}   # 3M: Im = T3 - T
 def test_contract_pair_3m(env, shape, layout, batch, prec):
     """3M products (T1 = ArBr, T2 = AiBi, T3 = (Ar+Ai)(Br+Bi); Re = T1 - T2,
     Im = T3 - T1 - T2) on the tensor cores, A gathered (random storage order)
-    or fetched by TMA ([k..., m...] order), against the FP64 contraction."""
+    or fetched by TMA ([k..., m...] order), against the FP64 contraction; three
+    smaller ones, which the CUDA cores run as 4M."""
     tn, torch = env
     nm, nk, nn = shape
     rng = np.random.default_rng(zlib.crc32(repr((shape, layout)).encode()) % 1000 + batch)
@@ -508,6 +530,7 @@ def test_contract_pair_3m(env, shape, layout, batch, prec):
     tc = torch.empty((batch, 2 ** len(c_w)), dtype=torch.complex64, device="cuda")
     tn.contract_pair(ta, a_w, tb, b_w, tc, c_w, batch=batch, precision=prec, complex_mult=3)
     torch.cuda.synchronize()
+    assert shape not in TC_SHAPES or _on_tensor_cores(tn, torch, tc, ta, a_w, tb, b_w, c_w, batch)
     got = tc.cpu().numpy()
     for i in range(batch):
         want = pairwise.contract_pair(a[i], a_w, b[i], b_w, c_w)
@@ -548,7 +571,7 @@ def test_contract_pair_converted_a_many_inputs(env, prec, cm):
 
 @pytest.mark.parametrize("cm", [4, 3])
 @pytest.mark.parametrize("mag", [2.0 ** -20, 2.0 ** -40, 2.0 ** 20])
-@pytest.mark.parametrize("shape", [(12, 5, 3), (9, 6, 7), (8, 14, 5)])
+@pytest.mark.parametrize("shape", [(12, 8, 5), (9, 9, 7), (8, 14, 5)])
 def test_contract_pair_fp16x3_scaling(env, shape, mag, cm):
     """FP16 hi/lo operands cover magnitudes far outside the FP16 range because
     each operand is scaled by a power of two before the split and the product
@@ -567,8 +590,10 @@ def test_contract_pair_fp16x3_scaling(env, shape, mag, cm):
     def run(x, y):
         dev = lambda t: torch.from_numpy(np.ascontiguousarray(t)).cuda()
         tc = torch.empty(2 ** len(c_w), dtype=torch.complex64, device="cuda")
-        tn.contract_pair(dev(x), a_w, dev(y), b_w, tc, c_w, precision="fp16x3", complex_mult=cm)
+        tx, ty = dev(x), dev(y)
+        tn.contract_pair(tx, a_w, ty, b_w, tc, c_w, precision="fp16x3", complex_mult=cm)
         torch.cuda.synchronize()
+        assert _on_tensor_cores(tn, torch, tc, tx, a_w, ty, b_w, c_w, 1)
         return tc.cpu().numpy()
 
     base = run(a, b)
@@ -579,11 +604,11 @@ def test_contract_pair_fp16x3_scaling(env, shape, mag, cm):
 
 
 @pytest.mark.parametrize("prec", ["tf32", "bf16x3", "fp16x3"])
-@pytest.mark.parametrize("shape", [(8, 4, 3, 1), (10, 4, 6, 3), (12, 5, 7, 1), (8, 8, 8, 2), (9, 13, 3, 1),
-                                   (8, 14, 5, 3), (11, 6, 2, 1)])
+@pytest.mark.parametrize("shape", [(8, 14, 3, 1), (10, 7, 8, 3), (12, 7, 7, 1), (8, 9, 8, 2), (9, 13, 3, 1),
+                                   (8, 14, 5, 3), (11, 12, 2, 1), (12, 5, 10, 1)])
 def test_contract_pair_sm_pairs_a_by_tma(env, shape, prec):
-    """4M products with two or more full 128-row m tiles run on SM pairs; here
-    with A stored [k, m] (fetched by tensor-map loads, then split in shared
+    """4M products with two or more full 128-row m tiles and more than 64 k or 256
+    columns run on SM pairs; here with A stored [k, m] (fetched by tensor-map loads, then split in shared
     memory) and C in a random order: one pair, several pairs, batched
     instances, 8- to 128-column tiles, split-K over a long k."""
     tn, torch = env
@@ -596,8 +621,10 @@ def test_contract_pair_sm_pairs_a_by_tma(env, shape, prec):
     b = (rng.normal(size=(batch, 2 ** len(b_w))) + 1j * rng.normal(size=(batch, 2 ** len(b_w)))) / 2
     dev = lambda x: torch.from_numpy(np.ascontiguousarray(x.astype(np.complex64))).cuda()
     tc = torch.empty((batch, 2 ** len(c_w)), dtype=torch.complex64, device="cuda")
-    tn.contract_pair(dev(a), a_w, dev(b), b_w, tc, c_w, batch=batch, precision=prec)
+    ta, tb = dev(a), dev(b)
+    tn.contract_pair(ta, a_w, tb, b_w, tc, c_w, batch=batch, precision=prec)
     tn.device_sync()
+    assert _on_tensor_cores(tn, torch, tc, ta, a_w, tb, b_w, c_w, batch)
     got = tc.cpu().numpy()
     for i in range(batch):
         want = pairwise.contract_pair(a[i], a_w, b[i], b_w, c_w)
@@ -606,7 +633,7 @@ def test_contract_pair_sm_pairs_a_by_tma(env, shape, prec):
 
 
 @pytest.mark.parametrize("prec", ["tf32", "bf16x3", "fp16x3"])
-@pytest.mark.parametrize("shape", [(3, 12, 3, 64), (4, 10, 6, 16), (5, 8, 7, 8), (6, 15, 3, 32), (6, 9, 9, 4)])
+@pytest.mark.parametrize("shape", [(4, 12, 3, 64), (4, 10, 6, 35), (5, 8, 7, 37), (6, 15, 3, 32), (6, 9, 9, 4)])
 def test_contract_pair_short_tiles_by_tma(env, shape, prec):
     """A stored [k, m] with fewer than 128 rows per instance: tensor-map tiles
     of 2^m rows (the rest of the 128-row MMA tile is dropped), batched."""
@@ -620,8 +647,10 @@ def test_contract_pair_short_tiles_by_tma(env, shape, prec):
     b = (rng.normal(size=(batch, 2 ** len(b_w))) + 1j * rng.normal(size=(batch, 2 ** len(b_w)))) / 2
     dev = lambda x: torch.from_numpy(np.ascontiguousarray(x.astype(np.complex64))).cuda()
     tc = torch.empty((batch, 2 ** len(c_w)), dtype=torch.complex64, device="cuda")
-    tn.contract_pair(dev(a), a_w, dev(b), b_w, tc, c_w, batch=batch, precision=prec)
+    ta, tb = dev(a), dev(b)
+    tn.contract_pair(ta, a_w, tb, b_w, tc, c_w, batch=batch, precision=prec)
     torch.cuda.synchronize()
+    assert _on_tensor_cores(tn, torch, tc, ta, a_w, tb, b_w, c_w, batch)
     got = tc.cpu().numpy()
     for i in range(batch):
         want = pairwise.contract_pair(a[i], a_w, b[i], b_w, c_w)
