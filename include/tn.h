@@ -280,8 +280,8 @@ tn_status tn_contract_slices(tn_plan_t* plan, uint64_t slice_first, uint64_t sli
  * and, when kernel_out is not NULL, the kernel used by each step into
  * kernel_out[n_steps]: 0-2 FP32 SIMT tiles (64x64, 128x16, 256x4), then the
  * tcgen05 kernels 3 TF32 4M, 4 BF16x3 4M, 5 TF32 3M, 6 BF16x3 3M, 7 FP16x3 4M,
- * 8 FP16x3 3M, then 9-10 further FP32 SIMT tiles (128x64, 32x32).  Used for plan reports and roofline measurements; synchronises
- * `stream`. */
+ * 8 FP16x3 3M, then 9-10 further FP32 SIMT tiles (128x64, 32x32).  Used for
+ * plan reports and roofline measurements; synchronises `stream`. */
 tn_status tn_plan_step_times(tn_plan_t* plan, int32_t reps, double* ms_out, int32_t* kernel_out,
                              void* stream);
 
@@ -367,15 +367,18 @@ tn_status tn_plan_rank(const tn_network_t* net, const tn_plan_opts* opts, int32_
  * tn_contract_slices call; TN_ERR_ARG before): leaf select, every
  * slice-dependent step's kernels (tensor-core steps: B' image + GEMM [+ split-K
  * reduction]; CUDA-core steps: one) and the slice sum.  Steps that depend on no
- * slice run once per plan or per batch and are not counted.  Host only. */
+ * slice run once per plan or per batch and are not counted.  Chunks that run
+ * side by side (tn_contract_slices) share these launches, but for the kernels
+ * of tensor-core steps, which each chunk launches.  Host only. */
 tn_status tn_plan_chunk_launches(const tn_plan_t* plan, int32_t* launches);
 
 /* Kernels the per-batch prologue launches (after the first tn_contract_slices
  * call; TN_ERR_ARG before): the steps that depend on the closed output bits
  * but on no slice run once for every new batch bitstring (main text, section
  * III: the part of the network shared by a batch's slices is contracted once),
- * each with its kernels as in tn_plan_chunk_launches, on the leaf select of
- * the batch's first chunk; 0 when the plan has no such step.  Host only. */
+ * each with its kernels as in tn_plan_chunk_launches (and shared by chunks
+ * side by side as there), on the leaf select of the batch's first chunk; 0 when
+ * the plan has no such step.  Host only. */
 tn_status tn_plan_batch_launches(const tn_plan_t* plan, int32_t* launches);
 
 /* Wait for the plan's work on `stream` and return its sticky device error, if any. */

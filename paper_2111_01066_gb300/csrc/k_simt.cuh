@@ -52,21 +52,20 @@ constexpr int SIMT_MAX_SPLIT = 8;   // CTAs of one split-K cluster (the portable
 
 // A tiling: TM x TN outputs per CTA, TK of k per stage, RM x RN outputs per
 // thread, KG groups of threads that each take 1/KG of a stage's k (their sums
-// are added at the end), MINB CTAs per SM that the registers are kept to, NST
-// stages, filled by asynchronous copies NST - 1 chunks ahead or (REGS) through
-// registers one chunk ahead.  Copies need no registers, which the small tilings'
+// are added at the end), MINB CTAs per SM that the registers are kept to, two
+// stages, filled one chunk ahead by asynchronous copies or (REGS) through registers.  Copies need no registers, which the small tilings'
 // short loops want; they move 4 bytes at a time (the two planes of A), twice the L1
 // requests of the register path's 16-byte loads, which is faster where a loop is
 // long (2^17 x 256 x 256: 1198 us against 1310 with 128x64).  A is staged as two planes
 // (re, im) whose consecutive rows make the packed pairs.
-template <int TM_, int TN_, int TK_, int RM_, int RN_, int KG_, int MINB_, int NST_, bool REGS_>
+template <int TM_, int TN_, int TK_, int RM_, int RN_, int KG_, int MINB_, bool REGS_>
 struct SimtCfg {
   static constexpr int TM = TM_, TN = TN_, TK = TK_, RM = RM_, RN = RN_, KG = KG_, MINB = MINB_;
-  static constexpr int NST = NST_;
   static constexpr bool REGS = REGS_;
   static constexpr int NTX = TM / RM, NTY = TN / RN;
   static_assert(NTX * NTY * KG == SIMT_THREADS, "one thread per RM x RN outputs and k group");
-  static constexpr int RG = RM < 4 ? RM : 4;           // consecutive rows of a thread
+  static constexpr int RG = 4;                         // consecutive rows of a thread
+  static_assert(RM % RG == 0, "whole runs of rows");
   static constexpr int AS = TM + 4;                    // plane row stride: k-fastest stores stay conflict-free
   static constexpr bool SPLIT = KG > 1;                // partial tiles: k groups, and CTAs of a split-K cluster
   struct Stage {
@@ -78,7 +77,7 @@ struct SimtCfg {
 template <class Cfg>
 struct SimtSmem {
   union alignas(16) {
-    typename Cfg::Stage st[Cfg::NST];
+    typename Cfg::Stage st[2];
     // partial tiles of the k groups (column-major); the first one then takes their sum
     float2 part[Cfg::SPLIT ? Cfg::KG : 1][Cfg::SPLIT ? Cfg::TN : 1][Cfg::SPLIT ? Cfg::TM + 2 : 1];
   };
@@ -90,11 +89,11 @@ struct SimtSmem {
   int64_t kdB[KMAXR];
 };
 
-using SimtBig = SimtCfg<128, 64, 8, 8, 4, 1, 2, 2, true>;
-using Simt64 = SimtCfg<64, 64, 8, 4, 4, 1, 3, 2, true>;
-using Simt128x16 = SimtCfg<128, 16, 16, 4, 2, 1, 3, 2, false>;
-using Simt256x4 = SimtCfg<256, 4, 8, 4, 1, 1, 4, 2, false>;
-using Simt32 = SimtCfg<32, 32, 32, 4, 4, 4, 2, 2, false>;
+using SimtBig = SimtCfg<128, 64, 8, 8, 4, 1, 2, true>;
+using Simt64 = SimtCfg<64, 64, 8, 4, 4, 1, 3, true>;
+using Simt128x16 = SimtCfg<128, 16, 16, 4, 2, 1, 3, false>;
+using Simt256x4 = SimtCfg<256, 4, 8, 4, 1, 1, 4, false>;
+using Simt32 = SimtCfg<32, 32, 32, 4, 4, 4, 2, false>;
 
 // One thread's pairs of tile elements (2p, 2p + 1) of an operand: the elements
 // of a tile are numbered by the tile bits in ascending memory position, so
@@ -283,17 +282,12 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
 #pragma unroll
       for (int gq = 0; gq < RM / RG; ++gq) {
         const int r0 = (gq * NTX + tx) * RG;
-        if constexpr (RG == 4) {
-          const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(&st.ar[kk][r0]);
-          const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(&st.ai[kk][r0]);
-          ar[2 * gq] = x.x;
-          ar[2 * gq + 1] = x.y;
-          ai[2 * gq] = y.x;
-          ai[2 * gq + 1] = y.y;
-        } else {
-          ar[gq] = *reinterpret_cast<const f32x2*>(&st.ar[kk][r0]);
-          ai[gq] = *reinterpret_cast<const f32x2*>(&st.ai[kk][r0]);
-        }
+        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(&st.ar[kk][r0]);
+        const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(&st.ai[kk][r0]);
+        ar[2 * gq] = x.x;
+        ar[2 * gq + 1] = x.y;
+        ai[2 * gq] = y.x;
+        ai[2 * gq + 1] = y.y;
       }
 #pragma unroll
       for (int j = 0; j < RN; ++j) {
@@ -311,9 +305,8 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
         }
       }
     };
-    constexpr int NST = Cfg::NST;
     if constexpr (Cfg::REGS) {
-      static_assert(!Cfg::REGS || (Cfg::KG == 1 && NST == 2), "one k group, two stages");
+      static_assert(!Cfg::REGS || Cfg::KG == 1, "one k group");
       float4 la[AP], lb[BP];
       const bool va = g.a_tbits > 0 && g.a_tpos[0] == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
       const bool vb = g.b_tbits > 0 && g.b_tpos[0] == 0 && (reinterpret_cast<uintptr_t>(g.B) & 15) == 0;
@@ -362,8 +355,8 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
         __syncthreads();
       }
     } else {
-      // NST - 1 chunks in flight ahead of the one being multiplied; a chunk's stage
-      // was last read before the barrier that lets its copies be issued
+      // one chunk in flight ahead of the one being multiplied; a chunk's stage was last
+      // read before the barrier that lets its copies be issued
       auto next = [&](int c) {   // chunk c's copies, as one group (empty past the end)
         if (c < kc_per) {
           if (c > 0) {
@@ -371,17 +364,16 @@ __device__ __forceinline__ void simt_tile(const GemmArgs& g, int bx, int by, int
             A += sm.kdA[t];
             B += sm.kdB[t];
           }
-          issue(sm.st[c % NST]);
+          issue(sm.st[c & 1]);
         }
         cp_async_commit_group();
       };
-#pragma unroll
-      for (int c = 0; c < NST - 1; ++c) next(c);
+      next(0);
       for (int c = 0; c < kc_per; ++c) {
-        cp_async_wait_groups<NST - 2>();
+        cp_async_wait_groups<0>();
         __syncthreads();
-        next(c + NST - 1);
-        const typename Cfg::Stage& st = sm.st[c % NST];
+        next(c + 1);
+        const typename Cfg::Stage& st = sm.st[c & 1];
         if (TKv == TK) {
 #pragma unroll 8
           for (int kk = 0; kk < TK / Cfg::KG; ++kk) step(st, kk * Cfg::KG + kg);

@@ -95,15 +95,7 @@ __device__ __forceinline__ void amax_update(float* amax_c, float m) {
 }
 __device__ __forceinline__ float cabs_max(float2 v) { return fmaxf(fabsf(v.x), fabsf(v.y)); }
 
-// sum over bits i >= from of bit_{i-from}(x) << pos[i]
-__device__ __forceinline__ int64_t deposit_hi(uint64_t x, const int8_t* pos, int from, int to) {
-  int64_t r = 0;
-  for (int i = from; i < to; ++i)
-    if ((x >> (i - from)) & 1) r += (int64_t)1 << pos[i];
-  return r;
-}
-
-// the same for from = 0, to = n <= N, unrolled (no loop over the argument bank)
+// Sum over bits i < n <= N of bit_i(x) << pos[i], unrolled (no loop over the argument bank)
 template <int N>
 __device__ __forceinline__ int64_t deposit_lo(uint32_t x, const int8_t* pos, int n) {
   int64_t r = 0;

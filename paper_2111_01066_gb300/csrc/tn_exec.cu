@@ -150,11 +150,11 @@ static GemmArgs make_args(const StepDesc& d, int kid, const float2* A, const flo
   return g;
 }
 
-// Launch with programmatic dependent launch where `overlap` (the kernel calls
-// pdl_wait), on clusters of `cluster` CTAs along x where that is above 1.
+// Launch with programmatic dependent launch (the kernel calls pdl_wait), on
+// clusters of `cluster` CTAs along x where that is above 1.
 template <class... KArgs, class... Args>
 static void klaunch(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t s, int cluster,
-                    bool overlap, Args&&... args) {
+                    Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
@@ -162,7 +162,7 @@ static void klaunch(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem,
   cfg.stream = s;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = (unsigned)cluster;
   at[1].val.clusterDim.y = 1;
@@ -174,7 +174,7 @@ static void klaunch(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem,
 
 template <class Cfg>
 static void launch_simt_cfg(const GemmArgs& g, dim3 grid, int split, cudaStream_t s) {
-  klaunch(k_cgemm_simt<Cfg>, grid, SIMT_THREADS, 0, s, split, true, g, split);
+  klaunch(k_cgemm_simt<Cfg>, grid, SIMT_THREADS, 0, s, split, g, split);
 }
 static void launch_simt(const GemmArgs& g, int kid, cudaStream_t s) {
   if (g.n_inst <= 0) return;
@@ -528,7 +528,7 @@ static void launch_prep(const TcArgs& t, cudaStream_t s) {
   const int64_t threads = ((int64_t)t.g.n_inst * t.n_nt * t.n_kc) << (ls_cols + TcPrep<MODE, CM>::LS_KT);
   const int64_t grid = (threads + PREP_THREADS - 1) / PREP_THREADS;
   if (grid > 0x7fffffff) fail(TN_ERR_UNSUPPORTED, "B' image grid too large");
-  klaunch(k_tc_prep_b<MODE, CM>, dim3((unsigned)grid), PREP_THREADS, 0, s, 1, true, t, ls_cols);
+  klaunch(k_tc_prep_b<MODE, CM>, dim3((unsigned)grid), PREP_THREADS, 0, s, 1, t, ls_cols);
 }
 static void launch_prep_kid(const TcArgs& t, int kid, cudaStream_t s) {
   switch (kid) {
@@ -569,9 +569,9 @@ static void launch_tc_kernel(const TcArgs& t, const StepLaunch& L, int grid, cud
   if constexpr (PAIR) {
     // clusters of two CTAs, each pair persistent over the work units
     const int clusters = (int)std::min<int64_t>(t.n_tiles, pair_clusters<MODE, PAIR>());
-    klaunch(k_cgemm_tc<MODE, CM, PAIR, SEG>, dim3(2 * clusters), TC_THREADS, L.smem, s, 2, true, t, L.tma);
+    klaunch(k_cgemm_tc<MODE, CM, PAIR, SEG>, dim3(2 * clusters), TC_THREADS, L.smem, s, 2, t, L.tma);
   } else {
-    klaunch(k_cgemm_tc<MODE, CM, PAIR, SEG>, dim3(grid), TC_THREADS, L.smem, s, 1, true, t, L.tma);
+    klaunch(k_cgemm_tc<MODE, CM, PAIR, SEG>, dim3(grid), TC_THREADS, L.smem, s, 1, t, L.tma);
   }
 }
 template <int MODE, int CM, bool PAIR>
@@ -630,7 +630,7 @@ static void launch_step(StepLaunch& L, uint8_t* ws, int32_t* err, cudaStream_t s
   }
   if (t.n_split > 1) {
     const int rb = (int)std::min<int64_t>((L.c_total + 255) / 256, (int64_t)sm_count() * 8);
-    klaunch(k_split_reduce, dim3(rb), 256, 0, s, 1, true, (const float2*)t.c_part, (int)t.n_split, t.c_part_stride, t.g.C,
+    klaunch(k_split_reduce, dim3(rb), 256, 0, s, 1, (const float2*)t.c_part, (int)t.n_split, t.c_part_stride, t.g.C,
             L.c_total, t.g.amax_c);
   }
 }
@@ -766,7 +766,7 @@ static int simt_multi_tiling(int kid) {
 
 static void launch_simt_multi(const DeviceState& ds, const GroupRun::Multi& m, cudaStream_t s) {
   const uint8_t* buf = ds.group_buf;
-  klaunch(k_cgemm_simt_multi, dim3((unsigned)m.blocks), SIMT_THREADS, 0, s, m.cluster, true,
+  klaunch(k_cgemm_simt_multi, dim3((unsigned)m.blocks), SIMT_THREADS, 0, s, m.cluster,
           reinterpret_cast<const GemmArgs*>(buf + m.args_at), reinterpret_cast<const int32_t*>(buf + m.start_at),
           reinterpret_cast<const int8_t*>(buf + m.tiling_at), reinterpret_cast<const int8_t*>(buf + m.split_at), (int32_t)m.n);
 }
@@ -1209,9 +1209,8 @@ static void launch_leaf_select(Plan& p, cudaStream_t s, int classes, int ls) {
       z1 = nl + i + 1;
     }
   }
-  klaunch(k_leaf_select, dim3((unsigned)std::max(1, std::min(nl, 4096)), 1u << ls), 128, 0, s, 1, true,
-          (const float2*)ds.leaf_data,
-          (const LeafDesc*)ds.leaf_desc, nl, ds.arena, (const ChunkParam*)ds.params, (const unsigned*)ds.counter,
+  klaunch(k_leaf_select, dim3((unsigned)std::max(1, std::min(nl, 4096)), 1u << ls), 128, 0, s, 1,
+          (const float2*)ds.leaf_data, (const LeafDesc*)ds.leaf_desc, nl, ds.arena, (const ChunkParam*)ds.params, (const unsigned*)ds.counter,
           ds.lane_stride, ds.amax, ds.amax_nodes, z0, z1);
 }
 
@@ -1254,7 +1253,7 @@ static void run_chunk(Plan& p, cudaStream_t s, LaunchSet& st, bool new_batch) {
   launch_class(p, s, st, [](int f) { return (f & 1) != 0; });   // slice-dependent steps
   const bool one = ((int64_t)1 << p.root.rank) <= (int64_t)ds.root_blocks * 256;   // amplitude per thread
   klaunch(one ? k_root_sum<1> : k_root_sum<4>, dim3((unsigned)ds.root_blocks, (unsigned)ds.root_groups, 1u << st.ls),
-          256, 0, s, 1, true, (const float2*)ds.arena, p.root, p.log2_batch, ds.root_groups, ds.root_part,
+          256, 0, s, 1, (const float2*)ds.arena, p.root, p.log2_batch, ds.root_groups, ds.root_part,
           (const ChunkParam*)ds.params, ds.counter, ds.root_tickets, ds.lane_stride);
 }
 

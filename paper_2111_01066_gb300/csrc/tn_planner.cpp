@@ -931,13 +931,13 @@ Plan* build_plan(const Network& net, const tn_plan_opts& o) {
       // nor the closed output bits (run once per plan), in post-order; then
       // those that depend on the closed bits only (run once per batch); then
       // the slice-dependent ones (run in every chunk).  Within the last two
-      // classes, the small steps (under 2^20 multiply-adds per chunk: the
-      // CUDA-core kernels) whose subtree holds only such steps, leaves and
-      // results of earlier classes come first, one group per dependency level
-      // (a group's steps are independent and run as one launch); then the
-      // other steps of the class in post-order, where the remaining small
-      // steps are deferred and emitted the same way, level by level, right
-      // before the first step that reads one of them.
+      // classes, the small steps (under 2^20 multiply-adds per chunk; the CUDA
+      // cores also run steps up to 2^25, one launch each) whose subtree holds
+      // only such steps, leaves and results of earlier classes come first, one
+      // group per dependency level (a group's steps are independent and run as
+      // one launch); then the other steps of the class in post-order, where the
+      // remaining small steps are deferred and emitted the same way, level by
+      // level, right before the first step that reads one of them.
       exec.clear();
       exec_group.clear();
       std::vector<char> pend(nm, 0), hoist(nm, 0);

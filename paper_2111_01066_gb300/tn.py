@@ -159,7 +159,6 @@ def _check(status: int) -> None:
 
 def _ints(seq):
     """int32 buffer of a sequence of integers and its address (the buffer must outlive the call)."""
-    n = len(seq)
     if type(seq) is list or type(seq) is tuple:
         try:
             buf = array.array("i", seq)
@@ -167,7 +166,7 @@ def _ints(seq):
         except (TypeError, OverflowError):   # other numbers
             pass
     # one by one, wrapped to 32 bits (array.array would take bytes for the items' memory)
-    buf = array.array("i", _i32(seq)[:n])
+    buf = array.array("i", _i32(seq)[:len(seq)])
     return buf, buf.buffer_info()[0]
 
 
