@@ -367,7 +367,7 @@ __global__ void k_permute_gather(const float2* __restrict__ in, float2* __restri
 // tile.  A persistent block loads its next tile into registers before it writes
 // the current one out.  HBM-bound: what counts is bytes in flight (32 KB a block
 // of 4096 elements, loads of the next tile among them) and the lengths of the
-// runs; a random permutation of 2^27 elements takes 375 us, 5.7 TB/s (557 us,
+// runs; a random permutation of 2^27 elements takes 338 us, 6.4 TB/s (557 us,
 // 3.9 TB/s, with 8 KB tiles, 8-byte accesses and no load in flight across the
 // write-back).
 template <int NT>

@@ -63,14 +63,14 @@ static bool is_simt(int kid) { return kid >= 0 && kid < K_COUNT && !(kid >= K_TC
 
 // CUDA-core tiling of a step, from times on a GB300 (us a launch, log2 m, k, n):
 //  * few outputs (at most two 32x32 tiles per SM): 32x32, whose k groups and
-//    split-K clusters keep the SMs busy -- (7, 10, 6): 8.6 against 148 with 64x64;
-//    (10, 6, 8): 8.1 against 14; with more tiles the larger ones win, (12, 4, 9): 36
-//    against 12 with 128x64;
-//  * n <= 4: 256x4, n <= 16: 128x16 -- (20, 3, 1): 44 with 256x4, 96 with 128x16;
+//    split-K clusters keep the SMs busy -- (7, 10, 6): 8.5 against 149 with 64x64;
+//    (10, 6, 8): 7.8 against 11.5; with more tiles the larger ones win, (12, 4, 9): 32
+//    against 11 with 128x64;
+//  * n <= 4: 256x4, n <= 16: 128x16 -- (20, 3, 1): 45 with 256x4, 96 with 128x16;
 //    (16, 5, 4): 15 with 128x16, 30 with 64x64;
-//  * n = 32 with k >= 64: 32x32 -- (15, 8, 5): 70 against 105 with 64x64;
-//  * otherwise 128x64 where its tiles fill the SMs -- (12, 10, 12): 2513 against
-//    2639 with 64x64 -- and 64x64 where they do not.
+//  * n = 32 with k >= 64: 32x32 -- (15, 8, 5): 70 against 108 with 64x64;
+//  * otherwise 128x64 where its tiles fill the SMs -- (12, 10, 12): 2424 against
+//    2705 with 64x64 -- and 64x64 where they do not.
 static int pick_simt(const StepDesc& d, int64_t n_inst) {
   auto tiles = [&](int tm, int tn) {
     return ((int64_t)1 << (std::max(d.nm, tm) - tm)) * ((int64_t)1 << (std::max(d.nn, tn) - tn)) * n_inst;
@@ -86,9 +86,8 @@ static int pick_simt(const StepDesc& d, int64_t n_inst) {
 
 // CTAs of a cluster that share a tile's k loop (1: no split): as many as leave
 // each at least two k chunks and the grid within two CTAs per SM.  A cluster
-// costs 2-4 us, a 32-k chunk of a lone CTA 1-1.5 (in a chain of launches without
-// overlap (8, 8, 6) took 16 us unsplit, 8.3 over 4 CTAs with 2 chunks each, 9.1 over
-// 8; (7, 10, 6) 52, 17 and 12).
+// costs 2-4 us, a 32-k chunk of a lone CTA 1-1.5 (back to back (8, 8, 6) takes 11.5 us
+// unsplit, 5.6 over 4 CTAs with 2 chunks each, 5.8 over 8; (7, 10, 6) 40, 12.7 and 8.5).
 static int simt_split(const GemmArgs& g, int kid) {
   if (kid != K_SIMT_32x32) return 1;
   // of one lane: the same sums however many chunks run side by side
@@ -362,7 +361,7 @@ static bool pair_pays(int ls_kc, int ls_nt) { return ls_kc > 2 || ls_nt > 1; }
 // Default tile width (log2 complex columns): 128, or 64 or 32 where the tiles are
 // few and that takes less modeled time: narrower tiles spread over more SMs and
 // leave room for more accumulators of a divided k (2048 x 256 x 1024: 36 us with 128
-// columns and four partial results, 23 with 64 columns and four accumulators).
+// columns and four partial results, 25 with 64 columns and four accumulators).
 static int tc_tile(int kid, int nm, int nk, int nn, int64_t n_inst, int64_t c_total, int64_t cap_bytes, bool pairs) {
   const KernelCfg& k = kCfg[kid];
   const int tm = std::min(k.tm, nm), tk = std::min(k.tk, nk), widest = std::min(k.tn, nn);
@@ -724,9 +723,9 @@ static int tc_kernel(int precision, int cmult) {
 // TF32 / BF16X3 / FP16X3 modes, from 2^25 multiply-adds over all instances; the
 // rest (and the FP32 mode) on the CUDA cores, which always form 4M products in
 // FP32.  A tensor-core step has a B' image launch, a pipeline to fill and an
-// accumulator to drain, 7-8 us at least in a chain of launches; at 2^20 the CUDA
-// cores take 3.1 us against 8.0, at 2^22 5-6 against 8-10, at 2^24 7.6-9.2 against
-// 9.1-11.8 (16 columns or fewer: 10-16 against 9-17), at 2^25 11.6 against 9.3.
+// accumulator to drain, about 7 us at least back to back (BF16x3): at 2^20 the CUDA
+// cores take 4.3 us against 7.4, at 2^22 4-5 against 7-9, at 2^24 8-9 against 7-10 (16
+// columns: 8-12 against 7-10), at 2^25 13.1 against 12.5 (16 columns: 21 against 12).
 static int pick_kernel(int precision, int cmult, const StepDesc& d, int64_t n_inst) {
   if (precision == TN_PREC_FP32) return pick_simt(d, n_inst);
   const double macs = std::ldexp((double)n_inst, d.nm + d.nk + d.nn);
@@ -1977,8 +1976,8 @@ extern "C" tn_status tn_permute(const float* in, float* out, int32_t rank, const
     k_permute_gather<<<blocks, 256, 0, (cudaStream_t)stream>>>(reinterpret_cast<const float2*>(in),
                                                                reinterpret_cast<float2*>(out), rank, pa, total);
   } else {
-    // tiles of 2^12 elements where they give every SM at least four (5.2 TB/s at
-    // rank 24, 5.7 from 28 on; 3.2 and 3.9 with 2^10), else 2^10 (rank 20: 1.5
+    // tiles of 2^12 elements where they give every SM at least four (5.4 TB/s at
+    // rank 24, 6.0-6.4 from 26 on; 3.2 and 3.9 with 2^10), else 2^10 (rank 20: 2.5
     // TB/s, its 8 MB a few microseconds of latency)
     const int nt = rank >= 12 && (batch << (rank - 12)) >= 4 * (int64_t)sm_count() ? 12 : 10;
     permute_tile(pa, rank, perm, nt);
